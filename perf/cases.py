@@ -1,0 +1,509 @@
+"""Measured cases of the library: what its users have it do, through nebem.py's public calls.
+
+A user has a detector cell (a THGEM unit cell with its periodic copies, or a closed
+conductor) and
+  * solves it for the charge densities, in FP64 or in mixed precision;
+  * asks for potential and field at points: the few hundred points of a drift line's next
+    steps, a map of some ten thousand points, a volume of some hundred thousand;
+  * factors a dense matrix of its own and solves with it;
+  * sums the space charge of a carrier cloud, and lets the cloud drift in its own field;
+  * makes weighting-field maps of the readout electrodes and looks them up;
+  * serves many small field queries at once.
+Each kind of case below stands for one of these; sizes are those of the repository's tests
+and benchmark (meshes of 384 to 10,000 elements, 5 x 5 copies) and the range between them.
+"""
+import math
+
+import numpy as np
+import torch
+
+from paper_2606_24154_gb300 import inputs as I
+from paper_2606_24154_gb300 import nebem as N
+
+PREC = {"fp64": N.NEBEM_FP64, "mixed": N.NEBEM_MIXED}
+EPS0 = 8.8541878128e-12
+KE = 1.0 / (4.0 * math.pi * EPS0)
+
+
+# ----------------------------------------------------------------------------- the cases
+def listed():
+    full = {"n_phi": 96, "n_r": 9, "n_zc": 2, "n_zf": 18, "n_plane": 9}    # 9,996 elements, the benchmark's cell
+    half = {"n_phi": 60, "n_r": 7, "n_zc": 2, "n_zf": 10, "n_plane": 6}    # 4,632 elements
+    small = {"n_phi": 36, "n_r": 5, "n_zc": 1, "n_zf": 8, "n_plane": 5}    # 2,100 elements
+    tiny = {"n_phi": 24, "n_r": 3, "n_zc": 1, "n_zf": 4, "n_plane": 3}     # 828 elements, the tests' cell
+    return [
+        # the capacitance of a cube (384 elements) and the field on a grid around it, all in
+        # FP64 from numpy arrays: the smallest whole call, where launches and latency count
+        {"name": "cube_solve_eval_f64", "kind": "cube", "edge_cells": 8, "grid": "20x20x25"},
+        # the next steps of a few drift lines: an odd handful of points, FP32 tiers with refinement
+        {"name": "eval_mixed_257", "kind": "eval", **full, "points": 257, "precision": "mixed", "with_err": False},
+        # a field map's points, with their error estimates
+        {"name": "eval_mixed_20011", "kind": "eval", **full, "points": 20011, "precision": "mixed", "with_err": True},
+        # a filled volume, the shape of the benchmark's headline
+        {"name": "eval_mixed_200k", "kind": "eval", **full, "points": 200000, "precision": "mixed",
+         "with_err": False},
+        # a coarser cell in plain FP64: a check of a sample of points
+        {"name": "eval_f64_1500", "kind": "eval", **half, "points": 1500, "precision": "fp64", "with_err": False},
+        # a new geometry solved from its element records: fill, factorisation, substitution
+        {"name": "solve_f64_4632", "kind": "solve", **half, "precision": "fp64"},
+        {"name": "solve_mixed_9996", "kind": "solve", **full, "precision": "mixed"},
+        # a caller's own dense system, factored and solved on the device in FP64
+        {"name": "lu_f64_6145", "kind": "lu", "n": 6145},
+        # the direct sum of a carrier cloud at its own carriers, self excluded
+        {"name": "space_charge_100k", "kind": "cloud", **tiny, "carriers": 100000},
+        # self-consistent drift steps of a cloud in a solved cell
+        {"name": "drift_steps_20k", "kind": "drift", **small, "carriers": 20000, "steps": 3},
+        # weighting fields of every electrode as maps, then lookups along tracks
+        {"name": "weighting_maps", "kind": "maps", **small, "readouts": 4, "grid": "17x17x41", "points": 500000},
+        # a burst of small queries to three resident cells
+        {"name": "serve_burst_12", "kind": "serve", "requests": 12, "lo": 20, "hi": 1500},
+    ]
+
+
+def _spread(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def _mesh(rng, most):
+    """A THGEM mesh of up to `most` elements, element counts spread over their logarithm."""
+    while True:
+        want = _spread(rng, 500, most)
+        m = {"n_phi": 12 * rng.randint(1, 8), "n_r": rng.randint(2, 9), "n_zc": rng.randint(1, 2),
+             "n_zf": rng.randint(3, 18), "n_plane": rng.randint(3, 9)}
+        if 0.8 * want <= _elements(m) <= min(most, 1.25 * want):
+            return m
+
+
+def draw(rng):
+    kind = rng.choice(["eval", "eval", "eval", "solve", "solve", "lu", "cloud", "drift", "maps", "serve", "cube"])
+    if kind == "cube":
+        g = rng.randint(7, 21), rng.randint(7, 21), rng.randint(7, 25)
+        return {"kind": kind, "edge_cells": rng.randint(3, 12), "grid": "%dx%dx%d" % g}
+    if kind == "eval":
+        prec = rng.choice(["mixed", "mixed", "fp64"])
+        m = _mesh(rng, 10000 if prec == "mixed" else 4632)
+        pairs = 9996 * 200000 if prec == "mixed" else 4632 * 1500
+        return {"kind": kind, **m, "points": _spread(rng, 60, min(200000, pairs // _elements(m))), "precision": prec,
+                "with_err": prec == "mixed" and rng.random() < 0.5}
+    if kind == "solve":
+        prec = rng.choice(["mixed", "fp64"])
+        return {"kind": kind, **_mesh(rng, 9996 if prec == "mixed" else 4632), "precision": prec}
+    if kind == "lu":
+        return {"kind": kind, "n": _spread(rng, 150, 6145)}
+    if kind == "cloud":
+        return {"kind": kind, **_mesh(rng, 1500), "carriers": _spread(rng, 2000, 100000)}
+    if kind == "drift":
+        return {"kind": kind, **_mesh(rng, 2100), "carriers": _spread(rng, 1000, 20000), "steps": rng.randint(1, 3)}
+    if kind == "maps":
+        g = rng.randint(5, 17), rng.randint(5, 17), rng.randint(9, 41)
+        return {"kind": kind, **_mesh(rng, 2100), "readouts": rng.randint(1, 4), "grid": "%dx%dx%d" % g,
+                "points": _spread(rng, 5000, 500000)}
+    return {"kind": kind, "requests": rng.randint(4, 12), "lo": 20, "hi": _spread(rng, 200, 1500)}
+
+
+def _elements(c):
+    return c["n_phi"] * (8 * c["n_r"] + 2 * c["n_zc"] + c["n_zf"]) + 12 * c["n_plane"] ** 2
+
+
+# ------------------------------------------------------------------------------- inputs
+def _geometry(case, gen):
+    """The case's THGEM cell; hole, foil and voltages vary from seed to seed."""
+    spec = I.PlateSpec(hole_d=1e-3 * gen.uniform(0.45, 0.55), fr4=1e-3 * gen.uniform(0.45, 0.55),
+                       n_phi=case["n_phi"], n_r=case["n_r"], n_zc=case["n_zc"], n_zf=case["n_zf"])
+    v = gen.uniform(0.9, 1.1, 4)
+    return I.thgem(spec, n_plane=case["n_plane"], v_top=-500.0 * v[0], v_bot=500.0 * v[1], v_drift=-1100.0 * v[2],
+                   v_ind=1700.0 * v[3])
+
+
+def _shape(case):
+    return tuple(int(k) for k in case["grid"].split("x"))
+
+
+def _serving(case, gen):
+    geoms = [I.cube(edge=0.01 * gen.uniform(0.9, 1.1), n_per_edge=8),
+             _geometry({"n_phi": 24, "n_r": 3, "n_zc": 1, "n_zf": 4, "n_plane": 3}, gen),
+             _geometry({"n_phi": 36, "n_r": 5, "n_zc": 1, "n_zf": 8, "n_plane": 5}, gen)]
+    # the trace's sizes and cells belong to the case, the points to the seed
+    trace = np.random.Generator(np.random.PCG64([20261203, case["requests"], case["hi"]]))
+    _, sizes, geo = I.serving_trace(case["requests"], trace, lo=case["lo"], hi=case["hi"])
+    return geoms, [(int(k), I.cell_points(geoms[k], int(m), gen)) for k, m in zip(geo, sizes)]
+
+
+def _inputs(case, seed):
+    """Everything a case's run starts from, as numpy arrays and geometries, from the seed."""
+    gen = np.random.Generator(np.random.PCG64([20261203, int(seed)]))
+    k = case["kind"]
+    if k == "cube":
+        g = I.cube(edge=0.01 * gen.uniform(0.9, 1.1), n_per_edge=case["edge_cells"], voltage=gen.uniform(0.5, 2.0))
+        return {"geometry": g, "points": I.cube_grid_points(0.01, _shape(case)) * gen.uniform(0.97, 0.99)}
+    if k == "serve":
+        geoms, reqs = _serving(case, gen)
+        return {"geometries": geoms, "requests": reqs}
+    if k == "lu":
+        return {}
+    g = _geometry(case, gen)
+    if k == "eval":
+        return {"geometry": g, "points": I.cell_points(g, case["points"], gen)}
+    if k in ("cloud", "drift"):
+        pos, q = I.carrier_cloud(g, case["carriers"], gen, center=(0.0, 0.0, gen.uniform(-5e-5, 5e-5)))
+        # carriers are macro charges of 1 to 4 elementary charges
+        return {"geometry": g, "pos": pos, "q": q * gen.integers(1, 5, q.shape[0])}
+    if k == "maps":
+        nx, ny, nz = _shape(case)
+        # the cell's box, a hair inside the planes and off the mesh's own lines
+        axes = (np.linspace(-0.4931e-3, 0.4957e-3, nx), np.linspace(-0.5679e-3, 0.5701e-3, ny),
+                np.linspace(g.z_range[0] * 0.9973, g.z_range[1] * 0.9959, nz))
+        return {"geometry": g, "axes": axes, "points": I.cell_points(g, case["points"], gen)}
+    return {"geometry": g}
+
+
+def _matrix(case, seed):
+    gen = torch.Generator(device="cuda").manual_seed(int(seed))
+    n = case["n"]
+    a = torch.randn((n, n), dtype=torch.float64, device="cuda", generator=gen)
+    return a, torch.randn(n, dtype=torch.float64, device="cuda", generator=gen)
+
+
+def _solved(g, precision=N.NEBEM_MIXED):
+    ctx = N.Context().set_geometry(g)
+    ctx.solve(precision)
+    return ctx
+
+
+def prepare(case, seed):
+    k, s = case["kind"], {"case": case, "stream": torch.cuda.Stream()}
+    s.update(_inputs(case, seed))
+    f64 = dict(dtype=torch.float64, device="cuda")
+    if k == "eval":
+        s["ctx"] = _solved(s["geometry"])
+        s["pts"] = torch.from_numpy(s["points"]).cuda()
+        n = case["points"]
+        s["phi"], s["E"], s["err"] = torch.empty(n, **f64), torch.empty((n, 3), **f64), torch.empty((n, 2), **f64)
+    elif k in ("solve", "cube"):
+        s["ctx"] = N.Context()
+    elif k == "lu":
+        s["ctx"] = N.Context()
+        s["A"], s["b"] = _matrix(case, seed)
+        s["LU"], s["x"] = torch.empty_like(s["A"]), torch.empty_like(s["b"])
+        s["piv"] = torch.empty(case["n"], dtype=torch.int32, device="cuda")
+    elif k == "cloud":
+        s["ctx"] = N.Context().set_geometry(s["geometry"])
+        N.nebem_space_charge(s["ctx"].h, s["pos"], s["q"], 1e-6)
+    elif k == "drift":
+        s["ctx"] = _solved(s["geometry"])
+    elif k == "maps":
+        s["ctx"] = _solved(s["geometry"])
+        s["pts"] = torch.from_numpy(s["points"]).cuda()
+        n, r = case["points"], case["readouts"]
+        s["phi"], s["E"] = torch.empty((r, n), **f64), torch.empty((r, n, 3), **f64)
+    elif k == "serve":
+        s["ctxs"] = [_solved(g) for g in s["geometries"]]
+        s["server"] = N.nebem_server_create([c.h for c in s["ctxs"]])
+        s["outs"] = [(np.empty(p.shape[0]), np.empty((p.shape[0], 3))) for _, p in s["requests"]]
+        s["guard"] = _Server(s["server"])
+    torch.cuda.synchronize()
+    return s
+
+
+class _Server:
+    """Destroys the server with the state that holds it, before the state's contexts."""
+
+    def __init__(self, handle):
+        self.handle = handle
+
+    def __del__(self):
+        N.nebem_server_destroy(self.handle)
+
+
+# ---------------------------------------------------------------------------------- run
+def run(s):
+    case, k = s["case"], s["case"]["kind"]
+    stream = s["stream"].cuda_stream
+    if k == "eval":
+        args = s["ctx"].h, s["pts"].data_ptr(), case["points"], s["phi"].data_ptr(), s["E"].data_ptr()
+        if case["with_err"]:
+            N.nebem_eval_device_err(*args, s["err"].data_ptr(), stream)
+            return {"phi": s["phi"], "E": s["E"], "err": s["err"]}
+        N.nebem_eval_device(*args, PREC[case["precision"]], stream)
+        return {"phi": s["phi"], "E": s["E"]}
+    if k == "solve":
+        sigma, _, _ = s["ctx"].set_geometry(s["geometry"]).solve(PREC[case["precision"]])
+        return {"sigma": sigma}
+    if k == "cube":
+        sigma, _, _ = s["ctx"].set_geometry(s["geometry"]).solve(N.NEBEM_FP64)
+        phi, E = s["ctx"].eval(s["points"], N.NEBEM_FP64)
+        return {"sigma": sigma, "phi": phi, "E": E}
+    if k == "lu":
+        with torch.cuda.stream(s["stream"]):
+            s["LU"].copy_(s["A"])  # the caller keeps its matrix
+            s["x"].copy_(s["b"])
+        N.nebem_lu_factor_device(s["ctx"].h, s["LU"].data_ptr(), case["n"], s["piv"].data_ptr(), stream)
+        N.nebem_lu_solve_device(s["ctx"].h, s["LU"].data_ptr(), case["n"], s["piv"].data_ptr(), s["x"].data_ptr(),
+                                stream)
+        return {"LU": s["LU"], "piv": s["piv"], "x": s["x"]}
+    if k == "cloud":
+        phi, E = N.nebem_space_charge_eval(s["ctx"].h, s["pos"], N.NEBEM_MIXED, exclude_self=True)
+        return {"phi": phi, "E": E}
+    if k == "drift":
+        ctx = s["ctx"]
+        N.nebem_space_charge(ctx.h, s["pos"], s["q"], 1e-6)
+        pos = N.nebem_step(ctx.h, case["steps"], 1e-4, 1e-9, N.NEBEM_MIXED, case["carriers"])
+        return {"move": pos - s["pos"]}
+    if k == "maps":
+        ctx, n = s["ctx"], case["points"]
+        maps, _ = N.nebem_weighting_fastvol_build(ctx.h, np.arange(case["readouts"]), *s["axes"], N.NEBEM_MIXED)
+        for j, m in enumerate(maps):
+            m.eval_device(s["pts"].data_ptr(), n, s["phi"][j].data_ptr(), s["E"][j].data_ptr(), stream)
+        s["stream"].synchronize()  # a map is freed only after its lookups
+        for m in maps:
+            m.close()
+        return {"phi": s["phi"], "E": s["E"]}
+    ids = [N.nebem_server_submit(s["server"], g, p, o[0], o[1], N.NEBEM_MIXED)
+           for (g, p), o in zip(s["requests"], s["outs"])]
+    for i in ids:
+        N.nebem_server_wait(s["server"], i)
+    return {"phi": np.concatenate([o[0] for o in s["outs"]]), "E": np.concatenate([o[1] for o in s["outs"]])}
+
+
+# --------------------------------------------------------------------------------- work
+# Floating-point operations that one pair cannot do without: an element seen from a point
+# is four distances to its corners, four logarithms and a solid angle (phi and field); a
+# point charge is a difference, a square, an inverse root and four sums.
+PAIR_FLOPS, CHARGE_FLOPS = 100, 20
+
+
+def work(case):
+    k = case["kind"]
+    if k == "lu":
+        n = case["n"]
+        return {"bytes": 8 * (2 * n * n + 3 * n), "flops": 2 * n ** 3 / 3 + 2 * n * n}
+    if k == "cube":
+        n, p = 6 * case["edge_cells"] ** 2, math.prod(_shape(case))
+        return {"bytes": 128 * n + 8 * n + 56 * p, "flops": PAIR_FLOPS * n * (n + p) + 2 * n ** 3 / 3}
+    if k == "serve":
+        points = case["requests"] * (case["hi"] - case["lo"]) / math.log(case["hi"] / case["lo"])
+        n_pairs = (384 + 25 * 828 + 25 * 2100) / 3
+        return {"bytes": 56 * points + 128 * 3312, "flops": PAIR_FLOPS * points * n_pairs}
+    n = _elements(case)
+    if k == "eval":
+        p = case["points"]
+        return {"bytes": 136 * n + (72 if case["with_err"] else 56) * p, "flops": PAIR_FLOPS * 25 * n * p}
+    if k == "solve":
+        return {"bytes": 136 * n, "flops": PAIR_FLOPS * 25 * n * n + 2 * n ** 3 / 3}
+    if k == "cloud":
+        m = case["carriers"]
+        return {"bytes": 64 * m, "flops": CHARGE_FLOPS * m * m}
+    if k == "drift":
+        m = case["carriers"]
+        per = CHARGE_FLOPS * m * (m + n) + PAIR_FLOPS * 25 * n * m + 2 * n * n
+        return {"bytes": 56 * m + 136 * n, "flops": case["steps"] * per}
+    nodes = math.prod(_shape(case))
+    r, p = case["readouts"], case["points"]
+    return {"bytes": 136 * n + p * (24 + 32 * r), "flops": r * (PAIR_FLOPS * 25 * n * nodes + 56 * p + 2 * n * n)}
+
+
+# -------------------------------------------------------------------------------- exact
+# The closed forms in 64 bits, written with torch: potential and field of a flat polygon
+# from its corners (edges: artanh of length over the sum of the end distances; solid angle:
+# one arctangent per fan triangle).
+def _frame(g):
+    v = torch.tensor(np.array(g.elements["v"]), dtype=torch.float64, device="cuda")
+    tri = torch.tensor(np.array(g.elements["kind"]) == I.KIND_TRI, device="cuda")
+    v = torch.where(tri[:, None, None] & (torch.arange(4, device="cuda") == 3)[None, :, None], v[:, 2:3], v)
+    n = torch.linalg.cross(v[:, 1] - v[:, 0], v[:, 2] - v[:, 0])
+    c = torch.where(tri[:, None], v[:, :3].mean(1), v.mean(1))
+    return v, n / n.norm(dim=1, keepdim=True), c
+
+
+def _images(g):
+    if g.lattice is None:
+        return torch.zeros((1, 3), dtype=torch.float64, device="cuda")
+    r = range(g.img_lo, g.img_hi + 1)
+    t = [i * g.lattice[0] + j * g.lattice[1] for i in r for j in r]
+    return torch.tensor(np.array(t), dtype=torch.float64, device="cuda")
+
+
+def _dot(a, b):
+    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]
+
+
+def _cross(a, b):
+    return [a[1] * b[2] - a[2] * b[1], a[2] * b[0] - a[0] * b[2], a[0] * b[1] - a[1] * b[0]]
+
+
+def _influence(v, n, P, own=None):
+    """phi' and E' of elements v [m, 4, 3] (normals n) at points P [p, 3]: each [p, m].  own: True where
+    the point is the element's own centroid."""
+    corner = [[v[None, :, i, a] - P[:, None, a] for a in range(3)] for i in range(4)]
+    R = [torch.sqrt(_dot(c, c)) for c in corner]
+    nn = [n[None, :, a] for a in range(3)]
+    h = -_dot(corner[0], nn)  # height of the point over the element's plane
+    phi, Ex = 0.0, [0.0, 0.0, 0.0]
+    for i in range(4):
+        j = (i + 1) % 4
+        e = [v[None, :, j, a] - v[None, :, i, a] for a in range(3)]
+        length = torch.sqrt(_dot(e, e))
+        live = length > 0
+        safe = torch.where(live, length, 1.0)
+        t = [x / safe for x in e]
+        m = _cross(t, nn)  # outward normal of the edge, in the plane
+        L = torch.where(live, 2 * torch.atanh(torch.clamp(length / (R[i] + R[j]), max=1 - 1e-16)), 0.0)
+        phi = phi + _dot(corner[i], m) * L
+        Ex = [x + y * L for x, y in zip(Ex, m)]
+    om = 0.0
+    for i, j in ((1, 2), (2, 3)):
+        a, b, c = corner[0], corner[i], corner[j]
+        # the doubled area times the height: no cancellation in the far field
+        u = [v[None, :, i, q] - v[None, :, 0, q] for q in range(3)]
+        w = [v[None, :, j, q] - v[None, :, 0, q] for q in range(3)]
+        num = _dot(_cross(u, w), nn) * h
+        den = R[0] * R[i] * R[j] + _dot(a, b) * R[j] + _dot(a, c) * R[i] + _dot(b, c) * R[0]
+        om = om + 2 * torch.atan2(num, den)
+    if own is not None:
+        om = torch.where(own, 0.0, om)
+    phi = phi - h * om
+    return phi, [x + om * y for x, y in zip(Ex, nn)]
+
+
+def _field(g, sigma, P):
+    """phi [p, k], E [p, 3, k] of densities sigma [n, k] with all copies."""
+    v, n, _ = _frame(g)
+    phi = torch.zeros((P.shape[0], sigma.shape[1]), dtype=torch.float64, device="cuda")
+    E = torch.zeros((P.shape[0], 3, sigma.shape[1]), dtype=torch.float64, device="cuda")
+    step = max(1, 30_000_000 // v.shape[0])
+    for t in _images(g):
+        for a in range(0, P.shape[0], step):
+            f, e = _influence(v, n, P[a:a + step] - t)
+            phi[a:a + step] += KE * (f @ sigma)
+            for q in range(3):
+                E[a:a + step, q] += KE * (e[q] @ sigma)
+    return phi, E
+
+
+def _influence_matrix(g):
+    v, n, c = _frame(g)
+    bc = torch.tensor(np.array(g.elements["bc"]), device="cuda") == I.BC_CONDUCTOR
+    m = v.shape[0]
+    K = torch.zeros((m, m), dtype=torch.float64, device="cuda")
+    step = max(1, 30_000_000 // m)
+    for t in _images(g):
+        base = float(t.abs().max()) == 0.0
+        for a in range(0, m, step):
+            P = c[a:a + step] - t
+            own = (torch.arange(a, a + P.shape[0], device="cuda")[:, None] == torch.arange(m, device="cuda")) if base \
+                else None
+            f, e = _influence(v, n, P, own)
+            normal = sum(n[a:a + step, q, None] * e[q] for q in range(3))
+            K[a:a + step] += KE * torch.where(bc[a:a + step, None], f, normal)
+    ea, eb = (torch.tensor(np.array(g.elements[q]), device="cuda") for q in ("eps_a", "eps_b"))
+    K.diagonal().add_(torch.where(bc, 0.0, (ea + eb) / (2 * EPS0 * torch.where(bc, 1.0, eb - ea))))
+    return K, bc
+
+
+def _densities(g, rhs=None):
+    K, bc = _influence_matrix(g)
+    if rhs is None:
+        cond = torch.tensor(np.array(g.elements["conductor"]), device="cuda").clamp(min=0).long()
+        rhs = torch.where(bc, torch.tensor(g.voltages, dtype=torch.float64, device="cuda")[cond], 0.0)[:, None]
+    return torch.linalg.solve(K, rhs)
+
+
+def _unit_readouts(g, k):
+    cond = torch.tensor(np.array(g.elements["conductor"]), device="cuda")
+    bc = torch.tensor(np.array(g.elements["bc"]), device="cuda") == I.BC_CONDUCTOR
+    return torch.stack([torch.where(bc & (cond == j), 1.0, 0.0) for j in range(k)], 1).double()
+
+
+def _charges(P, pos, q, own):
+    phi = torch.empty(P.shape[0], dtype=torch.float64, device="cuda")
+    E = torch.empty((P.shape[0], 3), dtype=torch.float64, device="cuda")
+    step = max(1, 100_000_000 // pos.shape[0])
+    for a in range(0, P.shape[0], step):
+        d = [P[a:a + step, None, i] - pos[None, :, i] for i in range(3)]
+        w = q[None] / torch.sqrt(_dot(d, d) + 1e-12)
+        r2 = 1.0 / (_dot(d, d) + 1e-12)
+        if own:
+            i = torch.arange(w.shape[0], device="cuda")
+            w[i, a + i] = 0.0
+        phi[a:a + step] = KE * w.sum(1)
+        for c in range(3):
+            E[a:a + step, c] = KE * (w * r2 * d[c]).sum(1)
+    return phi, E
+
+
+def _lookup(axes, values, P):
+    """Trilinear interpolation of values [nx, ny, nz, ...], points clamped to the box."""
+    at, fr = [], []
+    for i, ax in enumerate(axes):
+        x = torch.tensor(ax, dtype=torch.float64, device="cuda")
+        p = P[:, i].clamp(x[0], x[-1])
+        c = (torch.searchsorted(x, p, right=True) - 1).clamp(0, len(ax) - 2)
+        at.append(c)
+        fr.append((p - x[c]) / (x[c + 1] - x[c]))
+    out = 0.0
+    for corner in range(8):
+        b = [(corner >> i) & 1 for i in range(3)]
+        w = math.prod(f if q else 1 - f for f, q in zip(fr, b))
+        v = values[at[0] + b[0], at[1] + b[1], at[2] + b[2]]
+        out = out + w.reshape(-1, *[1] * (v.dim() - 1)) * v
+    return out
+
+
+def exact(case, seed):
+    k = case["kind"]
+    if k == "lu":
+        a, b = _matrix(case, seed)
+        # the library's matrix is column-major: its A is this tensor's transpose
+        lu, piv = torch.linalg.lu_factor(a.T)
+        x = torch.linalg.lu_solve(lu, piv, b[:, None])[:, 0]
+        return {"LU": lu.T.contiguous(), "piv": None, "x": x}
+    if k == "cloud" and case["carriers"] > 150000 or k == "eval" and _elements(case) * case["points"] > 4e8:
+        return None  # over about 20 seconds in plain torch
+    s = _inputs(case, seed)
+    if k == "cube":
+        sigma = _densities(s["geometry"])
+        phi, E = _field(s["geometry"], sigma, torch.from_numpy(s["points"]).cuda())
+        return {"sigma": sigma[:, 0], "phi": phi[:, 0], "E": E[:, :, 0].contiguous()}
+    if k == "serve":
+        fields = [_field(s["geometries"][i], _densities(s["geometries"][i]),
+                         torch.cat([torch.from_numpy(p) for q, p in s["requests"] if q == i] or
+                                   [torch.zeros((0, 3), dtype=torch.float64)]).cuda()) for i in range(3)]
+        at, phi, E = [0, 0, 0], [], []
+        for i, p in s["requests"]:
+            a, at[i] = at[i], at[i] + p.shape[0]
+            phi.append(fields[i][0][a:at[i], 0])
+            E.append(fields[i][1][a:at[i], :, 0])
+        return {"phi": torch.cat(phi), "E": torch.cat(E)}
+    g = s["geometry"]
+    if k == "solve":
+        return {"sigma": _densities(g)[:, 0]}
+    if k == "eval":
+        phi, E = _field(g, _densities(g), torch.from_numpy(s["points"]).cuda())
+        # an error estimate is the library's own statement
+        return {"phi": phi[:, 0], "E": E[:, :, 0].contiguous(), **({"err": None} if case["with_err"] else {})}
+    if k == "cloud":
+        pos, q = torch.from_numpy(s["pos"]).cuda(), torch.from_numpy(s["q"]).cuda()
+        phi, E = _charges(pos, pos, q, True)
+        return {"phi": phi, "E": E}
+    if k == "drift":
+        pos, q = torch.from_numpy(s["pos"]).cuda(), torch.from_numpy(s["q"]).cuda()
+        K, bc = _influence_matrix(g)
+        cond = torch.tensor(np.array(g.elements["conductor"]), device="cuda").clamp(min=0).long()
+        V = torch.tensor(g.voltages, dtype=torch.float64, device="cuda")[cond]
+        _, n, c = _frame(g)
+        lu, piv = torch.linalg.lu_factor(K)
+        start = pos
+        for _ in range(case["steps"]):
+            f, e = _charges(c, pos, q, False)
+            rhs = torch.where(bc, V - f, -(n * e).sum(1))
+            sigma = torch.linalg.lu_solve(lu, piv, rhs[:, None])
+            E = _field(g, sigma, pos)[1][:, :, 0] + _charges(pos, pos, q, True)[1]
+            pos = pos + 1e-4 * 1e-9 * torch.sign(q)[:, None] * E
+        return {"move": pos - start}
+    nodes = torch.cartesian_prod(*[torch.tensor(a, dtype=torch.float64, device="cuda") for a in s["axes"]])
+    phi, E = _field(g, _densities(g, _unit_readouts(g, case["readouts"])), nodes)
+    P = torch.from_numpy(s["points"]).cuda()
+    shape = _shape(case)
+    f = _lookup(s["axes"], phi.reshape(*shape, -1), P)
+    e = _lookup(s["axes"], E.reshape(*shape, 3, -1), P)
+    return {"phi": f.T.contiguous(), "E": e.permute(2, 0, 1).contiguous()}
