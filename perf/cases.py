@@ -36,14 +36,13 @@ def listed():
         # FP64 from numpy arrays: the smallest whole call, where launches and latency count
         {"name": "cube_solve_eval_f64", "kind": "cube", "edge_cells": 8, "grid": "20x20x25"},
         # the next steps of a few drift lines: an odd handful of points, FP32 tiers with refinement
-        {"name": "eval_mixed_257", "kind": "eval", **full, "points": 257, "precision": "mixed", "with_err": False},
-        # a field map's points, with their error estimates
-        {"name": "eval_mixed_20011", "kind": "eval", **full, "points": 20011, "precision": "mixed", "with_err": True},
+        {"name": "eval_mixed_257", "kind": "eval", **full, "points": 257, "precision": "mixed"},
+        # a field map's points
+        {"name": "eval_mixed_20011", "kind": "eval", **full, "points": 20011, "precision": "mixed"},
         # a filled volume, the shape of the benchmark's headline
-        {"name": "eval_mixed_200k", "kind": "eval", **full, "points": 200000, "precision": "mixed",
-         "with_err": False},
+        {"name": "eval_mixed_200k", "kind": "eval", **full, "points": 200000, "precision": "mixed"},
         # a coarser cell in plain FP64: a check of a sample of points
-        {"name": "eval_f64_1500", "kind": "eval", **half, "points": 1500, "precision": "fp64", "with_err": False},
+        {"name": "eval_f64_1500", "kind": "eval", **half, "points": 1500, "precision": "fp64"},
         # a new geometry solved from its element records: fill, factorisation, substitution
         {"name": "solve_f64_4632", "kind": "solve", **half, "precision": "fp64"},
         {"name": "solve_mixed_9996", "kind": "solve", **full, "precision": "mixed"},
@@ -83,8 +82,7 @@ def draw(rng):
         prec = rng.choice(["mixed", "mixed", "fp64"])
         m = _mesh(rng, 10000 if prec == "mixed" else 4632)
         pairs = 9996 * 200000 if prec == "mixed" else 4632 * 1500
-        return {"kind": kind, **m, "points": _spread(rng, 60, min(200000, pairs // _elements(m))), "precision": prec,
-                "with_err": prec == "mixed" and rng.random() < 0.5}
+        return {"kind": kind, **m, "points": _spread(rng, 60, min(200000, pairs // _elements(m))), "precision": prec}
     if kind == "solve":
         prec = rng.choice(["mixed", "fp64"])
         return {"kind": kind, **_mesh(rng, 9996 if prec == "mixed" else 4632), "precision": prec}
@@ -178,7 +176,7 @@ def prepare(case, seed):
         s["ctx"] = _solved(s["geometry"])
         s["pts"] = torch.from_numpy(s["points"]).cuda()
         n = case["points"]
-        s["phi"], s["E"], s["err"] = torch.empty(n, **f64), torch.empty((n, 3), **f64), torch.empty((n, 2), **f64)
+        s["phi"], s["E"] = torch.empty(n, **f64), torch.empty((n, 3), **f64)
     elif k in ("solve", "cube"):
         s["ctx"] = N.Context()
     elif k == "lu":
@@ -220,11 +218,8 @@ def run(s):
     case, k = s["case"], s["case"]["kind"]
     stream = s["stream"].cuda_stream
     if k == "eval":
-        args = s["ctx"].h, s["pts"].data_ptr(), case["points"], s["phi"].data_ptr(), s["E"].data_ptr()
-        if case["with_err"]:
-            N.nebem_eval_device_err(*args, s["err"].data_ptr(), stream)
-            return {"phi": s["phi"], "E": s["E"], "err": s["err"]}
-        N.nebem_eval_device(*args, PREC[case["precision"]], stream)
+        N.nebem_eval_device(s["ctx"].h, s["pts"].data_ptr(), case["points"], s["phi"].data_ptr(), s["E"].data_ptr(),
+                            PREC[case["precision"]], stream)
         return {"phi": s["phi"], "E": s["E"]}
     if k == "solve":
         sigma, _, _ = s["ctx"].set_geometry(s["geometry"]).solve(PREC[case["precision"]])
@@ -287,7 +282,7 @@ def work(case):
     n = _elements(case)
     if k == "eval":
         p = case["points"]
-        return {"bytes": 136 * n + (72 if case["with_err"] else 56) * p, "flops": PAIR_FLOPS * 25 * n * p}
+        return {"bytes": 136 * n + 56 * p, "flops": PAIR_FLOPS * 25 * n * p}
     if k == "solve":
         return {"bytes": 136 * n, "flops": PAIR_FLOPS * 25 * n * n + 2 * n ** 3 / 3}
     if k == "cloud":
@@ -479,8 +474,7 @@ def exact(case, seed):
         return {"sigma": _densities(g)[:, 0]}
     if k == "eval":
         phi, E = _field(g, _densities(g), torch.from_numpy(s["points"]).cuda())
-        # an error estimate is the library's own statement
-        return {"phi": phi[:, 0], "E": E[:, :, 0].contiguous(), **({"err": None} if case["with_err"] else {})}
+        return {"phi": phi[:, 0], "E": E[:, :, 0].contiguous()}
     if k == "cloud":
         pos, q = torch.from_numpy(s["pos"]).cuda(), torch.from_numpy(s["q"]).cuda()
         phi, E = _charges(pos, pos, q, True)
