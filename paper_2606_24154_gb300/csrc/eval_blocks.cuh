@@ -53,7 +53,6 @@ constexpr int kEvalThreads = 128;  // threads per block (one target each)
 constexpr int kTileMax = 16;       // elements per shared-memory tile (mixed)
 constexpr int kCjkMax = 512;       // (element, image) centres per tile (mixed)
 constexpr int kGroup = 8;          // elements per FP32 partial sum (mixed)
-constexpr int kTile64 = 32;        // elements per shared-memory tile (FP64)
 constexpr int kChunkEl = 1024;     // elements per chunk of the far sums (multiple of every tile width)
 
 // Squared FP32 distance between a point (two floats per coordinate) and an image centroid;
@@ -365,41 +364,35 @@ __device__ __forceinline__ void near_point(const GeomView& g, const ImageTable& 
     }
 }
 
-__device__ __forceinline__ void load_elem_tile(Elem* s_el, const Elem* __restrict__ el, int64_t base, int cnt) {
-    const double2* src = reinterpret_cast<const double2*>(el + base);
-    double2* dst = reinterpret_cast<double2*>(s_el);
-    for (int i = threadIdx.x; i < cnt * 16; i += blockDim.x) dst[i] = src[i];
-}
-
 // Raw FP64 sums (before the factor ke) of the closed forms of one point over the elements
 // [e0, e1) and all images.  Called by every thread of the block (shared-memory tiles).
 __device__ __forceinline__ Sum4 f64_range(const Elem* __restrict__ el, const double* __restrict__ sigma, int64_t e0,
                                           int64_t e1, const ImageTable& img, double Px, double Py, double Pz) {
-    __shared__ Elem s_el[kTile64];
-    __shared__ double s_sig[kTile64];
+    __shared__ Tile64 s_t;
     double aphi = 0.0, aEx = 0.0, aEy = 0.0, aEz = 0.0;
     for (int64_t base = e0; base < e1; base += kTile64) {
         const int cnt = (int)min((int64_t)kTile64, e1 - base);
-        __syncthreads();
-        load_elem_tile(s_el, el, base, cnt);
-        if (threadIdx.x < cnt) s_sig[threadIdx.x] = sigma[base + threadIdx.x];
-        __syncthreads();
+        load_tile64(s_t, el, base, cnt, img);
         for (int jj = 0; jj < cnt; ++jj) {
-            const Elem& e = s_el[jj];
+            const Elem& e = s_t.el[jj];
+            double X0, Y0, Z0;
+            to_local(e, __dsub_rn(Px, e.o[0]), __dsub_rn(Py, e.o[1]), __dsub_rn(Pz, e.o[2]), X0, Y0, Z0);
             double lphi = 0.0, lx = 0.0, ly = 0.0, lz = 0.0;
             for (int k = 0; k < img.n; ++k) {
+                const double* tau = s_t.tau[jj][k];
                 double f, gx, gy, gz;
-                elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, gx, gy, gz);
-                lphi += f;
-                lx += gx;
-                ly += gy;
-                lz += gz;
+                elem_at_f64<true, true>(e, s_t.edge[jj], __dsub_rn(X0, tau[0]), __dsub_rn(Y0, tau[1]),
+                                        __dsub_rn(Z0, tau[2]), f, gx, gy, gz);
+                lphi = __dadd_rn(lphi, f);
+                lx = __dadd_rn(lx, gx);
+                ly = __dadd_rn(ly, gy);
+                lz = __dadd_rn(lz, gz);
             }
-            const double s = s_sig[jj];
-            aphi = fma(s, lphi, aphi);
-            aEx = fma(s, fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0])), aEx);
-            aEy = fma(s, fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1])), aEy);
-            aEz = fma(s, fma(lx, e.ex[2], fma(ly, e.ey[2], lz * e.ez[2])), aEz);
+            const double s = sigma[base + jj];
+            aphi = __fma_rn(s, lphi, aphi);
+            aEx = __fma_rn(s, __fma_rn(lx, e.ex[0], __fma_rn(ly, e.ey[0], __dmul_rn(lz, e.ez[0]))), aEx);
+            aEy = __fma_rn(s, __fma_rn(lx, e.ex[1], __fma_rn(ly, e.ey[1], __dmul_rn(lz, e.ez[1]))), aEy);
+            aEz = __fma_rn(s, __fma_rn(lx, e.ex[2], __fma_rn(ly, e.ey[2], __dmul_rn(lz, e.ez[2]))), aEz);
         }
     }
     return Sum4{aphi, aEx, aEy, aEz};
