@@ -54,9 +54,25 @@ int check_count(int64_t n, const char* what) {
     return 0;
 }
 
+cudaError_t Ctx::ensure_pool() {
+    if (pool) return cudaSuccess;
+    cudaMemPoolProps p{};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = device;
+    cudaError_t e = cudaMemPoolCreate(&pool, &p);
+    if (e != cudaSuccess) {
+        pool = nullptr;
+        return e;
+    }
+    uint64_t keep = kPoolKeep;
+    return cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
 Ctx::~Ctx() {
     // the device buffers free themselves after this body, on the device set here
     cudaSetDevice(device);
+    if (pool) cudaMemPoolDestroy(pool);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);
     for (cudaEvent_t e : ev_eval)

@@ -50,6 +50,11 @@ struct Ctx {
     bool eval_timed = false;
     int64_t eval_points_n = 0;
     cudaDeviceProp props{};
+    // stream-ordered scratch of the FP64 evaluation (see eval_f64 in solve.cpp): made on first
+    // use, keeps at most kPoolKeep bytes between calls, freed with the context
+    static constexpr uint64_t kPoolKeep = 256ull << 20;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t ensure_pool();
 
     // geometry
     int64_t n = 0;

@@ -309,131 +309,89 @@ __device__ __forceinline__ void store_acc(int64_t p, const Sum6& tot, double* __
                                0.f, 0.f);
 }
 
+// The far sums of one point over whole pieces of the summation tree.
+template <int L, int M>
+__device__ __forceinline__ Sum6 acc_sum(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
+                                        const float (&pl)[3], int64_t e0, int64_t e1) {
+    Sum6 tot{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int64_t c0 = e0; c0 < e1; c0 += kChunkEl) {
+        const int64_t c1 = min(c0 + (int64_t)kChunkEl, e1);
+        Sum6 ch{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int64_t l = c0; l < c1; l += kLeafEl)
+            add_sum(ch, acc_range<L, M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
+        add_sum(tot, ch);
+    }
+    return tot;
+}
+
 // Far part of every listed point at level L, thread per point, kAT points (a group) per
-// block pass.  The G = ceil(*n_list / kAT) groups are split so that every resident block
-// gets the same work: the first Gm = floor(G / gridDim) * gridDim groups are taken whole,
-// round-robin; the R = G - Gm left over are cut into R * nch pieces (group, element chunk of
-// kChunkEl), also round-robin, whose Sum6 go to part[chunk * cap + (group - Gm) * kAT + t]
-// for k_acc_reduce.  A whole group adds its chunks' sums in chunk order, as k_acc_reduce
-// does, so a point gets the same bits whichever way it is taken.  M: which quantities the
-// pass re-evaluates (kBoth, kPhiOnly, kEOnly).
+// block pass.  The ceil(*n_list / kAT) groups are dealt by split_plan: whole groups, then the
+// pieces of the left-over groups, whose Sum6 go to part[(i - Gm kAT) np + piece] of list entry
+// i for k_acc_reduce.  A point gets the same bits whichever way it is taken.  M: which
+// quantities the pass re-evaluates (kBoth, kPhiOnly, kEOnly).
 template <int L, int M>
 __global__ void __launch_bounds__(kAT, kATBlocks)
     k_eval_acc_far(const AccView A, int nimg, int te, const double* __restrict__ pts,
-                   const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int nch, int64_t cap,
+                   const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
                    Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
                    double* __restrict__ err, float4* __restrict__ bound) {
     extern __shared__ float4 sm[];
     const int64_t count = *n_list;
-    const int64_t gb = gridDim.x;
-    const int64_t G = (count + kAT - 1) / kAT;
-    const int64_t Gm = (G / gb) * gb;
-    for (int64_t g = blockIdx.x; g < Gm; g += gb) {
-        const int64_t base = g * kAT;
-        const bool active = base + threadIdx.x < count;
-        const int64_t p = active ? (int64_t)list[base + threadIdx.x] : 0;
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
+    const int64_t units = plan.Gm + plan.R * plan.np;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const SplitUnit t = split_unit(plan, u, A.n_el);
+        const int64_t i = t.group * kAT + threadIdx.x;
+        const bool active = i < count;
+        const int64_t p = active ? (int64_t)list[i] : 0;
         float ph[3], pl[3];
         load_point_2f(pts, p, active, ph[0], ph[1], ph[2], pl[0], pl[1], pl[2]);
-        Sum6 tot{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int64_t e0 = 0; e0 < A.n_el; e0 += kChunkEl)
-            add6(tot, acc_range<L, M>(A, nimg, te, sm, ph, pl, e0, min(e0 + (int64_t)kChunkEl, A.n_el)));
-        if (active) store_acc<L, M>(p, tot, phi, E, err, bound);
-    }
-    const int64_t R = G - Gm;
-    for (int64_t q = blockIdx.x; q < R * nch; q += gb) {
-        const int64_t r = q % R, ch = q / R;  // consecutive blocks: the same chunk, other groups
-        const int64_t base = (Gm + r) * kAT;
-        const bool active = base + threadIdx.x < count;
-        const int64_t p = active ? (int64_t)list[base + threadIdx.x] : 0;
-        float ph[3], pl[3];
-        load_point_2f(pts, p, active, ph[0], ph[1], ph[2], pl[0], pl[1], pl[2]);
-        const int64_t e0 = ch * kChunkEl;
-        const Sum6 c = acc_range<L, M>(A, nimg, te, sm, ph, pl, e0, min(e0 + (int64_t)kChunkEl, A.n_el));
-        if (active) part[ch * cap + r * kAT + threadIdx.x] = c;
+        const Sum6 tot = acc_sum<L, M>(A, nimg, te, sm, ph, pl, t.e0, t.e1);
+        if (!active) continue;
+        if (t.whole)
+            store_acc<L, M>(p, tot, phi, E, err, bound);
+        else
+            part[(t.r * kAT + threadIdx.x) * plan.np + t.piece] = tot;
     }
 }
 
-// The left-over groups of k_eval_acc_far launched with gb blocks: adds each point's chunk
-// sums in chunk order and stores them.
+// The left-over groups of k_eval_acc_far: their pieces added along the summation tree, a warp
+// per point.
 template <int L, int M>
 __global__ void __launch_bounds__(256)
-    k_acc_reduce(const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb, int nch,
-                 int64_t cap, const Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
+    k_acc_reduce(int64_t n_el, const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
+                 const Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
                  double* __restrict__ err, float4* __restrict__ bound) {
     const int64_t count = *n_list;
-    const int64_t G = (count + kAT - 1) / kAT;
-    const int64_t Gm = (G / gb) * gb;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap || Gm * kAT + i >= count) return;
-    const int64_t p = list[Gm * kAT + i];
-    Sum6 tot{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int k = 0; k < nch; ++k) add6(tot, part[(int64_t)k * cap + i]);
-    store_acc<L, M>(p, tot, phi, E, err, bound);
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, n_el);
+    const int64_t first = plan.Gm * kAT, warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; first + w < count; w += warps) {
+        const Sum6 tot = split_reduce(part + w * plan.np, plan.np, plan.leaf);
+        if ((threadIdx.x & 31) == 0) store_acc<L, M>(list[first + w], tot, phi, E, err, bound);
+    }
 }
 
-__global__ void __launch_bounds__(kEvalThreads)
-    k_eval_acc_near1(const GeomView g, const ImageTable img, const double* __restrict__ pts,
-                     const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, double* __restrict__ phi,
-                     double* __restrict__ E) {
-    const int64_t count = *n_list;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-        near_point(g, img, pts, list[i], phi, E);
-}
+// FP64 near pairs of every listed point, a warp per point (near_point_warp): level 1 with
+// the FP32 pass's near radii, level 2 with the fill's.
+struct NearFill {
+    const FillEl* fe;
+    __device__ __forceinline__ float operator()(int32_t j) const { return fe[j].hdr.z; }
+};
 
-// Level-2 near part (FP64 closed forms of the pairs nearer than kFillRatioC radii, found
-// through the fill's cell list) of every listed point; adds ke * sum to phi / E.
-__global__ void __launch_bounds__(128)
+template <int L>
+__global__ void __launch_bounds__(kAT)
     k_eval_acc_near(const AccView A, const ImageTable img, const double* __restrict__ pts,
                     const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, double* __restrict__ phi,
                     double* __restrict__ E) {
-    const int64_t count = *n_list;
-    const int nimg = img.n;
-    const double ke = 1.0 / (4.0 * kPi * kEps0);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = list[i];
-        const double Px = pts[3 * p], Py = pts[3 * p + 1], Pz = pts[3 * p + 2];
-        float phx, phy, phz, plx, ply, plz;
-        split2f(Px, phx, plx);
-        split2f(Py, phy, ply);
-        split2f(Pz, phz, plz);
-        const NearGrid& grid = A.grid;
-        int cc[3];
-        const double P[3] = {Px, Py, Pz};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double f = floor((P[a] - grid.origin[a]) * grid.inv_h);
-            f = fmin(fmax(f, -2.0), (double)grid.dims[a] + 1.0);
-            cc[a] = (int)f;
-        }
-        double aphi = 0.0, aEx = 0.0, aEy = 0.0, aEz = 0.0;
-        for (int z = max(cc[2] - 1, 0); z <= min(cc[2] + 1, grid.dims[2] - 1); ++z)
-            for (int y = max(cc[1] - 1, 0); y <= min(cc[1] + 1, grid.dims[1] - 1); ++y)
-                for (int x = max(cc[0] - 1, 0); x <= min(cc[0] + 1, grid.dims[0] - 1); ++x) {
-                    const int64_t cell = ((int64_t)z * grid.dims[1] + y) * grid.dims[0] + x;
-                    for (int32_t it = A.cell_start[cell]; it < A.cell_start[cell + 1]; ++it) {
-                        const int32_t jk = A.cell_items[it];
-                        const int32_t j = jk / nimg, k = jk - j * nimg;
-                        float dx, dy, dz;
-                        const float d2 = pair_d2(phx, phy, phz, plx, ply, plz, A.cjk[2 * (int64_t)jk],
-                                                 A.cjk[2 * (int64_t)jk + 1], dx, dy, dz);
-                        if (!(d2 < A.fe[j].hdr.z)) continue;  // far pair: k_eval_acc_far<2>
-                        const Elem& e = A.el[j];
-                        double f, ux, uy, uz;
-                        elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, ux, uy, uz);
-                        const double s = A.sigma[j];
-                        aphi = fma(s, f, aphi);
-                        aEx = fma(s, fma(ux, e.ex[0], fma(uy, e.ey[0], uz * e.ez[0])), aEx);
-                        aEy = fma(s, fma(ux, e.ex[1], fma(uy, e.ey[1], uz * e.ez[1])), aEy);
-                        aEz = fma(s, fma(ux, e.ex[2], fma(uy, e.ey[2], uz * e.ez[2])), aEz);
-                    }
-                }
-        if (phi) phi[p] += ke * aphi;
-        if (E) {
-            E[3 * p] += ke * aEx;
-            E[3 * p + 1] += ke * aEy;
-            E[3 * p + 2] += ke * aEz;
-        }
+    __shared__ int32_t s_queue[kAT / 32][kNearQueue];
+    const int64_t count = *n_list, warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < count; w += warps) {
+        if constexpr (L == 1)
+            near_point_warp(A.el, A.sigma, A.cjk, A.view.grid, A.view.cell_start, A.view.cell_items, img,
+                            NearFar{A.far}, pts, list[w], phi, E, s_queue[threadIdx.x >> 5]);
+        else
+            near_point_warp(A.el, A.sigma, A.cjk, A.grid, A.cell_start, A.cell_items, img, NearFill{A.fe}, pts,
+                            list[w], phi, E, s_queue[threadIdx.x >> 5]);
     }
 }
 
@@ -490,23 +448,6 @@ __global__ void __launch_bounds__(256)
     if (f) list[s_base + s_warp[w] + __popc(ballot & ((1u << lane) - 1u))] = p;
 }
 
-// Blocks of a far launch and the partial-sum layout of its left-over groups, from the
-// largest possible list (npts points): gb resident blocks at most (kATBlocks per SM), no more than
-// there are pieces; cap >= kAT * R for any list length (R < gb, and R <= the groups of npts).
-struct RefineGrid {
-    int64_t gb, cap;
-    int nch;
-};
-
-RefineGrid refine_grid(int64_t npts, int sms, int64_t n_el) {
-    RefineGrid r;
-    const int64_t want = std::max<int64_t>(1, (npts + kAT - 1) / kAT);
-    r.nch = (int)std::max<int64_t>(1, (n_el + kChunkEl - 1) / kChunkEl);
-    r.gb = std::max<int64_t>(1, std::min<int64_t>(want * r.nch, kATBlocks * (int64_t)sms));
-    r.cap = std::min(want, r.gb) * kAT;
-    return r;
-}
-
 template <int L, int M>
 cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* pts, int64_t npts, double* phi,
                          double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list, int sms,
@@ -516,27 +457,25 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
     int te = 16;
     while (te > 1 && acc_tile_f4(te, img.n, Lv::kStaged, Lv::kHdr) * (int)sizeof(float4) > 40 * 1024) te /= 2;
     const size_t smem = (size_t)acc_tile_f4(te, img.n, Lv::kStaged, Lv::kHdr) * sizeof(float4);
-    const RefineGrid rg = refine_grid(npts, sms, A.n_el);
+    const int64_t gb = kATBlocks * (int64_t)sms, want = (npts + kAT - 1) / kAT;
+    const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
     cudaError_t e =
         cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_eval_acc_far<L, M><<<(unsigned)rg.gb, kAT, smem, s>>>(A, img.n, te, pts, list, n_list, rg.nch, rg.cap, part,
-                                                            phi, E, err, bound);
+    k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, gb, part, phi,
+                                                                        E, err, bound);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_acc_reduce<L, M><<<(unsigned)((rg.cap + 255) / 256), 256, 0, s>>>(list, n_list, rg.gb, rg.nch, rg.cap, part,
-                                                                         phi, E, err, bound);
+    const int64_t left = std::min(want, 2 * gb) * kAT;  // points of the left-over groups, at most
+    k_acc_reduce<L, M><<<(unsigned)std::min<int64_t>((left + 7) / 8, 8 * (int64_t)sms), 256, 0, s>>>(
+        A.n_el, list, n_list, gb, part, phi, E, err, bound);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the FP64 near pairs, added to the quantities this pass re-evaluated only
     double* nphi = (M == kEOnly) ? nullptr : phi;
     double* nE = (M == kPhiOnly) ? nullptr : E;
-    const int64_t want = (npts + kAT - 1) / kAT;
-    const unsigned gn = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 8 * (int64_t)sms));
-    if (L == 1)
-        k_eval_acc_near1<<<gn, kEvalThreads, 0, s>>>(A.view, img, pts, list, n_list, nphi, nE);
-    else
-        k_eval_acc_near<<<gn, 128, 0, s>>>(A, img, pts, list, n_list, nphi, nE);
+    const unsigned gn = (unsigned)std::min<int64_t>((npts + kAT / 32 - 1) / (kAT / 32), 16 * (int64_t)sms);
+    k_eval_acc_near<L><<<gn, kAT, 0, s>>>(A, img, pts, list, n_list, nphi, nE);
     return cudaGetLastError();
 }
 
@@ -545,8 +484,7 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
 ErrModel default_err_model() { return ErrModel{kErrGammaR, kErrGammaB, kErrGammaS}; }
 
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el) {
-    const RefineGrid rg = refine_grid(npts, sms, n_el);
-    return sizeof(Sum6) * (size_t)rg.cap * (size_t)rg.nch;
+    return sizeof(Sum6) * (size_t)split_parts((npts + kAT - 1) / kAT, kATBlocks * (int64_t)sms, n_el);
 }
 
 cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const double* pts, int64_t npts,

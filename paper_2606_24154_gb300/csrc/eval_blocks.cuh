@@ -53,7 +53,71 @@ constexpr int kEvalThreads = 128;  // threads per block (one target each)
 constexpr int kTileMax = 16;       // elements per shared-memory tile (mixed)
 constexpr int kCjkMax = 512;       // (element, image) centres per tile (mixed)
 constexpr int kGroup = 8;          // elements per FP32 partial sum (mixed)
-constexpr int kChunkEl = 1024;     // elements per chunk of the far sums (multiple of every tile width)
+
+// Summation tree over the elements, the same in every launch: leaves of kLeafEl elements
+// (a multiple of every tile width), added in order to chunks of kChunkEl, added in order to
+// the total.  A launch may take a point's whole sum, or its chunks or its leaves as separate
+// pieces on different blocks (SplitPlan); the tree, and so every bit, stays the same.
+constexpr int kLeafEl = 32;
+constexpr int kChunkEl = 256;
+static_assert(kChunkEl % kLeafEl == 0 && kLeafEl % kTileMax == 0 && kLeafEl % kTile64 == 0, "summation tree");
+
+// How G groups of kEvalThreads points are dealt to the gb blocks that the device holds at once:
+// the first Gm groups whole, floor(G / gb) - 1 rounds of gb; the R < 2 gb left over in R * np
+// pieces (group, chunk), or (group, leaf) where the chunks would give a block fewer than
+// kSplitRounds pieces.  (With the last full round whole too, its slowest groups ran on alone:
+// 169 ms instead of 144 for the FP32 pass over 233,472 points, exactly two rounds.)  One thread walks all (element, image) pairs of its point in turn, about
+// 0.29 us a pair whatever else the SM does, so a launch cannot end before its longest piece:
+// 250,000 pairs (72 ms) for a whole point of a 10,000-element cell with 25 copies, 1.9 ms for a
+// chunk, 0.23 ms for a leaf.  The leaves cost eight times the chunks' partial sums (48 B per
+// point and piece), which is why they are kept for launches that are short of pieces.
+constexpr int kSplitRounds = 4;
+struct SplitPlan {
+    int64_t Gm, R, np;
+    int leaf;  // 1: pieces are leaves, 0: chunks
+};
+// pieces of `len` elements (at least one: an empty set has one empty piece)
+__host__ __device__ __forceinline__ int64_t split_count(int64_t n_el, int64_t len) {
+    return n_el > 0 ? (n_el + len - 1) / len : 1;
+}
+__host__ __device__ __forceinline__ SplitPlan split_plan(int64_t G, int64_t gb, int64_t n_el) {
+    SplitPlan s;
+    s.Gm = G >= 2 * gb ? (G / gb - 1) * gb : 0;
+    s.R = G - s.Gm;
+    const int64_t nch = split_count(n_el, kChunkEl);
+    s.leaf = s.R * nch < kSplitRounds * gb;
+    s.np = s.leaf ? split_count(n_el, kLeafEl) : nch;
+    return s;
+}
+// partial sums (one per point and piece) of the largest left-over part of up to G groups
+inline int64_t split_parts(int64_t G, int64_t gb, int64_t n_el) {
+    const int64_t nch = split_count(n_el, kChunkEl), nleaf = split_count(n_el, kLeafEl);
+    const int64_t r = G < 2 * gb ? G : 2 * gb;                      // groups left over, at most
+    const int64_t rl = (kSplitRounds * gb + nch - 1) / nch;          // the most that go by leaves
+    const int64_t a = r * nch, b = (r < rl ? r : rl) * nleaf;
+    return (a > b ? a : b) * kEvalThreads;
+}
+// The piece that unit u (< Gm + R np) stands for: its group and element range.
+struct SplitUnit {
+    int64_t group, e0, e1, r, piece;
+    bool whole;
+};
+__device__ __forceinline__ SplitUnit split_unit(const SplitPlan& s, int64_t u, int64_t n_el) {
+    SplitUnit t;
+    t.whole = u < s.Gm;
+    if (t.whole) {
+        t.group = u, t.e0 = 0, t.e1 = n_el, t.r = 0, t.piece = 0;
+        return t;
+    }
+    // consecutive units: the same piece of other groups, whose element data then stay in L2
+    t.piece = (u - s.Gm) / s.R;
+    t.r = (u - s.Gm) - t.piece * s.R;
+    t.group = s.Gm + t.r;
+    const int64_t len = s.leaf ? kLeafEl : kChunkEl;
+    t.e0 = t.piece * len;
+    t.e1 = t.e0 + len < n_el ? t.e0 + len : n_el;
+    return t;
+}
 
 // Squared FP32 distance between a point (two floats per coordinate) and an image centroid;
 // the operation sequence is pinned (no contraction) so both kernels agree bit for bit.
@@ -99,16 +163,69 @@ __device__ __forceinline__ void pairs0_reg(const float4 (&q)[2 * kPairs0], float
     node_pairs<kPairs0>(q, dx, dy, dz, ph, ex, ey, ez);
 }
 
-// Raw FP64 sums (phi, E; before the factor ke) of the far pairs of one point over the
-// elements [e0, e1).  Called by every thread of the block (shared-memory tiles); the
-// inactive threads' sums are unused.
-struct Sum4 {
+// Raw FP64 sums (phi, E; before the factor ke) of one point.
+struct __align__(16) Sum4 {
     double phi, x, y, z;
 };
 // far sums plus the error scales B_phi, B_E (raw, before the factor ke)
-struct Sum6 {
+struct __align__(16) Sum6 {
     double phi, x, y, z, bphi, bE;
 };
+// far sums of the FP32 pass with its four FP32 error scales (bound_slot)
+struct __align__(16) SumB {
+    Sum4 s;
+    float4 b;
+};
+__device__ __forceinline__ void add_sum(Sum4& t, const Sum4& c) {
+    t.phi += c.phi;
+    t.x += c.x;
+    t.y += c.y;
+    t.z += c.z;
+}
+__device__ __forceinline__ void add_sum(Sum6& t, const Sum6& c) {
+    t.phi += c.phi;
+    t.x += c.x;
+    t.y += c.y;
+    t.z += c.z;
+    t.bphi += c.bphi;
+    t.bE += c.bE;
+}
+__device__ __forceinline__ void add_sum(SumB& t, const SumB& c) {
+    add_sum(t.s, c.s);
+    t.b.x += c.b.x;
+    t.b.y += c.b.y;
+    t.b.z += c.b.z;
+    t.b.w += c.b.w;
+}
+// The total of one point's np pieces (leaves or chunks), added along the summation tree by
+// one warp: lane l adds the leaves of chunk l, then every lane adds the chunks in order.
+template <class T>
+__device__ __forceinline__ T split_reduce(const T* __restrict__ part, int64_t np, int leaf) {
+    constexpr int kPer = kChunkEl / kLeafEl, kWords = sizeof(T) / 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t nch = leaf ? (np + kPer - 1) / kPer : np;
+    T tot{};
+    for (int64_t c0 = 0; c0 < nch; c0 += 32) {
+        const int64_t c = c0 + lane;
+        T own{};
+        if (c < nch) {
+            if (leaf) {
+                for (int64_t l = c * kPer; l < c * kPer + kPer && l < np; ++l) add_sum(own, part[l]);
+            } else {
+                own = part[c];
+            }
+        }
+        const int m = (int)(nch - c0 < 32 ? nch - c0 : 32);
+        for (int k = 0; k < m; ++k) {
+            T v;
+#pragma unroll
+            for (int w = 0; w < kWords; ++w)
+                reinterpret_cast<int*>(&v)[w] = __shfl_sync(0xffffffffu, reinterpret_cast<const int*>(&own)[w], k);
+            add_sum(tot, v);
+        }
+    }
+    return tot;
+}
 
 // Per-thread error scales of the far pass, raw (before the factor ke): (B_phi, B_E, the
 // sums of squares of the terms b_j of B_phi and B_E, each term scaled by kScaleSq first).
@@ -123,12 +240,18 @@ __device__ __forceinline__ float4* bound_slot() {
     return &s_bnd[threadIdx.x];
 }
 __device__ __forceinline__ void bound_reset() { *bound_slot() = make_float4(0.f, 0.f, 0.f, 0.f); }
-// the point's scales summed over its element chunks (in chunk order), also in shared memory
-__device__ __forceinline__ float4* bound_total_slot() {
-    __shared__ float4 s_btot[kEvalThreads];
-    return &s_btot[threadIdx.x];
+// Per-thread slots of the chunk and of the total of far_sum, in shared memory too.
+__device__ __forceinline__ SumB* chunk_slot() {
+    __shared__ SumB s_chunk[kEvalThreads];
+    return &s_chunk[threadIdx.x];
+}
+__device__ __forceinline__ SumB* total_slot() {
+    __shared__ SumB s_total[kEvalThreads];
+    return &s_total[threadIdx.x];
 }
 
+// Raw FP64 sums of the far pairs of one point over the elements [e0, e1).  Called by every
+// thread of the block (shared-memory tiles); the inactive threads' sums are unused.
 __device__ __forceinline__ Sum4 far_range(const GeomView& g, float phx, float phy, float phz, float plx, float ply,
                                           float plz, int64_t e0, int64_t e1) {
     const FarNodes* __restrict__ far = g.far;
@@ -258,27 +381,31 @@ __device__ __forceinline__ void store_bound(float4* __restrict__ bound, int64_t 
         bound[p] = make_float4((float)(ke * b.x), (float)(ke * b.y), (float)(ke * inv * sqrt((double)b.z)),
                                (float)(ke * inv * sqrt((double)b.w)));
 }
-__device__ __forceinline__ void add4f(float4& t, const float4& c) {
-    t.x += c.x;
-    t.y += c.y;
-    t.z += c.z;
-    t.w += c.w;
+
+// The far sums and scales of one point over the elements [e0, e1) (whole pieces of the
+// summation tree), left in total_slot(); every thread of the block takes part.
+__device__ __forceinline__ void far_sum(const GeomView& g, float phx, float phy, float phz, float plx, float ply,
+                                        float plz, int64_t e0, int64_t e1) {
+    SumB* tot = total_slot();
+    SumB* ch = chunk_slot();
+    *tot = SumB{};
+    for (int64_t c0 = e0; c0 < e1; c0 += kChunkEl) {
+        const int64_t c1 = min(c0 + (int64_t)kChunkEl, e1);
+        *ch = SumB{};
+        for (int64_t l = c0; l < c1; l += kLeafEl) {
+            bound_reset();
+            SumB leaf;
+            leaf.s = far_range(g, phx, phy, phz, plx, ply, plz, l, min(l + (int64_t)kLeafEl, c1));
+            leaf.b = *bound_slot();
+            add_sum(*ch, leaf);
+        }
+        add_sum(*tot, *ch);
+    }
 }
 
-// Far part (FP32 tiers) of `count` targets; writes ke * sum (overwrites phi / E).  Thread
-// t takes point idx[base + t] (or base + t when idx is null) of pts / phi / E.  The
-// elements are summed in chunks of kChunkEl whose FP64 sums are added in order, so that
-// a launch split over element chunks (the server's small requests) gives the same bits.
-// `bound` (may be null) receives ke * (B_phi, B_E, S_phi, S_E) per point.
-__device__ __forceinline__ void add6(Sum6& t, const Sum6& c) {
-    t.phi += c.phi;
-    t.x += c.x;
-    t.y += c.y;
-    t.z += c.z;
-    t.bphi += c.bphi;
-    t.bE += c.bE;
-}
-
+// Far part (FP32 tiers) of `count` targets over every element; writes ke * sum (overwrites
+// phi / E).  Thread t takes point idx[base + t] (or base + t when idx is null) of pts / phi /
+// E.  `bound` (may be null) receives ke * (B_phi, B_E, S_phi, S_E) per point.
 __device__ __forceinline__ void far_block(const GeomView& g, const double* __restrict__ pts,
                                           const int32_t* __restrict__ idx, int64_t base, int count,
                                           double* __restrict__ phi, double* __restrict__ E,
@@ -287,35 +414,32 @@ __device__ __forceinline__ void far_block(const GeomView& g, const double* __res
     const int64_t p = active ? (idx ? (int64_t)idx[base + threadIdx.x] : base + threadIdx.x) : 0;
     float phx, phy, phz, plx, ply, plz;
     load_point_2f(pts, p, active, phx, phy, phz, plx, ply, plz);
-    Sum4 tot{0.0, 0.0, 0.0, 0.0};
-    float4* btot = bound_total_slot();  // chunk scales added in chunk order (as the server does)
-    *btot = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t e0 = 0; e0 < g.n_el; e0 += kChunkEl) {
-        bound_reset();
-        const Sum4 c = far_range(g, phx, phy, phz, plx, ply, plz, e0, min(e0 + (int64_t)kChunkEl, g.n_el));
-        tot.phi += c.phi;
-        tot.x += c.x;
-        tot.y += c.y;
-        tot.z += c.z;
-        add4f(*btot, *bound_slot());
-    }
+    far_sum(g, phx, phy, phz, plx, ply, plz, 0, g.n_el);
     if (active) {
-        store_far(pts, phi, E, p, tot);
-        store_bound(bound, p, *btot);
+        store_far(pts, phi, E, p, total_slot()->s);
+        store_bound(bound, p, total_slot()->b);
     }
 }
 
-// Near part (FP64 closed forms) of one target; adds ke * sum to phi[p] / E[p].
-__device__ __forceinline__ void near_point(const GeomView& g, const ImageTable& img, const double* __restrict__ pts,
-                                           int64_t p, double* __restrict__ phi, double* __restrict__ E) {
-    const Elem* __restrict__ el = g.el;
-    const FarNodes* __restrict__ far = g.far;
-    const float4* __restrict__ cjk = g.cjk;
-    const double* __restrict__ sigma = g.sigma;
-    const int32_t* __restrict__ cell_start = g.cell_start;
-    const int32_t* __restrict__ cell_items = g.cell_items;
-    const int nimg = g.nimg;
-    const NearGrid& grid = g.grid;
+// Near part (FP64 closed forms) of target p, by one warp; adds ke * sum to phi[p] / E[p].
+// The image centroids in the 27 cells around the point are tested 32 at a time (a row of
+// three cells is contiguous in cell_items), the near ones are queued in `queue` (kNearQueue
+// entries of shared memory of the warp) and evaluated 32 at a time: an FP64 instruction holds
+// the SM's FP64 pipe as long for one lane as for 32, so a lane that met its near pairs one by
+// one (a thread per point) made the pipe do mostly empty work and left one point's pairs
+// in one serial chain (200,000 points: 8.6 ms a thread per point, 1.4 ms a warp).  near2 gives the squared near radius of an element.  The order of the sums
+// depends on the point and the tables only.
+constexpr int kNearQueue = 64;
+template <class Near2>
+__device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, const double* __restrict__ sigma,
+                                                const float4* __restrict__ cjk, const NearGrid& grid,
+                                                const int32_t* __restrict__ cell_start,
+                                                const int32_t* __restrict__ cell_items, const ImageTable& img,
+                                                const Near2& near2, const double* __restrict__ pts, int64_t p,
+                                                double* __restrict__ phi, double* __restrict__ E,
+                                                int32_t* __restrict__ queue) {
+    const int lane = threadIdx.x & 31;
+    const int nimg = img.n;
     const double Px = pts[3 * p], Py = pts[3 * p + 1], Pz = pts[3 * p + 2];
     float phx, phy, phz, plx, ply, plz;
     split2f(Px, phx, plx);
@@ -330,38 +454,90 @@ __device__ __forceinline__ void near_point(const GeomView& g, const ImageTable& 
         f = fmin(fmax(f, -2.0), (double)grid.dims[a] + 1.0);
         cc[a] = (int)f;
     }
+    const int x0 = max(cc[0] - 1, 0), x1 = min(cc[0] + 1, grid.dims[0] - 1);
     double aphi = 0.0, aEx = 0.0, aEy = 0.0, aEz = 0.0;
     bool any = false;
-    for (int z = max(cc[2] - 1, 0); z <= min(cc[2] + 1, grid.dims[2] - 1); ++z)
-        for (int y = max(cc[1] - 1, 0); y <= min(cc[1] + 1, grid.dims[1] - 1); ++y)
-            for (int x = max(cc[0] - 1, 0); x <= min(cc[0] + 1, grid.dims[0] - 1); ++x) {
-                const int64_t cell = ((int64_t)z * grid.dims[1] + y) * grid.dims[0] + x;
-                for (int32_t it = cell_start[cell]; it < cell_start[cell + 1]; ++it) {
-                    const int32_t jk = cell_items[it];
-                    const int32_t j = jk / nimg, k = jk - j * nimg;
-                    float dx, dy, dz;
-                    const float d2 = pair_d2(phx, phy, phz, plx, ply, plz, cjk[2 * (int64_t)jk], cjk[2 * (int64_t)jk + 1],
-                                             dx, dy, dz);
-                    if (!(d2 < far[j].hdr.w)) continue;
-                    const Elem& e = el[j];
-                    double f, ux, uy, uz;
-                    elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, ux, uy, uz);
-                    const double s = sigma[j];
-                    aphi = fma(s, f, aphi);
-                    aEx = fma(s, fma(ux, e.ex[0], fma(uy, e.ey[0], uz * e.ez[0])), aEx);
-                    aEy = fma(s, fma(ux, e.ex[1], fma(uy, e.ey[1], uz * e.ez[1])), aEy);
-                    aEz = fma(s, fma(ux, e.ex[2], fma(uy, e.ey[2], uz * e.ez[2])), aEz);
-                    any = true;
+    int row = 0, nq = 0;  // rows (y, z) of the neighbourhood taken so far; queued pairs
+    int32_t it = 0, end = 0;
+    bool more = x0 <= x1;
+    while (more || nq > 0) {
+        while (more && nq < 32) {
+            if (it >= end) {
+                if (row == 9) {
+                    more = false;
+                    break;
                 }
+                const int y = cc[1] - 1 + row % 3, z = cc[2] - 1 + row / 3;
+                ++row;
+                if (y < 0 || y >= grid.dims[1] || z < 0 || z >= grid.dims[2]) continue;
+                const int64_t cell = ((int64_t)z * grid.dims[1] + y) * grid.dims[0];
+                it = cell_start[cell + x0];
+                end = cell_start[cell + x1 + 1];
+                continue;
             }
-    if (!any) return;
-    const double ke = 1.0 / (4.0 * kPi * kEps0);
-    if (phi) phi[p] += ke * aphi;
-    if (E) {
-        E[3 * p] += ke * aEx;
-        E[3 * p + 1] += ke * aEy;
-        E[3 * p + 2] += ke * aEz;
+            bool hit = false;
+            int32_t jk = 0;
+            if (it + lane < end) {
+                jk = cell_items[it + lane];
+                float dx, dy, dz;
+                const float d2 = pair_d2(phx, phy, phz, plx, ply, plz, cjk[2 * (int64_t)jk], cjk[2 * (int64_t)jk + 1],
+                                         dx, dy, dz);
+                hit = d2 < near2(jk / nimg);
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            if (hit) queue[nq + __popc(m & ((1u << lane) - 1u))] = jk;
+            nq += __popc(m);
+            it += 32;
+        }
+        __syncwarp();
+        const int take = min(nq, 32);
+        if (lane < take) {
+            const int32_t jk = queue[lane];
+            const int32_t j = jk / nimg, k = jk - j * nimg;
+            const Elem& e = el[j];
+            double f, ux, uy, uz;
+            elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, ux, uy, uz);
+            const double s = sigma[j];
+            aphi = fma(s, f, aphi);
+            aEx = __fma_rn(s, __fma_rn(ux, e.ex[0], __fma_rn(uy, e.ey[0], __dmul_rn(uz, e.ez[0]))), aEx);
+            aEy = __fma_rn(s, __fma_rn(ux, e.ex[1], __fma_rn(uy, e.ey[1], __dmul_rn(uz, e.ez[1]))), aEy);
+            aEz = __fma_rn(s, __fma_rn(ux, e.ex[2], __fma_rn(uy, e.ey[2], __dmul_rn(uz, e.ez[2]))), aEz);
+        }
+        any = any || take > 0;
+        nq -= take;
+        const int32_t rest = lane < nq ? queue[32 + lane] : 0;
+        __syncwarp();
+        if (lane < nq) queue[lane] = rest;
+        __syncwarp();
     }
+    if (!any) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        aphi += __shfl_xor_sync(0xffffffffu, aphi, o);
+        aEx += __shfl_xor_sync(0xffffffffu, aEx, o);
+        aEy += __shfl_xor_sync(0xffffffffu, aEy, o);
+        aEz += __shfl_xor_sync(0xffffffffu, aEz, o);
+    }
+    if (lane != 0) return;
+    const double ke = 1.0 / (4.0 * kPi * kEps0);
+    if (phi) phi[p] = __fma_rn(ke, aphi, phi[p]);
+    if (E) {
+        E[3 * p] = __fma_rn(ke, aEx, E[3 * p]);
+        E[3 * p + 1] = __fma_rn(ke, aEy, E[3 * p + 1]);
+        E[3 * p + 2] = __fma_rn(ke, aEz, E[3 * p + 2]);
+    }
+}
+
+// squared near radii of the FP32 pass
+struct NearFar {
+    const FarNodes* far;
+    __device__ __forceinline__ float operator()(int32_t j) const { return far[j].hdr.w; }
+};
+__device__ __forceinline__ void near_point(const GeomView& g, const ImageTable& img, const double* __restrict__ pts,
+                                           int64_t p, double* __restrict__ phi, double* __restrict__ E) {
+    __shared__ int32_t s_queue[kEvalThreads / 32][kNearQueue];
+    near_point_warp(g.el, g.sigma, g.cjk, g.grid, g.cell_start, g.cell_items, img, NearFar{g.far}, pts, p, phi, E,
+                    s_queue[threadIdx.x >> 5]);
 }
 
 // Raw FP64 sums (before the factor ke) of the closed forms of one point over the elements
@@ -398,9 +574,22 @@ __device__ __forceinline__ Sum4 f64_range(const Elem* __restrict__ el, const dou
     return Sum4{aphi, aEx, aEy, aEz};
 }
 
-// FP64 closed forms for every pair of `count` targets (overwrites phi / E).  Sums over
-// kChunkEl-element chunks are added in order, so that a launch split over element chunks
-// (the server's small requests) gives the same bits.
+// The same over whole pieces of the summation tree, left in total_slot()->s.
+__device__ __forceinline__ void f64_sum(const Elem* __restrict__ el, const double* __restrict__ sigma, int64_t e0,
+                                        int64_t e1, const ImageTable& img, double Px, double Py, double Pz) {
+    Sum4* tot = &total_slot()->s;
+    Sum4* ch = &chunk_slot()->s;
+    *tot = Sum4{};
+    for (int64_t c0 = e0; c0 < e1; c0 += kChunkEl) {
+        const int64_t c1 = min(c0 + (int64_t)kChunkEl, e1);
+        *ch = Sum4{};
+        for (int64_t l = c0; l < c1; l += kLeafEl)
+            add_sum(*ch, f64_range(el, sigma, l, min(l + (int64_t)kLeafEl, c1), img, Px, Py, Pz));
+        add_sum(*tot, *ch);
+    }
+}
+
+// FP64 closed forms for every pair of `count` targets (overwrites phi / E).
 __device__ __forceinline__ void f64_block(const Elem* __restrict__ el, const double* __restrict__ sigma, int64_t n_el,
                                           const ImageTable& img, const double* __restrict__ pts, int count,
                                           double* __restrict__ phi, double* __restrict__ E) {
@@ -412,15 +601,8 @@ __device__ __forceinline__ void f64_block(const Elem* __restrict__ el, const dou
         Py = pts[3 * p + 1];
         Pz = pts[3 * p + 2];
     }
-    Sum4 tot{0.0, 0.0, 0.0, 0.0};
-    for (int64_t e0 = 0; e0 < n_el; e0 += kChunkEl) {
-        const Sum4 c = f64_range(el, sigma, e0, min(e0 + (int64_t)kChunkEl, n_el), img, Px, Py, Pz);
-        tot.phi += c.phi;
-        tot.x += c.x;
-        tot.y += c.y;
-        tot.z += c.z;
-    }
-    if (active) store_far(pts, phi, E, p, tot);
+    f64_sum(el, sigma, 0, n_el, img, Px, Py, Pz);
+    if (active) store_far(pts, phi, E, p, total_slot()->s);
 }
 
 }  // namespace nb

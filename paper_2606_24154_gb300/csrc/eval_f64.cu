@@ -18,14 +18,39 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kFillCols = 64;
+constexpr int kF64Blocks = 3;  // resident evaluation blocks per SM (168 registers a thread)
 
-__global__ void __launch_bounds__(kThreads, 3) k_eval_f64(const Elem* __restrict__ el, const double* __restrict__ sigma,
-                                                       int64_t n_el, const ImageTable img,
-                                                       const double* __restrict__ pts, int64_t npts,
-                                                       double* __restrict__ phi, double* __restrict__ E) {
-    const int64_t base = (int64_t)blockIdx.x * blockDim.x;
-    const int count = (int)min((int64_t)blockDim.x, npts - base);
-    f64_block(el, sigma, n_el, img, pts + 3 * base, count, phi ? phi + base : nullptr, E ? E + 3 * base : nullptr);
+// Block u takes unit u of `plan`: whole groups of points, then element pieces of the left-over
+// groups (see split_plan).  1,500 points x 4,632 elements x 25 copies: 516 ms with a thread per
+// point in 12 blocks, 42 ms in pieces.
+__global__ void __launch_bounds__(kEvalThreads, kF64Blocks)
+    k_eval_f64(const Elem* __restrict__ el, const double* __restrict__ sigma, int64_t n_el, const ImageTable img,
+               const double* __restrict__ pts, int64_t npts, const SplitPlan plan, Sum4* __restrict__ part,
+               double* __restrict__ phi, double* __restrict__ E) {
+    const SplitUnit t = split_unit(plan, blockIdx.x, n_el);
+    const int64_t p = t.group * kEvalThreads + threadIdx.x;
+    {
+        const bool active = p < npts;
+        const double Px = active ? pts[3 * p] : 0.0, Py = active ? pts[3 * p + 1] : 0.0,
+                     Pz = active ? pts[3 * p + 2] : 0.0;
+        f64_sum(el, sigma, t.e0, t.e1, img, Px, Py, Pz);
+    }
+    if (p >= npts) return;
+    if (t.whole)
+        store_far(pts, phi, E, p, total_slot()->s);
+    else
+        part[(t.r * kEvalThreads + threadIdx.x) * plan.np + t.piece] = total_slot()->s;
+}
+
+// the left-over groups' points: their pieces added along the summation tree, a warp per point
+__global__ void __launch_bounds__(256) k_f64_reduce(const double* __restrict__ pts, int64_t npts, const SplitPlan plan,
+                                                    const Sum4* __restrict__ part, double* __restrict__ phi,
+                                                    double* __restrict__ E) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t p = plan.Gm * kEvalThreads + w;
+    if (p >= npts) return;
+    const Sum4 tot = split_reduce(part + w * plan.np, plan.np, plan.leaf);
+    if ((threadIdx.x & 31) == 0) store_far(pts, phi, E, p, tot);
 }
 
 // Bound by the FP64 pipe: 4,632 elements x 25 copies take 121 ms, 4.4e9 pairs a second, where
@@ -103,11 +128,24 @@ __global__ void k_element_influence(const Elem* __restrict__ el, int64_t n_el, c
 
 }  // namespace
 
+size_t f64_part_bytes(int64_t npts, int sms, int64_t n_el) {
+    const int64_t G = (npts + kEvalThreads - 1) / kEvalThreads, gb = kF64Blocks * (int64_t)sms;
+    const SplitPlan plan = split_plan(G, gb, n_el);
+    return sizeof(Sum4) * (size_t)(plan.R * plan.np * kEvalThreads);
+}
+
 cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
-                            const double* pts, int64_t npts, double* phi, double* E, cudaStream_t s) {
+                            const double* pts, int64_t npts, double* phi, double* E, int sms, void* part,
+                            cudaStream_t s) {
     if (npts == 0) return cudaSuccess;
-    const int64_t blocks = (npts + kThreads - 1) / kThreads;
-    k_eval_f64<<<(unsigned)blocks, kThreads, 0, s>>>(el, sigma, n_el, img, pts, npts, phi, E);
+    const int64_t gb = kF64Blocks * (int64_t)sms;
+    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
+    const int64_t units = plan.Gm + plan.R * plan.np;
+    k_eval_f64<<<(unsigned)units, kEvalThreads, 0, s>>>(el, sigma, n_el, img, pts, npts, plan,
+                                                        static_cast<Sum4*>(part), phi, E);
+    if (plan.R > 0)
+        k_f64_reduce<<<(unsigned)((plan.R * kEvalThreads + 7) / 8), 256, 0, s>>>(
+            pts, npts, plan, static_cast<const Sum4*>(part), phi, E);
     return cudaGetLastError();
 }
 

@@ -8,22 +8,59 @@ namespace nb {
 
 namespace {
 
-__global__ void __launch_bounds__(kEvalThreads, 6) k_eval_far(const GeomView g, const double* __restrict__ pts,
-                                                            const int32_t* __restrict__ order, int64_t npts,
-                                                            double* __restrict__ phi, double* __restrict__ E,
-                                                            float4* __restrict__ bound) {
-    const int64_t base = (int64_t)blockIdx.x * blockDim.x;
-    const int count = (int)min((int64_t)blockDim.x, npts - base);
-    far_block(g, pts, order, base, count, phi, E, bound);
+constexpr int kFarBlocks = 6;  // resident far blocks per SM (80 registers a thread)
+
+// Far part of every point: block u takes unit u of `plan` (whole groups, then pieces of the
+// left-over groups).  Bound by the FP32 pipe where every SM has its six
+// blocks; a thread's own chain of pairs takes as long on an idle SM as on a full one, so few
+// points are spread over element pieces (see split_plan): 257 points of the 9,996-element
+// cell x 25 copies took 71.2 ms in 3 blocks and take 0.64 ms in 939; 20,000 points 69 and 15 ms,
+// 200,000 points 162 and 126 ms, 1e6 points 644 and 610 ms (with binning and near pairs).
+__global__ void __launch_bounds__(kEvalThreads, kFarBlocks)
+    k_eval_far(const GeomView g, const double* __restrict__ pts, const int32_t* __restrict__ order, int64_t npts,
+               const SplitPlan plan, SumB* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
+               float4* __restrict__ bound) {
+    const int64_t n_el = g.n_el;
+    const SplitUnit t = split_unit(plan, blockIdx.x, n_el);
+    const int64_t i = t.group * kEvalThreads + threadIdx.x;
+    {
+        const bool active = i < npts;
+        float phx, phy, phz, plx, ply, plz;
+        load_point_2f(pts, active ? (int64_t)order[i] : 0, active, phx, phy, phz, plx, ply, plz);
+        far_sum(g, phx, phy, phz, plx, ply, plz, t.e0, t.e1);
+    }
+    if (i >= npts) return;
+    if (t.whole) {
+        const int64_t p = order[i];
+        store_far(pts, phi, E, p, total_slot()->s);
+        store_bound(bound, p, total_slot()->b);
+    } else {
+        part[(t.r * kEvalThreads + threadIdx.x) * plan.np + t.piece] = *total_slot();
+    }
+}
+
+// the left-over groups' points: their pieces added along the summation tree, a warp per point
+__global__ void __launch_bounds__(256) k_far_reduce(const double* __restrict__ pts, const int32_t* __restrict__ order,
+                                                    int64_t npts, const SplitPlan plan,
+                                                    const SumB* __restrict__ part, double* __restrict__ phi,
+                                                    double* __restrict__ E, float4* __restrict__ bound) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t i = plan.Gm * kEvalThreads + w;
+    if (i >= npts) return;
+    const SumB tot = split_reduce(part + w * plan.np, plan.np, plan.leaf);
+    if ((threadIdx.x & 31) != 0) return;
+    const int64_t p = order[i];
+    store_far(pts, phi, E, p, tot.s);
+    store_bound(bound, p, tot.b);
 }
 
 __global__ void __launch_bounds__(kEvalThreads) k_eval_near(const GeomView g, const ImageTable img,
                                                           const double* __restrict__ pts,
                                                           const int32_t* __restrict__ order, int64_t npts,
                                                           double* __restrict__ phi, double* __restrict__ E) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= npts) return;
-    near_point(g, img, pts, order ? (int64_t)order[i] : i, phi, E);
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= npts) return;
+    near_point(g, img, pts, (int64_t)order[w], phi, E);
 }
 
 // ---- spatial binning of the targets: counting sort by the Morton index of a 64^3 grid
@@ -59,28 +96,49 @@ __global__ void k_bin_keys(const double* __restrict__ pts, int64_t n, const Near
     atomicAdd(&count[k], 1);
 }
 
-// Exclusive scan of kBins counts by one block of 1024 threads (kBins / 1024 per thread):
-// per-thread sums, a block scan of those, then each thread rewrites its range in place.
-__global__ void __launch_bounds__(1024) k_bin_scan(int32_t* __restrict__ count) {
-    constexpr int per = kBins / 1024;
-    __shared__ int32_t part[1024];
-    int32_t* mine = count + threadIdx.x * per;
-    int32_t s = 0;
-    for (int j = 0; j < per; ++j) s += mine[j];
-    part[threadIdx.x] = s;
+// Exclusive scan of the kBins counts in two launches of kBins / 1024 blocks: every block's
+// sum of its 1024 counts, then every block scans its own counts from the sum of the blocks before
+// it.  (One block for all 262,144 counts took 0.30 ms, in a chain of dependent loads.)
+constexpr int kScanBlocks = kBins / 1024;
+static_assert(kScanBlocks <= 1024, "one thread per block sum");
+
+__device__ __forceinline__ int32_t warp_sum(int32_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__global__ void __launch_bounds__(256) k_bin_sums(const int32_t* __restrict__ count, int32_t* __restrict__ sums) {
+    __shared__ int32_t s_w[8];
+    const int4 c = reinterpret_cast<const int4*>(count)[blockIdx.x * 256 + threadIdx.x];
+    const int32_t v = warp_sum(c.x + c.y + c.z + c.w);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int32_t v = (threadIdx.x >= (unsigned)off) ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t t = 0;
+        for (int k = 0; k < 8; ++k) t += s_w[k];
+        sums[blockIdx.x] = t;
     }
-    int32_t run = part[threadIdx.x] - s;  // exclusive prefix of this thread's range
-    for (int j = 0; j < per; ++j) {
-        const int32_t c = mine[j];
-        mine[j] = run;
-        run += c;
+}
+
+__global__ void __launch_bounds__(1024) k_bin_scan(int32_t* __restrict__ count, const int32_t* __restrict__ sums) {
+    __shared__ int32_t s_w[32], s_b[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int32_t before = ((int)threadIdx.x < kScanBlocks && threadIdx.x < blockIdx.x) ? sums[threadIdx.x] : 0;
+    const int32_t bs = warp_sum(before);
+    const int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+    const int32_t c = count[i];
+    int32_t inc = c;  // inclusive scan of the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
     }
+    if (lane == 31) s_w[w] = inc;
+    if (lane == 0) s_b[w] = bs;
+    __syncthreads();
+    const int32_t base = warp_sum(s_b[lane]) + warp_sum(lane < w ? s_w[lane] : 0);
+    count[i] = base + inc - c;
 }
 
 __global__ void k_bin_scatter(const int32_t* __restrict__ key, int64_t n, int32_t* __restrict__ next,
@@ -182,19 +240,25 @@ MixedScratch mixed_scratch(void* base, int64_t npts) {
     m.list_e = reinterpret_cast<int32_t*>(p);
     p += align256(sizeof(int32_t) * n);
     m.n_list = reinterpret_cast<int32_t*>(p);
+    p += 256;
+    m.bin_sums = reinterpret_cast<int32_t*>(p);
     return m;
 }
 
 size_t eval_mixed_scratch_bytes(int64_t npts) {
     const size_t n = (size_t)npts;
     return align256(sizeof(int32_t) * kBins) + 6 * align256(sizeof(int32_t) * n) + align256(sizeof(float4) * n) +
-           256;
+           256 + align256(sizeof(int32_t) * kScanBlocks);
+}
+
+size_t far_part_bytes(int64_t npts, int sms, int64_t n_el) {
+    return sizeof(SumB) * (size_t)split_parts((npts + kEvalThreads - 1) / kEvalThreads, kFarBlocks * (int64_t)sms, n_el);
 }
 
 cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4* cjk, const double* sigma,
                               int64_t n_el, const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
                               const int32_t* cell_items, const double* pts, int64_t npts, double* phi, double* E,
-                              const MixedScratch& ms, cudaStream_t s) {
+                              const MixedScratch& ms, int sms, void* part, cudaStream_t s) {
     if (npts == 0) return cudaSuccess;
     if (npts > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
     const GeomView g = make_view(el, far, cjk, sigma, n_el, img, grid, cell_start, cell_items);
@@ -202,13 +266,21 @@ cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4*
     cudaError_t e = cudaMemsetAsync(ms.count, 0, sizeof(int32_t) * kBins, s);
     if (e != cudaSuccess) return e;
     k_bin_keys<<<pblocks, 256, 0, s>>>(pts, npts, grid, ms.key, ms.count);
-    k_bin_scan<<<1, 1024, 0, s>>>(ms.count);
+    k_bin_sums<<<kScanBlocks, 256, 0, s>>>(ms.count, ms.bin_sums);
+    k_bin_scan<<<kScanBlocks, 1024, 0, s>>>(ms.count, ms.bin_sums);
     k_bin_scatter<<<pblocks, 256, 0, s>>>(ms.key, npts, ms.count, ms.order);
-    const unsigned blocks = (unsigned)((npts + kEvalThreads - 1) / kEvalThreads);
-    k_eval_far<<<blocks, kEvalThreads, 0, s>>>(g, pts, ms.order, npts, phi, E, ms.bound);
+    const int64_t gb = kFarBlocks * (int64_t)sms;
+    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
+    const int64_t units = plan.Gm + plan.R * plan.np;
+    k_eval_far<<<(unsigned)units, kEvalThreads, 0, s>>>(g, pts, ms.order, npts, plan, static_cast<SumB*>(part), phi, E,
+                                                        ms.bound);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_eval_near<<<blocks, kEvalThreads, 0, s>>>(g, img, pts, ms.order, npts, phi, E);
+    if (plan.R > 0)
+        k_far_reduce<<<(unsigned)((plan.R * kEvalThreads + 7) / 8), 256, 0, s>>>(
+            pts, ms.order, npts, plan, static_cast<const SumB*>(part), phi, E, ms.bound);
+    const int64_t near_blocks = (npts + kEvalThreads / 32 - 1) / (kEvalThreads / 32);
+    k_eval_near<<<(unsigned)near_blocks, kEvalThreads, 0, s>>>(g, img, pts, ms.order, npts, phi, E);
     return cudaGetLastError();
 }
 

@@ -133,8 +133,11 @@ GeomView make_view(const Elem* el, const FarNodes* far, const float4* cjk, const
 
 // ------------------------------------------------------------------ launchers (.cu)
 // Each returns cudaSuccess or the launch error.
+// FP64 evaluation; part: f64_part_bytes(npts, sms, n_el) bytes of device scratch (NULL when 0)
+size_t f64_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
-                            const double* pts, int64_t npts, double* phi, double* E, cudaStream_t s);
+                            const double* pts, int64_t npts, double* phi, double* E, int sms, void* part,
+                            cudaStream_t s);
 // Scratch of one mixed evaluation of npts points: binning (bin counts, keys, the binned
 // order), the FP32 pass's error scales ke * (B_phi, B_E, S_phi, S_E) per point, and the
 // list and count of the points the refinement re-evaluates.
@@ -148,15 +151,19 @@ struct MixedScratch {
     int32_t* list_p; // npts: points of the first level, phi only
     int32_t* list_e; // npts: points of the first level, E only
     int32_t* n_list; // 4: the lengths of list, list2, list_p, list_e
+    int32_t* bin_sums;  // block sums of the bin scan
 };
 MixedScratch mixed_scratch(void* base, int64_t npts);
 // scratch bytes a mixed evaluation (FP32 pass and refinement) needs for npts points
 size_t eval_mixed_scratch_bytes(int64_t npts);
-// FP32 pass (binning, far tiers, FP64 near pairs); fills ms.order and ms.bound
+// bytes of the partial sums of the point groups that the FP32 pass splits over element pieces
+size_t far_part_bytes(int64_t npts, int sms, int64_t n_el);
+// FP32 pass (binning, far tiers, FP64 near pairs); fills ms.order and ms.bound.  part:
+// far_part_bytes(npts, sms, n_el) bytes of device scratch; sms = multiprocessors.
 cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4* cjk, const double* sigma,
                               int64_t n_el, const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
                               const int32_t* cell_items, const double* pts, int64_t npts, double* phi, double* E,
-                              const MixedScratch& ms, cudaStream_t s);
+                              const MixedScratch& ms, int sms, void* part, cudaStream_t s);
 // Tables of the two-float evaluation (the mixed fill's): element records, node records,
 // tau = t_k . frame, two-float image centroids, and the cell list with the near radius
 // kFillRatioC rho.

@@ -6,7 +6,7 @@
 // points are copied into the arena, its remaining point-block counter is set, and its
 // items are appended to the ring in host-mapped memory before `tail` is advanced.  An
 // item is 128 points over all elements; a request of up to 16384 points instead gets one
-// item per (point block, chunk of 1024 elements), so that its points still spread over
+// item per (point block, chunk of 256 elements), so that its points still spread over
 // many CTAs (its latency would otherwise be one CTA's pass over all elements).  A persistent kernel (relaunched whenever admitted work exists and no
 // instance is running) claims items as they appear, so requests admitted while others
 // run join the running launch.  On completion the outputs are copied to the caller's
@@ -300,7 +300,7 @@ struct Server {
         CK(launch_serve(d_geoms.as<ServeGeom>(), h_ring, ring_cap, h_tail, d_head.as<unsigned long long>(),
                         d_pts.as<double>(), d_phi.as<double>(), d_E.as<double>(), d_bound.as<float4>(),
                         d_remaining.as<int>(), h_done,
-                        d_partials.as<double>(), d_pcount.as<int>(), max_chunks, (uint64_t)opt.idle_us * 1000ull,
+                        d_partials.ptr, d_pcount.as<int>(), max_chunks, (uint64_t)opt.idle_us * 1000ull,
                         opt.workers, compute));
         CK(cudaEventRecord(kernel_done, compute));
         kernel_launched = true;
@@ -402,8 +402,7 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         (e = s->d_E.ensure(sizeof(double) * 3 * cap)) != cudaSuccess ||
         (e = s->d_head.ensure(3 * sizeof(unsigned long long))) != cudaSuccess ||  // claimed, finished, closing
         (e = s->d_remaining.ensure(sizeof(int) * o.max_requests)) != cudaSuccess ||
-        (e = s->d_partials.ensure(sizeof(double) * kPartialDoubles * kItemPoints * (size_t)kPartialBlocks *
-                                  s->max_chunks)) != cudaSuccess ||
+        (e = s->d_partials.ensure((size_t)kPartialBytes * kItemPoints * (size_t)kPartialBlocks * s->max_chunks)) != cudaSuccess ||
         (e = s->d_bound.ensure(sizeof(float4) * cap)) != cudaSuccess ||
         (e = s->d_list.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_list2.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||

@@ -34,12 +34,22 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 static_assert(kChunkElements == kChunkEl, "server chunk width must match the evaluation bodies");
+static_assert(kPartialBytes == sizeof(SumB), "size of a point's chunk sums");
+
+// near pairs of the block's `count` points, each warp its own 32 points in turn (the values
+// that its lanes have just stored are added to after the warp barrier)
+__device__ __forceinline__ void near_points(const ServeGeom& G, const double* __restrict__ pts, int64_t base,
+                                            int count, double* __restrict__ phi, double* __restrict__ E) {
+    __syncwarp();
+    const int w0 = threadIdx.x & ~31;
+    for (int t = w0; t < min(w0 + 32, count); ++t) near_point(G.view, G.img, pts, base + t, phi, E);
+}
 
 __global__ void __launch_bounds__(kEvalThreads) k_serve(const ServeGeom* __restrict__ geoms, const WorkItem* ring,
                                                         int64_t ring_cap, int64_t* tail_mapped,
                                                         unsigned long long* head, const double* __restrict__ arena_pts,
                                                         double* __restrict__ arena_phi, double* __restrict__ arena_E,
-                                                        float4* __restrict__ arena_bound, int* remaining, int64_t* done_mapped, double* partials,
+                                                        float4* __restrict__ arena_bound, int* remaining, int64_t* done_mapped, SumB* partials,
                                                         int* pblock_count, int max_chunks, uint64_t idle_ns) {
     __shared__ WorkItem it;
     __shared__ int have;
@@ -83,8 +93,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_serve(const ServeGeom* __restr
                       arena_phi + it.offset, arena_E + 3 * it.offset);
         } else if (it.chunk < 0) {
             far_block(G.view, arena_pts, nullptr, it.offset, it.count, arena_phi, arena_E, arena_bound);
-            if ((int)threadIdx.x < it.count)
-                near_point(G.view, G.img, arena_pts, it.offset + threadIdx.x, arena_phi, arena_E);
+            near_points(G, arena_pts, it.offset, it.count, arena_phi, arena_E);
         } else {
             // one element chunk of a point block: raw sums to the partial area; the CTA that
             // finishes the block's last chunk adds the chunks in order (as far_block and
@@ -93,29 +102,18 @@ __global__ void __launch_bounds__(kEvalThreads) k_serve(const ServeGeom* __restr
             const int64_t p = it.offset + threadIdx.x;
             const int64_t e0 = (int64_t)it.chunk * kChunkEl;
             const int64_t e1 = min(e0 + (int64_t)kChunkEl, G.view.n_el);
-            Sum4 c;
-            float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
             if (mixed) {
                 float phx, phy, phz, plx, ply, plz;
                 load_point_2f(arena_pts, p, active, phx, phy, phz, plx, ply, plz);
-                bound_reset();
-                c = far_range(G.view, phx, phy, phz, plx, ply, plz, e0, e1);
-                b = *bound_slot();
+                far_sum(G.view, phx, phy, phz, plx, ply, plz, e0, e1);
             } else {
                 const double Px = active ? arena_pts[3 * p] : 0.0, Py = active ? arena_pts[3 * p + 1] : 0.0,
                              Pz = active ? arena_pts[3 * p + 2] : 0.0;
-                c = f64_range(G.view.el, G.view.sigma, e0, e1, G.img, Px, Py, Pz);
+                total_slot()->b = make_float4(0.f, 0.f, 0.f, 0.f);
+                f64_sum(G.view.el, G.view.sigma, e0, e1, G.img, Px, Py, Pz);
             }
-            constexpr int kP = kPartialDoubles;
-            double* part = partials + ((int64_t)it.pblock * max_chunks + it.chunk) * (kP * kEvalThreads);
-            part[kP * threadIdx.x] = c.phi;
-            part[kP * threadIdx.x + 1] = c.x;
-            part[kP * threadIdx.x + 2] = c.y;
-            part[kP * threadIdx.x + 3] = c.z;
-            part[kP * threadIdx.x + 4] = (double)b.x;  // exact
-            part[kP * threadIdx.x + 5] = (double)b.y;
-            part[kP * threadIdx.x + 6] = (double)b.z;
-            part[kP * threadIdx.x + 7] = (double)b.w;
+            SumB* part = partials + ((int64_t)it.pblock * max_chunks + it.chunk) * kEvalThreads;
+            part[threadIdx.x] = *total_slot();
             __threadfence();
             __syncthreads();
             if (threadIdx.x == 0) last = (atomicAdd(&pblock_count[it.pblock], 1) == it.nchunks - 1);
@@ -123,25 +121,21 @@ __global__ void __launch_bounds__(kEvalThreads) k_serve(const ServeGeom* __restr
             block_done = last;
             if (last) {
                 __threadfence();
-                Sum4 tot{0.0, 0.0, 0.0, 0.0};
-                float4 btot = make_float4(0.f, 0.f, 0.f, 0.f);  // FP32 sums in chunk order, as far_block
+                SumB tot{};  // in chunk order, as far_sum and f64_sum
                 for (int k = 0; k < it.nchunks; ++k) {
-                    const double* q = partials + ((int64_t)it.pblock * max_chunks + k) * (kP * kEvalThreads) +
-                                      kP * threadIdx.x;
-                    tot.phi += __ldcg(q);
-                    tot.x += __ldcg(q + 1);
-                    tot.y += __ldcg(q + 2);
-                    tot.z += __ldcg(q + 3);
-                    btot.x += (float)__ldcg(q + 4);
-                    btot.y += (float)__ldcg(q + 5);
-                    btot.z += (float)__ldcg(q + 6);
-                    btot.w += (float)__ldcg(q + 7);
+                    const SumB* q = partials + ((int64_t)it.pblock * max_chunks + k) * kEvalThreads + threadIdx.x;
+                    SumB v;
+                    const double2* d = reinterpret_cast<const double2*>(q);
+                    const double2 a = __ldcg(d), b = __ldcg(d + 1);
+                    v.s = Sum4{a.x, a.y, b.x, b.y};
+                    v.b = __ldcg(&q->b);
+                    add_sum(tot, v);
                 }
                 if (active) {
-                    store_far(arena_pts, arena_phi, arena_E, p, tot);
-                    if (mixed) store_bound(arena_bound, p, btot);
-                    if (mixed) near_point(G.view, G.img, arena_pts, p, arena_phi, arena_E);
+                    store_far(arena_pts, arena_phi, arena_E, p, tot.s);
+                    if (mixed) store_bound(arena_bound, p, tot.b);
                 }
+                if (mixed) near_points(G, arena_pts, it.offset, it.count, arena_phi, arena_E);
                 if (threadIdx.x == 0) pblock_count[it.pblock] = 0;
             }
         }
@@ -163,10 +157,10 @@ __global__ void __launch_bounds__(kEvalThreads) k_serve(const ServeGeom* __restr
 
 cudaError_t launch_serve(const ServeGeom* geoms, const WorkItem* ring, int64_t ring_cap, int64_t* tail_mapped,
                          unsigned long long* head, const double* arena_pts, double* arena_phi, double* arena_E,
-                         float4* arena_bound, int* remaining, int64_t* done_mapped, double* partials,
+                         float4* arena_bound, int* remaining, int64_t* done_mapped, void* partials,
                          int* pblock_count, int max_chunks, uint64_t idle_ns, int workers, cudaStream_t s) {
     k_serve<<<workers, kEvalThreads, 0, s>>>(geoms, ring, ring_cap, tail_mapped, head, arena_pts, arena_phi, arena_E,
-                                             arena_bound, remaining, done_mapped, partials, pblock_count, max_chunks, idle_ns);
+                                             arena_bound, remaining, done_mapped, static_cast<SumB*>(partials), pblock_count, max_chunks, idle_ns);
     return cudaGetLastError();
 }
 

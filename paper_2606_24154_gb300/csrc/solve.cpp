@@ -317,15 +317,36 @@ int weighting_solve(Ctx* c, const int32_t* readout, int k, int precision, nebem_
     return 0;
 }
 
+// FP64 evaluation with stream-ordered scratch from the context's own pool: unlike the mixed
+// evaluation's scratch it is the call's own, so FP64 calls on different streams of a context
+// share nothing, and a call can be captured into a graph.
+static int eval_f64(Ctx* c, const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
+                    const double* d_pts, int64_t n, double* d_phi, double* d_E, cudaStream_t s) {
+    const int sms = c->props.multiProcessorCount;
+    const size_t bytes = f64_part_bytes(n, sms, n_el);
+    void* part = nullptr;
+    if (bytes > 0) {
+        CK(c->ensure_pool());
+        CK(cudaMallocFromPoolAsync(&part, bytes, c->pool, s));
+    }
+    const cudaError_t e = launch_eval_f64(el, sigma, n_el, img, d_pts, n, d_phi, d_E, sms, part, s);
+    const cudaError_t ef = part ? cudaFreeAsync(part, s) : cudaSuccess;
+    if (e != cudaSuccess) return cuda_fail(e, "launch_eval_f64");
+    CK(ef);
+    return 0;
+}
+
 int eval_set(Ctx* c, const EvalSet& es, const double* d_pts, int64_t n, double* d_phi, double* d_E, int precision,
              cudaStream_t s) {
     if (precision == NEBEM_MIXED) {
-        CK(c->d_scratch.ensure(eval_mixed_scratch_bytes(n)));
+        const int sms = c->props.multiProcessorCount;
+        const size_t ms_bytes = eval_mixed_scratch_bytes(n);
+        CK(c->d_scratch.ensure(ms_bytes + far_part_bytes(n, sms, es.n)));
         CK(launch_eval_mixed(es.el, es.far, es.cjk.as<float4>(), es.sigma, es.n, es.img, es.grid,
                              es.cell_start.as<int32_t>(), es.cell_items.as<int32_t>(), d_pts, n, d_phi, d_E,
-                             mixed_scratch(c->d_scratch.ptr, n), s));
+                             mixed_scratch(c->d_scratch.ptr, n), sms, c->d_scratch.as<char>() + ms_bytes, s));
     } else {
-        CK(launch_eval_f64(es.el, es.sigma, es.n, es.img, d_pts, n, d_phi, d_E, s));
+        return eval_f64(c, es.el, es.sigma, es.n, es.img, d_pts, n, d_phi, d_E, s);
     }
     return 0;
 }
@@ -340,13 +361,16 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
             if (rc) return rc;
         }
         const size_t ms_bytes = eval_mixed_scratch_bytes(n);  // a multiple of 256
-        CK(c->d_scratch.ensure(ms_bytes + refine_part_bytes(n, c->props.multiProcessorCount, c->n)));
+        // the FP32 pass and the refinement levels use one partial-sum area in turn
+        const int sms = c->props.multiProcessorCount;
+        CK(c->d_scratch.ensure(ms_bytes + std::max(far_part_bytes(n, sms, c->n), refine_part_bytes(n, sms, c->n))));
+        void* part = c->d_scratch.as<char>() + ms_bytes;
         const MixedScratch ms = mixed_scratch(c->d_scratch.ptr, n);
         c->eval_timed = false;
         CK(cudaEventRecord(c->ev_eval[0], s));
         CK(launch_eval_mixed(c->d_el.as<Elem>(), c->d_far.as<FarNodes>(), c->d_cjk.as<float4>(),
                              c->d_sigma.as<double>(), c->n, c->img, c->grid, c->d_cell_start.as<int32_t>(),
-                             c->d_cell_items.as<int32_t>(), d_pts, n, d_phi, d_E, ms, s));
+                             c->d_cell_items.as<int32_t>(), d_pts, n, d_phi, d_E, ms, sms, part, s));
         CK(cudaEventRecord(c->ev_eval[1], s));
         if (refine || err) {
             AccView A;
@@ -364,8 +388,7 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
             A.grid = c->fill_grid;
             A.cell_start = c->d_fill_cell_start.as<int32_t>();
             A.cell_items = c->d_fill_cell_items.as<int32_t>();
-            CK(launch_eval_refine(A, c->img, d_pts, n, d_phi, d_E, err, c->opt.mixed_point_tol, c->err_model, ms, c->props.multiProcessorCount, s, &c->ev_eval[2],
-                                  static_cast<char*>(c->d_scratch.ptr) + ms_bytes));
+            CK(launch_eval_refine(A, c->img, d_pts, n, d_phi, d_E, err, c->opt.mixed_point_tol, c->err_model, ms, sms, s, &c->ev_eval[2], part));
             c->refine_list = ms.n_list;
         } else {
             CK(cudaMemsetAsync(ms.n_list, 0, 4 * sizeof(int32_t), s));
@@ -376,7 +399,7 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
         c->eval_timed = true;
         c->eval_points_n = n;
     } else {
-        CK(launch_eval_f64(c->d_el.as<Elem>(), c->d_sigma.as<double>(), c->n, c->img, d_pts, n, d_phi, d_E, s));
+        return eval_f64(c, c->d_el.as<Elem>(), c->d_sigma.as<double>(), c->n, c->img, d_pts, n, d_phi, d_E, s);
     }
     return 0;
 }
