@@ -198,7 +198,7 @@ int nebem_set_bc(nebem_ctx *ctx, const double *voltages, int32_t n_conductors);
  * charge densities; info (may be NULL) the report.
  * Errors: NEBEM_BAD_STATE (no geometry or no voltages), NEBEM_SINGULAR,
  * NEBEM_NOT_CONVERGED (sigma and info are still written), NEBEM_TIMEOUT (a bounded device
- * wait ran out -- see wait_polls: in the FP32 factorisation, nothing is written; in a
+ * wait ran out -- see wait_polls: in the factorisation, nothing is written; in a
  * triangular sweep, sigma_out is written with NaN in the 64-row blocks whose wait ran out,
  * and the context holds no valid charge densities until the next solve; every kernel has
  * returned, so the context stays usable), NEBEM_OUT_OF_MEMORY, NEBEM_CUDA. */
@@ -441,13 +441,16 @@ int nebem_step(nebem_ctx *ctx, int32_t steps, double mu, double dt, int32_t prec
  *          diagonal) and U.
  *   d_piv  device int32[n]; row k was swapped with row d_piv[k] at step k.
  * Runs on `stream` (NULL = the context stream) and synchronises it before returning.
- * Allocates its work buffer (about (lu_block + 1) * n doubles) on the context's device
- * for the duration of the call.  An exact zero pivot (the whole remaining column is zero)
+ * The trailing updates are formed exactly from integer digits on the tensor cores and
+ * rounded to FP64 once per panel; each panel is one cooperative launch (all CTAs resident,
+ * one bounded grid barrier per column) when the device supports it.
+ * Allocates its work buffer (about (lu_block + 257) * n doubles and 1.1 MB) on the context's
+ * device for the duration of the call.  An exact zero pivot (the whole remaining column is zero)
  * does not stop the factorisation: that column is left unscaled, the remaining columns
  * are factored, and the call returns NEBEM_SINGULAR naming the first such column in
  * nebem_last_error.  d_A and d_piv then hold complete factors, P A = L U, with an exact
  * zero on U's diagonal there (which nebem_lu_solve_device cannot use).  Other errors:
- * NEBEM_INVALID_ARG, NEBEM_OUT_OF_MEMORY, NEBEM_CUDA. */
+ * NEBEM_INVALID_ARG, NEBEM_OUT_OF_MEMORY, NEBEM_TIMEOUT (a bounded wait gave up), NEBEM_CUDA. */
 int nebem_lu_factor_device(nebem_ctx *ctx, double *d_A, int64_t n, int32_t *d_piv, void *stream);
 
 /* FP32 variant (Sec. 4.1, Alg. 1; the factorisation inside mixed solves): d_A is float, n x n column-major.

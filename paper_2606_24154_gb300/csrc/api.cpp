@@ -519,15 +519,16 @@ int nebem_lu_factor_device(nebem_ctx* ctx, double* d_A, int64_t n, int32_t* d_pi
     cudaStream_t s = stream ? (cudaStream_t)stream : c->stream;
     const int nb = c->opt.lu_block;
     DevBuf work, info;
-    CK(work.ensure(sizeof(double) * lu_work_elems(n, nb)));
+    CK(work.ensure(lu_work_bytes_f64(n, nb)));
     CK(info.ensure(2 * sizeof(int)));
-    CK(lu_factor_f64(d_A, n, d_piv, nb, work.as<double>(), info.as<int>(), s));
-    int h_info = 0;
-    CK(cudaMemcpyAsync(&h_info, info.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(lu_factor_f64(d_A, n, d_piv, nb, work.ptr, info.as<int>(), s));
+    int h2[2] = {0, 0};
+    CK(cudaMemcpyAsync(h2, info.ptr, sizeof(h2), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     work.release();
     info.release();
-    if (h_info) return fail(NEBEM_SINGULAR, "zero pivot at column " + std::to_string(h_info - 1));
+    if (h2[1]) return fail(NEBEM_TIMEOUT, "FP64 factorisation: a bounded wait gave up (panel barrier or tensor-core update)");
+    if (h2[0]) return fail(NEBEM_SINGULAR, "zero pivot at column " + std::to_string(h2[0] - 1));
     return NEBEM_OK;
 }
 

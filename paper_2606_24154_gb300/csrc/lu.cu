@@ -9,6 +9,7 @@
 //     apply the panel's swaps to the other columns;
 //     U12 = L11^-1 A12  (explicit inverse of the unit-lower nb x nb block, then a GEMM);
 //     A22 -= L21 U12    (GEMM).
+// A22 -= L21 U12 runs on the tensor cores in both precisions (lu_tc.cu, lu_tc64.cu).
 // Templated on the element type: double (FP64 solves) and float (mixed solves, the
 // FP64 iterative refinement lives in the caller).
 #include <algorithm>
@@ -270,11 +271,30 @@ constexpr int kCoopThreads = 256;
 constexpr int kCoopMaxG = 1024;
 constexpr long long kCoopSpinLimit = 1ll << 22;
 
+// A magnitude as it is compared: FP32 as it is, FP64 by its bits (non-negative doubles order as
+// their bits, and integer compares leave the FP64 pipe alone).  NaN never wins: -1.
+template <typename T>
+struct Mag;
+template <>
+struct Mag<float> {
+    typedef float Key;
+    static __device__ __forceinline__ Key of(float a) { return fabsf(a); }  // NaN fails every compare
+};
+template <>
+struct Mag<double> {
+    typedef long long Key;
+    static __device__ __forceinline__ Key of(double a) {
+        const long long m = __double_as_longlong(a) & 0x7fffffffffffffffll;
+        return m <= 0x7ff0000000000000ll ? m : -1;
+    }
+};
+
+template <typename T>
 struct CoopScratch {
-    float cval[2][kCoopMaxG];
+    typename Mag<T>::Key cval[2][kCoopMaxG];
     int cidx[2][kCoopMaxG];
-    float cand[2][kCoopMaxG][64];
-    float srow[2][64];
+    T cand[2][kCoopMaxG][64];
+    T srow[2][64];
     unsigned int bar[4];  // bar[0]: grid-barrier arrivals of the factorisation
     int err;
 };
@@ -295,7 +315,8 @@ __device__ __forceinline__ int ld_acquire_i(const int* p) {
 // waits until the count reaches `target` (this barrier's total), so one atomic and one
 // polled load make the barrier, and the last arrival publishes everyone's writes (the
 // acquire load that sees the final count synchronises with every add before it).
-__device__ bool coop_barrier(CoopScratch* cs, unsigned int target, bool* s_flag, long long limit) {
+template <typename T>
+__device__ bool coop_barrier(CoopScratch<T>* cs, unsigned int target, bool* s_flag, long long limit) {
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned int v;
@@ -318,15 +339,17 @@ __device__ bool coop_barrier(CoopScratch* cs, unsigned int target, bool* s_flag,
     return *s_flag;
 }
 
+template <typename T>
 __global__ void __launch_bounds__(kCoopThreads, 1)
-    k_panel_coop(float* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
-                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch* cs, unsigned int bar_base,
+    k_panel_coop(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
+                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch<T>* cs, unsigned int bar_base,
                  long long limit) {
+    typedef typename Mag<T>::Key Key;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ld_acquire_i(&cs->err)) return;  // an earlier panel gave up: leave the matrix as it is
     const int w = (int)(k1 - k0);
-    float* S = reinterpret_cast<float*>(smem_raw);  // R x w, column-major
-    __shared__ float prow[64];
+    T* S = reinterpret_cast<T*>(smem_raw);  // R x w, column-major
+    __shared__ T prow[64];
     __shared__ bool s_flag;
     const int G = gridDim.x, b = blockIdx.x;
     const int64_t rb0 = k0 + (int64_t)b * R;
@@ -337,15 +360,15 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     }
     __syncthreads();
     bool ok_piv = true;  // the previous pivot was nonzero
-    __shared__ float wv[kCoopThreads / 32];
+    __shared__ Key wv[kCoopThreads / 32];
     __shared__ int wi[kCoopThreads / 32];
     // (best, index) of the block: warp shuffles, then every thread over the warps' results;
     // the largest value with the lowest index on ties, so the order of the reduction does
     // not matter.  Magnitudes of FP32 values compare exactly in FP32 (no FP64 pipe), row
     // indices fit in 32 bits (n < 2^31).  Every thread returns with the result in (v, ix).
-    auto block_best = [&](float& v, int& ix) {
+    auto block_best = [&](Key& v, int& ix) {
         for (int o = 16; o > 0; o >>= 1) {
-            const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
+            const Key v2 = __shfl_xor_sync(0xffffffffu, v, o);
             const int i2 = __shfl_xor_sync(0xffffffffu, ix, o);
             if (v2 > v || (v2 == v && i2 < ix)) {
                 v = v2;
@@ -371,17 +394,17 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         const int par = jj & 1;
         // (a) + (b): column jj-1 scaled and its rank-1 update applied to this thread's rows
         // below it, then this thread's candidate for column jj from the same rows
-        float best = -1.0f;
+        Key best = (Key)-1;
         int bidx = INT_MAX;
-        const float inv = (jj > 0 && ok_piv) ? 1.0f / prow[jj - 1] : 0.f;
+        const T inv = (jj > 0 && ok_piv) ? (T)1 / prow[jj - 1] : (T)0;
         for (int r = threadIdx.x; r < nr; r += kCoopThreads) {
             if (rb0 + r < j) continue;
             if (jj > 0 && ok_piv) {
-                const float l = S[(jj - 1) * R + r] * inv;
+                const T l = S[(jj - 1) * R + r] * inv;
                 S[(jj - 1) * R + r] = l;
                 for (int c = jj; c < w; ++c) S[c * R + r] -= l * prow[c];
             }
-            const float v = fabsf(S[jj * R + r]);
+            const Key v = Mag<T>::of(S[jj * R + r]);
             if (v > best || (v == best && (int)(rb0 + r) < bidx)) {
                 best = v;
                 bidx = (int)(rb0 + r);
@@ -394,7 +417,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
             cs->cidx[par][b] = mine;
         }
         if (threadIdx.x < w) {
-            cs->cand[par][b][threadIdx.x] = (mine != INT_MAX) ? S[threadIdx.x * R + (int)(mine - rb0)] : 0.f;
+            cs->cand[par][b][threadIdx.x] = (mine != INT_MAX) ? S[threadIdx.x * R + (int)(mine - rb0)] : (T)0;
             if (j >= rb0 && j < rb0 + nr) cs->srow[par][threadIdx.x] = S[threadIdx.x * R + (int)(j - rb0)];
         }
         if (!coop_barrier(cs, bar_base + (unsigned)(jj + 1) * (unsigned)G, &s_flag, limit)) {
@@ -405,10 +428,10 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
             return;
         }
         // (c) the pivot: largest |a| over the candidates, lowest row on ties
-        best = -1.0f;
+        best = (Key)-1;
         bidx = INT_MAX;
         for (int q = threadIdx.x; q < G; q += kCoopThreads) {
-            const float v = __ldcg(&cs->cval[par][q]);
+            const Key v = __ldcg(&cs->cval[par][q]);
             const int ix = __ldcg(&cs->cidx[par][q]);
             if (v > best || (v == best && ix < bidx)) {
                 best = v;
@@ -421,10 +444,10 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         if (threadIdx.x < w) prow[threadIdx.x] = __ldcg(&cs->cand[par][owner][threadIdx.x]);
         if (b == 0 && threadIdx.x == 0) {
             piv[j] = (int32_t)p;
-            if (!(best > 0.0f) && *info == 0) *info = (int)(j + 1);
+            if (!(best > (Key)0) && *info == 0) *info = (int)(j + 1);
         }
         __syncthreads();
-        ok_piv = prow[jj] != 0.f;  // the scaling below is skipped for a zero pivot, as in k_panel_col
+        ok_piv = prow[jj] != (T)0;  // the scaling below is skipped for a zero pivot, as in k_panel_col
         if (threadIdx.x < w) {
             if (j >= rb0 && j < rb0 + nr) S[threadIdx.x * R + (int)(j - rb0)] = prow[threadIdx.x];
             if (p != j && p >= rb0 && p < rb0 + nr)
@@ -434,7 +457,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     }
     // scale the last panel column below the panel
     if (ok_piv) {
-        const float inv = 1.0f / prow[w - 1];
+        const T inv = (T)1 / prow[w - 1];
         for (int r = threadIdx.x; r < nr; r += kCoopThreads)
             if (rb0 + r >= k1) S[(w - 1) * R + r] *= inv;
     }
@@ -748,27 +771,27 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
     const int swap_smem = (int)(sizeof(T) * kSwapMax * kSwapThreads);
     NB_TRY(cudaFuncSetAttribute(k_laswp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, swap_smem));
     if (nb > 64) return cudaErrorInvalidValue;  // k_panel_col stages at most 64 row values
-    // FP32: the whole panel in one cooperative launch when every CTA's rows fit in shared
+    // the whole panel in one cooperative launch when every CTA's rows fit in shared
     // memory (R rows x 64 columns, R = max(64, rows / SMs)) and all CTAs can be resident
     int gmax = 0;
-    CoopScratch* cs = static_cast<CoopScratch*>(coop);
-    if constexpr (sizeof(T) == 4) {
+    CoopScratch<T>* cs = static_cast<CoopScratch<T>*>(coop);
+    if (cs) {
         int dev = 0, sms = 0, can = 0;
-        if (cs && cudaGetDevice(&dev) == cudaSuccess &&
+        if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && can) {
             const int g = std::min(kCoopMaxG, sms);
             const int64_t R0 = std::max<int64_t>(64, (n + g - 1) / g);
-            const int smem0 = (int)(R0 * 64 * sizeof(float));
+            const int64_t smem0 = R0 * 64 * (int64_t)sizeof(T);
             int per_sm = 0;
             if (smem0 <= 200 * 1024 &&
-                cudaFuncSetAttribute(k_panel_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, smem0) ==
+                cudaFuncSetAttribute(k_panel_coop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) ==
                     cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_coop, kCoopThreads, smem0) ==
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_coop<T>, kCoopThreads, (size_t)smem0) ==
                     cudaSuccess &&
                 per_sm >= 1) {
                 gmax = g;
-                NB_TRY(cudaMemsetAsync(cs, 0, sizeof(CoopScratch), s));
+                NB_TRY(cudaMemsetAsync(cs, 0, sizeof(CoopScratch<T>), s));
             }
         }
         cudaGetLastError();  // a refused attribute or query leaves the per-column path
@@ -808,15 +831,15 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                 const int64_t rows = n - k0;
                 const int R = (int)std::max<int64_t>(64, (rows + gmax - 1) / gmax);
                 const int G = (int)((rows + R - 1) / R);
-                float* Af = reinterpret_cast<float*>(A);
+                T* Af = A;
                 int64_t nn = n, kk0 = k0, kk1 = k1;
                 int RR = R;
                 int* tmo = d_info + 1;
                 unsigned int base = arrivals;
                 long long lim = polls > 0 ? polls : kCoopSpinLimit;
                 void* args[] = {&Af, &nn, &kk0, &kk1, &RR, &piv, &d_info, &tmo, &cs, &base, &lim};
-                NB_TRY(cudaLaunchCooperativeKernel((const void*)k_panel_coop, dim3((unsigned)G), dim3(kCoopThreads),
-                                                   args, (size_t)R * w * sizeof(float), s));
+                NB_TRY(cudaLaunchCooperativeKernel((const void*)k_panel_coop<T>, dim3((unsigned)G), dim3(kCoopThreads),
+                                                   args, (size_t)R * w * sizeof(T), s));
                 arrivals += (unsigned int)G * (unsigned int)w;
             } else {
                 // columns k0..k1-1: update by the previous column + pivot of this one; then the
@@ -833,7 +856,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
             k_swap_perm<<<1, 32, 0, s>>>(piv, n, k0, k1, swap_perm);
             k_laswp<T><<<(unsigned)((n + kSwapThreads - 1) / kSwapThreads), kSwapThreads, swap_smem, s>>>(A, n, k0,
                                                                                                     k1, swap_perm);
-            if (super && (k1 < K1 || K1 < n)) {
+            const bool tc64 = sizeof(T) == 8 && split;  // FP64 with the tensor-core update
+            if ((super && (k1 < K1 || K1 < n)) || (tc64 && w == 64 && k1 < n)) {
                 // the panel's unit-lower inverse, kept in its slot for the block row's U12
                 T* slot = Linv + (size_t)((k0 - K0) / nb) * nb * nb;
                 const int tri_smem = (int)(2 * sizeof(T) * w * (w + 1));
@@ -843,7 +867,7 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
             }
             if (k1 < e1) {
                 const int64_t m = n - k1, mc = e1 - k1;
-                if (super)
+                if (super || (tc64 && w == 64))
                     NB_TRY(trsm_block(k0, 1, Linv + (size_t)((k0 - K0) / nb) * nb * nb, k1, e1));
                 else
                     NB_TRY(trsm_rows(k0, w, k1, e1));
@@ -856,6 +880,10 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                                              reinterpret_cast<float*>(A + k1 + k1 * n), n, split, d_info + 1, s));
                         continue;
                     }
+                } else if (tc64) {
+                    NB_TRY(tc_update_f64(m, mc, w, A + k1 + k0 * n, n, A + k0 + k1 * n, n, A + k1 + k1 * n, n, split,
+                                         d_info + 1, s));
+                    continue;
                 }
                 NB_TRY(gemm<T>(m, mc, w, (T)-1, A + k1 + k0 * n, n, A + k0 + k1 * n, n, (T)1, A + k1 + k1 * n, n, s));
             }
@@ -1518,14 +1546,27 @@ size_t lu_work_elems(int64_t n, int nb) {
            (2 * kSwapMax + 16);
 }
 
-cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, double* work, int* d_info, cudaStream_t s) {
+cudaError_t lu_factor_f64_small(double* A, int64_t n, int32_t* piv, int nb, double* work, int* d_info,
+                                cudaStream_t s) {
     return lu_factor<double>(A, n, piv, nb, work, d_info, nullptr, nullptr, s, 0);
+}
+static size_t digits_offset(int64_t n, int nb) { return (sizeof(double) * lu_work_elems(n, nb) + 255) & ~(size_t)255; }
+static size_t coop64_offset(int64_t n, int nb) {
+    return (digits_offset(n, nb) + tc64_work_bytes(n, n) + 255) & ~(size_t)255;
+}
+size_t lu_work_bytes_f64(int64_t n, int nb) { return coop64_offset(n, nb) + sizeof(CoopScratch<double>); }
+cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, void* work, int* d_info, cudaStream_t s) {
+    // work: panel staging, then the digits of the tensor-core update, then the cooperative
+    // panel's candidates and barrier
+    char* w = static_cast<char*>(work);
+    return lu_factor<double>(A, n, piv, nb, reinterpret_cast<double*>(w), d_info, w + digits_offset(n, nb),
+                             w + coop64_offset(n, nb), s, 0);
 }
 static size_t split_offset(int64_t n, int nb) { return (sizeof(float) * lu_work_elems(n, nb) + 255) & ~(size_t)255; }
 static size_t coop_offset(int64_t n, int nb) {
     return (split_offset(n, nb) + tc_split_bytes(n, n, kSuperPanels) + 255) & ~(size_t)255;
 }
-size_t lu_work_bytes_f32(int64_t n, int nb) { return coop_offset(n, nb) + sizeof(CoopScratch); }
+size_t lu_work_bytes_f32(int64_t n, int nb) { return coop_offset(n, nb) + sizeof(CoopScratch<float>); }
 cudaError_t lu_factor_f32(float* A, int64_t n, int32_t* piv, int nb, float* work, int* d_info, cudaStream_t s,
                           long long polls) {
     // work: lu_work_bytes_f32(n, nb) bytes, 256-byte aligned: panel staging, then the

@@ -56,8 +56,8 @@ extern "C" int nebem_lu_factor_device_noalloc(double* d_A, int64_t n, int32_t* d
     if (rc) return rc;
     int* info = reinterpret_cast<int*>(scratch + kWorkDoubles);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = lu_factor_f64(d_A, n, d_piv, kNoAllocBlock, scratch, info, s);  // clears the flag first
-    if (e != cudaSuccess) return cuda_fail(e, "lu_factor_f64");
+    cudaError_t e = lu_factor_f64_small(d_A, n, d_piv, kNoAllocBlock, scratch, info, s);  // clears the flag first
+    if (e != cudaSuccess) return cuda_fail(e, "lu_factor_f64_small");
     int h_info = 0;
     e = cudaMemcpyAsync(&h_info, info, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

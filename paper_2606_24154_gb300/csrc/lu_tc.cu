@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "nb_internal.h"
+#include "tcgen05.cuh"
 
 namespace nb {
 
@@ -36,12 +37,7 @@ constexpr uint32_t kSBO = (kTK / 4) * kCoreBytes;    // next 8-row group: 2048 B
 constexpr uint32_t kABytes = kTM * kTK * 4;          // 32 KB per A operand tile
 constexpr uint32_t kBBytes = kTN * kTK * 4;          // 16 KB per B operand tile
 constexpr uint32_t kSmemBytes = 2 * kABytes + 2 * kBBytes + 64;
-constexpr long long kSpinLimit = 1ll << 24;
 constexpr int kTilesN = 4;                           // 64-column tiles of C per CTA
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 
 // byte offset of element (row r, k) in a K-major non-swizzled operand tile
 __device__ __forceinline__ uint32_t kmajor_off(int r, int k) {
@@ -271,31 +267,6 @@ constexpr uint32_t kBSplit = 2 * kBBytes;            // 32 KB per 64-column oper
 constexpr uint32_t kCTile = kTM * kTN * 4;           // 32 KB
 constexpr uint32_t kBulkSmem = kASplit + 2 * kBSplit + 2 * kCTile + 128;
 
-__device__ __forceinline__ void mbar_init(uint64_t* b) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(b)));
-}
-__device__ __forceinline__ void mbar_expect(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-// bounded wait for completion `parity` of barrier b; 1 = completed
-__device__ __forceinline__ int mbar_wait(uint64_t* b, uint32_t parity) {
-    uint32_t done = 0;
-    for (long long it = 0; it < kSpinLimit && !done; ++it) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(smem_u32(b)), "r"(parity)
-            : "memory");
-    }
-    return (int)done;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(b))
-        : "memory");
-}
 __device__ __forceinline__ void tma_reduce_add_c(const CUtensorMap* map, int x, int y, const void* src) {
     asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
                      reinterpret_cast<uint64_t>(map)),

@@ -88,15 +88,18 @@ int ensure_factors(Ctx* c, int precision, double* ms) {
         if (c->fac64_valid) return 0;
         CK(c->d_LU64.ensure(sizeof(double) * n * n));
         CK(c->d_piv64.ensure(sizeof(int32_t) * n));
-        CK(c->d_work.ensure(sizeof(double) * lu_work_elems(n, nb)));
+        CK(c->d_work.ensure(lu_work_bytes_f64(n, nb)));
         CK(c->d_small.ensure(256));
         CK(cudaEventRecord(c->ev0, c->stream));
         CK(cudaMemcpyAsync(c->d_LU64.ptr, c->d_K.ptr, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, c->stream));
-        CK(lu_factor_f64(c->d_LU64.as<double>(), n, c->d_piv64.as<int32_t>(), nb, c->d_work.as<double>(),
+        CK(lu_factor_f64(c->d_LU64.as<double>(), n, c->d_piv64.as<int32_t>(), nb, c->d_work.ptr,
                          c->d_small.as<int>(), c->stream));
         int rc = elapsed_ms(c, ms);
         if (rc) return rc;
-        CK(cudaMemcpy(&h_info, c->d_small.ptr, sizeof(int), cudaMemcpyDeviceToHost));
+        int h2[2] = {0, 0};
+        CK(cudaMemcpy(h2, c->d_small.ptr, sizeof(h2), cudaMemcpyDeviceToHost));
+        h_info = h2[0];
+        if (h2[1]) return fail(NEBEM_TIMEOUT, "FP64 factorisation: a bounded wait gave up (panel barrier or tensor-core update)");
         if (h_info) return fail(NEBEM_SINGULAR, "zero pivot at column " + std::to_string(h_info - 1));
         CK(c->d_perm64.ensure(sizeof(int32_t) * n));
         CK(lu_make_perm(c->d_piv64.as<int32_t>(), n, c->d_perm64.as<int32_t>(), c->stream));
