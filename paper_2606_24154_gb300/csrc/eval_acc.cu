@@ -46,7 +46,7 @@ namespace nb {
 namespace {
 
 constexpr int kAT = 128;             // threads (flagged points) per block
-constexpr int kATBlocks = 4;         // resident far blocks per SM (128 registers a thread)
+constexpr int kATBlocks = 5;         // resident far blocks per SM (96 registers a thread)
 constexpr double kErrGammaR = 1e-7;   // FP32 pass: share of the result
 constexpr double kErrGammaB = 7e-8;   // FP32 pass: share of B
 constexpr double kErrGammaS = 5e-7;   // FP32 pass: share of S
@@ -143,45 +143,216 @@ __device__ __forceinline__ void df_fma_acc(float ah, float al, float bh, float b
     Sl = __fadd_rn(Sl, __fadd_rn(t2, l));
 }
 
-// Two levels of re-evaluation, both two-float: level 1 takes the tiers of the FP32 pass
-// (nb_internal.h FarNodes: 2x2 / 4-point, 3x3 / 6-point, 4x4, 6x6 rules at ratio_0, ratio_a,
-// ratio_b, ratio_near radii; FP64 closed forms nearer), whose truncation stays near 1e-10 of
-// B; level 2 takes the fill's tiers (truncation below ~3e-12 of each pair, FP64 within
-// kFillRatioC radii).  Staged in shared memory per element: the level's most frequent node
-// set (tier 0 for level 1, tier a for level 2) and, for level 1, the tier radii.
-template <int L>
-struct Level;
-template <>
-struct Level<1> {
-    static constexpr int kStaged = 4 * kFillPairs0;  // float4 of the staged node set
-    static constexpr int kStagedOff = kFillOff0;
-    static constexpr int kHdr = 1;                   // FarNodes radii per element
-};
-template <>
-struct Level<2> {
-    static constexpr int kStaged = 4 * kFillPairsA;
-    static constexpr int kStagedOff = 0;
-    static constexpr int kHdr = 0;
-};
-
-// dynamic shared memory per tile of te elements: FillEl (9 float4), the staged node set,
-// tau and image centroids (2 float4 each per image), the level-1 tier radii
-__host__ __device__ constexpr int acc_tile_f4(int te, int nimg, int staged, int hdr) {
-    return te * (9 + staged + 4 * nimg + hdr);
+// Two levels of re-evaluation, both two-float: level 1 takes the pairs from kMomRatio radii on by
+// their moments (mom_pair2) and the nearer ones by the tiers of the FP32 pass (nb_internal.h
+// FarNodes: 3x3 / 6-point, 4x4, 6x6 rules at ratio_a, ratio_b, ratio_near radii; FP64 closed forms
+// nearer); its truncation stays near 1e-10 of B.  Level 2 takes the fill's tiers (truncation below
+// ~3e-12 of each pair, FP64 within kFillRatioC radii).
+//
+// dynamic shared memory per tile of te elements.  Level 1: FillEl (9 float4), the moments, the tier
+// radii, and tau as six planes of nimg (padded to even) floats (x, y, z negated: hi, then lo).
+// Level 2: FillEl, the tier-a nodes, tau and image centroids (2 float4 each per image).
+__host__ __device__ constexpr int acc_pad(int nimg) { return (nimg + 1) & ~1; }
+__host__ __device__ constexpr int acc_tile_f4(int level, int te, int nimg) {
+    return level == 1 ? te * (9 + kMomF4 + 1) + (te * 6 * acc_pad(nimg) + 3) / 4
+                      : te * (9 + 4 * kFillPairsA + 4 * nimg);
 }
 
-// Raw sums (before ke) of the far pairs of one point over the elements [e0, e1) at level L,
+// One pair that level 1 does not take by moments, by its tier's nodes: Phi' and E' (local) added to the
+// element's FP64 sums.  About one pair in a hundred; kept out of line and out of the image loop, whose
+// registers it would otherwise crowd.
+template <int M>
+__device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr, int na, int64_t j, int nimg, int k,
+                                            const float (&ph)[3], const float (&pl)[3], float x0h, float x0l, float y0h,
+                                            float y0l, float z0h, float z0l, const float* __restrict__ tau, int np2,
+                                            double& fphi, double& lx, double& ly, double& lz) {
+    const int64_t jk = j * nimg + k;
+    float dx, dy, dz;
+    const float d2 = pair_d2(ph[0], ph[1], ph[2], pl[0], pl[1], pl[2], A.cjk[2 * jk], A.cjk[2 * jk + 1], dx, dy, dz);
+    if (!(d2 >= hdr.w)) return;  // near pair: the FP64 kernel
+    const float4* nd = A.nodes + j * kFillNodeRec;
+    int np = na;
+    if (!(d2 >= hdr.y)) {
+        const bool b = d2 >= hdr.z;
+        nd += b ? kFillOffB : kFillOffC;
+        np = b ? kFillPairsB : kFillPairsC;
+    }
+    float xh, xl, yh, yl, zh, zl, d2h, d2l;
+    df_sub(x0h, x0l, -tau[k], -tau[3 * np2 + k], xh, xl);
+    df_sub(y0h, y0l, -tau[np2 + k], -tau[4 * np2 + k], yh, yl);
+    df_sub(z0h, z0l, -tau[2 * np2 + k], -tau[5 * np2 + k], zh, zl);
+    df_norm2(xh, xl, yh, yl, zh, zl, d2h, d2l);
+    PairDF2 P;
+    P.xh = bc2(xh), P.nxh = bc2(-xh), P.xl = bc2(xl);
+    P.zh = bc2(zh), P.nzh = bc2(-zh), P.zl = bc2(zl);
+    P.d2h = bc2(d2h), P.d2l = bc2(d2l);
+    PairSums2 S{bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
+    float2 sh = bc2(0.f), snl = bc2(0.f);
+    nodes_acc2<M>(nd, np, P, sh, snl, S);
+    auto sum = [](const float2& h, const float2& nl) {
+        return ((double)h.x - (double)nl.x) + ((double)h.y - (double)nl.y);
+    };
+    if constexpr (M != kEOnly) fphi += sum(sh, snl);
+    if constexpr (M != kPhiOnly) {
+        const double s0 = sum(S.s0, S.ns0);
+        lx = fma((double)xh + (double)xl, s0, fma(0.5, sum(S.sx, S.nsx), lx));
+        ly = fma((double)yh + (double)yl, s0, ly);
+        lz = fma((double)zh + (double)zl, s0, fma(0.5, sum(S.sz, S.nsz), lz));
+    }
+}
+
+// Level 1, 1e6 points of the 9,996-element cell x 25 copies (320,000 of them refined): 1,490 ms with
+// every pair by Gauss nodes in two-float arithmetic, 629 ms so, with an error 10 to 25 times smaller
+// (E: 2.0e-10 B before, 1.7e-11 B now, the largest of 665 refined points).  The FP32 pipe is busy for
+// about two thirds of it; 5 blocks per SM (96 registers) beat 4 by 3 %, 6 are the same.
+//
+// Raw sums (before ke) of the far pairs of one point over the elements [e0, e1) at level 1,
 // with the error scales, of phi and E (M = kBoth), phi only or E only (the other sums stay
 // 0); all threads of the block take part (tiles).
-template <int L, int M>
-__device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
+template <int M>
+__device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
+                                           const float (&pl)[3], int64_t e0, int64_t e1) {
+    FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
+    float4* s_mom = sm + 9 * te;
+    float4* s_hdr = s_mom + kMomF4 * te;
+    float* s_tau = reinterpret_cast<float*>(s_hdr + te);
+    const int np2 = acc_pad(nimg);
+    Sum6 acc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    float bphi = 0.f, bE = 0.f;  // the leaf's error scales
+    for (int64_t base = e0; base < e1; base += te) {
+        const int cnt = (int)min((int64_t)te, e1 - base);
+        __syncthreads();
+        {
+            const float4* src = reinterpret_cast<const float4*>(A.fe + base);
+            float4* dst = reinterpret_cast<float4*>(s_fe);
+            for (int i = threadIdx.x; i < 9 * cnt; i += blockDim.x) dst[i] = src[i];
+        }
+        for (int i = threadIdx.x; i < kMomF4 * cnt; i += blockDim.x) s_mom[i] = A.mom[base * kMomF4 + i];
+        for (int i = threadIdx.x; i < cnt; i += blockDim.x) s_hdr[i] = A.far[base + i].hdr;
+        for (int i = threadIdx.x; i < cnt * np2; i += blockDim.x) {
+            const int jj = i / np2, k = min(i - jj * np2, nimg - 1);
+            const float4 h = A.tau[2 * ((base + jj) * nimg + k)], l = A.tau[2 * ((base + jj) * nimg + k) + 1];
+            float* d = s_tau + jj * 6 * np2 + (i - jj * np2);
+            d[0] = -h.x, d[np2] = -h.y, d[2 * np2] = -h.z;
+            d[3 * np2] = -l.x, d[4 * np2] = -l.y, d[5 * np2] = -l.z;
+        }
+        __syncthreads();
+        for (int jj = 0; jj < cnt; ++jj) {
+            const FillEl& F = s_fe[jj];
+            const int64_t j = base + jj;
+            const float4 hdr = s_hdr[jj];
+            // squared distance from which the moments are taken; never inside the near radius, which
+            // the two classifications of a pair (here and in the near kernel) round differently
+            const float mom2 = fmaxf(F.hdr.x * (float)(kMomRatio * kMomRatio / (kFillRatioA * kFillRatioA)),
+                                     hdr.w * 1.0001f);
+            float dh[3], dl[3];
+            df_sub(ph[0], pl[0], F.ch.x, F.cl.x, dh[0], dl[0]);
+            df_sub(ph[1], pl[1], F.ch.y, F.cl.y, dh[1], dl[1]);
+            df_sub(ph[2], pl[2], F.ch.z, F.cl.z, dh[2], dl[2]);
+            float x0h, x0l, y0h, y0l, z0h, z0l;
+            df_dot3(dh, dl, F.exh, F.exl, x0h, x0l);
+            df_dot3(dh, dl, F.eyh, F.eyl, y0h, y0l);
+            df_dot3(dh, dl, F.ezh, F.ezl, z0h, z0l);
+            MomSum2 S{};
+            double fphi = 0.0, lx = 0.0, ly = 0.0, lz = 0.0;  // the nearer pairs
+            const float* tau = s_tau + jj * 6 * np2;
+            uint32_t nearer = 0;  // images of the group of 32 at hand whose pair is not taken by moments
+            for (int k = 0; k < np2; k += 2) {
+                auto plane = [&](int q) { return *reinterpret_cast<const float2*>(tau + q * np2 + k); };
+                // X = X0 - tau, two floats
+                auto diff = [&](float ah, float al, int q, float2& h, float2& l) {
+                    float2 t;
+                    two_sum2(bc2(ah), plane(q), h, t);
+                    l = __fadd2_rn(t, __fadd2_rn(bc2(al), plane(q + 3)));
+                };
+                float2 xh, xl, yh, yl, zh, zl;
+                diff(x0h, x0l, 0, xh, xl);
+                diff(y0h, y0l, 1, yh, yl);
+                diff(z0h, z0l, 2, zh, zl);
+                const float2 m1 = bc2(-1.f);
+                float2 px = __fmul2_rn(xh, xh), py = __fmul2_rn(yh, yh), pz = __fmul2_rn(zh, zh);
+                float2 ex = __ffma2_rn(xh, xh, make_float2(-px.x, -px.y)), ey = __ffma2_rn(yh, yh, make_float2(-py.x, -py.y)),
+                       ez = __ffma2_rn(zh, zh, make_float2(-pz.x, -pz.y));
+                ex = __ffma2_rn(__fadd2_rn(xh, xh), xl, ex);
+                ey = __ffma2_rn(__fadd2_rn(yh, yh), yl, ey);
+                ez = __ffma2_rn(__fadd2_rn(zh, zh), zl, ez);
+                float2 s, t1, t2, d2h;
+                two_sum2(px, py, s, t1);
+                two_sum2(s, pz, d2h, t2);
+                const float2 d2l = __fadd2_rn(__fadd2_rn(ex, ey), __fadd2_rn(ez, __fadd2_rn(t1, t2)));
+                const bool two = k + 1 < nimg;
+                const bool far0 = d2h.x >= mom2, far1 = two && d2h.y >= mom2;
+                mom_pair2<M != kEOnly, M != kPhiOnly>(s_mom + kMomF4 * jj, xh, xl, yh, yl, zh, zl, d2h, d2l, far0,
+                                                      far1, S);
+                nearer |= ((far0 ? 0u : 1u) | (far1 || !two ? 0u : 2u)) << (k & 31);
+                if ((k & 31) == 30 || k + 2 >= np2) {
+                    for (uint32_t m = nearer; m; m &= m - 1) {
+                        const int kk = (k & ~31) + __ffs(m) - 1;
+                        acc_pair_nodes<M>(A, hdr, (int)F.hdr.w, j, nimg, kk, ph, pl, x0h, x0l, y0h, y0l, z0h, z0l, tau,
+                                          np2, fphi, lx, ly, lz);
+                    }
+                    nearer = 0;
+                }
+            }
+            // element j: A x (sum over the images) + the other terms as two floats, then FP64:
+            // rotated to the global frame and weighted by sigma_j.  A conversion takes the FP64 pipe
+            // like an addition does, so each quantity crosses over once, as two values; the
+            // error scales stay in FP32.
+            const double s = A.sigma[j];
+            const float4 tail = s_mom[kMomF4 * jj + kMomF4 - 1];
+            // sign: -1 where the high parts are kept negated
+            auto total = [&](float sign, const float2& h, const float2& l, const float2& c, float& oh, float& ol) {
+                float sh, t, p, e;
+                two_sum(h.x, h.y, sh, t);
+                sh *= sign;
+                const float sl = __fmaf_rn(sign, t, __fadd_rn(l.x, l.y));
+                two_prod(sh, tail.z, p, e);
+                e = __fmaf_rn(sh, tail.w, __fmaf_rn(sl, tail.z, e));
+                oh = p;
+                ol = __fadd_rn(e, __fadd_rn(c.x, c.y));
+            };
+            if constexpr (M != kEOnly) {
+                float h, l;
+                total(1.f, S.ph, S.pl, S.fc, h, l);
+                fphi += (double)h + (double)l;
+                acc.phi = fma(s, fphi, acc.phi);
+                bphi = fmaf(fabsf((float)s), fabsf((float)fphi), bphi);
+            }
+            if constexpr (M != kPhiOnly) {
+                float h, l;
+                total(-1.f, S.xh, S.xl, S.ex, h, l);
+                lx += (double)h + (double)l;
+                total(-1.f, S.yh, S.yl, S.ey, h, l);
+                ly += (double)h + (double)l;
+                total(-1.f, S.zh, S.zl, S.ez, h, l);
+                lz += (double)h + (double)l;
+                const Elem& e = A.el[j];
+                const double gx = fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0]));
+                const double gy = fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1]));
+                const double gz = fma(lx, e.ex[2], fma(ly, e.ey[2], lz * e.ez[2]));
+                acc.x = fma(s, gx, acc.x);
+                acc.y = fma(s, gy, acc.y);
+                acc.z = fma(s, gz, acc.z);
+                bE = fmaf(fabsf((float)s), fabsf((float)gx) + fabsf((float)gy) + fabsf((float)gz), bE);
+            }
+        }
+    }
+    acc.bphi = (double)bphi;
+    acc.bE = (double)bE;
+    return acc;
+}
+
+// Raw sums (before ke) of the far pairs of one point over the elements [e0, e1) at level 2,
+// with the error scales, of phi and E (M = kBoth), phi only or E only (the other sums stay
+// 0); all threads of the block take part (tiles).
+template <int M>
+__device__ __forceinline__ Sum6 acc_range2(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
                                           const float (&pl)[3], int64_t e0, int64_t e1) {
-    using Lv = Level<L>;
+    constexpr int kStaged = 4 * kFillPairsA;
     FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
     float4* s_na = sm + 9 * te;
-    float4* s_tau = s_na + Lv::kStaged * te;
+    float4* s_tau = s_na + kStaged * te;
     float4* s_c = s_tau + 2 * nimg * te;
-    float4* s_hdr = s_c + 2 * nimg * te;
     Sum6 acc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int64_t base = e0; base < e1; base += te) {
         const int cnt = (int)min((int64_t)te, e1 - base);
@@ -191,23 +362,21 @@ __device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, fl
             float4* dst = reinterpret_cast<float4*>(s_fe);
             for (int i = threadIdx.x; i < 9 * cnt; i += blockDim.x) dst[i] = src[i];
         }
-        for (int e = threadIdx.x; e < cnt * Lv::kStaged; e += blockDim.x) {
-            const int jj = e / Lv::kStaged, q = e - jj * Lv::kStaged;
-            s_na[e] = A.nodes[(base + jj) * kFillNodeRec + Lv::kStagedOff + q];
+        for (int e = threadIdx.x; e < cnt * kStaged; e += blockDim.x) {
+            const int jj = e / kStaged, q = e - jj * kStaged;
+            s_na[e] = A.nodes[(base + jj) * kFillNodeRec + q];
         }
         for (int i = threadIdx.x; i < 2 * cnt * nimg; i += blockDim.x) {
             s_tau[i] = A.tau[2 * base * nimg + i];
             s_c[i] = A.cjk[2 * base * nimg + i];
         }
-        if (Lv::kHdr)
-            for (int i = threadIdx.x; i < cnt; i += blockDim.x) s_hdr[i] = A.far[base + i].hdr;
         __syncthreads();
         for (int jj = 0; jj < cnt; ++jj) {
             const FillEl& F = s_fe[jj];
             const int64_t j = base + jj;
             // squared tier radii, largest first, and the nearest (FP64) radius
-            const float4 hdr = Lv::kHdr ? s_hdr[jj] : F.hdr;
-            const float near2 = Lv::kHdr ? hdr.w : hdr.z;
+            const float4 hdr = F.hdr;
+            const float near2 = hdr.z;
             const int na = (int)F.hdr.w;
             float dh[3], dl[3];
             df_sub(ph[0], pl[0], F.ch.x, F.cl.x, dh[0], dl[0]);
@@ -237,12 +406,9 @@ __device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, fl
                 const float4* nd;
                 int np;
                 if (d2 >= hdr.x) {  // the staged set
-                    nd = s_na + jj * Lv::kStaged;
-                    np = (L == 1) ? kFillPairs0 : na;
-                } else if (L == 1 && d2 >= hdr.y) {
-                    nd = A.nodes + j * kFillNodeRec;
+                    nd = s_na + jj * kStaged;
                     np = na;
-                } else if (d2 >= (L == 1 ? hdr.z : hdr.y)) {
+                } else if (d2 >= hdr.y) {
                     nd = A.nodes + j * kFillNodeRec + kFillOffB;
                     np = kFillPairsB;
                 } else {
@@ -318,7 +484,10 @@ __device__ __forceinline__ Sum6 acc_sum(const AccView& A, int nimg, int te, floa
         const int64_t c1 = min(c0 + (int64_t)kChunkEl, e1);
         Sum6 ch{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         for (int64_t l = c0; l < c1; l += kLeafEl)
-            add_sum(ch, acc_range<L, M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
+            if constexpr (L == 1)
+                add_sum(ch, acc_range1<M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
+            else
+                add_sum(ch, acc_range2<M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
         add_sum(tot, ch);
     }
     return tot;
@@ -452,11 +621,10 @@ template <int L, int M>
 cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* pts, int64_t npts, double* phi,
                          double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list, int sms,
                          Sum6* part, cudaStream_t s) {
-    using Lv = Level<L>;
     // element tile: a power of two (divides the chunk width), at most 16, within ~40 KB
-    int te = 16;
-    while (te > 1 && acc_tile_f4(te, img.n, Lv::kStaged, Lv::kHdr) * (int)sizeof(float4) > 40 * 1024) te /= 2;
-    const size_t smem = (size_t)acc_tile_f4(te, img.n, Lv::kStaged, Lv::kHdr) * sizeof(float4);
+    int te = L == 1 ? kLeafEl : 16;
+    while (te > 1 && acc_tile_f4(L, te, img.n) * (int)sizeof(float4) > 40 * 1024) te /= 2;
+    const size_t smem = (size_t)acc_tile_f4(L, te, img.n) * sizeof(float4);
     const int64_t gb = kATBlocks * (int64_t)sms, want = (npts + kAT - 1) / kAT;
     const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
     cudaError_t e =
@@ -479,7 +647,50 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
     return cudaGetLastError();
 }
 
+// ElemMom records (twofloat.cuh) from the elements' 36-node rules, which integrate degree 4 exactly.
+__global__ void k_elem_moments(const float4* __restrict__ nodes, int64_t n, float4* __restrict__ mom) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const float4* nd = nodes + j * kFillNodeRec + kFillOffC;
+    double A = 0.0, M2[3] = {}, M3[4] = {}, M4[5] = {};
+    for (int q = 0; q < kFillPairsC; ++q) {
+        const float4 h0 = nd[4 * q], h1 = nd[4 * q + 1], l0 = nd[4 * q + 2], l1 = nd[4 * q + 3];
+        for (int lane = 0; lane < 2; ++lane) {
+            // u = node - centroid = -s, stored as 2 s
+            const double x = -0.5 * (lane ? (double)h0.y + (double)l0.y : (double)h0.x + (double)l0.x);
+            const double z = -0.5 * (lane ? (double)h0.w + (double)l0.w : (double)h0.z + (double)l0.z);
+            const double w = lane ? (double)h1.w + (double)l1.w : (double)h1.z + (double)l1.z;
+            A += w;
+            M2[0] += w * x * x, M2[1] += w * x * z, M2[2] += w * z * z;
+            M3[0] += w * x * x * x, M3[1] += w * x * x * z, M3[2] += w * x * z * z, M3[3] += w * z * z * z;
+            M4[0] += w * x * x * x * x, M4[1] += w * x * x * x * z, M4[2] += w * x * x * z * z;
+            M4[3] += w * x * z * z * z, M4[4] += w * z * z * z * z;
+        }
+    }
+    const double t2 = M2[0] + M2[2], q0 = 0.375 * (M4[0] + 2 * M4[2] + M4[4]);
+    const double c[22] = {3 * M2[0], 3 * M2[1], 3 * M2[2], -0.5 * t2,
+                          7.5 * M3[0], 7.5 * M3[1], 7.5 * M3[2], 7.5 * M3[3],
+                          -1.5 * (M3[0] + M3[2]), -1.5 * (M3[1] + M3[3]),
+                          17.5 * M4[0], 17.5 * M4[1], 17.5 * M4[3], 17.5 * M4[4], 52.5 * M4[1], 52.5 * M4[2],
+                          52.5 * M4[3], -7.5 * (M4[0] + M4[2]), -7.5 * (M4[1] + M4[3]), -7.5 * (M4[2] + M4[4]),
+                          q0, 5 * q0};
+    float4* out = mom + j * kMomF4;
+    for (int q = 0; q < kMomF4 - 1; ++q) {
+        const float a = (float)c[2 * q], b = (float)c[2 * q + 1];
+        out[q] = make_float4(a, a, b, b);
+    }
+    const float t3 = (float)(-1.5 * t2), ah = (float)A;
+    out[kMomF4 - 1] = make_float4(t3, t3, ah, (float)(A - (double)ah));
+}
+
 }  // namespace
+
+size_t elem_moments_bytes(int64_t n) { return sizeof(float4) * kMomF4 * (size_t)n; }
+cudaError_t launch_elem_moments(const float4* nodes, int64_t n, float4* mom, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    k_elem_moments<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(nodes, n, mom);
+    return cudaGetLastError();
+}
 
 ErrModel default_err_model() { return ErrModel{kErrGammaR, kErrGammaB, kErrGammaS}; }
 

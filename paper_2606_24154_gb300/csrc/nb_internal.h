@@ -83,13 +83,9 @@ constexpr double kFillRatioC = 6.0;
 constexpr int kFillPairsA = 5;  // capacity (3 used by triangles)
 constexpr int kFillPairsB = 8;
 constexpr int kFillPairsC = 18;
-// tier 0 of the mixed evaluation (2x2 / 4-point rule) in the same two-float form, appended
-// for the two-float re-evaluation of eval_acc.cu (the fill does not use it)
-constexpr int kFillPairs0 = 2;
 constexpr int kFillOffB = 4 * kFillPairsA;
 constexpr int kFillOffC = 4 * (kFillPairsA + kFillPairsB);
-constexpr int kFillOff0 = 4 * (kFillPairsA + kFillPairsB + kFillPairsC);
-constexpr int kFillNodeRec = kFillOff0 + 4 * kFillPairs0;  // float4 per element
+constexpr int kFillNodeRec = 4 * (kFillPairsA + kFillPairsB + kFillPairsC);  // float4 per element
 // Per element: centroid c and frame (ex, ey, ez) as hi + lo floats; hdr = squared tier
 // distances (a, b, c) in m^2 and the tier-a node-pair count.
 struct __align__(16) FillEl {
@@ -173,6 +169,7 @@ struct AccView {
     const FarNodes* far;
     const FillEl* fe;
     const float4* nodes;
+    const float4* mom;  // elem_moments_bytes: planar moments (ElemMom of twofloat.cuh)
     const float4* tau;
     const float4* cjk;
     const double* sigma;
@@ -198,6 +195,8 @@ ErrModel default_err_model();
 cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const double* pts, int64_t npts,
                                double* phi, double* E, double* err, double tol, const ErrModel& em,
                                const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part);
+size_t elem_moments_bytes(int64_t n);
+cudaError_t launch_elem_moments(const float4* nodes, int64_t n, float4* mom, cudaStream_t s);
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_pair_tiers(const FarNodes* far, const float4* cjk, int64_t n_el, int nimg, const double* pts,
                               int64_t npts, uint8_t* codes, cudaStream_t s);

@@ -51,6 +51,8 @@ int ensure_fill_tables(Ctx* c) {
                        cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->d_fill_cell_items.ptr, cell_items.data(), sizeof(int32_t) * cell_items.size(),
                        cudaMemcpyHostToDevice, c->stream));
+    CK(c->d_fill_mom.ensure(elem_moments_bytes(c->n)));
+    CK(launch_elem_moments(c->d_fill_nodes.as<float4>(), c->n, c->d_fill_mom.as<float4>(), c->stream));
     CK(cudaStreamSynchronize(c->stream));  // the host vectors go out of scope
     c->fill_tables = true;
     return 0;
@@ -384,6 +386,7 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
             A.el = c->d_el.as<Elem>();
             A.fe = c->d_fill_el.as<FillEl>();
             A.nodes = c->d_fill_nodes.as<float4>();
+            A.mom = c->d_fill_mom.as<float4>();
             A.tau = c->d_fill_tau.as<float4>();
             A.cjk = c->d_cjk.as<float4>();
             A.sigma = c->d_sigma.as<double>();

@@ -127,4 +127,130 @@ __device__ __forceinline__ void node_rinv2(const PairDF2& P, const float4& q0, c
     nyl = __fmul2_rn(__fmul2_rn(bc2(-0.5f), y0), h);
 }
 
+// ---------------------------------------------------------------- far pairs by moments
+// A pair far from its element (d >= kMomRatio radii) by the element's planar moments about its
+// centroid, two images per packed instruction.  With n = D / d, y = 1 / d,
+//   Phi' = A y + y^3 (f2 + y f3 + y^2 f4),   E' = A D y^3 + y^4 [(r2 + y r3 + y^2 r4) n - (w2 + y w3 + y^2 w4)],
+// the monopole and the terms of degree 2 to 4 of the multipole series of 1 / |D - u| over the
+// element's points u (degree 1 vanishes about the centroid).  Only the monopole needs two-float
+// arithmetic: the rest is below (rho / d)^2 / 5 of the pair, so plain FP32 leaves an error of about
+// 1e-7 of that (1e-11 of the pair at 64 radii).  190 FP32 lane operations per pair for Phi' and E' (124
+// for Phi' alone) and one MUFU root, where four Gauss nodes in two-float arithmetic took 549
+// (283) and four roots, six 743 and nine 1131.  What the series leaves out (odd moments of a
+// triangle: degree 5) is 2.8e-9 of the pair at 24 radii, where the 6-point rule has 1.9e-9, 1.3e-9 at
+// kMomRatio = 28, and 2e-11 at 64 radii, where the 4-point rules have 3e-9 (worst over triangles,
+// slivers, 10:1 strips and skewed quadrilaterals, 400 directions).
+// ElemMom per element: every constant twice (both lanes), two constants per float4:
+//   3 M20, 3 M11 | 3 M02, -t2 / 2 | k30, k21 | k12, k03 | -tx, -tz | K40, K31 | K13, K04 | T31, T22 | T13, P20 |
+//   P11, P02 | q0, 5 q0 | -3 t2 / 2, then the area A as hi, lo
+// with M the moments of u = node - centroid in the element plane, t2 = M20 + M02, k = 7.5 M, (tx, tz) = 1.5
+// (M30 + M12, M21 + M03), K = 17.5 M, T = 3 K, P = -7.5 (M40 + M22, M31 + M13, M22 + M04), q0 = 0.375 (M40 +
+// 2 M22 + M04).
+constexpr double kMomRatio = 28.0;
+constexpr int kMomF4 = 12;
+
+struct MomSum2 {  // sums over the images of an element, both lanes
+    float2 ph, pl;                        // y, two floats (times A: the monopole's potential)
+    float2 xh, xl, yh, yl, zh, zl;        // D y^3, two floats: minus the high part, the low part
+    float2 fc, ex, ey, ez;                // the other terms, FP32
+};
+
+__device__ __forceinline__ float2 lane2(const float4& v, int i) {
+    return i ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+}
+
+// One step: local differences X, Y, Z (two floats each) of two images; lanes with far = false add 0.
+// Returns nothing for them: the caller evaluates those pairs itself.  d2h is |D|^2's high part.
+template <bool kPhi, bool kField>
+__device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float2 xh, float2 xl, float2 yh, float2 yl,
+                                          float2 zh, float2 zl, float2 d2h, float2 d2l, bool far0, bool far1,
+                                          MomSum2& S) {
+    const float2 m1 = bc2(-1.f);
+    const float2 y0 = make_float2(far0 ? rsqrtf(d2h.x) : 0.f, far1 ? rsqrtf(d2h.y) : 0.f);
+    // y = y0 + ye: one Newton step in two floats (h = 1 - d2 y0^2)
+    const float2 ny0 = __fmul2_rn(y0, m1);
+    const float2 a = __fmul2_rn(y0, y0), na = __fmul2_rn(ny0, y0);
+    const float2 nae = __ffma2_rn(ny0, y0, a);  // a - y0^2
+    const float2 b = __fmul2_rn(d2h, a);
+    const float2 nbe = __ffma2_rn(d2h, na, b);
+    float2 h = __ffma2_rn(b, m1, bc2(1.f));
+    h = __fadd2_rn(h, nbe);
+    h = __ffma2_rn(d2h, nae, h);
+    h = __ffma2_rn(d2l, na, h);
+    // a lane that is not far has y0 = 0, so h = 1 and ye = 0
+    const float2 ye = __fmul2_rn(__fmul2_rn(bc2(0.5f), y0), h);
+    float2 t;
+    if constexpr (kPhi) {
+        two_sum2(S.ph, y0, S.ph, t);
+        S.pl = __fadd2_rn(S.pl, __fadd2_rn(t, ye));
+    }
+    const float2 c3 = __fmul2_rn(a, y0);
+    if constexpr (kField) {
+        // y^3 = c3 + cl, y^2 = a + (2 y0 ye - nae)
+        const float2 y2l = __ffma2_rn(nae, m1, __fmul2_rn(__fadd2_rn(y0, y0), ye));
+        const float2 nc3 = __fmul2_rn(na, y0);
+        float2 cl = __ffma2_rn(a, y0, nc3);
+        cl = __ffma2_rn(a, ye, cl);
+        cl = __ffma2_rn(y2l, y0, cl);
+        auto add = [&](float2 vh, float2 vl, float2& nSh, float2& Sl) {
+            const float2 np = __fmul2_rn(vh, nc3);  // -(v c3), whose error the fma below gives
+            float2 e = __ffma2_rn(vh, c3, np);
+            e = __ffma2_rn(vh, cl, e);
+            e = __ffma2_rn(vl, c3, e);
+            float2 u;
+            two_sum2(nSh, np, nSh, u);
+            Sl = __fadd2_rn(Sl, __ffma2_rn(u, m1, e));
+        };
+        add(xh, xl, S.xh, S.xl);
+        add(yh, yl, S.yh, S.yl);
+        add(zh, zl, S.zh, S.zl);
+    }
+    // degrees 2 to 4 in FP32
+    const float2 nx = __fmul2_rn(xh, y0), nz = __fmul2_rn(zh, y0);
+    const float2 qxx = __fmul2_rn(nx, nx), qxz = __fmul2_rn(nx, nz), qzz = __fmul2_rn(nz, nz);
+    const float2 qd = __fadd2_rn(qxz, qxz);
+    const float4 m0 = mom[0], m1_ = mom[1];
+    const float2 w2x = __ffma2_rn(lane2(m0, 0), nx, __fmul2_rn(lane2(m0, 1), nz));
+    const float2 w2z = __ffma2_rn(lane2(m0, 1), nx, __fmul2_rn(lane2(m1_, 0), nz));
+    const float2 T2 = __ffma2_rn(w2x, nx, __fmul2_rn(w2z, nz));
+    const float4 m2 = mom[2], m3 = mom[3], m4 = mom[4];
+    const float2 ntx = lane2(m4, 0), ntz = lane2(m4, 1);
+    const float2 w3x =
+        __ffma2_rn(lane2(m2, 0), qxx, __ffma2_rn(lane2(m2, 1), qd, __ffma2_rn(lane2(m3, 0), qzz, ntx)));
+    const float2 w3z =
+        __ffma2_rn(lane2(m2, 1), qxx, __ffma2_rn(lane2(m3, 0), qd, __ffma2_rn(lane2(m3, 1), qzz, ntz)));
+    const float2 W3 = __ffma2_rn(w3x, nx, __fmul2_rn(w3z, nz));
+    const float2 ntn = __ffma2_rn(ntx, nx, __fmul2_rn(ntz, nz));
+    const float4 m5 = mom[5], m6 = mom[6], m7 = mom[7], m8 = mom[8], m9 = mom[9], m10 = mom[10];
+    const float2 T22 = lane2(m7, 1), P20 = lane2(m8, 1), P11 = lane2(m9, 0), P02 = lane2(m9, 1);
+    const float2 gx =
+        __ffma2_rn(lane2(m5, 0), qxx, __ffma2_rn(lane2(m7, 0), qxz, __ffma2_rn(T22, qzz, P20)));
+    const float2 gz =
+        __ffma2_rn(lane2(m6, 1), qzz, __ffma2_rn(lane2(m8, 0), qxz, __ffma2_rn(T22, qxx, P02)));
+    const float2 w4x = __ffma2_rn(nx, gx, __fmul2_rn(nz, __ffma2_rn(lane2(m6, 0), qzz, P11)));
+    const float2 w4z = __ffma2_rn(nz, gz, __fmul2_rn(nx, __ffma2_rn(lane2(m5, 1), qxx, P11)));
+    const float2 W4 = __ffma2_rn(w4x, nx, __fmul2_rn(w4z, nz));
+    const float2 Q = __ffma2_rn(P20, qxx, __ffma2_rn(P11, qd, __fmul2_rn(P02, qzz)));
+    if constexpr (kPhi) {
+        const float2 f2 = __ffma2_rn(bc2(0.5f), T2, lane2(m1_, 1));
+        const float2 f3 = __ffma2_rn(bc2(1.f / 3.f), W3, __fmul2_rn(bc2(2.f / 3.f), ntn));
+        const float2 f4 = __ffma2_rn(bc2(0.25f), __fadd2_rn(W4, Q), lane2(m10, 0));
+        const float2 f = __ffma2_rn(a, f4, __ffma2_rn(y0, f3, f2));
+        S.fc = __ffma2_rn(c3, f, S.fc);
+    }
+    if constexpr (kField) {
+        const float2 ny = __fmul2_rn(yh, y0);
+        const float2 r2 = __ffma2_rn(bc2(2.5f), T2, lane2(mom[11], 0));
+        const float2 r3 = __ffma2_rn(bc2(7.f / 3.f), W3, __fmul2_rn(bc2(8.f / 3.f), ntn));
+        const float2 r4 = __ffma2_rn(bc2(2.25f), W4, __ffma2_rn(bc2(1.25f), Q, lane2(m10, 1)));
+        const float2 r = __ffma2_rn(a, r4, __ffma2_rn(y0, r3, r2));
+        const float2 wx = __ffma2_rn(a, w4x, __ffma2_rn(y0, w3x, w2x));
+        const float2 wz = __ffma2_rn(a, w4z, __ffma2_rn(y0, w3z, w2z));
+        const float2 y4 = __fmul2_rn(a, a), ny4 = __fmul2_rn(na, a), s = __fmul2_rn(y4, r);
+        S.ex = __ffma2_rn(ny4, wx, __ffma2_rn(s, nx, S.ex));
+        S.ey = __ffma2_rn(s, ny, S.ey);
+        S.ez = __ffma2_rn(ny4, wz, __ffma2_rn(s, nz, S.ez));
+    }
+}
+
 }  // namespace nb
