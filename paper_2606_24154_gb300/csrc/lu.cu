@@ -254,217 +254,219 @@ __global__ void __launch_bounds__(kPivThreads, 2) k_panel_col(T* __restrict__ A,
     }
 }
 
-// The whole panel of the FP32 factorisation in one cooperative launch (all CTAs resident).
-// CTA b holds rows [k0 + b R, k0 + (b+1) R) of the panel columns in shared memory
-// (column-major, R rows); per column j of the panel:
-//   (a) scale column j-1 by the previous pivot and apply its rank-1 update to the rows
-//       below it (the same per-element arithmetic as k_panel_col);
-//   (b) each CTA finds its largest |a_ij| (lowest row on ties) and publishes it with its
-//       row (candidate slot of parity j & 1); the CTA holding row j publishes row j;
-//   (c) one grid barrier; every CTA reduces the candidates to the pivot p, reads the
-//       pivot row, and the holders of rows j and p swap them in shared memory.
-// The candidate slots alternate between two parities: a CTA writes slot j+1 only after it
-// has passed barrier j, by which time every CTA has finished reading slot j-1.  The grid
-// barrier (a cumulative arrival counter) waits a bounded number of polls; on giving up a
-// CTA records *err and leaves the panel (the host reports a timeout).
+// The whole panel in one cooperative launch (all CTAs resident), FP32 and FP64.  CTA b holds rows
+// [k0 + b R, k0 + (b+1) R) of the panel columns in shared memory (column-major, R rows); per
+// column j of the panel:
+//   (a) the rank-1 update of column j-1 on the rows below it (the per-element arithmetic of
+//       k_panel_col), the columns dealt to groups of threads where the rows do not fill the block.
+//       L's columns stay unscaled in shared memory, scaled where they are used and when they
+//       are written back;
+//   (b) each CTA finds its largest |a_ij| (lowest row on ties) and warp 0 publishes it: the row and
+//       a 16-byte slot (magnitude, row index) of parity j & 1; the CTA that holds row j publishes
+//       row j too.  Then the grid barrier: one acquire-release add to an arrival counter that
+//       counts all arrivals of the factorisation, and polls of it until this column's total;
+//   (c) thread q of every CTA reads slot q; the CTA reduces them to the pivot p, reads the pivot
+//       row, and the holders of rows j and p swap them in shared memory.
+// The slots alternate between two parities: a CTA writes slot j+1 only after it has passed
+// barrier j, by which time every CTA has finished reading slot j-1.  A poll gives up after `limit`
+// reads; the CTA records *err and leaves the panel (the host reports a timeout), and the others
+// follow.
+//
+// Bound by latency: per column four block barriers and three L2 round trips in turn (arrival,
+// slots, pivot row).  A column takes 2.7 us in FP32 (n = 9996; 3.4 with shuffles for the
+// reductions, a barrier after each, L scaled and stored at once) and 3.1 us in FP64 (n = 6145;
+// 5.1 with one thread per row and the reciprocal taken by every thread).  Polling the CTAs' tagged
+// slots in place of the counter was slower on many CTAs (152: 3.9 us).
 constexpr int kCoopThreads = 256;
-constexpr int kCoopMaxG = 1024;
+constexpr int kCoopMaxG = kCoopThreads;  // one reading thread per CTA of the grid
 constexpr long long kCoopSpinLimit = 1ll << 22;
 
-// A magnitude as it is compared: FP32 as it is, FP64 by its bits (non-negative doubles order as
-// their bits, and integer compares leave the FP64 pipe alone).  NaN never wins: -1.
+// A magnitude as it is compared: its bits (non-negative numbers order as their bits, and integer
+// compares leave the FP64 pipe alone).  NaN never wins: -1.
 template <typename T>
 struct Mag;
 template <>
 struct Mag<float> {
-    typedef float Key;
-    static __device__ __forceinline__ Key of(float a) { return fabsf(a); }  // NaN fails every compare
+    static __device__ __forceinline__ long long of(float a) {
+        const int m = __float_as_int(a) & 0x7fffffff;
+        return m <= 0x7f800000 ? m : -1;
+    }
 };
 template <>
 struct Mag<double> {
-    typedef long long Key;
-    static __device__ __forceinline__ Key of(double a) {
+    static __device__ __forceinline__ long long of(double a) {
         const long long m = __double_as_longlong(a) & 0x7fffffffffffffffll;
         return m <= 0x7ff0000000000000ll ? m : -1;
     }
 };
 
+// rows a CTA holds at least: FP64 updates are bound by the FP64 pipe (one warp of rows), FP32 ones are not
+template <typename T>
+constexpr int64_t kCoopMinRows = sizeof(T) == 8 ? 32 : 64;
+
+struct __align__(16) CoopSlot {
+    long long key;
+    int idx, pad;
+};
 template <typename T>
 struct CoopScratch {
-    typename Mag<T>::Key cval[2][kCoopMaxG];
-    int cidx[2][kCoopMaxG];
-    T cand[2][kCoopMaxG][64];
-    T srow[2][64];
-    unsigned int bar[4];  // bar[0]: grid-barrier arrivals of the factorisation
+    CoopSlot slot[2][kCoopMaxG];
+    alignas(16) T cand[2][kCoopMaxG][64];
+    alignas(16) T srow[2][64];
+    unsigned int bar;  // arrivals of the factorisation
     int err;
 };
 
-__device__ __forceinline__ unsigned int ld_acquire_u(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ int ld_acquire_i(const int* p) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-
-// every CTA of the grid arrives; false if the wait gave up.  bar[0] counts all arrivals
-// of the factorisation (never reset): each CTA adds 1 with acquire-release semantics and
-// waits until the count reaches `target` (this barrier's total), so one atomic and one
-// polled load make the barrier, and the last arrival publishes everyone's writes (the
-// acquire load that sees the final count synchronises with every add before it).
-template <typename T>
-__device__ bool coop_barrier(CoopScratch<T>* cs, unsigned int target, bool* s_flag, long long limit) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned int v;
-        asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(v) : "l"(&cs->bar[0]) : "memory");
-        bool ok = true;
-        if (v + 1u < target) {
-            long long spins = 0;
-            while (ld_acquire_u(&cs->bar[0]) < target) {
-                // give up after the poll limit, or at once when another CTA has given up
-                if (++spins > limit || ((spins & 1023) == 0 && ld_acquire_i(&cs->err))) {
-                    ok = false;
-                    break;
-                }
-                __nanosleep(20);
-            }
-        }
-        *s_flag = ok;
-    }
-    __syncthreads();
-    return *s_flag;
+__device__ __forceinline__ unsigned int ld_acquire_u(const unsigned int* p) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// largest key of the warp with the lowest index on ties, in every lane
+__device__ __forceinline__ void warp_best(long long& key, int& idx) {
+    const int hi = (int)(key >> 32);
+    const int mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned int lo = hi == mh ? (unsigned int)key : 0u;
+    const unsigned int ml = __reduce_max_sync(0xffffffffu, lo);
+    const bool mine = hi == mh && (unsigned int)key == ml;
+    idx = __reduce_min_sync(0xffffffffu, mine ? idx : INT_MAX);
+    key = ((long long)mh << 32) | ml;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kCoopThreads, 1)
     k_panel_coop(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
-                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch<T>* cs, unsigned int bar_base,
-                 long long limit) {
-    typedef typename Mag<T>::Key Key;
+                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch<T>* cs, unsigned int bar_base, long long limit) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ld_acquire_i(&cs->err)) return;  // an earlier panel gave up: leave the matrix as it is
     const int w = (int)(k1 - k0);
     T* S = reinterpret_cast<T*>(smem_raw);  // R x w, column-major
-    __shared__ T prow[64];
-    __shared__ bool s_flag;
-    const int G = gridDim.x, b = blockIdx.x;
+    constexpr int kWarps = kCoopThreads / 32;
+    __shared__ T prow[64], sinv[64];
+    __shared__ long long wk[2][kWarps];
+    __shared__ int wi[2][kWarps];
+    __shared__ int s_fail;
+    const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int64_t rb0 = k0 + (int64_t)b * R;
     const int nr = (int)max((int64_t)0, min((int64_t)R, n - rb0));
-    for (int idx = threadIdx.x; idx < nr * w; idx += kCoopThreads) {
+    if (tid == 0) s_fail = 0;
+    for (int idx = tid; idx < nr * w; idx += kCoopThreads) {
         const int r = idx % nr, c = idx / nr;
         S[c * R + r] = A[(rb0 + r) + (k0 + c) * n];
     }
     __syncthreads();
-    bool ok_piv = true;  // the previous pivot was nonzero
-    __shared__ Key wv[kCoopThreads / 32];
-    __shared__ int wi[kCoopThreads / 32];
-    // (best, index) of the block: warp shuffles, then every thread over the warps' results;
-    // the largest value with the lowest index on ties, so the order of the reduction does
-    // not matter.  Magnitudes of FP32 values compare exactly in FP32 (no FP64 pipe), row
-    // indices fit in 32 bits (n < 2^31).  Every thread returns with the result in (v, ix).
-    auto block_best = [&](Key& v, int& ix) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const Key v2 = __shfl_xor_sync(0xffffffffu, v, o);
-            const int i2 = __shfl_xor_sync(0xffffffffu, ix, o);
-            if (v2 > v || (v2 == v && i2 < ix)) {
-                v = v2;
-                ix = i2;
-            }
-        }
-        if ((threadIdx.x & 31) == 0) {
-            wv[threadIdx.x >> 5] = v;
-            wi[threadIdx.x >> 5] = ix;
+    // thread -> row and group of columns: `step` rows at a time, `groups` column groups
+    const int step = R <= kCoopThreads / 2 ? (R + 31) & ~31 : kCoopThreads;
+    const int groups = kCoopThreads / step, grp = tid / step, row0 = tid - grp * step;
+    // (key, index) of the block, in every thread, through buffer q
+    auto block_best = [&](int q, long long& key, int& idx) {
+        warp_best(key, idx);
+        if (lane == 0) {
+            wk[q][tid >> 5] = key;
+            wi[q][tid >> 5] = idx;
         }
         __syncthreads();
-        v = wv[0];
-        ix = wi[0];
-        for (int q = 1; q < kCoopThreads / 32; ++q)
-            if (wv[q] > v || (wv[q] == v && wi[q] < ix)) {
-                v = wv[q];
-                ix = wi[q];
-            }
-        __syncthreads();  // wv / wi are rewritten by the next reduction
+        key = lane < kWarps ? wk[q][lane] : -1;
+        idx = lane < kWarps ? wi[q][lane] : INT_MAX;
+        warp_best(key, idx);
     };
+    bool ok_piv = true;  // the previous pivot was nonzero
     for (int jj = 0; jj < w; ++jj) {
         const int64_t j = k0 + jj;
         const int par = jj & 1;
-        // (a) + (b): column jj-1 scaled and its rank-1 update applied to this thread's rows
-        // below it, then this thread's candidate for column jj from the same rows
-        Key best = (Key)-1;
+        // (a) column jj-1's rank-1 update, then this thread's candidate for column jj
+        long long best = -1;
         int bidx = INT_MAX;
-        const T inv = (jj > 0 && ok_piv) ? (T)1 / prow[jj - 1] : (T)0;
-        for (int r = threadIdx.x; r < nr; r += kCoopThreads) {
-            if (rb0 + r < j) continue;
-            if (jj > 0 && ok_piv) {
-                const T l = S[(jj - 1) * R + r] * inv;
-                S[(jj - 1) * R + r] = l;
-                for (int c = jj; c < w; ++c) S[c * R + r] -= l * prow[c];
+        const T inv = jj > 0 ? sinv[jj - 1] : (T)0;
+        if (grp < groups)
+            for (int r = row0; r < nr; r += step) {
+                if (rb0 + r < j) continue;
+                if (jj > 0 && ok_piv) {
+                    const T l = S[(jj - 1) * R + r] * inv;
+#pragma unroll 4
+                    for (int c = jj + grp; c < w; c += groups) S[c * R + r] -= l * prow[c];
+                }
+                if (grp == 0) {
+                    const long long v = Mag<T>::of(S[jj * R + r]);
+                    if (v > best) {  // rows in increasing order: the first of equal ones stays
+                        best = v;
+                        bidx = (int)(rb0 + r);
+                    }
+                }
             }
-            const Key v = Mag<T>::of(S[jj * R + r]);
-            if (v > best || (v == best && (int)(rb0 + r) < bidx)) {
-                best = v;
-                bidx = (int)(rb0 + r);
+        block_best(0, best, bidx);
+        // (b) warp 0 publishes the candidate row (and row j), then the slot
+        if (tid < 32) {
+            const int mine = bidx != INT_MAX ? (int)(bidx - rb0) : -1;
+            const bool own = j >= rb0 && j < rb0 + nr;
+            for (int c = lane; c < w; c += 32) {
+                cs->cand[par][b][c] = mine >= 0 ? S[c * R + mine] : (T)0;
+                if (own) cs->srow[par][c] = S[c * R + (int)(j - rb0)];
+            }
+            __syncwarp();
+            if (lane == 0) {
+                __stcg(reinterpret_cast<int4*>(&cs->slot[par][b]),
+                       make_int4((int)best, (int)(best >> 32), bidx, 0));
+                // the barrier: the release half publishes the warp's stores (cumulative over the
+                // warp barrier), the acquire of the final count everyone's
+                const unsigned int target = bar_base + (unsigned)(jj + 1) * (unsigned)G;
+                unsigned int v;
+                asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(v) : "l"(&cs->bar) : "memory");
+                long long spins = 0;
+                while (v + 1u < target && ld_acquire_u(&cs->bar) < target) {
+                    // give up after the poll limit, or when another CTA has given up
+                    if (++spins > limit || ((spins & 1023) == 0 && ld_acquire_i(&cs->err))) {
+                        s_fail = 1;
+                        break;
+                    }
+                    __nanosleep(20);
+                }
             }
         }
-        block_best(best, bidx);
-        const int mine = bidx;
-        if (threadIdx.x == 0) {
-            cs->cval[par][b] = best;
-            cs->cidx[par][b] = mine;
+        __syncthreads();
+        // (c) every CTA's candidate
+        best = -1;
+        bidx = INT_MAX;
+        if (tid < G) {
+            const int4 q = __ldcg(reinterpret_cast<const int4*>(&cs->slot[par][tid]));
+            best = ((long long)q.y << 32) | (unsigned int)q.x;
+            bidx = q.z;
         }
-        if (threadIdx.x < w) {
-            cs->cand[par][b][threadIdx.x] = (mine != INT_MAX) ? S[threadIdx.x * R + (int)(mine - rb0)] : (T)0;
-            if (j >= rb0 && j < rb0 + nr) cs->srow[par][threadIdx.x] = S[threadIdx.x * R + (int)(j - rb0)];
-        }
-        if (!coop_barrier(cs, bar_base + (unsigned)(jj + 1) * (unsigned)G, &s_flag, limit)) {
-            if (threadIdx.x == 0) {
+        block_best(1, best, bidx);
+        if (s_fail) {
+            if (tid == 0) {
                 atomicExch(&cs->err, 1);
                 atomicExch(tmo, 1);
             }
             return;
         }
-        // (c) the pivot: largest |a| over the candidates, lowest row on ties
-        best = (Key)-1;
-        bidx = INT_MAX;
-        for (int q = threadIdx.x; q < G; q += kCoopThreads) {
-            const Key v = __ldcg(&cs->cval[par][q]);
-            const int ix = __ldcg(&cs->cidx[par][q]);
-            if (v > best || (v == best && ix < bidx)) {
-                best = v;
-                bidx = ix;
-            }
+        // no candidate (a column of NaN): row j stays where it is
+        const bool any = (int64_t)bidx >= j && (int64_t)bidx < n;
+        const int64_t p = any ? (int64_t)bidx : j;
+        if (tid < w) {
+            const T v = __ldcg(any ? &cs->cand[par][(int)((p - k0) / R)][tid] : &cs->srow[par][tid]);
+            prow[tid] = v;
+            if (j >= rb0 && j < rb0 + nr) S[tid * R + (int)(j - rb0)] = v;
+            if (p != j && p >= rb0 && p < rb0 + nr) S[tid * R + (int)(p - rb0)] = __ldcg(&cs->srow[par][tid]);
+            // a zero pivot leaves its column unscaled and skips its update, as in k_panel_col
+            if (tid == jj) sinv[jj] = v != (T)0 ? (T)1 / v : (T)1;
         }
-        block_best(best, bidx);
-        const int64_t p = ((int64_t)bidx >= j && (int64_t)bidx < n) ? (int64_t)bidx : j;
-        const int owner = (int)((p - k0) / R);
-        if (threadIdx.x < w) prow[threadIdx.x] = __ldcg(&cs->cand[par][owner][threadIdx.x]);
-        if (b == 0 && threadIdx.x == 0) {
+        if (b == 0 && tid == 0) {
             piv[j] = (int32_t)p;
-            if (!(best > (Key)0) && *info == 0) *info = (int)(j + 1);
+            if (!(best > 0) && *info == 0) *info = (int)(j + 1);
         }
         __syncthreads();
-        ok_piv = prow[jj] != (T)0;  // the scaling below is skipped for a zero pivot, as in k_panel_col
-        if (threadIdx.x < w) {
-            if (j >= rb0 && j < rb0 + nr) S[threadIdx.x * R + (int)(j - rb0)] = prow[threadIdx.x];
-            if (p != j && p >= rb0 && p < rb0 + nr)
-                S[threadIdx.x * R + (int)(p - rb0)] = __ldcg(&cs->srow[par][threadIdx.x]);
-        }
-        __syncthreads();
+        ok_piv = prow[jj] != (T)0;
     }
-    // scale the last panel column below the panel
-    if (ok_piv) {
-        const T inv = (T)1 / prow[w - 1];
-        for (int r = threadIdx.x; r < nr; r += kCoopThreads)
-            if (rb0 + r >= k1) S[(w - 1) * R + r] *= inv;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nr * w; idx += kCoopThreads) {
+    for (int idx = tid; idx < nr * w; idx += kCoopThreads) {
         const int r = idx % nr, c = idx / nr;
-        A[(rb0 + r) + (k0 + c) * n] = S[c * R + r];
+        const T v = S[c * R + r];
+        A[(rb0 + r) + (k0 + c) * n] = rb0 + r > k0 + c ? v * sinv[c] : v;
     }
 }
 
@@ -475,66 +477,48 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
 // panel rows (slot r - k0) and the distinct pivot rows below the panel (found by a
 // warp-wide search of the list so far).  A pivot outside [r, n) is a row no panel wrote (its
 // panel gave up a bounded wait) and is skipped, as in the swaps themselves.
+// Each of 128 threads follows one touched row's content through the swaps: thread t < 64 the
+// panel row k0 + t, thread 64 + t the pivot row of step t below the panel, where no earlier
+// step has it.  (One warp searching its list of rows once per swap took 20 us, this 3.)
 constexpr int kSwapMax = 128;
 
-__global__ void __launch_bounds__(32) k_swap_perm(const int32_t* __restrict__ piv, int64_t n, int64_t k0, int64_t k1,
-                                                  int32_t* __restrict__ perm) {
-    __shared__ int64_t row_of[kSwapMax];  // slot -> row
-    __shared__ int32_t content[kSwapMax]; // slot -> slot whose original row is there now
-    __shared__ int32_t pv[kSwapMax / 2];  // the panel's pivots
-    __shared__ int n_slots;
-    const int lane = threadIdx.x;
-    const int w = (int)(k1 - k0);
-    for (int q = lane; q < w; q += 32) pv[q] = piv[k0 + q];
-    for (int s = lane; s < kSwapMax; s += 32) {
-        row_of[s] = s < w ? k0 + s : -1;
-        content[s] = s;
+__global__ void __launch_bounds__(kSwapMax) k_swap_perm(const int32_t* __restrict__ piv, int64_t n, int64_t k0,
+                                                        int64_t k1, int32_t* __restrict__ perm) {
+    __shared__ int64_t pv[kSwapMax / 2];
+    __shared__ int s_cnt;
+    const int w = (int)(k1 - k0), t = threadIdx.x;
+    if (t == 0) s_cnt = 0;
+    if (t < w) {
+        const int64_t r = k0 + t, p = piv[r];
+        pv[t] = (p > r && p < n) ? p : r;
     }
-    if (lane == 0) n_slots = w;
-    __syncwarp();
-    for (int64_t r = k0; r < k1; ++r) {
-        const int64_t p = pv[r - k0];
-        if (!(p != r && p > r && p < n)) continue;
-        int sp;
-        if (p < k1) {
-            sp = (int)(p - k0);
-        } else {
-            const int ns = n_slots;
-            int found = -1;
-            for (int base = w; base < ns && found < 0; base += 32) {
-                const int s = base + lane;
-                const unsigned hit = __ballot_sync(0xffffffffu, s < ns && row_of[s] == p);
-                if (hit) found = base + __ffs(hit) - 1;
-            }
-            if (found < 0) {
-                found = ns;
-                if (lane == 0) {
-                    row_of[ns] = p;
-                    n_slots = ns + 1;
-                }
-            }
-            sp = found;
-        }
-        __syncwarp();
-        if (lane == 0) {
-            const int sr = (int)(r - k0);
-            const int t = content[sr];
-            content[sr] = content[sp];
-            content[sp] = t;
-        }
-        __syncwarp();
+    __syncthreads();
+    int64_t src = -1;
+    if (t < w) {
+        src = k0 + t;
+    } else if (t >= kSwapMax / 2 && t - kSwapMax / 2 < w) {
+        const int q = t - kSwapMax / 2;
+        src = pv[q] >= k1 ? pv[q] : -1;
+        for (int r = 0; r < q; ++r)
+            if (pv[r] == src) src = -1;
     }
+    int64_t at = src;
+    if (src >= 0)
+        for (int r = 0; r < w; ++r) {
+            const int64_t p = pv[r];
+            if (at == k0 + r)
+                at = p;
+            else if (at == p)
+                at = k0 + r;
+        }
     // moved rows: (dst, src) pairs after the count
-    if (lane == 0) {
-        int c = 0;
-        for (int s = 0; s < n_slots; ++s)
-            if (content[s] != s) {
-                perm[1 + 2 * c] = (int32_t)row_of[s];
-                perm[2 + 2 * c] = (int32_t)row_of[content[s]];
-                ++c;
-            }
-        perm[0] = c;
+    if (at != src) {
+        const int c = atomicAdd(&s_cnt, 1);
+        perm[1 + 2 * c] = (int32_t)at;
+        perm[2 + 2 * c] = (int32_t)src;
     }
+    __syncthreads();
+    if (t == 0) perm[0] = s_cnt;
 }
 
 // The composed swaps applied to every column outside the panel: each thread loads all the
@@ -564,35 +548,34 @@ __global__ void __launch_bounds__(kSwapThreads) k_laswp(T* __restrict__ A, int64
     for (int i = 0; i < cnt; ++i) col[perm[1 + 2 * i]] = vals[i * kSwapThreads + threadIdx.x];
 }
 
-// Inverse of the unit-lower nb x nb diagonal block at (k0, k0) into W (nb x nb, ld nb):
-// X = I, then for q = 0 .. nb-2 (row q of X is final) X[r][c] -= L[r][q] X[q][c] for
-// r > q, c <= q -- forward substitution of all columns at once, one block barrier per q,
-// L and X in shared memory.
+// Inverse of the unit-lower nb x nb diagonal block at (k0, k0) into W (nb x nb, ld nb), nb <= 64:
+// a warp per column c, lane l holding rows l and l + 32 of it: X = e_c, then for q = c .. nb-2 (X[q]
+// is final) X[r] -= L[r][q] X[q] for r > q.  The columns are independent, so nb / 8 blocks share
+// the work without block barriers; one block for all, a barrier per q, took 28 us in FP32 and
+// 35 us in FP64 (where one SM's FP64 pipe was the bound).
+constexpr int kTriWarps = 8;
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_trtri_unit_lower(const T* __restrict__ A, int64_t n, int64_t k0, int nb,
-                                                          T* __restrict__ W) {
-    extern __shared__ unsigned char smem_raw[];
+__global__ void __launch_bounds__(32 * kTriWarps) k_trtri_unit_lower(const T* __restrict__ A, int64_t n, int64_t k0,
+                                                                    int nb, T* __restrict__ W) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ld = nb + 1;
-    T* L = reinterpret_cast<T*>(smem_raw);  // nb x (nb+1)
-    T* X = L + nb * ld;                       // nb x (nb+1)
+    T* L = reinterpret_cast<T*>(smem_raw);  // nb x (nb+1), column q at L + q ld
     for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-        const int r = idx % nb, c = idx / nb;
-        L[r + c * ld] = A[(k0 + r) + (k0 + c) * n];
-        X[r + c * ld] = (r == c) ? (T)1 : (T)0;
+        const int r = idx % nb, q = idx / nb;
+        L[r + q * ld] = A[(k0 + r) + (k0 + q) * n];
     }
     __syncthreads();
-    for (int q = 0; q + 1 < nb; ++q) {
-        const int rows = nb - 1 - q;
-        for (int idx = threadIdx.x; idx < rows * (q + 1); idx += blockDim.x) {
-            const int r = q + 1 + idx % rows, c = idx / rows;
-            X[r + c * ld] -= L[r + q * ld] * X[q + c * ld];
-        }
-        __syncthreads();
+    const int c = blockIdx.x * kTriWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (c >= nb) return;
+    T x0 = lane == c ? (T)1 : (T)0, x1 = lane + 32 == c ? (T)1 : (T)0;
+    for (int q = c; q + 1 < nb; ++q) {
+        const T xq = __shfl_sync(0xffffffffu, q < 32 ? x0 : x1, q & 31);
+        if (lane > q && lane < nb) x0 -= L[lane + q * ld] * xq;
+        if (lane + 32 > q && lane + 32 < nb) x1 -= L[lane + 32 + q * ld] * xq;
     }
-    for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
-        const int r = idx % nb, c = idx / nb;
-        W[r + (int64_t)c * nb] = X[r + c * ld];
-    }
+    if (lane < nb) W[lane + (int64_t)c * nb] = x0;
+    if (lane + 32 < nb) W[lane + 32 + (int64_t)c * nb] = x1;
 }
 
 // C = alpha * A * B + beta * C; column-major, M x N x K; 64 x 64 tiles, 256 threads, 4x4
@@ -781,7 +764,7 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && can) {
             const int g = std::min(kCoopMaxG, sms);
-            const int64_t R0 = std::max<int64_t>(64, (n + g - 1) / g);
+            const int64_t R0 = std::max<int64_t>(kCoopMinRows<T>, (n + g - 1) / g);
             const int64_t smem0 = R0 * 64 * (int64_t)sizeof(T);
             int per_sm = 0;
             if (smem0 <= 200 * 1024 &&
@@ -796,7 +779,7 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
         }
         cudaGetLastError();  // a refused attribute or query leaves the per-column path
     }
-    unsigned int arrivals = 0;  // grid-barrier arrivals of the cooperative panels so far
+    unsigned int arrivals = 0;
     // FP32 with the bulk tensor-core path: two-level blocking.  Super-panels of kSuperPanels
     // panels; inside one, each panel's U12 and update stop at the super-panel's last column;
     // after it, the block row's U12 by block forward substitution and one trailing update of
@@ -807,9 +790,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
     auto trsm_rows = [&](int64_t r0, int wr, int64_t c0, int64_t c1) -> cudaError_t {
         // A[r0 : r0 + wr, c0 : c1] = L(r0 block)^-1 A[r0 : r0 + wr, c0 : c1] (unit lower wr x wr)
         const int64_t m = c1 - c0;
-        const int tri_smem = (int)(2 * sizeof(T) * wr * (wr + 1));
-        NB_TRY(cudaFuncSetAttribute(k_trtri_unit_lower<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, tri_smem));
-        k_trtri_unit_lower<T><<<1, 256, tri_smem, s>>>(A, n, r0, wr, Linv);
+        k_trtri_unit_lower<T><<<(unsigned)((wr + kTriWarps - 1) / kTriWarps), 32 * kTriWarps,
+                                sizeof(T) * wr * (wr + 1), s>>>(A, n, r0, wr, Linv);
         NB_TRY(gemm<T>(wr, m, wr, (T)1, Linv, wr, A + r0 + c0 * n, n, (T)0, W, wr, s));
         k_copy_block<T><<<(unsigned)((wr * m + 255) / 256), 256, 0, s>>>(W, wr, A + r0 + c0 * n, n, wr, m);
         return cudaGetLastError();
@@ -829,18 +811,18 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
             const int w = (int)(k1 - k0);
             if (gmax > 0) {
                 const int64_t rows = n - k0;
-                const int R = (int)std::max<int64_t>(64, (rows + gmax - 1) / gmax);
+                const int R = (int)std::max<int64_t>(kCoopMinRows<T>, (rows + gmax - 1) / gmax);
                 const int G = (int)((rows + R - 1) / R);
                 T* Af = A;
                 int64_t nn = n, kk0 = k0, kk1 = k1;
                 int RR = R;
                 int* tmo = d_info + 1;
                 unsigned int base = arrivals;
+                arrivals += (unsigned int)G * (unsigned int)w;
                 long long lim = polls > 0 ? polls : kCoopSpinLimit;
                 void* args[] = {&Af, &nn, &kk0, &kk1, &RR, &piv, &d_info, &tmo, &cs, &base, &lim};
                 NB_TRY(cudaLaunchCooperativeKernel((const void*)k_panel_coop<T>, dim3((unsigned)G), dim3(kCoopThreads),
                                                    args, (size_t)R * w * sizeof(T), s));
-                arrivals += (unsigned int)G * (unsigned int)w;
             } else {
                 // columns k0..k1-1: update by the previous column + pivot of this one; then the
                 // last column's scaling of the rows below the panel
@@ -853,17 +835,15 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                 }
             }
             NB_TRY(cudaGetLastError());
-            k_swap_perm<<<1, 32, 0, s>>>(piv, n, k0, k1, swap_perm);
+            k_swap_perm<<<1, kSwapMax, 0, s>>>(piv, n, k0, k1, swap_perm);
             k_laswp<T><<<(unsigned)((n + kSwapThreads - 1) / kSwapThreads), kSwapThreads, swap_smem, s>>>(A, n, k0,
                                                                                                     k1, swap_perm);
             const bool tc64 = sizeof(T) == 8 && split;  // FP64 with the tensor-core update
             if ((super && (k1 < K1 || K1 < n)) || (tc64 && w == 64 && k1 < n)) {
                 // the panel's unit-lower inverse, kept in its slot for the block row's U12
                 T* slot = Linv + (size_t)((k0 - K0) / nb) * nb * nb;
-                const int tri_smem = (int)(2 * sizeof(T) * w * (w + 1));
-                NB_TRY(cudaFuncSetAttribute(k_trtri_unit_lower<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            tri_smem));
-                k_trtri_unit_lower<T><<<1, 256, tri_smem, s>>>(A, n, k0, w, slot);
+                k_trtri_unit_lower<T><<<(unsigned)((w + kTriWarps - 1) / kTriWarps), 32 * kTriWarps,
+                                        sizeof(T) * w * (w + 1), s>>>(A, n, k0, w, slot);
             }
             if (k1 < e1) {
                 const int64_t m = n - k1, mc = e1 - k1;
