@@ -40,17 +40,12 @@ double elem_area(const Elem& e) { return (e.nv == 4) ? 0.5 * (e.twoA[0] + e.twoA
 // copy es.el) under the image set es.img.
 int finish_set(Ctx* c, const std::vector<Elem>& h_el, EvalSet& es) {
     std::string why;
-    std::vector<int32_t> cell_start, cell_items;
-    int rc = build_near_grid(h_el, es.img, c->opt.ratio_near, es.grid, cell_start, cell_items, why);
+    int rc = near_grid_box(h_el, es.img, c->opt.ratio_near, es.grid, why);
     if (rc) return fail(rc, why);
     CK(es.cjk.ensure(sizeof(float4) * 2 * es.n * es.img.n));
     CK(launch_image_centroids(es.el, es.n, es.img, es.cjk.as<float4>(), c->stream));
-    CK(es.cell_start.ensure(sizeof(int32_t) * cell_start.size()));
-    CK(es.cell_items.ensure(sizeof(int32_t) * cell_items.size()));
-    CK(cudaMemcpyAsync(es.cell_start.ptr, cell_start.data(), sizeof(int32_t) * cell_start.size(),
-                       cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(es.cell_items.ptr, cell_items.data(), sizeof(int32_t) * cell_items.size(),
-                       cudaMemcpyHostToDevice, c->stream));
+    rc = make_cell_list(c, es.el, es.n, es.img, es.grid, es.cell_start, es.cell_items);
+    if (rc) return rc;
     return 0;
 }
 

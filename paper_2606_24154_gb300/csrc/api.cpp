@@ -199,8 +199,7 @@ int nebem_set_geometry(nebem_ctx* ctx, const nebem_element* el, int64_t n, const
         h_cond[i] = el[i].conductor;
     }
     NearGrid grid;
-    std::vector<int32_t> cell_start, cell_items;
-    rc = build_near_grid(h_el, img, c->opt.ratio_near, grid, cell_start, cell_items, why);
+    rc = near_grid_box(h_el, img, c->opt.ratio_near, grid, why);
     if (rc) return fail(rc, why);
     CK(cudaStreamSynchronize(c->stream));
     // invalidate everything that depends on the geometry
@@ -224,12 +223,8 @@ int nebem_set_geometry(nebem_ctx* ctx, const nebem_element* el, int64_t n, const
     CK(cudaMemcpyAsync(c->d_diag.ptr, h_diag.data(), sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
     CK(c->d_cjk.ensure(sizeof(float4) * 2 * n * img.n));
     CK(launch_image_centroids(c->d_el.as<Elem>(), n, img, c->d_cjk.as<float4>(), c->stream));
-    CK(c->d_cell_start.ensure(sizeof(int32_t) * cell_start.size()));
-    CK(c->d_cell_items.ensure(sizeof(int32_t) * cell_items.size()));
-    CK(cudaMemcpyAsync(c->d_cell_start.ptr, cell_start.data(), sizeof(int32_t) * cell_start.size(),
-                       cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->d_cell_items.ptr, cell_items.data(), sizeof(int32_t) * cell_items.size(),
-                       cudaMemcpyHostToDevice, c->stream));
+    rc = make_cell_list(c, c->d_el.as<Elem>(), n, img, grid, c->d_cell_start, c->d_cell_items);
+    if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));
     c->grid = grid;
     c->img = img;

@@ -65,6 +65,7 @@ struct Ctx {
     DevBuf d_el, d_far, d_diag;
     DevBuf d_cjk, d_cell_start, d_cell_items;  // mixed eval: two-float image centroids, near cell list
     NearGrid grid{};
+    DevBuf d_tab_work;  // scratch of the cell lists
 
     // boundary conditions and solution
     std::vector<double> voltages;
@@ -138,6 +139,9 @@ int solve_with_factors(Ctx* c, int precision, nebem_solve_info* info);
 // k weighting-field solutions (unit potential on readout[j], 0 on the other conductors, no
 // known charges) into c->d_wX (n x k, column-major) with the retained factors
 int weighting_solve(Ctx* c, const int32_t* readout, int k, int precision, nebem_solve_info* info);
+// the cell list of an element table with images (its grid set), into start / items (grown)
+int make_cell_list(Ctx* c, const Elem* d_el, int64_t n, const ImageTable& img, const NearGrid& grid, DevBuf& start,
+                   DevBuf& items);
 // two-float tables of the mixed fill and of the refined evaluation (built on first use)
 int ensure_fill_tables(Ctx* c);
 // elements only (with images); err (may be NULL, n x 2): per-point error estimates of a

@@ -542,11 +542,6 @@ __global__ void __launch_bounds__(256)
 
 // FP64 near pairs of every listed point, a warp per point (near_point_warp): level 1 with
 // the FP32 pass's near radii, level 2 with the fill's.
-struct NearFill {
-    const FillEl* fe;
-    __device__ __forceinline__ float operator()(int32_t j) const { return fe[j].hdr.z; }
-};
-
 template <int L>
 __global__ void __launch_bounds__(kAT)
     k_eval_acc_near(const AccView A, const ImageTable img, const double* __restrict__ pts,

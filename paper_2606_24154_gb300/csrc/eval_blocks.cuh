@@ -421,30 +421,22 @@ __device__ __forceinline__ void far_block(const GeomView& g, const double* __res
     }
 }
 
-// Near part (FP64 closed forms) of target p, by one warp; adds ke * sum to phi[p] / E[p].
-// The image centroids in the 27 cells around the point are tested 32 at a time (a row of
-// three cells is contiguous in cell_items), the near ones are queued in `queue` (kNearQueue
-// entries of shared memory of the warp) and evaluated 32 at a time: an FP64 instruction holds
-// the SM's FP64 pipe as long for one lane as for 32, so a lane that met its near pairs one by
-// one (a thread per point) made the pipe do mostly empty work and left one point's pairs
-// in one serial chain (200,000 points: 8.6 ms a thread per point, 1.4 ms a warp).  near2 gives the squared near radius of an element.  The order of the sums
-// depends on the point and the tables only.
+// The near pairs of the target (Px, Py, Pz) (ph, pl: its two floats), by one warp.  The image centroids in
+// the 27 cells around the point are tested 32 at a time (a row of three cells is contiguous in
+// cell_items), the near ones are queued in `queue` (kNearQueue entries of shared memory of the warp)
+// and handed out 32 at a time: eval(live, jk) by every lane.  An FP64 instruction holds the SM's FP64 pipe
+// as long for one lane as for 32, so a lane that met its near pairs one by one (a thread per point)
+// made the pipe do mostly empty work and left one point's pairs in one serial chain (200,000
+// points: 8.6 ms a thread per point, 1.4 ms a warp).  near2 gives the squared near radius of an
+// element.  The order of the pairs depends on the point and the tables only.
 constexpr int kNearQueue = 64;
-template <class Near2>
-__device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, const double* __restrict__ sigma,
-                                                const float4* __restrict__ cjk, const NearGrid& grid,
-                                                const int32_t* __restrict__ cell_start,
-                                                const int32_t* __restrict__ cell_items, const ImageTable& img,
-                                                const Near2& near2, const double* __restrict__ pts, int64_t p,
-                                                double* __restrict__ phi, double* __restrict__ E,
-                                                int32_t* __restrict__ queue) {
+template <class Near2, class Eval>
+__device__ __forceinline__ void near_pairs_warp(double Px, double Py, double Pz, float phx, float phy, float phz,
+                                                float plx, float ply, float plz, const float4* __restrict__ cjk,
+                                                const NearGrid& grid, const int32_t* __restrict__ cell_start,
+                                                const int32_t* __restrict__ cell_items, int nimg, const Near2& near2,
+                                                int32_t* __restrict__ queue, const Eval& eval) {
     const int lane = threadIdx.x & 31;
-    const int nimg = img.n;
-    const double Px = pts[3 * p], Py = pts[3 * p + 1], Pz = pts[3 * p + 2];
-    float phx, phy, phz, plx, ply, plz;
-    split2f(Px, phx, plx);
-    split2f(Py, phy, ply);
-    split2f(Pz, phz, plz);
     // cell of the point, clamped (a point more than one cell outside has no near pair)
     int cc[3];
     const double P[3] = {Px, Py, Pz};
@@ -455,8 +447,6 @@ __device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, con
         cc[a] = (int)f;
     }
     const int x0 = max(cc[0] - 1, 0), x1 = min(cc[0] + 1, grid.dims[0] - 1);
-    double aphi = 0.0, aEx = 0.0, aEy = 0.0, aEz = 0.0;
-    bool any = false;
     int row = 0, nq = 0;  // rows (y, z) of the neighbourhood taken so far; queued pairs
     int32_t it = 0, end = 0;
     bool more = x0 <= x1;
@@ -491,25 +481,47 @@ __device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, con
         }
         __syncwarp();
         const int take = min(nq, 32);
-        if (lane < take) {
-            const int32_t jk = queue[lane];
-            const int32_t j = jk / nimg, k = jk - j * nimg;
-            const Elem& e = el[j];
-            double f, ux, uy, uz;
-            elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, ux, uy, uz);
-            const double s = sigma[j];
-            aphi = fma(s, f, aphi);
-            aEx = __fma_rn(s, __fma_rn(ux, e.ex[0], __fma_rn(uy, e.ey[0], __dmul_rn(uz, e.ez[0]))), aEx);
-            aEy = __fma_rn(s, __fma_rn(ux, e.ex[1], __fma_rn(uy, e.ey[1], __dmul_rn(uz, e.ez[1]))), aEy);
-            aEz = __fma_rn(s, __fma_rn(ux, e.ex[2], __fma_rn(uy, e.ey[2], __dmul_rn(uz, e.ez[2]))), aEz);
-        }
-        any = any || take > 0;
+        if (take == 0) break;
+        eval(lane < take, lane < take ? queue[lane] : 0);
         nq -= take;
         const int32_t rest = lane < nq ? queue[32 + lane] : 0;
         __syncwarp();
         if (lane < nq) queue[lane] = rest;
         __syncwarp();
     }
+}
+
+// Near part (FP64 closed forms) of target p, by one warp; adds ke * sum to phi[p] / E[p].
+template <class Near2>
+__device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, const double* __restrict__ sigma,
+                                                const float4* __restrict__ cjk, const NearGrid& grid,
+                                                const int32_t* __restrict__ cell_start,
+                                                const int32_t* __restrict__ cell_items, const ImageTable& img,
+                                                const Near2& near2, const double* __restrict__ pts, int64_t p,
+                                                double* __restrict__ phi, double* __restrict__ E,
+                                                int32_t* __restrict__ queue) {
+    const int nimg = img.n;
+    const double Px = pts[3 * p], Py = pts[3 * p + 1], Pz = pts[3 * p + 2];
+    float phx, phy, phz, plx, ply, plz;
+    split2f(Px, phx, plx);
+    split2f(Py, phy, ply);
+    split2f(Pz, phz, plz);
+    double aphi = 0.0, aEx = 0.0, aEy = 0.0, aEz = 0.0;
+    bool any = false;
+    near_pairs_warp(Px, Py, Pz, phx, phy, phz, plx, ply, plz, cjk, grid, cell_start, cell_items, nimg, near2, queue,
+                    [&](bool live, int32_t jk) {
+                        any = true;
+                        if (!live) return;
+                        const int32_t j = jk / nimg, k = jk - j * nimg;
+                        const Elem& e = el[j];
+                        double f, ux, uy, uz;
+                        elem_local_f64(e, Px - img.t[k][0], Py - img.t[k][1], Pz - img.t[k][2], false, f, ux, uy, uz);
+                        const double s = sigma[j];
+                        aphi = __fma_rn(s, f, aphi);
+                        aEx = __fma_rn(s, __fma_rn(ux, e.ex[0], __fma_rn(uy, e.ey[0], __dmul_rn(uz, e.ez[0]))), aEx);
+                        aEy = __fma_rn(s, __fma_rn(ux, e.ex[1], __fma_rn(uy, e.ey[1], __dmul_rn(uz, e.ez[1]))), aEy);
+                        aEz = __fma_rn(s, __fma_rn(ux, e.ex[2], __fma_rn(uy, e.ey[2], __dmul_rn(uz, e.ez[2]))), aEz);
+                    });
     if (!any) return;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -518,7 +530,7 @@ __device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, con
         aEy += __shfl_xor_sync(0xffffffffu, aEy, o);
         aEz += __shfl_xor_sync(0xffffffffu, aEz, o);
     }
-    if (lane != 0) return;
+    if ((threadIdx.x & 31) != 0) return;
     const double ke = 1.0 / (4.0 * kPi * kEps0);
     if (phi) phi[p] = __fma_rn(ke, aphi, phi[p]);
     if (E) {
@@ -528,6 +540,11 @@ __device__ __forceinline__ void near_point_warp(const Elem* __restrict__ el, con
     }
 }
 
+// squared near radii of the fill and of refinement level 2
+struct NearFill {
+    const FillEl* fe;
+    __device__ __forceinline__ float operator()(int32_t j) const { return fe[j].hdr.z; }
+};
 // squared near radii of the FP32 pass
 struct NearFar {
     const FarNodes* far;

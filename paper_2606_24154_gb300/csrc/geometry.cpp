@@ -1,8 +1,9 @@
 // geometry.cpp -- host-side FP64 construction of the device element table, the image
-// table and the FP32 far-field Gauss nodes (Sec. 2: flat rectangular / triangular
+// table, the near grid's box and the FP32 far-field Gauss nodes (Sec. 2: flat rectangular / triangular
 // elements, collocation at centroids; Sec. 5 Case 2: periodic virtual copies).
 #include "geometry.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -34,7 +35,7 @@ const double kTri3W[4] = {-27.0 / 48.0, 25.0 / 48.0, 25.0 / 48.0, 25.0 / 48.0};
 
 }  // namespace
 
-void gauss_legendre01(int m, double* x, double* w) {
+void gauss_legendre_newton(int m, double* x, double* w) {
     for (int i = 0; i < m; ++i) {
         // initial guess (Chebyshev-like) then Newton on the Legendre recurrence
         double t = std::cos(kPi * (i + 0.75) / (m + 0.5));
@@ -56,6 +57,20 @@ void gauss_legendre01(int m, double* x, double* w) {
         x[i] = 0.5 * (1.0 - t);
         w[i] = 1.0 / ((1.0 - t * t) * dp * dp);  // 2/((1-t^2) P'^2) on [-1,1], halved for [0,1]
     }
+}
+
+// The rule of m <= 16 nodes; each is made once (an element takes up to seven, and the Newton
+// iterations were two thirds of its cost on the host).
+void gauss_legendre01(int m, double* x, double* w) {
+    struct Rules {
+        double x[17][16], w[17][16];
+        Rules() {
+            for (int q = 1; q <= 16; ++q) gauss_legendre_newton(q, x[q], w[q]);
+        }
+    };
+    static const Rules rules;  // initialised once, whichever thread comes first
+    std::copy(rules.x[m], rules.x[m] + m, x);
+    std::copy(rules.w[m], rules.w[m] + m, w);
 }
 
 int build_element(const nebem_element& r, const nebem_options& opt, Elem& e, double& diag, FarNodes& fn,
@@ -309,167 +324,42 @@ int build_element(const nebem_element& r, const nebem_options& opt, Elem& e, dou
     return NEBEM_OK;
 }
 
-namespace {
-
-inline void split_f(double x, float& hi, float& lo) {
-    hi = (float)x;
-    lo = (float)(x - (double)hi);
-}
-
-inline float4 f4(float a, float b, float c, float d) {
-    float4 r;
-    r.x = a;
-    r.y = b;
-    r.z = c;
-    r.w = d;
-    return r;
-}
-
-// Two-float node record of the offset s = centroid - node (local frame) and weight w, for
-// a node pair (a, b): see nb_internal.h.
-struct FillNode {
-    double sx, sz, w;
-};
-
-inline void pack_fill_pairs(const FillNode* nd, int cnt, float4* dst) {
-    for (int p = 0; p < (cnt + 1) / 2; ++p) {
-        const FillNode a = nd[2 * p];
-        FillNode b = (2 * p + 1 < cnt) ? nd[2 * p + 1] : nd[2 * p];
-        if (2 * p + 1 >= cnt) b.w = 0.0;
-        float h[2][4], l[2][4];
-        const FillNode* ab[2] = {&a, &b};
-        for (int q = 0; q < 2; ++q) {
-            split_f(2.0 * ab[q]->sx, h[q][0], l[q][0]);
-            split_f(2.0 * ab[q]->sz, h[q][1], l[q][1]);
-            split_f(ab[q]->sx * ab[q]->sx + ab[q]->sz * ab[q]->sz, h[q][2], l[q][2]);
-            split_f(ab[q]->w, h[q][3], l[q][3]);
-        }
-        dst[4 * p + 0] = f4(h[0][0], h[1][0], h[0][1], h[1][1]);
-        dst[4 * p + 1] = f4(h[0][2], h[1][2], h[0][3], h[1][3]);
-        dst[4 * p + 2] = f4(l[0][0], l[1][0], l[0][1], l[1][1]);
-        dst[4 * p + 3] = f4(l[0][2], l[1][2], l[0][3], l[1][3]);
+GaussRules gauss_rules() {
+    GaussRules g;
+    gauss_legendre01(3, g.x3, g.w3);
+    gauss_legendre01(4, g.x4, g.w4);
+    gauss_legendre01(6, g.x6, g.w6);
+    for (int q = 0; q < 2; ++q) {
+        g.tri_a[q] = kTriA[q];
+        g.tri_w[q] = kTriW[q];
     }
+    return g;
 }
 
-}  // namespace
-
-void build_fill_tables(const std::vector<Elem>& el, const ImageTable& img, std::vector<FillEl>& fe,
-                       std::vector<float4>& nodes, std::vector<float4>& tau) {
-    const int64_t n = (int64_t)el.size();
-    const int m = img.n;
-    fe.assign((size_t)n, FillEl{});
-    nodes.assign((size_t)n * kFillNodeRec, f4(0.f, 0.f, 0.f, 0.f));
-    tau.assign((size_t)n * m * 2, f4(0.f, 0.f, 0.f, 0.f));
-    for (int64_t j = 0; j < n; ++j) {
-        const Elem& e = el[j];
-        FillEl& r = fe[j];
-        float h[3], l[3];
-        for (int a = 0; a < 3; ++a) split_f(e.c[a], h[a], l[a]);
-        r.ch = f4(h[0], h[1], h[2], 0.f);
-        r.cl = f4(l[0], l[1], l[2], 0.f);
-        const double* ax[3] = {e.ex, e.ey, e.ez};
-        float4* dh[3] = {&r.exh, &r.eyh, &r.ezh};
-        float4* dl[3] = {&r.exl, &r.eyl, &r.ezl};
-        for (int v = 0; v < 3; ++v) {
-            for (int a = 0; a < 3; ++a) split_f(ax[v][a], h[a], l[a]);
-            *dh[v] = f4(h[0], h[1], h[2], 0.f);
-            *dl[v] = f4(l[0], l[1], l[2], 0.f);
-        }
-        const double ra = kFillRatioA * e.rho, rb = kFillRatioB * e.rho, rc = kFillRatioC * e.rho;
-        const int nv = e.nv;
-        // centroid in the local frame (origin v0)
-        double d[3];
-        sub3(e.c, e.o, d);
-        const double cx = dot3(d, e.ex), cz = dot3(d, e.ez);
-        const double* qx = e.qx;
-        const double* qz = e.qz;
-        float4* out = nodes.data() + j * kFillNodeRec;
-        FillNode nd[36];
-        int cnt = 0;
-        auto put = [&](double px, double pz, double w) { nd[cnt++] = FillNode{cx - px, cz - pz, w}; };
-        int n_a = 0;  // tier-a node pairs
-        if (nv == 4) {
-            // tensor Gauss-Legendre on the bilinear map x(s, t) = q0 + s e1 + t e3 + s t tw,
-            // weight ws wt |x_s x x_t|
-            const double e1x = qx[1] - qx[0], e1z = qz[1] - qz[0];
-            const double e3x = qx[3] - qx[0], e3z = qz[3] - qz[0];
-            const double twx = qx[2] - qx[1] - e3x, twz = qz[2] - qz[1] - e3z;
-            auto tensor = [&](int mq, float4* dst) {
-                double x[16], w[16];
-                gauss_legendre01(mq, x, w);
-                cnt = 0;
-                for (int a = 0; a < mq; ++a)
-                    for (int b = 0; b < mq; ++b) {
-                        const double px = qx[0] + x[a] * e1x + x[b] * e3x + x[a] * x[b] * twx;
-                        const double pz = qz[0] + x[a] * e1z + x[b] * e3z + x[a] * x[b] * twz;
-                        const double sx = e1x + x[b] * twx, sz = e1z + x[b] * twz;
-                        const double tx = e3x + x[a] * twx, tz = e3z + x[a] * twz;
-                        put(px, pz, w[a] * w[b] * std::fabs(sx * tz - sz * tx));
-                    }
-                pack_fill_pairs(nd, cnt, dst);
-                return (cnt + 1) / 2;
-            };
-            n_a = tensor(3, out);
-            tensor(4, out + kFillOffB);
-            tensor(6, out + kFillOffC);
-        } else {
-            const double area = 0.5 * e.twoA[0];
-            cnt = 0;
-            for (int g2 = 0; g2 < 2; ++g2)
-                for (int rr = 0; rr < 3; ++rr) {
-                    double bc[3] = {kTriA[g2], kTriA[g2], kTriA[g2]};
-                    bc[rr] = 1.0 - 2.0 * kTriA[g2];
-                    const double px = bc[0] * qx[0] + bc[1] * qx[1] + bc[2] * qx[2];
-                    const double pz = bc[0] * qz[0] + bc[1] * qz[1] + bc[2] * qz[2];
-                    put(px, pz, kTriW[g2] * area);
-                }
-            pack_fill_pairs(nd, cnt, out);
-            n_a = (cnt + 1) / 2;
-            // collapsed (Duffy) product rules: x = q0 + s e1 + t (1 - s) e2, weight 2 ws wt (1 - s) A
-            auto collapsed = [&](int mq, float4* dst) {
-                double x[16], w[16];
-                gauss_legendre01(mq, x, w);
-                cnt = 0;
-                for (int a = 0; a < mq; ++a)
-                    for (int b = 0; b < mq; ++b) {
-                        const double sa = x[a], tb = x[b] * (1.0 - x[a]);
-                        const double px = qx[0] + sa * (qx[1] - qx[0]) + tb * (qx[2] - qx[0]);
-                        const double pz = qz[0] + sa * (qz[1] - qz[0]) + tb * (qz[2] - qz[0]);
-                        put(px, pz, 2.0 * w[a] * w[b] * (1.0 - x[a]) * area);
-                    }
-                pack_fill_pairs(nd, cnt, dst);
-            };
-            collapsed(4, out + kFillOffB);
-            collapsed(6, out + kFillOffC);
-        }
-        r.hdr = f4((float)(ra * ra), (float)(rb * rb), (float)(rc * rc), (float)n_a);
-        for (int k = 0; k < m; ++k) {
-            float th[3], tl[3];
-            for (int v = 0; v < 3; ++v) split_f(dot3(img.t[k], ax[v]), th[v], tl[v]);
-            tau[((size_t)j * m + k) * 2] = f4(th[0], th[1], th[2], 0.f);
-            tau[((size_t)j * m + k) * 2 + 1] = f4(tl[0], tl[1], tl[2], 0.f);
-        }
-    }
-}
-
-int build_near_grid(const std::vector<Elem>& el, const ImageTable& img, double ratio_near, NearGrid& grid,
-                    std::vector<int32_t>& cell_start, std::vector<int32_t>& cell_items, std::string& why) {
-    const int64_t n = (int64_t)el.size(), m = img.n, total = n * m;
-    if (total > (int64_t)INT32_MAX) {
+int near_grid_box(const std::vector<Elem>& el, const ImageTable& img, double ratio_near, NearGrid& grid,
+                  std::string& why) {
+    const int64_t n = (int64_t)el.size(), m = img.n;
+    if (n * m > (int64_t)INT32_MAX) {
         why = "too many element images for the near-pair grid";
         return NEBEM_TOO_LARGE;
     }
+    // the box of c_j + t_k: rounding keeps the order, so its ends come from the ends of c and t
     double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300}, rmax = 0.0;
-    std::vector<double> C((size_t)total * 3);
     for (int64_t j = 0; j < n; ++j) {
         rmax = std::fmax(rmax, ratio_near * el[j].rho);
-        for (int64_t k = 0; k < m; ++k)
-            for (int a = 0; a < 3; ++a) {
-                const double v = el[j].c[a] + img.t[k][a];
-                C[(j * m + k) * 3 + a] = v;
-                lo[a] = std::fmin(lo[a], v);
-                hi[a] = std::fmax(hi[a], v);
-            }
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = std::fmin(lo[a], el[j].c[a]);
+            hi[a] = std::fmax(hi[a], el[j].c[a]);
+        }
+    }
+    for (int a = 0; a < 3; ++a) {
+        double tl = 1e300, th = -1e300;
+        for (int64_t k = 0; k < m; ++k) {
+            tl = std::fmin(tl, img.t[k][a]);
+            th = std::fmax(th, img.t[k][a]);
+        }
+        lo[a] += tl;
+        hi[a] += th;
     }
     double h = 1.01 * rmax;
     if (!(h > 0.0)) h = 1.0;
@@ -486,23 +376,6 @@ int build_near_grid(const std::vector<Elem>& el, const ImageTable& img, double r
         grid.dims[a] = (int32_t)std::floor((hi[a] - grid.origin[a]) * grid.inv_h) + 2;
     }
     grid.pad = 0;
-    const int64_t ncell = (int64_t)grid.dims[0] * grid.dims[1] * grid.dims[2];
-    std::vector<int32_t> cell_of((size_t)total);
-    cell_start.assign((size_t)ncell + 1, 0);
-    for (int64_t i = 0; i < total; ++i) {
-        int64_t cc[3];
-        for (int a = 0; a < 3; ++a) {
-            const double f = std::floor((C[i * 3 + a] - grid.origin[a]) * grid.inv_h);
-            cc[a] = (int64_t)std::fmin(std::fmax(f, 0.0), (double)grid.dims[a] - 1.0);
-        }
-        const int64_t cell = (cc[2] * grid.dims[1] + cc[1]) * grid.dims[0] + cc[0];
-        cell_of[i] = (int32_t)cell;
-        cell_start[cell + 1]++;
-    }
-    for (int64_t c = 0; c < ncell; ++c) cell_start[c + 1] += cell_start[c];
-    cell_items.assign((size_t)total, 0);
-    std::vector<int32_t> fillp(cell_start.begin(), cell_start.end() - 1);
-    for (int64_t i = 0; i < total; ++i) cell_items[fillp[cell_of[i]]++] = (int32_t)i;  // stable: ascending j*m+k
     return NEBEM_OK;
 }
 

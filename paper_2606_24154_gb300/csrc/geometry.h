@@ -16,16 +16,17 @@ int build_element(const nebem_element& r, const nebem_options& opt, Elem& e, dou
 // Gauss-Legendre nodes and weights on [0, 1] (m <= 16), by Newton iteration on P_m.
 void gauss_legendre01(int m, double* x, double* w);
 
-// Cell list of the image centroids c_j + t_k (entry j * nimg + k) for the near-pair search;
-// near radius of element j = ratio_near * rho_j.  Cells in x-fastest order, CSR form.
-int build_near_grid(const std::vector<Elem>& el, const ImageTable& img, double ratio_near, NearGrid& grid,
-                    std::vector<int32_t>& cell_start, std::vector<int32_t>& cell_items, std::string& why);
+// Grid (box and cell edge) of the near-pair search over the image centroids c_j + t_k; near radius of
+// element j = ratio_near * rho_j.  The cell list itself is made on the device (launch_cell_list).
+int near_grid_box(const std::vector<Elem>& el, const ImageTable& img, double ratio_near, NearGrid& grid,
+                  std::string& why);
 
-// Tables of the mixed fill: per element the FillEl record and kFillNodeRec float4 of
-// two-float Gauss nodes (local frame); per (element, image) the two float4 of
-// tau = t_k . (ex, ey, ez) (hi, lo).
-void build_fill_tables(const std::vector<Elem>& el, const ImageTable& img, std::vector<FillEl>& fe,
-                       std::vector<float4>& nodes, std::vector<float4>& tau);
+// The rules of the fill's node tables (launch_fill_tables): Gauss-Legendre on [0, 1] with 3, 4 and 6
+// nodes, and the two orbits of the 6-point triangle rule (barycentric place, share of the area).
+struct GaussRules {
+    double x3[3], w3[3], x4[4], w4[4], x6[6], w6[6], tri_a[2], tri_w[2];
+};
+GaussRules gauss_rules();
 
 // Image translations t = k1 a1 + k2 a2, index (k1-lo)*m + (k2-lo); lattice NULL -> one
 // zero translation.

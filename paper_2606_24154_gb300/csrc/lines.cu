@@ -607,6 +607,16 @@ int64_t vox_pad_len(int64_t n) {
 
 int64_t vox_scan_blocks(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
 
+cudaError_t launch_sort_keys(long long* keys, int64_t P, cudaStream_t s) {
+    k_bitonic_presort<<<(unsigned)(P / kSortTile), kSortTile / 2, 0, s>>>(keys);
+    for (int64_t k = 2 * kSortTile; k <= P; k <<= 1) {
+        for (int64_t j = k >> 1; j >= kSortTile; j >>= 1)
+            k_bitonic_global<<<(unsigned)(P / 2 / 256), 256, 0, s>>>(keys, P / 2, k, j);
+        k_bitonic_merge<<<(unsigned)(P / kSortTile), kSortTile / 2, 0, s>>>(keys, k);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_voxelize(const double* pos, const double* q, int64_t n, const double d[3], const VoxWork& w,
                             cudaStream_t s) {
     if (n <= 0 || n > kVoxMaxPoints) return cudaErrorInvalidValue;
@@ -615,12 +625,7 @@ cudaError_t launch_voxelize(const double* pos, const double* q, int64_t n, const
     k_minmax_partial<<<mmb, kMM, 0, s>>>(pos, n, w.partial);
     k_minmax_final<<<1, kMMBlocks, 0, s>>>(w.partial, mmb, n, d[0], d[1], d[2], w.grid);
     k_vox_keys<<<(unsigned)(P / 256), 256, 0, s>>>(pos, n, P, w.grid, w.keys);
-    k_bitonic_presort<<<(unsigned)(P / kSortTile), kSortTile / 2, 0, s>>>(w.keys);
-    for (int64_t k = 2 * kSortTile; k <= P; k <<= 1) {
-        for (int64_t j = k >> 1; j >= kSortTile; j >>= 1)
-            k_bitonic_global<<<(unsigned)(P / 2 / 256), 256, 0, s>>>(w.keys, P / 2, k, j);
-        k_bitonic_merge<<<(unsigned)(P / kSortTile), kSortTile / 2, 0, s>>>(w.keys, k);
-    }
+    launch_sort_keys(w.keys, P, s);
     const unsigned nb256 = (unsigned)((n + 255) / 256);
     k_heads<<<nb256, 256, 0, s>>>(w.keys, n, w.flags);
     const int64_t nb = vox_scan_blocks(n);

@@ -200,6 +200,16 @@ cudaError_t launch_elem_moments(const float4* nodes, int64_t n, float4* mom, cud
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_pair_tiers(const FarNodes* far, const float4* cjk, int64_t n_el, int nimg, const double* pts,
                               int64_t npts, uint8_t* codes, cudaStream_t s);
+// tables.cu: cell list of the image centroids (entry j * nimg + k), cells in x-fastest order, CSR form:
+// cell_start (cells + 1), cell_items (n * images, ascending within a cell); work of
+// cell_list_work_bytes(n * images, cells) bytes
+size_t cell_list_work_bytes(int64_t total, int64_t ncell);
+cudaError_t launch_cell_list(const Elem* el, int64_t n, const ImageTable& img, const NearGrid& grid,
+                             int32_t* cell_start, int32_t* cell_items, void* work, cudaStream_t s);
+// Tables of the mixed fill: per element the FillEl record and kFillNodeRec float4 of two-float
+// Gauss nodes (local frame); per (element, image) the two float4 of tau = t_k . (ex, ey, ez) (hi, lo)
+cudaError_t launch_fill_tables(const Elem* el, int64_t n, const ImageTable& img, FillEl* fe, float4* nodes,
+                               float4* tau, cudaStream_t s);
 cudaError_t launch_image_centroids(const Elem* el, int64_t n, const ImageTable& img, float4* cjk, cudaStream_t s);
 cudaError_t launch_fill_f64(const Elem* el, const double* diag, int64_t n, const ImageTable& img, double* K,
                             cudaStream_t s);
@@ -330,6 +340,8 @@ struct VoxWork {
 };
 int64_t vox_pad_len(int64_t n);     // sort length: power of two >= max(n, 2048)
 int64_t vox_scan_blocks(int64_t n);
+// ascending sort of P = vox_pad_len(n) keys
+cudaError_t launch_sort_keys(long long* keys, int64_t P, cudaStream_t s);
 constexpr int64_t kVoxMaxPoints = (int64_t)1 << 26;
 cudaError_t launch_voxelize(const double* pos, const double* q, int64_t n, const double d[3], const VoxWork& w,
                             cudaStream_t s);

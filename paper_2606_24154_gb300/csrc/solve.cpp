@@ -29,31 +29,32 @@ static int elapsed_ms(Ctx* c, double* ms) {
     return 0;
 }
 
+int make_cell_list(Ctx* c, const Elem* d_el, int64_t n, const ImageTable& img, const NearGrid& grid, DevBuf& start,
+                   DevBuf& items) {
+    const int64_t total = n * img.n, ncell = (int64_t)grid.dims[0] * grid.dims[1] * grid.dims[2];
+    CK(start.ensure(sizeof(int32_t) * (size_t)(ncell + 1)));
+    CK(items.ensure(sizeof(int32_t) * (size_t)std::max<int64_t>(total, 1)));
+    CK(c->d_tab_work.ensure(cell_list_work_bytes(total, ncell)));
+    CK(launch_cell_list(d_el, n, img, grid, start.as<int32_t>(), items.as<int32_t>(), c->d_tab_work.ptr, c->stream));
+    return 0;
+}
+
 int ensure_fill_tables(Ctx* c) {
     if (c->fill_tables) return 0;
-    std::vector<FillEl> fe;
-    std::vector<float4> nodes, tau;
-    build_fill_tables(c->h_el, c->img, fe, nodes, tau);
-    std::vector<int32_t> cell_start, cell_items;
+    const int64_t n = c->n;
     std::string why;
-    int rc = build_near_grid(c->h_el, c->img, kFillRatioC, c->fill_grid, cell_start, cell_items, why);
+    int rc = near_grid_box(c->h_el, c->img, kFillRatioC, c->fill_grid, why);
     if (rc) return fail(rc, why);
-    CK(c->d_fill_el.ensure(sizeof(FillEl) * fe.size()));
-    CK(c->d_fill_nodes.ensure(sizeof(float4) * nodes.size()));
-    CK(c->d_fill_tau.ensure(sizeof(float4) * tau.size()));
-    CK(c->d_fill_cell_start.ensure(sizeof(int32_t) * cell_start.size()));
-    CK(c->d_fill_cell_items.ensure(sizeof(int32_t) * cell_items.size()));
-    CK(cudaMemcpyAsync(c->d_fill_el.ptr, fe.data(), sizeof(FillEl) * fe.size(), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->d_fill_nodes.ptr, nodes.data(), sizeof(float4) * nodes.size(), cudaMemcpyHostToDevice,
-                       c->stream));
-    CK(cudaMemcpyAsync(c->d_fill_tau.ptr, tau.data(), sizeof(float4) * tau.size(), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->d_fill_cell_start.ptr, cell_start.data(), sizeof(int32_t) * cell_start.size(),
-                       cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->d_fill_cell_items.ptr, cell_items.data(), sizeof(int32_t) * cell_items.size(),
-                       cudaMemcpyHostToDevice, c->stream));
-    CK(c->d_fill_mom.ensure(elem_moments_bytes(c->n)));
-    CK(launch_elem_moments(c->d_fill_nodes.as<float4>(), c->n, c->d_fill_mom.as<float4>(), c->stream));
-    CK(cudaStreamSynchronize(c->stream));  // the host vectors go out of scope
+    CK(c->d_fill_el.ensure(sizeof(FillEl) * n));
+    CK(c->d_fill_nodes.ensure(sizeof(float4) * kFillNodeRec * n));
+    CK(c->d_fill_tau.ensure(sizeof(float4) * 2 * n * c->img.n));
+    CK(c->d_fill_mom.ensure(elem_moments_bytes(n)));
+    CK(launch_fill_tables(c->d_el.as<Elem>(), n, c->img, c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(),
+                          c->d_fill_tau.as<float4>(), c->stream));
+    CK(launch_elem_moments(c->d_fill_nodes.as<float4>(), n, c->d_fill_mom.as<float4>(), c->stream));
+    rc = make_cell_list(c, c->d_el.as<Elem>(), n, c->img, c->fill_grid, c->d_fill_cell_start, c->d_fill_cell_items);
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(c->stream));  // evaluations on other streams use the tables too
     c->fill_tables = true;
     return 0;
 }
