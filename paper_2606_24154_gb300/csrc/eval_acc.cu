@@ -158,14 +158,18 @@ __host__ __device__ constexpr int acc_tile_f4(int level, int te, int nimg) {
                       : te * (9 + 4 * kFillPairsA + 4 * nimg);
 }
 
-// One pair that level 1 does not take by moments, by its tier's nodes: Phi' and E' (local) added to the
-// element's FP64 sums.  About one pair in a hundred; kept out of line and out of the image loop, whose
-// registers it would otherwise crowd.
+// Sums of an element's nearer pairs (those not taken by moments), two floats each.
+struct NearerSum {
+    float ph, pl, xh, xl, yh, yl, zh, zl;
+};
+
+// One such pair by its tier's nodes: Phi' and E' (local) added to N.  About one pair in a hundred; kept
+// out of line and out of the image loop, whose registers it would otherwise crowd.
 template <int M>
 __device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr, int na, int64_t j, int nimg, int k,
                                             const float (&ph)[3], const float (&pl)[3], float x0h, float x0l, float y0h,
                                             float y0l, float z0h, float z0l, const float* __restrict__ tau, int np2,
-                                            double& fphi, double& lx, double& ly, double& lz) {
+                                            NearerSum& N) {
     const int64_t jk = j * nimg + k;
     float dx, dy, dz;
     const float d2 = pair_d2(ph[0], ph[1], ph[2], pl[0], pl[1], pl[2], A.cjk[2 * jk], A.cjk[2 * jk + 1], dx, dy, dz);
@@ -189,15 +193,20 @@ __device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr,
     PairSums2 S{bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
     float2 sh = bc2(0.f), snl = bc2(0.f);
     nodes_acc2<M>(nd, np, P, sh, snl, S);
-    auto sum = [](const float2& h, const float2& nl) {
-        return ((double)h.x - (double)nl.x) + ((double)h.y - (double)nl.y);
-    };
-    if constexpr (M != kEOnly) fphi += sum(sh, snl);
+    if constexpr (M != kEOnly) {
+        float h, l, t;
+        lanes_to_df(sh, snl, 1.f, h, l);
+        two_sum(N.ph, h, N.ph, t);
+        N.pl = __fadd_rn(N.pl, __fadd_rn(t, l));
+    }
     if constexpr (M != kPhiOnly) {
-        const double s0 = sum(S.s0, S.ns0);
-        lx = fma((double)xh + (double)xl, s0, fma(0.5, sum(S.sx, S.nsx), lx));
-        ly = fma((double)yh + (double)yl, s0, ly);
-        lz = fma((double)zh + (double)zl, s0, fma(0.5, sum(S.sz, S.nsz), lz));
+        float s0h, s0l, sxh, sxl, szh, szl;
+        lanes_to_df(S.s0, S.ns0, 1.f, s0h, s0l);
+        lanes_to_df(S.sx, S.nsx, 0.5f, sxh, sxl);
+        lanes_to_df(S.sz, S.nsz, 0.5f, szh, szl);
+        df_fma_acc(xh, xl, s0h, s0l, sxh, sxl, N.xh, N.xl);
+        df_fma_acc(yh, yl, s0h, s0l, 0.f, 0.f, N.yh, N.yl);
+        df_fma_acc(zh, zl, s0h, s0l, szh, szl, N.zh, N.zl);
     }
 }
 
@@ -254,7 +263,8 @@ __device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, f
             df_dot3(dh, dl, F.eyh, F.eyl, y0h, y0l);
             df_dot3(dh, dl, F.ezh, F.ezl, z0h, z0l);
             MomSum2 S{};
-            double fphi = 0.0, lx = 0.0, ly = 0.0, lz = 0.0;  // the nearer pairs
+            NearerSum nr{};
+            bool any_nearer = false;
             const float* tau = s_tau + jj * 6 * np2;
             uint32_t nearer = 0;  // images of the group of 32 at hand whose pair is not taken by moments
             for (int k = 0; k < np2; k += 2) {
@@ -282,15 +292,16 @@ __device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, f
                 const float2 d2l = __fadd2_rn(__fadd2_rn(ex, ey), __fadd2_rn(ez, __fadd2_rn(t1, t2)));
                 const bool two = k + 1 < nimg;
                 const bool far0 = d2h.x >= mom2, far1 = two && d2h.y >= mom2;
-                mom_pair2<M != kEOnly, M != kPhiOnly>(s_mom + kMomF4 * jj, xh, xl, yh, yl, zh, zl, d2h, d2l, far0,
+                mom_pair2<M != kEOnly, M != kPhiOnly>(s_mom + kMomF4 * jj, F.ch.w, xh, xl, yh, yl, zh, zl, d2h, d2l, far0,
                                                       far1, S);
                 nearer |= ((far0 ? 0u : 1u) | (far1 || !two ? 0u : 2u)) << (k & 31);
                 if ((k & 31) == 30 || k + 2 >= np2) {
                     for (uint32_t m = nearer; m; m &= m - 1) {
                         const int kk = (k & ~31) + __ffs(m) - 1;
                         acc_pair_nodes<M>(A, hdr, (int)F.hdr.w, j, nimg, kk, ph, pl, x0h, x0l, y0h, y0l, z0h, z0l, tau,
-                                          np2, fphi, lx, ly, lz);
+                                          np2, nr);
                     }
+                    any_nearer = any_nearer || nearer;
                     nearer = 0;
                 }
             }
@@ -300,8 +311,8 @@ __device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, f
             // error scales stay in FP32.
             const double s = A.sigma[j];
             const float4 tail = s_mom[kMomF4 * jj + kMomF4 - 1];
-            // sign: -1 where the high parts are kept negated
-            auto total = [&](float sign, const float2& h, const float2& l, const float2& c, float& oh, float& ol) {
+            // sign: -1 where the high parts are kept negated; unit: what c is kept over
+            auto total = [&](float sign, float unit, const float2& h, const float2& l, const float2& c, float& oh, float& ol) {
                 float sh, t, p, e;
                 two_sum(h.x, h.y, sh, t);
                 sh *= sign;
@@ -309,23 +320,30 @@ __device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, f
                 two_prod(sh, tail.z, p, e);
                 e = __fmaf_rn(sh, tail.w, __fmaf_rn(sl, tail.z, e));
                 oh = p;
-                ol = __fadd_rn(e, __fadd_rn(c.x, c.y));
+                ol = __fmaf_rn(__fadd_rn(c.x, c.y), unit, e);
             };
+            const float rho = F.ch.w;
             if constexpr (M != kEOnly) {
                 float h, l;
-                total(1.f, S.ph, S.pl, S.fc, h, l);
-                fphi += (double)h + (double)l;
+                total(1.f, rho * rho, S.ph, S.pl, S.fc, h, l);
+                double fphi = (double)h + (double)l;
+                if (any_nearer) fphi += (double)nr.ph + (double)nr.pl;
                 acc.phi = fma(s, fphi, acc.phi);
                 bphi = fmaf(fabsf((float)s), fabsf((float)fphi), bphi);
             }
             if constexpr (M != kPhiOnly) {
                 float h, l;
-                total(-1.f, S.xh, S.xl, S.ex, h, l);
-                lx += (double)h + (double)l;
-                total(-1.f, S.yh, S.yl, S.ey, h, l);
-                ly += (double)h + (double)l;
-                total(-1.f, S.zh, S.zl, S.ez, h, l);
-                lz += (double)h + (double)l;
+                total(-1.f, rho, S.xh, S.xl, S.ex, h, l);
+                double lx = (double)h + (double)l;
+                total(-1.f, rho, S.yh, S.yl, S.ey, h, l);
+                double ly = (double)h + (double)l;
+                total(-1.f, rho, S.zh, S.zl, S.ez, h, l);
+                double lz = (double)h + (double)l;
+                if (any_nearer) {
+                    lx += (double)nr.xh + (double)nr.xl;
+                    ly += (double)nr.yh + (double)nr.yl;
+                    lz += (double)nr.zh + (double)nr.zl;
+                }
                 const Elem& e = A.el[j];
                 const double gx = fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0]));
                 const double gy = fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1]));
@@ -643,17 +661,18 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
 }
 
 // ElemMom records (twofloat.cuh) from the elements' 36-node rules, which integrate degree 4 exactly.
-__global__ void k_elem_moments(const float4* __restrict__ nodes, int64_t n, float4* __restrict__ mom) {
+__global__ void k_elem_moments(const FillEl* __restrict__ fe, const float4* __restrict__ nodes, int64_t n,
+                               float4* __restrict__ mom) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const float4* nd = nodes + j * kFillNodeRec + kFillOffC;
+    const double half = -0.5 / (double)fe[j].ch.w;  // u = (node - centroid) / rho = -s / rho, stored as 2 s
     double A = 0.0, M2[3] = {}, M3[4] = {}, M4[5] = {};
     for (int q = 0; q < kFillPairsC; ++q) {
         const float4 h0 = nd[4 * q], h1 = nd[4 * q + 1], l0 = nd[4 * q + 2], l1 = nd[4 * q + 3];
         for (int lane = 0; lane < 2; ++lane) {
-            // u = node - centroid = -s, stored as 2 s
-            const double x = -0.5 * (lane ? (double)h0.y + (double)l0.y : (double)h0.x + (double)l0.x);
-            const double z = -0.5 * (lane ? (double)h0.w + (double)l0.w : (double)h0.z + (double)l0.z);
+            const double x = half * (lane ? (double)h0.y + (double)l0.y : (double)h0.x + (double)l0.x);
+            const double z = half * (lane ? (double)h0.w + (double)l0.w : (double)h0.z + (double)l0.z);
             const double w = lane ? (double)h1.w + (double)l1.w : (double)h1.z + (double)l1.z;
             A += w;
             M2[0] += w * x * x, M2[1] += w * x * z, M2[2] += w * z * z;
@@ -681,9 +700,9 @@ __global__ void k_elem_moments(const float4* __restrict__ nodes, int64_t n, floa
 }  // namespace
 
 size_t elem_moments_bytes(int64_t n) { return sizeof(float4) * kMomF4 * (size_t)n; }
-cudaError_t launch_elem_moments(const float4* nodes, int64_t n, float4* mom, cudaStream_t s) {
+cudaError_t launch_elem_moments(const FillEl* fe, const float4* nodes, int64_t n, float4* mom, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    k_elem_moments<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(nodes, n, mom);
+    k_elem_moments<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(fe, nodes, n, mom);
     return cudaGetLastError();
 }
 

@@ -86,7 +86,7 @@ constexpr int kFillPairsC = 18;
 constexpr int kFillOffB = 4 * kFillPairsA;
 constexpr int kFillOffC = 4 * (kFillPairsA + kFillPairsB);
 constexpr int kFillNodeRec = 4 * (kFillPairsA + kFillPairsB + kFillPairsC);  // float4 per element
-// Per element: centroid c and frame (ex, ey, ez) as hi + lo floats; hdr = squared tier
+// Per element: centroid c and frame (ex, ey, ez) as hi + lo floats (ch.w = rho); hdr = squared tier
 // distances (a, b, c) in m^2 and the tier-a node-pair count.
 struct __align__(16) FillEl {
     float4 ch, cl;
@@ -196,7 +196,7 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
                                double* phi, double* E, double* err, double tol, const ErrModel& em,
                                const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part);
 size_t elem_moments_bytes(int64_t n);
-cudaError_t launch_elem_moments(const float4* nodes, int64_t n, float4* mom, cudaStream_t s);
+cudaError_t launch_elem_moments(const FillEl* fe, const float4* nodes, int64_t n, float4* mom, cudaStream_t s);
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_pair_tiers(const FarNodes* far, const float4* cjk, int64_t n_el, int nimg, const double* pts,
                               int64_t npts, uint8_t* codes, cudaStream_t s);

@@ -51,7 +51,7 @@ int ensure_fill_tables(Ctx* c) {
     CK(c->d_fill_mom.ensure(elem_moments_bytes(n)));
     CK(launch_fill_tables(c->d_el.as<Elem>(), n, c->img, c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(),
                           c->d_fill_tau.as<float4>(), c->stream));
-    CK(launch_elem_moments(c->d_fill_nodes.as<float4>(), n, c->d_fill_mom.as<float4>(), c->stream));
+    CK(launch_elem_moments(c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(), n, c->d_fill_mom.as<float4>(), c->stream));
     rc = make_cell_list(c, c->d_el.as<Elem>(), n, c->img, c->fill_grid, c->d_fill_cell_start, c->d_fill_cell_items);
     if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));  // evaluations on other streams use the tables too

@@ -112,6 +112,7 @@ __global__ void k_fill_records(const Elem* __restrict__ el, int64_t n, FillEl* _
     const Elem& e = el[j];
     FillEl r;
     r.ch = hi4(e.c), r.cl = lo4(e.c, r.ch);
+    r.ch.w = (float)e.rho;
     r.exh = hi4(e.ex), r.exl = lo4(e.ex, r.exh);
     r.eyh = hi4(e.ey), r.eyl = lo4(e.ey, r.eyh);
     r.ezh = hi4(e.ez), r.ezl = lo4(e.ez, r.ezh);

@@ -130,7 +130,8 @@ __device__ __forceinline__ void node_rinv2(const PairDF2& P, const float4& q0, c
 // ---------------------------------------------------------------- far pairs by moments
 // A pair far from its element (d >= kMomRatio radii) by the element's planar moments about its
 // centroid, two images per packed instruction.  With n = D / d, y = 1 / d,
-//   Phi' = A y + y^3 (f2 + y f3 + y^2 f4),   E' = A D y^3 + y^4 [(r2 + y r3 + y^2 r4) n - (w2 + y w3 + y^2 w4)],
+//   Phi' = A y + y^3 rho^2 (f2 + s f3 + s^2 f4),
+//   E' = A D y^3 + y^3 s rho [(r2 + s r3 + s^2 r4) n - (w2 + s w3 + s^2 w4)],   s = y rho,
 // the monopole and the terms of degree 2 to 4 of the multipole series of 1 / |D - u| over the
 // element's points u (degree 1 vanishes about the centroid).  Only the monopole needs two-float
 // arithmetic: the rest is below (rho / d)^2 / 5 of the pair, so plain FP32 leaves an error of about
@@ -143,7 +144,8 @@ __device__ __forceinline__ void node_rinv2(const PairDF2& P, const float4& q0, c
 // ElemMom per element: every constant twice (both lanes), two constants per float4:
 //   3 M20, 3 M11 | 3 M02, -t2 / 2 | k30, k21 | k12, k03 | -tx, -tz | K40, K31 | K13, K04 | T31, T22 | T13, P20 |
 //   P11, P02 | q0, 5 q0 | -3 t2 / 2, then the area A as hi, lo
-// with M the moments of u = node - centroid in the element plane, t2 = M20 + M02, k = 7.5 M, (tx, tz) = 1.5
+// with M the moments of u = (node - centroid) / rho in the element plane (scaled by the element's radius, so
+// that they are FP32 numbers at any size of the geometry), t2 = M20 + M02, k = 7.5 M, (tx, tz) = 1.5
 // (M30 + M12, M21 + M03), K = 17.5 M, T = 3 K, P = -7.5 (M40 + M22, M31 + M13, M22 + M04), q0 = 0.375 (M40 +
 // 2 M22 + M04).
 constexpr double kMomRatio = 28.0;
@@ -152,7 +154,7 @@ constexpr int kMomF4 = 12;
 struct MomSum2 {  // sums over the images of an element, both lanes
     float2 ph, pl;                        // y, two floats (times A: the monopole's potential)
     float2 xh, xl, yh, yl, zh, zl;        // D y^3, two floats: minus the high part, the low part
-    float2 fc, ex, ey, ez;                // the other terms, FP32
+    float2 fc, ex, ey, ez;                // the other terms, FP32, over rho^2 and rho
 };
 
 __device__ __forceinline__ float2 lane2(const float4& v, int i) {
@@ -162,7 +164,7 @@ __device__ __forceinline__ float2 lane2(const float4& v, int i) {
 // One step: local differences X, Y, Z (two floats each) of two images; lanes with far = false add 0.
 // Returns nothing for them: the caller evaluates those pairs itself.  d2h is |D|^2's high part.
 template <bool kPhi, bool kField>
-__device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float2 xh, float2 xl, float2 yh, float2 yl,
+__device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float rho, float2 xh, float2 xl, float2 yh, float2 yl,
                                           float2 zh, float2 zl, float2 d2h, float2 d2l, bool far0, bool far1,
                                           MomSum2& S) {
     const float2 m1 = bc2(-1.f);
@@ -206,6 +208,7 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float2
         add(zh, zl, S.zh, S.zl);
     }
     // degrees 2 to 4 in FP32
+    const float2 s = __fmul2_rn(y0, bc2(rho)), s2 = __fmul2_rn(s, s);
     const float2 nx = __fmul2_rn(xh, y0), nz = __fmul2_rn(zh, y0);
     const float2 qxx = __fmul2_rn(nx, nx), qxz = __fmul2_rn(nx, nz), qzz = __fmul2_rn(nz, nz);
     const float2 qd = __fadd2_rn(qxz, qxz);
@@ -235,7 +238,7 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float2
         const float2 f2 = __ffma2_rn(bc2(0.5f), T2, lane2(m1_, 1));
         const float2 f3 = __ffma2_rn(bc2(1.f / 3.f), W3, __fmul2_rn(bc2(2.f / 3.f), ntn));
         const float2 f4 = __ffma2_rn(bc2(0.25f), __fadd2_rn(W4, Q), lane2(m10, 0));
-        const float2 f = __ffma2_rn(a, f4, __ffma2_rn(y0, f3, f2));
+        const float2 f = __ffma2_rn(s2, f4, __ffma2_rn(s, f3, f2));
         S.fc = __ffma2_rn(c3, f, S.fc);
     }
     if constexpr (kField) {
@@ -243,13 +246,13 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float2
         const float2 r2 = __ffma2_rn(bc2(2.5f), T2, lane2(mom[11], 0));
         const float2 r3 = __ffma2_rn(bc2(7.f / 3.f), W3, __fmul2_rn(bc2(8.f / 3.f), ntn));
         const float2 r4 = __ffma2_rn(bc2(2.25f), W4, __ffma2_rn(bc2(1.25f), Q, lane2(m10, 1)));
-        const float2 r = __ffma2_rn(a, r4, __ffma2_rn(y0, r3, r2));
-        const float2 wx = __ffma2_rn(a, w4x, __ffma2_rn(y0, w3x, w2x));
-        const float2 wz = __ffma2_rn(a, w4z, __ffma2_rn(y0, w3z, w2z));
-        const float2 y4 = __fmul2_rn(a, a), ny4 = __fmul2_rn(na, a), s = __fmul2_rn(y4, r);
-        S.ex = __ffma2_rn(ny4, wx, __ffma2_rn(s, nx, S.ex));
-        S.ey = __ffma2_rn(s, ny, S.ey);
-        S.ez = __ffma2_rn(ny4, wz, __ffma2_rn(s, nz, S.ez));
+        const float2 r = __ffma2_rn(s2, r4, __ffma2_rn(s, r3, r2));
+        const float2 wx = __ffma2_rn(s2, w4x, __ffma2_rn(s, w3x, w2x));
+        const float2 wz = __ffma2_rn(s2, w4z, __ffma2_rn(s, w3z, w2z));
+        const float2 k = __fmul2_rn(c3, s), nk = __fmul2_rn(k, m1), kr = __fmul2_rn(k, r);
+        S.ex = __ffma2_rn(nk, wx, __ffma2_rn(kr, nx, S.ex));
+        S.ey = __ffma2_rn(kr, ny, S.ey);
+        S.ez = __ffma2_rn(nk, wz, __ffma2_rn(kr, nz, S.ez));
     }
 }
 

@@ -1,5 +1,5 @@
 """The refinement's first level: pairs from 28 radii on by the element's moments, nearer ones by Gauss
-nodes, against the FP64 path; one element of each kind, with 1, 9, 25 and 121 copies (an odd count
+nodes, against the FP64 path; one element of each kind (of 20 um, and scaled by 1e-5 and 1e5), with 1, 9, 25 and 121 copies (an odd count
 leaves half of the last packed step empty).
 
 Tolerance (derived before the first run): the series ends at degree 4, and the terms left out are
@@ -22,12 +22,12 @@ SHAPES = {
 }
 
 
-@pytest.mark.parametrize("half", [0, 1, 2, 5])
+@pytest.mark.parametrize("half, scale", [(0, 1.0), (1, 1.0), (2, 1.0), (5, 1.0), (1, 1e-5), (1, 1e5)])
 @pytest.mark.parametrize("name", list(SHAPES))
-def test_level1_against_fp64(name, half):
+def test_level1_against_fp64(name, half, scale):
     from paper_2606_24154_gb300 import build, nebem as N
     build.build()
-    kind, verts = SHAPES[name]
+    kind, verts = SHAPES[name][0], scale * np.array(SHAPES[name][1], float)
     el = np.zeros(1, dtype=I.ELEMENT_DTYPE)
     el["kind"], el["eps_a"], el["eps_b"] = kind, 1.0, 1.0
     v = np.zeros((4, 3))
@@ -43,7 +43,7 @@ def test_level1_against_fp64(name, half):
     pts = c + r[:, None] * d
     # level 1 for every point: an estimate above the tolerance after the FP32 pass, below it after level 1
     ctx = N.Context(mixed_point_tol=1e-6)
-    lattice = np.array([2000.0 * U, 0, 0, 0, 2000.0 * U, 0]) if half else None
+    lattice = scale * np.array([2000.0 * U, 0, 0, 0, 2000.0 * U, 0]) if half else None
     N.nebem_set_geometry(ctx.h, el, lattice, -half, half)
     ctx.n = 1
     ctx.set_sigma(np.array([1e-6]))
