@@ -91,7 +91,7 @@ struct Ctx {
 
     // mixed fill tables (built on the first mixed fill of a geometry): element records,
     // two-float nodes, tau = t_k . frame, and the cell list for its near radius
-    DevBuf d_fill_el, d_fill_nodes, d_fill_mom, d_fill_tau, d_fill_cell_start, d_fill_cell_items;
+    DevBuf d_fill_el, d_fill_nodes, d_fill_mom, d_fill_phimom, d_fill_tau, d_fill_cell_start, d_fill_cell_items;
     NearGrid fill_grid{};
     bool fill_tables = false;
 

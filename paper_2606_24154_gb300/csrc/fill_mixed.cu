@@ -111,19 +111,53 @@ __device__ __forceinline__ void stage(float4* dst, const float4* __restrict__ sr
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) dst[i] = src[i];
 }
 
-// Dynamic shared memory per tile of te elements: FillEl (9 float4), tier-a nodes (18 float4),
-// tau and image centroids (2 float4 each per image).
-__host__ __device__ constexpr int fill_tile_f4(int te, int nimg) { return te * (9 + 4 * kFillPairsA + 4 * nimg); }
+// Dynamic shared memory per tile of te elements: FillEl (9 float4), FillMom, and tau as six planes of
+// nimg (padded to even) floats (x, y, z negated: hi, then lo).
+__host__ __device__ constexpr int fill_pad(int nimg) { return (nimg + 1) & ~1; }
+__host__ __device__ constexpr int fill_tile_f4(int te, int nimg) {
+    return te * (9 + kFillMomF4) + (te * 6 * fill_pad(nimg) + 3) / 4;
+}
 
+// The pair (row i, element j, image k) by its tier's nodes where it is nearer than the moments reach (one
+// to three pairs in a hundred); a near pair is left to k_fill_near.
+__device__ __noinline__ void fill_pair_nodes(const float4* __restrict__ nd, const float4* __restrict__ cjk2,
+                                             const float4& hdr, const float (&ch)[3], const float (&cl)[3], const float (&Xh)[3],
+                                             const float (&Xl)[3], bool iface, const FillRow& R, float2& sh,
+                                             float2& snl) {
+    float dx, dy, dz;
+    if (!(pair_d2(ch[0], ch[1], ch[2], cl[0], cl[1], cl[2], cjk2[0], cjk2[1], dx, dy, dz) >= hdr.z)) return;
+    float d2h, d2l;
+    df_norm2(Xh[0], Xl[0], Xh[1], Xl[1], Xh[2], Xl[2], d2h, d2l);
+    PairDF2 P;
+    P.xh = bc2(Xh[0]), P.nxh = bc2(-Xh[0]), P.xl = bc2(Xl[0]);
+    P.zh = bc2(Xh[2]), P.nzh = bc2(-Xh[2]), P.zl = bc2(Xl[2]);
+    P.d2h = bc2(d2h), P.d2l = bc2(d2l);
+    if (!iface) {
+        nodes_phi2(nd + kFillOffC, kFillPairsC, P, sh, snl);
+        return;
+    }
+    NormDF2 Nn;
+    Nn.nxh = bc2(R.nxh), Nn.nnxh = bc2(-R.nxh), Nn.nxl = bc2(R.nxl);
+    Nn.nzh = bc2(R.nzh), Nn.nnzh = bc2(-R.nzh), Nn.nzl = bc2(R.nzl);
+    float ndh, ndl;
+    df_dot3(Xh, Xl, make_float4(R.nxh, R.nyh, R.nzh, 0.f), make_float4(R.nxl, R.nyl, R.nzl, 0.f), ndh, ndl);
+    Nn.ndh = bc2(ndh), Nn.ndl = bc2(ndl);
+    const bool b = d2h >= hdr.y;
+    nodes_nE2(nd + (b ? kFillOffB : kFillOffC), b ? kFillPairsB : kFillPairsC, P, Nn, sh, snl);
+}
+
+// Far pairs of a block's 128 rows and kFillCols columns: the moments from 32 radii on (interface rows:
+// 52), nodes nearer.  9,996 elements x 25 copies (18 % interface rows) took 71 ms with nodes
+// for every pair and 35 ms so; bound by the FP32 pipe.
 __global__ void __launch_bounds__(kFT, 4)
-    k_fill_far(const FillEl* __restrict__ fe, const float4* __restrict__ nodes, const float4* __restrict__ tau,
-               const float4* __restrict__ cjk, const double* __restrict__ diag_in, int64_t n, int nimg, int te,
-               double* __restrict__ K) {
+    k_fill_far(const FillEl* __restrict__ fe, const float4* __restrict__ nodes, const float4* __restrict__ mom,
+               const float4* __restrict__ tau, const float4* __restrict__ cjk, const double* __restrict__ diag_in,
+               int64_t n, int nimg, int te, double* __restrict__ K) {
     extern __shared__ float4 sm[];
     FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
-    float4* s_na = sm + 9 * te;
-    float4* s_tau = s_na + 4 * kFillPairsA * te;
-    float4* s_c = s_tau + 2 * nimg * te;
+    float4* s_mom = sm + 9 * te;
+    float* s_tau = reinterpret_cast<float*>(s_mom + kFillMomF4 * te);
+    const int np2 = fill_pad(nimg);
 
     const int64_t i = (int64_t)blockIdx.x * kFT + threadIdx.x;
     const bool active = i < n;
@@ -147,18 +181,20 @@ __global__ void __launch_bounds__(kFT, 4)
         const int cnt = (int)min((int64_t)te, j1 - base);
         __syncthreads();
         stage(reinterpret_cast<float4*>(s_fe), reinterpret_cast<const float4*>(fe + base), 9 * cnt);
-        for (int e = threadIdx.x; e < cnt * 4 * kFillPairsA; e += blockDim.x) {
-            const int jj = e / (4 * kFillPairsA), q = e - jj * 4 * kFillPairsA;
-            s_na[e] = nodes[(base + jj) * kFillNodeRec + q];
+        stage(s_mom, mom + base * kFillMomF4, kFillMomF4 * cnt);
+        for (int q = threadIdx.x; q < cnt * np2; q += blockDim.x) {
+            const int jj = q / np2, k = min(q - jj * np2, nimg - 1);
+            const float4 h = tau[2 * ((base + jj) * nimg + k)], l = tau[2 * ((base + jj) * nimg + k) + 1];
+            float* d = s_tau + jj * 6 * np2 + (q - jj * np2);
+            d[0] = -h.x, d[np2] = -h.y, d[2 * np2] = -h.z;
+            d[3 * np2] = -l.x, d[4 * np2] = -l.y, d[5 * np2] = -l.z;
         }
-        stage(s_tau, tau + 2 * base * nimg, 2 * cnt * nimg);
-        stage(s_c, cjk + 2 * base * nimg, 2 * cnt * nimg);
         __syncthreads();
         for (int jj = 0; jj < cnt; ++jj) {
             const FillEl& E = s_fe[jj];
+            const float4* M = s_mom + kFillMomF4 * jj;
             const int64_t j = base + jj;
-            const float4 hdr = E.hdr;
-            const int na = (int)hdr.w;
+            const float* nt = s_tau + jj * 6 * np2;
             // c_i - c_j and its local components
             float dh[3], dl[3];
             df_sub(ch[0], cl[0], E.ch.x, E.cl.x, dh[0], dl[0]);
@@ -168,62 +204,135 @@ __global__ void __launch_bounds__(kFT, 4)
             df_dot3(dh, dl, E.exh, E.exl, x0h, x0l);
             df_dot3(dh, dl, E.eyh, E.eyl, y0h, y0l);
             df_dot3(dh, dl, E.ezh, E.ezl, z0h, z0l);
-            float nxh = 0.f, nxl = 0.f, nyh = 0.f, nyl = 0.f, nzh = 0.f, nzl = 0.f;
+            FillRow R;
             if (iface) {
-                df_dot3(nh, nl, E.exh, E.exl, nxh, nxl);
-                df_dot3(nh, nl, E.eyh, E.eyl, nyh, nyl);
-                df_dot3(nh, nl, E.ezh, E.ezl, nzh, nzl);
+                df_dot3(nh, nl, E.exh, E.exl, R.nxh, R.nxl);
+                df_dot3(nh, nl, E.eyh, E.eyl, R.nyh, R.nyl);
+                df_dot3(nh, nl, E.ezh, E.ezl, R.nzh, R.nzl);
+                // gx = 2 a1 n_x + a2 n_z, gz = a2 n_x + 2 a3 n_z
+                auto dot2 = [](float ah, float al, float bh, float bl, float xh, float xl, float zh, float zl, float& h,
+                               float& l) {
+                    float p, e, q, f, t;
+                    two_prod(ah, xh, p, e);
+                    two_prod(bh, zh, q, f);
+                    two_sum(p, q, h, t);
+                    e = __fmaf_rn(ah, xl, __fmaf_rn(al, xh, e));
+                    f = __fmaf_rn(bh, zl, __fmaf_rn(bl, zh, f));
+                    l = __fadd_rn(t, __fadd_rn(e, f));
+                };
+                dot2(M[0].x + M[0].x, M[0].z + M[0].z, M[1].x, M[1].z, R.nxh, R.nxl, R.nzh, R.nzl, R.gxh, R.gxl);
+                dot2(M[1].x, M[1].z, M[2].x + M[2].x, M[2].z + M[2].z, R.nxh, R.nxl, R.nzh, R.nzl, R.gzh, R.gzl);
             }
-            NormDF2 Nn;
-            if (iface) {
-                Nn.nxh = bc2(nxh), Nn.nnxh = bc2(-nxh), Nn.nxl = bc2(nxl);
-                Nn.nzh = bc2(nzh), Nn.nnzh = bc2(-nzh), Nn.nzl = bc2(nzl);
-            }
-            float2 sh = bc2(0.f), snl = bc2(0.f);  // sum: hi, negated lo
-            for (int k = 0; k < nimg; ++k) {
-                float dx, dy, dz;
-                const float d2 = pair_d2(ch[0], ch[1], ch[2], cl[0], cl[1], cl[2], s_c[2 * (jj * nimg + k)],
-                                         s_c[2 * (jj * nimg + k) + 1], dx, dy, dz);
-                if (!(d2 >= hdr.z)) continue;  // near pair: k_fill_near
-                const float4 th = s_tau[2 * (jj * nimg + k)], tl = s_tau[2 * (jj * nimg + k) + 1];
-                float xh, xl, yh, yl, zh, zl, d2h, d2l;
-                df_sub(x0h, x0l, th.x, tl.x, xh, xl);
-                df_sub(y0h, y0l, th.y, tl.y, yh, yl);
-                df_sub(z0h, z0l, th.z, tl.z, zh, zl);
-                df_norm2(xh, xl, yh, yl, zh, zl, d2h, d2l);
-                PairDF2 P;
-                P.xh = bc2(xh), P.nxh = bc2(-xh), P.xl = bc2(xl);
-                P.zh = bc2(zh), P.nzh = bc2(-zh), P.zl = bc2(zl);
-                P.d2h = bc2(d2h), P.d2l = bc2(d2l);
-                const float4* nd;
-                int np;
-                if (d2 >= hdr.x) {
-                    nd = s_na + jj * 4 * kFillPairsA;
-                    np = na;
-                } else if (d2 >= hdr.y) {
-                    nd = nodes + j * kFillNodeRec + kFillOffB;
-                    np = kFillPairsB;
-                } else {
-                    nd = nodes + j * kFillNodeRec + kFillOffC;
-                    np = kFillPairsC;
-                }
-                if (!iface) {
-                    nodes_phi2(nd, np, P, sh, snl);
-                } else {
-                    const float Xh[3] = {xh, yh, zh}, Xl[3] = {xl, yl, zl};
-                    float ndh, ndl;
-                    df_dot3(Xh, Xl, make_float4(nxh, nyh, nzh, 0.f), make_float4(nxl, nyl, nzl, 0.f), ndh, ndl);
-                    Nn.ndh = bc2(ndh), Nn.ndl = bc2(ndl);
-                    nodes_nE2(nd, np, P, Nn, sh, snl);
+            float2 sh = bc2(0.f), snl = bc2(0.f);  // node sums: hi, negated lo
+            float2 Sh = bc2(0.f), Sl = bc2(0.f);   // moment sums
+            const float mom2 = iface ? E.hdr.y * (float)(kFillMomField * kFillMomField / (kFillRatioB * kFillRatioB))
+                                     : E.hdr.y;
+            uint32_t nearer = 0;  // images of the group of 32 at hand that the moments do not reach
+            for (int k = 0; k < np2; k += 2) {
+                auto diff = [&](float ah, float al, int q, float2& h, float2& l) {
+                    float2 t;
+                    two_sum2(bc2(ah), *reinterpret_cast<const float2*>(nt + q * np2 + k), h, t);
+                    l = __fadd2_rn(t, __fadd2_rn(bc2(al), *reinterpret_cast<const float2*>(nt + (q + 3) * np2 + k)));
+                };
+                auto square = [](float2 h, float2 l, float2& p, float2& e) {
+                    p = __fmul2_rn(h, h);
+                    e = __ffma2_rn(__fadd2_rn(h, h), l, __ffma2_rn(h, h, make_float2(-p.x, -p.y)));
+                };
+                FillPair2 P;
+                float2 yh, yl, py, ey, s, t1, t2;
+                diff(x0h, x0l, 0, P.xh, P.xl);
+                diff(y0h, y0l, 1, yh, yl);
+                diff(z0h, z0l, 2, P.zh, P.zl);
+                square(P.xh, P.xl, P.px, P.ex);
+                square(yh, yl, py, ey);
+                square(P.zh, P.zl, P.pz, P.ez);
+                two_sum2(P.px, py, s, t1);
+                two_sum2(s, P.pz, P.d2h, t2);
+                P.d2l = __fadd2_rn(__fadd2_rn(P.ex, ey), __fadd2_rn(P.ez, __fadd2_rn(t1, t2)));
+                const bool two = k + 1 < nimg;
+                const bool far0 = P.d2h.x >= mom2, far1 = two && P.d2h.y >= mom2;
+                if (iface)
+                    fill_mom_field2(M, R, P, yh, yl, far0, far1, Sh, Sl);
+                else
+                    fill_mom_phi2(M, P, far0, far1, Sh, Sl);
+                nearer |= ((far0 ? 0u : 1u) | (far1 || !two ? 0u : 2u)) << (k & 31);
+                if ((k & 31) == 30 || k + 2 >= np2) {
+                    for (uint32_t m = nearer; m; m &= m - 1) {
+                        const int kk = (k & ~31) + __ffs(m) - 1;
+                        float Xh[3], Xl[3];
+                        df_sub(x0h, x0l, -nt[kk], -nt[3 * np2 + kk], Xh[0], Xl[0]);
+                        df_sub(y0h, y0l, -nt[np2 + kk], -nt[4 * np2 + kk], Xh[1], Xl[1]);
+                        df_sub(z0h, z0l, -nt[2 * np2 + kk], -nt[5 * np2 + kk], Xh[2], Xl[2]);
+                        fill_pair_nodes(nodes + j * kFillNodeRec, cjk + 2 * (j * nimg + kk), E.hdr, ch, cl, Xh, Xl,
+                                        iface, R, sh, snl);
+                    }
+                    nearer = 0;
                 }
             }
             if (active) {
-                // the two lanes' sums (hi + lo each) in FP64
-                const double acc = ((double)sh.x - (double)snl.x) + ((double)sh.y - (double)snl.y);
+                // A (sum over the images) in two floats; the node sums' lanes (hi + lo each) in FP64
+                const float4 area = M[kFillMomF4 - 1];
+                float h, t, p, e;
+                two_sum(Sh.x, Sh.y, h, t);
+                const float l = __fadd_rn(t, __fadd_rn(Sl.x, Sl.y));
+                two_prod(h, area.x, p, e);
+                e = __fmaf_rn(h, area.y, __fmaf_rn(l, area.x, e));
+                const double acc = ((double)p + (double)e) + (((double)sh.x - (double)snl.x) + ((double)sh.y - (double)snl.y));
                 K[i + j * n] = (i == j) ? fma(ke, acc, diag) : ke * acc;
             }
         }
     }
+}
+
+// FillMom records (twofloat.cuh) from the elements' 36-node rules, which integrate degree 6 exactly:
+//   |u|^l P_l(cos(D, u)) = sum_m c_lm (D.u / d)^(l - 2m) |u|^2m,  c_lm = (-1)^m (2l - 2m)! / (2^l m! (l-m)! (l-2m)!).
+__global__ void k_fill_moments(const FillEl* __restrict__ fe, const float4* __restrict__ nodes, int64_t n,
+                               float4* __restrict__ mom) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const double s = exp2(ceil(log2((double)fe[j].ch.w)));
+    const float4* nd = nodes + j * kFillNodeRec + kFillOffC;
+    double M[7][7];  // moments of ((node - centroid) / s)_x^a (..)_z^b, over A below
+    for (int a = 0; a < 7; ++a)
+        for (int b = 0; b < 7; ++b) M[a][b] = 0.0;
+    for (int q = 0; q < 2 * kFillPairsC; ++q) {
+        const float4* r = nd + 4 * (q / 2);
+        const bool o = q & 1;
+        const double x = -0.5 / s * (o ? (double)r[0].y + (double)r[2].y : (double)r[0].x + (double)r[2].x);
+        const double z = -0.5 / s * (o ? (double)r[0].w + (double)r[2].w : (double)r[0].z + (double)r[2].z);
+        double px = o ? (double)r[1].w + (double)r[3].w : (double)r[1].z + (double)r[3].z;  // w x^a z^b
+        for (int a = 0; a < 7; ++a, px *= x) {
+            double v = px;
+            for (int b = 0; a + b < 7; ++b, v *= z) M[a][b] += v;
+        }
+    }
+    const double A = M[0][0];
+    const double fact[13] = {1, 1, 2, 6, 24, 120, 720, 5040, 40320, 362880, 3628800, 39916800, 479001600};
+    double c[8 + kFillMomCoef + 1];
+    const double quad[4] = {1.5 * M[2][0] / A, 3.0 * M[1][1] / A, 1.5 * M[0][2] / A, -0.5 * (M[2][0] + M[0][2]) / A};
+    for (int q = 0; q < 4; ++q) {
+        c[2 * q] = quad[q];
+        c[2 * q + 1] = quad[q] - (double)__double2float_rn(quad[q]);
+    }
+    for (int i = 0; i < 7; ++i)
+        for (int k = i; k < 7; ++k)
+            for (int t = 0; t < fill_mom_terms(k); ++t) {
+                const int jz = k - i, m = fill_mom_m0(k) + t, l = k + 2 * m;
+                double v = 0.0;  // integral of u_x^i u_z^jz |u|^2m
+                for (int r = 0; r <= m; ++r)
+                    v += fact[m] / (fact[r] * fact[m - r]) * M[i + 2 * r][jz + 2 * (m - r)];
+                const double clm = (m & 1 ? -1.0 : 1.0) * fact[2 * l - 2 * m] /
+                                   ((double)(1 << l) * fact[m] * fact[l - m] * fact[k]);
+                c[8 + fill_mom_off(i, jz) + t] = clm * fact[k] / (fact[i] * fact[jz]) * v / A;
+            }
+    c[8 + kFillMomCoef] = 0.0;
+    float4* out = mom + j * kFillMomF4;
+    for (int q = 0; q < kFillMomF4 - 1; ++q) {
+        const float a = (float)c[2 * q], b = (float)c[2 * q + 1];
+        out[q] = make_float4(a, a, b, b);
+    }
+    const float ah = (float)A;
+    out[kFillMomF4 - 1] = make_float4(ah, (float)(A - (double)ah), (float)s, (float)(s * s));
 }
 
 // Near pairs of row i by one warp: found and queued 32 at a time as in near_point_warp, evaluated 32 at a
@@ -279,10 +388,17 @@ __global__ void __launch_bounds__(128) k_fill_near(const Elem* __restrict__ el, 
 
 }  // namespace
 
-cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* nodes, const float4* tau,
-                              const float4* cjk, const double* diag, int64_t n, const ImageTable& img,
-                              const NearGrid& grid, const int32_t* cell_start, const int32_t* cell_items, double* K,
-                              cudaStream_t s) {
+size_t fill_moments_bytes(int64_t n) { return sizeof(float4) * kFillMomF4 * (size_t)n; }
+cudaError_t launch_fill_moments(const FillEl* fe, const float4* nodes, int64_t n, float4* mom, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    k_fill_moments<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(fe, nodes, n, mom);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* nodes, const float4* mom,
+                              const float4* tau, const float4* cjk, const double* diag, int64_t n,
+                              const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
+                              const int32_t* cell_items, double* K, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     // column tile: as many elements as fit in ~40 KB (four blocks per SM), at most 16
     int te = 16;
@@ -291,7 +407,7 @@ cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* no
     cudaError_t e = cudaFuncSetAttribute(k_fill_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 g1((unsigned)((n + kFT - 1) / kFT), (unsigned)((n + kFillCols - 1) / kFillCols));
-    k_fill_far<<<g1, kFT, smem, s>>>(fe, nodes, tau, cjk, diag, n, img.n, te, K);
+    k_fill_far<<<g1, kFT, smem, s>>>(fe, nodes, mom, tau, cjk, diag, n, img.n, te, K);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_fill_near<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(el, fe, cjk, n, img, grid, cell_start, cell_items, K);

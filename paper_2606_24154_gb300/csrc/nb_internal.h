@@ -216,10 +216,13 @@ cudaError_t launch_fill_f64(const Elem* el, const double* diag, int64_t n, const
 // Mixed fill: far pairs (tiers a-c) write K; near pairs (grid of image centroids with
 // the near radius kFillRatioC rho) add their FP64 closed forms afterwards.  tau[j][k] =
 // t_k . (ex_j, ey_j, ez_j) as (hi, lo) float4 pairs; nodes of kFillNodeRec float4 per element.
-cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* nodes, const float4* tau,
-                              const float4* cjk, const double* diag, int64_t n, const ImageTable& img,
-                              const NearGrid& grid, const int32_t* cell_start, const int32_t* cell_items, double* K,
-                              cudaStream_t s);
+// mom: fill_moments_bytes(n) bytes from launch_fill_moments.
+size_t fill_moments_bytes(int64_t n);
+cudaError_t launch_fill_moments(const FillEl* fe, const float4* nodes, int64_t n, float4* mom, cudaStream_t s);
+cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* nodes, const float4* mom,
+                              const float4* tau, const float4* cjk, const double* diag, int64_t n,
+                              const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
+                              const int32_t* cell_items, double* K, cudaStream_t s);
 cudaError_t launch_element_influence(const Elem* el, int64_t n_el, const double* pts, int64_t npts,
                                      double* phi, double* E, cudaStream_t s);
 

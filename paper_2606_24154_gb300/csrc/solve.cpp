@@ -52,6 +52,9 @@ int ensure_fill_tables(Ctx* c) {
     CK(launch_fill_tables(c->d_el.as<Elem>(), n, c->img, c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(),
                           c->d_fill_tau.as<float4>(), c->stream));
     CK(launch_elem_moments(c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(), n, c->d_fill_mom.as<float4>(), c->stream));
+    CK(c->d_fill_phimom.ensure(fill_moments_bytes(n)));
+    CK(launch_fill_moments(c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(), n, c->d_fill_phimom.as<float4>(),
+                           c->stream));
     rc = make_cell_list(c, c->d_el.as<Elem>(), n, c->img, c->fill_grid, c->d_fill_cell_start, c->d_fill_cell_items);
     if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));  // evaluations on other streams use the tables too
@@ -70,7 +73,7 @@ int ensure_fill(Ctx* c, int precision, double* ms) {
     CK(cudaEventRecord(c->ev0, c->stream));
     if (precision == NEBEM_MIXED)
         CK(launch_fill_mixed(c->d_el.as<Elem>(), c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(),
-                             c->d_fill_tau.as<float4>(), c->d_cjk.as<float4>(), c->d_diag.as<double>(), n, c->img,
+                             c->d_fill_phimom.as<float4>(), c->d_fill_tau.as<float4>(), c->d_cjk.as<float4>(), c->d_diag.as<double>(), n, c->img,
                              c->fill_grid, c->d_fill_cell_start.as<int32_t>(), c->d_fill_cell_items.as<int32_t>(),
                              c->d_K.as<double>(), c->stream));
     else

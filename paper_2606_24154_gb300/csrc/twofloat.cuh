@@ -256,4 +256,221 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float 
     }
 }
 
+// ---------------------------------------------------------------- far pairs of the fill by moments
+// Phi' or n . E' of a pair from kFillRatioB = 32 radii on, to the fill's accuracy, two images per packed
+// instruction.  With y = 1 / |D|, p = y^2, N = n . D and all moments over the area A:
+//   Phi' / A   = y (1 + W + F),  W = q p Q,  Q = a1 X^2 + a2 X Z + a3 Z^2 - w |D|^2 (degree 2),
+//   n . E' / A = y p (N (1 + 5 W + G) - q H - s (n_x F_alpha + n_z F_beta)),  H = n . grad Q,
+//   F(alpha, beta, q) = terms of degree 3 to 6,  alpha = X p s, beta = Z p s, q = p s^2,
+//   G = F + 2 (alpha F_alpha + beta F_beta + q F_q).
+// s = the power of two above the element's radius: the moments, of (node - centroid) / s, stay FP32 numbers
+// at any size of the geometry, and q is exact.
+// The monopole and the quadrupole (below 1.5e-4 of the pair) are in two-float arithmetic, F (below
+// 1.5e-6) in FP32; the terms left out (degree 7) are below 3e-13 at 32 radii.  In the field they count
+// eight times as much, so interface rows use the moments from kFillMomField = 52 radii on.  About 200 (Phi') and 360
+// (n . E') FP32 lane operations and one MUFU root per pair, where the 6, 9 and 16 nodes of the Gauss
+// rules took 480 to 1009 and 650 to 1500 and as many roots.
+// FillMom per element, every constant twice (both lanes), two per float4: a1, a2, a3, -w as hi, lo, then
+// the coefficients of F in the order of fill_mom_off, then A as hi, lo, s, s^2.
+constexpr double kFillMomField = 52.0;
+constexpr int kFillMomCoef = 43;
+constexpr int kFillMomF4 = (8 + kFillMomCoef + 1) / 2 + 1;
+// F's monomials alpha^i beta^j, i + j = k <= 6: coefficient q^m0 (C + C' q), m0 and the number of terms
+__host__ __device__ constexpr int fill_mom_m0(int k) { return k == 0 ? 2 : k <= 2 ? 1 : 0; }
+__host__ __device__ constexpr int fill_mom_terms(int k) { return k <= 4 ? 2 : 1; }
+__host__ __device__ constexpr int fill_mom_off(int i, int j) {
+    int o = 0;
+    for (int b = 0; b < 7; ++b)
+        for (int a = 0; a + b < 7; ++a) {
+            if (a == i && b == j) return o;
+            o += fill_mom_terms(a + b);
+        }
+    return o;
+}
+static_assert(fill_mom_off(0, 6) + 1 == kFillMomCoef, "coefficient count");
+
+// (vh, vl) = (ah, al) (vh, vl)
+__device__ __forceinline__ void df_times2(float2 ah, float2 al, float2& vh, float2& vl) {
+    const float2 t = __fmul2_rn(ah, vh);
+    const float2 e = __ffma2_rn(ah, vh, __fmul2_rn(t, bc2(-1.f)));
+    vl = __ffma2_rn(ah, vl, __ffma2_rn(al, vh, e));
+    vh = t;
+}
+
+// Two targets (lanes) of an element: X, Z and |D|^2 with the squares that it was summed from.
+struct FillPair2 {
+    float2 xh, xl, zh, zl, px, ex, pz, ez, d2h, d2l;
+};
+// A conductor row's sum; the interface row's takes the normal and H's constants in the element's frame.
+struct FillRow {
+    float nxh, nxl, nyh, nyl, nzh, nzl;  // n in the element's frame
+    float gxh, gxl, gzh, gzl;            // 2 a1 n_x + a2 n_z, a2 n_x + 2 a3 n_z
+};
+
+// 1 / |D| of the lanes that are far (0 of the others) as y0 + ye, its square p as a + al, q and W
+__device__ __forceinline__ void fill_mom_head2(const float4* __restrict__ mom, const FillPair2& P, bool far0, bool far1,
+                                               float2& y0, float2& ye, float2& a, float2& al, float2& q, float2& ql, float2& W,
+                                               float2& lo) {
+    const float2 m1 = bc2(-1.f);
+    auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
+    y0 = make_float2(far0 ? rsqrtf(P.d2h.x) : 0.f, far1 ? rsqrtf(P.d2h.y) : 0.f);
+    const float2 ny0 = __fmul2_rn(y0, m1);
+    a = __fmul2_rn(y0, y0);
+    const float2 na = __fmul2_rn(ny0, y0);
+    const float2 nae = __ffma2_rn(ny0, y0, a);  // a - y0^2
+    const float2 b = __fmul2_rn(P.d2h, a);
+    const float2 nbe = __ffma2_rn(P.d2h, na, b);
+    float2 h = __ffma2_rn(b, m1, bc2(1.f));
+    h = __fadd2_rn(h, nbe);
+    h = __ffma2_rn(P.d2h, nae, h);
+    h = __ffma2_rn(P.d2l, na, h);
+    ye = __fmul2_rn(__fmul2_rn(bc2(0.5f), y0), h);
+    al = __ffma2_rn(nae, m1, __fmul2_rn(__fadd2_rn(y0, y0), ye));
+    // Q: four products of two-float numbers, summed with their errors
+    const float2 pxz = __fmul2_rn(P.xh, P.zh);
+    float2 exz = __ffma2_rn(P.xh, P.zh, __fmul2_rn(pxz, m1));
+    exz = __ffma2_rn(P.xh, P.zl, __ffma2_rn(P.xl, P.zh, exz));
+    lo = bc2(0.f);
+    auto product = [&](int i, float2 vh, float2 vl) {
+        const float2 ch = con(2 * i), cl = con(2 * i + 1);
+        const float2 t = __fmul2_rn(ch, vh);
+        lo = __fadd2_rn(lo, __ffma2_rn(ch, vh, __fmul2_rn(t, m1)));
+        lo = __ffma2_rn(ch, vl, __ffma2_rn(cl, vh, lo));
+        return t;
+    };
+    const float2 t1 = product(0, P.px, P.ex), t2 = product(1, pxz, exz), t3 = product(2, P.pz, P.ez),
+                 t4 = product(3, P.d2h, P.d2l);
+    float2 e1, e2, e3;
+    two_sum2(t1, t3, W, e1);
+    two_sum2(W, t2, W, e2);
+    two_sum2(W, t4, W, e3);
+    lo = __fadd2_rn(lo, __fadd2_rn(e1, __fadd2_rn(e2, e3)));
+    const float2 ss = bc2(mom[kFillMomF4 - 1].w);
+    q = __fmul2_rn(a, ss), ql = __fmul2_rn(al, ss);
+    df_times2(a, al, W, lo);
+    df_times2(q, ql, W, lo);
+}
+
+// (Sh, Sl) += y (1 + W + F) of the lanes that are far
+__device__ __forceinline__ void fill_mom_phi2(const float4* __restrict__ mom, const FillPair2& P, bool far0,
+                                              bool far1, float2& Sh, float2& Sl) {
+    auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
+    float2 y0, ye, a, al, q, ql, W, lo;
+    fill_mom_head2(mom, P, far0, far1, y0, ye, a, al, q, ql, W, lo);
+    df_times2(y0, ye, W, lo);
+    const float2 pr = __fmul2_rn(a, bc2(mom[kFillMomF4 - 1].z)), qq = __fmul2_rn(q, q);
+    const float2 al1 = __fmul2_rn(P.xh, pr), be1 = __fmul2_rn(P.zh, pr);
+    float2 F = bc2(0.f);
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        float2 R = bc2(0.f);
+#pragma unroll
+        for (int i = 6 - j; i >= 0; --i) {
+            const int o = 8 + fill_mom_off(i, j), k = i + j;
+            float2 c = con(o);
+            if (fill_mom_terms(k) == 2) c = __ffma2_rn(con(o + 1), q, c);
+            if (fill_mom_m0(k) == 1) c = __fmul2_rn(c, q);
+            if (fill_mom_m0(k) == 2) c = __fmul2_rn(c, qq);
+            R = i == 6 - j ? c : __ffma2_rn(R, al1, c);
+        }
+        F = j == 6 ? R : __ffma2_rn(F, be1, R);
+    }
+    float2 u1, u2;
+    two_sum2(Sh, y0, Sh, u1);
+    two_sum2(Sh, W, Sh, u2);
+    lo = __fadd2_rn(lo, __fadd2_rn(ye, __fadd2_rn(u1, u2)));
+    Sl = __fadd2_rn(Sl, __ffma2_rn(y0, F, lo));
+}
+
+// (Sh, Sl) += n . E' / A of the lanes that are far; (yh, yl) = the targets' Y
+__device__ __forceinline__ void fill_mom_field2(const float4* __restrict__ mom, const FillRow& R,
+                                                const FillPair2& P, float2 yh, float2 yl, bool far0, bool far1,
+                                                float2& Sh, float2& Sl) {
+    const float2 m1 = bc2(-1.f);
+    auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
+    auto product = [&](float ch, float cl, float2 vh, float2 vl, float2& e) {  // its hi; e += its lo
+        const float2 t = __fmul2_rn(bc2(ch), vh);
+        e = __fadd2_rn(e, __ffma2_rn(bc2(ch), vh, __fmul2_rn(t, m1)));
+        e = __ffma2_rn(bc2(ch), vl, __ffma2_rn(bc2(cl), vh, e));
+        return t;
+    };
+    float2 y0, ye, a, al, q, ql, W, wl;
+    fill_mom_head2(mom, P, far0, far1, y0, ye, a, al, q, ql, W, wl);
+    float2 Nh, Nl = bc2(0.f), e1, e2;
+    const float2 n1 = product(R.nxh, R.nxl, P.xh, P.xl, Nl), n2 = product(R.nyh, R.nyl, yh, yl, Nl),
+                 n3 = product(R.nzh, R.nzl, P.zh, P.zl, Nl);
+    two_sum2(n1, n2, Nh, e1);
+    two_sum2(Nh, n3, Nh, e2);
+    Nl = __fadd2_rn(Nl, __fadd2_rn(e1, e2));
+    // q H, H = gx X + gz Z - 2 w N
+    float2 Hh, Hl = bc2(0.f);
+    const float2 h1 = product(R.gxh, R.gxl, P.xh, P.xl, Hl), h2 = product(R.gzh, R.gzl, P.zh, P.zl, Hl);
+    float2 h3 = __fadd2_rn(con(6), con(6)), h3l = __fadd2_rn(con(7), con(7));  // -2 w
+    {
+        float2 vh = Nh, vl = Nl;
+        df_times2(h3, h3l, vh, vl);
+        h3 = vh;
+        Hl = __fadd2_rn(Hl, vl);
+    }
+    two_sum2(h1, h2, Hh, e1);
+    two_sum2(Hh, h3, Hh, e2);
+    Hl = __fadd2_rn(Hl, __fadd2_rn(e1, e2));
+    df_times2(q, ql, Hh, Hl);
+    // 5 W N
+    df_times2(bc2(5.f), bc2(0.f), W, wl);
+    df_times2(Nh, Nl, W, wl);
+    // G, F_alpha, F_beta
+    const float s = mom[kFillMomF4 - 1].z;
+    const float2 pr = __fmul2_rn(a, bc2(s)), qq = __fmul2_rn(q, q);
+    const float2 al1 = __fmul2_rn(P.xh, pr), be1 = __fmul2_rn(P.zh, pr);
+    float2 F = bc2(0.f), G = bc2(0.f), Fa = bc2(0.f), Fb = bc2(0.f);
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        float2 r = bc2(0.f), ra = bc2(0.f), rg = bc2(0.f);
+#pragma unroll
+        for (int i = 6 - j; i >= 0; --i) {
+            const int o = 8 + fill_mom_off(i, j), k = i + j;
+            const float f0 = (float)(1 + 2 * (k + fill_mom_m0(k)));
+            float2 c = con(o), g;
+            if (fill_mom_terms(k) == 2) {
+                const float2 c1 = __fmul2_rn(con(o + 1), q);
+                c = __fadd2_rn(c, c1);
+                g = __ffma2_rn(c1, bc2(2.f), __fmul2_rn(c, bc2(f0)));
+            } else {
+                g = __fmul2_rn(c, bc2(f0));
+            }
+            if (fill_mom_m0(k) == 1) c = __fmul2_rn(c, q), g = __fmul2_rn(g, q);
+            if (fill_mom_m0(k) == 2) c = __fmul2_rn(c, qq), g = __fmul2_rn(g, qq);
+            if (i == 6 - j) {
+                r = c, rg = g;
+            } else {
+                ra = i == 5 - j ? r : __ffma2_rn(ra, al1, r);
+                r = __ffma2_rn(r, al1, c);
+                rg = __ffma2_rn(rg, al1, g);
+            }
+        }
+        if (j == 6) {
+            F = r, G = rg;
+        } else {
+            Fb = j == 5 ? F : __ffma2_rn(Fb, be1, F);
+            F = __ffma2_rn(F, be1, r);
+            G = __ffma2_rn(G, be1, rg);
+            Fa = j == 5 ? ra : __ffma2_rn(Fa, be1, ra);
+        }
+    }
+    // T = N + 5 W N - q H + FP32 part, then y p T
+    float2 Th, Tl;
+    two_sum2(Nh, W, Th, e1);
+    two_sum2(Th, __fmul2_rn(Hh, m1), Th, e2);
+    Tl = __fadd2_rn(__fadd2_rn(Nl, wl), __fadd2_rn(e1, e2));
+    Tl = __ffma2_rn(Hl, m1, Tl);
+    const float2 D = __ffma2_rn(bc2(R.nxh), Fa, __fmul2_rn(bc2(R.nzh), Fb));
+    Tl = __fadd2_rn(Tl, __ffma2_rn(Nh, G, __fmul2_rn(D, bc2(-s))));
+    df_times2(a, al, Th, Tl);
+    df_times2(y0, ye, Th, Tl);
+    float2 u;
+    two_sum2(Sh, Th, Sh, u);
+    Sl = __fadd2_rn(Sl, __fadd2_rn(u, Tl));
+}
+
 }  // namespace nb
