@@ -42,6 +42,13 @@
 
 namespace nb {
 
+// 1 / sqrt(x) of a normal FP32 number: rsqrtf without its scaling of subnormal arguments (the same bits).
+__device__ __forceinline__ float rsqrt_normal(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // sqrt(a) for a normal a > 0: one third-order Householder step, a (y (1 + e/2 + 3 e^2/8)) with
 // e = 1 - a y^2, on the hardware's estimate y of 1 / sqrt(a) (about 20 bits, so the step
 // leaves the rounding of the last operations).  NaN for a = 0.

@@ -16,7 +16,11 @@
 // FP32 with rsqrt.  Runs of 32 sources are summed in FP32 and added to two-float
 // (hi + lo) running totals with an error-free two-sum; each thread takes two targets in
 // the lanes of the packed FP32x2 instructions.
-#include "nb_internal.h"
+#include <cooperative_groups.h>
+
+#include <cfloat>
+
+#include "influence.cuh"
 
 namespace nb {
 
@@ -93,16 +97,28 @@ __global__ void k_split2f(const double* __restrict__ pos, const double* __restri
     lo[i] = make_float4((float)(x - hx), (float)(y - hy), (float)(z - hz), 0.f);
 }
 
-// Mixed sum: each thread takes two targets, t and t + kSC2Threads of its block, held in
-// the two lanes of the packed FP32x2 instructions; a source tile is staged in shared
-// memory with every value negated and duplicated into both lanes, so that a pair
-// (target, source) costs the same rounded operations as the scalar form
+// Mixed sum: each thread takes P pairs of targets, a pair in the two lanes of the packed FP32x2
+// instructions; a source tile is staged in shared memory with every value negated and
+// duplicated into both lanes, so that a pair (target, source) costs the same rounded
+// operations as the scalar form
 //   d = (t_hi - s_hi) + (t_lo - s_lo),  r^2 = d.d + s^2,  q / r,  q d / r^3
-// at half the issue slots.  Partial sums over kFlush sources are added to running totals
-// kept as two floats (hi + lo, error-free two-sum), so no FP64 instruction runs per
-// source; the totals are converted to FP64 once per target.
-constexpr int kSC2Threads = 128;
-constexpr int kSC2Tile = 2 * kSC2Threads;  // targets per block = sources per tile
+// at half the issue slots (19 lane operations and one MUFU root).  Partial sums over kFlush sources
+// are added to running totals kept as two floats (hi + lo, error-free two-sum), so no FP64
+// instruction runs per source; the totals are converted to FP64 once per target.
+//
+// With SPLIT > 1 a cluster of SPLIT blocks shares a tile of targets: each sums a run of the sources, and
+// the runs' totals are added in FP64 in the order of the runs through distributed shared memory,
+// so the sums need neither scratch nor atomics.  The runs depend on the number of
+// sources alone, and P does not enter the arithmetic: a target's bits do not depend on the others.
+// Bound by the FP32 pipe with P = 2 (P = 1: by the four broadcast loads per source, 14 cycles of the
+// shared-memory port against 9.5 of the FP32 pipe), given enough warps: 20,000 x 20,000 took 1.26 ms with
+// one block per tile and P = 1, 0.40 ms in clusters of 8; 100,000 x 100,000 9.8 and 6.6 ms (4.8 ms
+// at the FP32 pipe's rate); 100,000 sources at one target 6.3 and 0.46 ms.
+constexpr int kSCT = 128;     // threads of a block
+constexpr int kSCSrc = 256;   // sources of a staged tile
+constexpr int kSCUnit = 128;  // the runs are whole units
+constexpr int kSCSplit = 8;
+constexpr int64_t kSCSplitFrom = 1024;
 
 struct F2Acc {  // two-float running total per lane: value = hi + lo
     float2 hi, lo;
@@ -121,32 +137,40 @@ __device__ __forceinline__ void acc_add(F2Acc& a, float2 x) {
     two_sum_add(a.hi.y, a.lo.y, x.y);
 }
 
-template <bool SELF>
-__device__ __forceinline__ void sc_tile_f32x2(const float4* __restrict__ A, const float4* __restrict__ B,
-                                              const float4* __restrict__ C, const float2* __restrict__ D, int k0,
-                                              int k1, float2 thx, float2 thy, float2 thz, float2 tlx, float2 tly,
-                                              float2 tlz, float2 s2, int self0, int self1, float2& ph, float2& ex,
-                                              float2& ey, float2& ez) {
-#pragma unroll 4
+// NORMAL: r^2 >= s^2 >= FLT_MIN, so the root needs no scaling of subnormal arguments (about eight
+// issue slots of 46 per pair of lanes; the same bits).
+template <bool SELF, bool NORMAL, int P>
+__device__ __forceinline__ void sc_run(const float4* __restrict__ A, const float4* __restrict__ B,
+                                       const float4* __restrict__ C, const float2* __restrict__ D, int k0, int k1,
+                                       const float2 (&th)[P][3], const float2 (&tl)[P][3], float2 s2,
+                                       const int (&self)[2 * P], float2 (&ph)[P], float2 (&ex)[P], float2 (&ey)[P],
+                                       float2 (&ez)[P]) {
+#pragma unroll(4 / P)
     for (int k = k0; k < k1; ++k) {
         const float4 a = A[k], b = B[k], c = C[k];
         const float2 d = D[k];
-        const float2 dx = __fadd2_rn(__fadd2_rn(thx, make_float2(a.x, a.y)), __fadd2_rn(tlx, make_float2(c.x, c.y)));
-        const float2 dy = __fadd2_rn(__fadd2_rn(thy, make_float2(a.z, a.w)), __fadd2_rn(tly, make_float2(c.z, c.w)));
-        const float2 dz = __fadd2_rn(__fadd2_rn(thz, make_float2(b.x, b.y)), __fadd2_rn(tlz, d));
-        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, s2)));
-        const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-        float2 qq = make_float2(b.z, b.w);
-        if (SELF) {
-            if (k == self0) qq.x = 0.f;
-            if (k == self1) qq.y = 0.f;
+#pragma unroll
+        for (int h = 0; h < P; ++h) {
+            const float2 dx =
+                __fadd2_rn(__fadd2_rn(th[h][0], make_float2(a.x, a.y)), __fadd2_rn(tl[h][0], make_float2(c.x, c.y)));
+            const float2 dy =
+                __fadd2_rn(__fadd2_rn(th[h][1], make_float2(a.z, a.w)), __fadd2_rn(tl[h][1], make_float2(c.z, c.w)));
+            const float2 dz = __fadd2_rn(__fadd2_rn(th[h][2], make_float2(b.x, b.y)), __fadd2_rn(tl[h][2], d));
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, s2)));
+            const float2 ri = NORMAL ? make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y))
+                                     : make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            float2 qq = make_float2(b.z, b.w);
+            if (SELF) {
+                if (k == self[2 * h]) qq.x = 0.f;
+                if (k == self[2 * h + 1]) qq.y = 0.f;
+            }
+            const float2 qr = __fmul2_rn(qq, ri);
+            const float2 qr3 = __fmul2_rn(qr, __fmul2_rn(ri, ri));
+            ph[h] = __fadd2_rn(ph[h], qr);
+            ex[h] = __ffma2_rn(qr3, dx, ex[h]);
+            ey[h] = __ffma2_rn(qr3, dy, ey[h]);
+            ez[h] = __ffma2_rn(qr3, dz, ez[h]);
         }
-        const float2 qr = __fmul2_rn(qq, ri);
-        const float2 qr3 = __fmul2_rn(qr, __fmul2_rn(ri, ri));
-        ph = __fadd2_rn(ph, qr);
-        ex = __ffma2_rn(qr3, dx, ex);
-        ey = __ffma2_rn(qr3, dy, ey);
-        ez = __ffma2_rn(qr3, dz, ez);
     }
 }
 
@@ -185,164 +209,80 @@ __device__ __forceinline__ void store_target(int64_t t, int accumulate, double k
     }
 }
 
-// Targets given as FP64 (split in-kernel); sources as two-float (hi, lo) arrays.
-__global__ void __launch_bounds__(kSC2Threads) k_sc_mixed(const float4* __restrict__ shq,
-                                                          const float4* __restrict__ slo, int64_t nsrc,
-                                                          const double* __restrict__ tgt, int64_t ntgt,
-                                                          int exclude_self, float s2, double ke, int accumulate,
-                                                          double* __restrict__ phi, double* __restrict__ E) {
-    __shared__ float4 sA[kSC2Tile], sB[kSC2Tile], sC[kSC2Tile];
-    __shared__ float2 sD[kSC2Tile];
-    const int64_t t0 = (int64_t)blockIdx.x * kSC2Tile + threadIdx.x;
-    const int64_t t1 = t0 + kSC2Threads;
-    float h0x, h0y, h0z, l0x, l0y, l0z, h1x, h1y, h1z, l1x, l1y, l1z;
-    load_target_2f(tgt, t0, t0 < ntgt, h0x, h0y, h0z, l0x, l0y, l0z);
-    load_target_2f(tgt, t1, t1 < ntgt, h1x, h1y, h1z, l1x, l1y, l1z);
-    const float2 thx = make_float2(h0x, h1x), thy = make_float2(h0y, h1y), thz = make_float2(h0z, h1z);
-    const float2 tlx = make_float2(l0x, l1x), tly = make_float2(l0y, l1y), tlz = make_float2(l0z, l1z);
-    const float2 s22 = make_float2(s2, s2);
-    const float2 zero = make_float2(0.f, 0.f);
-    F2Acc aph{zero, zero}, aex{zero, zero}, aey{zero, zero}, aez{zero, zero};
-    for (int64_t base = 0; base < nsrc; base += kSC2Tile) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kSC2Tile; i += kSC2Threads) {
-            const int64_t c = base + i;
-            if (c < nsrc) {
-                const float4 h = shq[c], l = slo[c];
-                sA[i] = make_float4(-h.x, -h.x, -h.y, -h.y);
-                sB[i] = make_float4(-h.z, -h.z, h.w, h.w);
-                sC[i] = make_float4(-l.x, -l.x, -l.y, -l.y);
-                sD[i] = make_float2(-l.z, -l.z);
-            }
-        }
-        __syncthreads();
-        const int cnt = (int)min((int64_t)kSC2Tile, nsrc - base);
-        // the tile that holds this block's own carriers (targets are the sources in order)
-        const bool self_tile = exclude_self && (base == (int64_t)blockIdx.x * kSC2Tile);
-        const int self0 = self_tile ? (int)threadIdx.x : -1;
-        const int self1 = self_tile ? (int)threadIdx.x + kSC2Threads : -1;
-        // FP32 partial sums over kFlush sources: the +/- charges cancel, so longer FP32
-        // runs would lose the result in the partial sums' rounding
-        for (int sub = 0; sub < cnt; sub += kFlush) {
-            const int m = min(kFlush, cnt - sub);
-            float2 fph = zero, fex = zero, fey = zero, fez = zero;
-            if (self_tile && ((self0 >= sub && self0 < sub + m) || (self1 >= sub && self1 < sub + m)))
-                sc_tile_f32x2<true>(sA, sB, sC, sD, sub, sub + m, thx, thy, thz, tlx, tly, tlz, s22, self0, self1, fph,
-                                    fex, fey, fez);
-            else
-                sc_tile_f32x2<false>(sA, sB, sC, sD, sub, sub + m, thx, thy, thz, tlx, tly, tlz, s22, -1, -1, fph,
-                                     fex, fey, fez);
-            acc_add(aph, fph);
-            acc_add(aex, fex);
-            acc_add(aey, fey);
-            acc_add(aez, fez);
-        }
-    }
-    if (t0 < ntgt)
-        store_target(t0, accumulate, ke, (double)aph.hi.x + (double)aph.lo.x, (double)aex.hi.x + (double)aex.lo.x,
-                     (double)aey.hi.x + (double)aey.lo.x, (double)aez.hi.x + (double)aez.lo.x, phi, E);
-    if (t1 < ntgt)
-        store_target(t1, accumulate, ke, (double)aph.hi.y + (double)aph.lo.y, (double)aex.hi.y + (double)aex.lo.y,
-                     (double)aey.hi.y + (double)aey.lo.y, (double)aez.hi.y + (double)aez.lo.y, phi, E);
-}
-
-// Four targets per thread for large target sets: two pairs of FP32x2 lanes, (t, t + 128)
-// and (t + 256, t + 384) of a 512-target block, share every source load from shared memory,
-// and the two independent chains give the scheduler more to overlap.  Per target the
-// operations, their order, the 32-source flush groups (tiles of 512 sources hold sixteen of
-// them, aligned as in the 256-source tiles) and the running totals are those of
-// k_sc_mixed, so the two kernels give the same bits.
-constexpr int kSC4Threads = 128;
-constexpr int kSC4Tile = 4 * kSC4Threads;
-
-template <bool SELF>
-__device__ __forceinline__ void sc_tile_f32x2x2(const float4* __restrict__ A, const float4* __restrict__ B,
-                                                const float4* __restrict__ C, const float2* __restrict__ D, int k0,
-                                                int k1, const float2 (&th)[2][3], const float2 (&tl)[2][3], float2 s2,
-                                                const int (&self)[4], float2 (&ph)[2], float2 (&ex)[2],
-                                                float2 (&ey)[2], float2 (&ez)[2]) {
-#pragma unroll 2
-    for (int k = k0; k < k1; ++k) {
-        const float4 a = A[k], b = B[k], c = C[k];
-        const float2 d = D[k];
+// Targets given as FP64 (split in-kernel); sources as two-float (hi, lo) arrays.  Grid: SPLIT blocks
+// per tile of 2 P kSCT targets, which are clusters for SPLIT > 1.
+template <int P, int SPLIT>
+__device__ __forceinline__ void sc_mixed(const float4* __restrict__ shq, const float4* __restrict__ slo, int64_t nsrc,
+                                         const double* __restrict__ tgt, int64_t ntgt, int exclude_self, float s2,
+                                         double ke, int accumulate, double* __restrict__ phi, double* __restrict__ E) {
+    constexpr int kTile = 2 * P * kSCT;
+    struct Stage {
+        float4 A[kSCSrc], B[kSCSrc], C[kSCSrc];
+        float2 D[kSCSrc];
+    };
+    __shared__ union {
+        Stage st;
+        double part[SPLIT > 1 ? 4 * kTile : 1];
+    } sm;
+    const int run = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
+    const int64_t first = (int64_t)(blockIdx.x / SPLIT) * kTile;
+    float2 th[P][3], tl[P][3];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 dx =
-                __fadd2_rn(__fadd2_rn(th[h][0], make_float2(a.x, a.y)), __fadd2_rn(tl[h][0], make_float2(c.x, c.y)));
-            const float2 dy =
-                __fadd2_rn(__fadd2_rn(th[h][1], make_float2(a.z, a.w)), __fadd2_rn(tl[h][1], make_float2(c.z, c.w)));
-            const float2 dz = __fadd2_rn(__fadd2_rn(th[h][2], make_float2(b.x, b.y)), __fadd2_rn(tl[h][2], d));
-            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, s2)));
-            const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-            float2 qq = make_float2(b.z, b.w);
-            if (SELF) {
-                if (k == self[2 * h]) qq.x = 0.f;
-                if (k == self[2 * h + 1]) qq.y = 0.f;
-            }
-            const float2 qr = __fmul2_rn(qq, ri);
-            const float2 qr3 = __fmul2_rn(qr, __fmul2_rn(ri, ri));
-            ph[h] = __fadd2_rn(ph[h], qr);
-            ex[h] = __ffma2_rn(qr3, dx, ex[h]);
-            ey[h] = __ffma2_rn(qr3, dy, ey[h]);
-            ez[h] = __ffma2_rn(qr3, dz, ez[h]);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kSC4Threads) k_sc_mixed4(const float4* __restrict__ shq,
-                                                           const float4* __restrict__ slo, int64_t nsrc,
-                                                           const double* __restrict__ tgt, int64_t ntgt,
-                                                           int exclude_self, float s2, double ke, int accumulate,
-                                                           double* __restrict__ phi, double* __restrict__ E) {
-    __shared__ float4 sA[kSC4Tile], sB[kSC4Tile], sC[kSC4Tile];
-    __shared__ float2 sD[kSC4Tile];
-    int64_t tq[4];
-    float2 th[2][3], tl[2][3];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < P; ++h) {
         float hx[2], hy[2], hz[2], lx[2], ly[2], lz[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            tq[2 * h + q] = (int64_t)blockIdx.x * kSC4Tile + threadIdx.x + (2 * h + q) * kSC4Threads;
-            load_target_2f(tgt, tq[2 * h + q], tq[2 * h + q] < ntgt, hx[q], hy[q], hz[q], lx[q], ly[q], lz[q]);
+            const int64_t t = first + threadIdx.x + (2 * h + q) * kSCT;
+            load_target_2f(tgt, t, t < ntgt, hx[q], hy[q], hz[q], lx[q], ly[q], lz[q]);
         }
         th[h][0] = make_float2(hx[0], hx[1]), th[h][1] = make_float2(hy[0], hy[1]), th[h][2] = make_float2(hz[0], hz[1]);
         tl[h][0] = make_float2(lx[0], lx[1]), tl[h][1] = make_float2(ly[0], ly[1]), tl[h][2] = make_float2(lz[0], lz[1]);
     }
     const float2 s22 = make_float2(s2, s2);
+    const bool normal = s2 >= FLT_MIN;
     const float2 zero = make_float2(0.f, 0.f);
-    F2Acc aph[2] = {{zero, zero}, {zero, zero}}, aex[2] = {{zero, zero}, {zero, zero}},
-          aey[2] = {{zero, zero}, {zero, zero}}, aez[2] = {{zero, zero}, {zero, zero}};
-    for (int64_t base = 0; base < nsrc; base += kSC4Tile) {
+    F2Acc aph[P], aex[P], aey[P], aez[P];
+#pragma unroll
+    for (int h = 0; h < P; ++h) aph[h] = aex[h] = aey[h] = aez[h] = F2Acc{zero, zero};
+    const int64_t units = (nsrc + kSCUnit - 1) / kSCUnit;
+    const int64_t c0 = SPLIT > 1 ? units * run / SPLIT * kSCUnit : 0;
+    const int64_t c1 = SPLIT > 1 ? min(nsrc, units * (run + 1) / SPLIT * kSCUnit) : nsrc;
+    for (int64_t base = c0; base < c1; base += kSCSrc) {
+        const int cnt = (int)min((int64_t)kSCSrc, c1 - base);
         __syncthreads();
-        for (int i = threadIdx.x; i < kSC4Tile; i += kSC4Threads) {
-            const int64_t c = base + i;
-            if (c < nsrc) {
-                const float4 h = shq[c], l = slo[c];
-                sA[i] = make_float4(-h.x, -h.x, -h.y, -h.y);
-                sB[i] = make_float4(-h.z, -h.z, h.w, h.w);
-                sC[i] = make_float4(-l.x, -l.x, -l.y, -l.y);
-                sD[i] = make_float2(-l.z, -l.z);
-            }
+        for (int i = threadIdx.x; i < cnt; i += kSCT) {
+            const float4 h = shq[base + i], l = slo[base + i];
+            sm.st.A[i] = make_float4(-h.x, -h.x, -h.y, -h.y);
+            sm.st.B[i] = make_float4(-h.z, -h.z, h.w, h.w);
+            sm.st.C[i] = make_float4(-l.x, -l.x, -l.y, -l.y);
+            sm.st.D[i] = make_float2(-l.z, -l.z);
         }
         __syncthreads();
-        const int cnt = (int)min((int64_t)kSC4Tile, nsrc - base);
-        const bool self_tile = exclude_self && (base == (int64_t)blockIdx.x * kSC4Tile);
-        int self[4];
+        // the block's own carriers (targets are the sources in order): source `self` of this tile
+        const bool own = exclude_self && base < first + kTile && first < base + cnt;
+        int self[2 * P];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) self[q] = self_tile ? (int)threadIdx.x + q * kSC4Threads : -1;
+        for (int q = 0; q < 2 * P; ++q) self[q] = own ? (int)(first - base) + (int)threadIdx.x + q * kSCT : -1;
+        // FP32 partial sums over kFlush sources: the +/- charges cancel, so longer FP32
+        // runs would lose the result in the partial sums' rounding
         for (int sub = 0; sub < cnt; sub += kFlush) {
             const int m = min(kFlush, cnt - sub);
-            float2 fph[2] = {zero, zero}, fex[2] = {zero, zero}, fey[2] = {zero, zero}, fez[2] = {zero, zero};
+            float2 fph[P], fex[P], fey[P], fez[P];
+#pragma unroll
+            for (int h = 0; h < P; ++h) fph[h] = fex[h] = fey[h] = fez[h] = zero;
             bool hit = false;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) hit |= self[q] >= sub && self[q] < sub + m;
+            for (int q = 0; q < 2 * P; ++q) hit |= self[q] >= sub && self[q] < sub + m;
             if (hit)
-                sc_tile_f32x2x2<true>(sA, sB, sC, sD, sub, sub + m, th, tl, s22, self, fph, fex, fey, fez);
+                sc_run<true, false, P>(sm.st.A, sm.st.B, sm.st.C, sm.st.D, sub, sub + m, th, tl, s22, self, fph, fex, fey, fez);
+            else if (normal)
+                sc_run<false, true, P>(sm.st.A, sm.st.B, sm.st.C, sm.st.D, sub, sub + m, th, tl, s22, self, fph, fex,
+                                       fey, fez);
             else
-                sc_tile_f32x2x2<false>(sA, sB, sC, sD, sub, sub + m, th, tl, s22, self, fph, fex, fey, fez);
+                sc_run<false, false, P>(sm.st.A, sm.st.B, sm.st.C, sm.st.D, sub, sub + m, th, tl, s22, self, fph, fex,
+                                        fey, fez);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < P; ++h) {
                 acc_add(aph[h], fph[h]);
                 acc_add(aex[h], fex[h]);
                 acc_add(aey[h], fey[h]);
@@ -350,17 +290,54 @@ __global__ void __launch_bounds__(kSC4Threads) k_sc_mixed4(const float4* __restr
             }
         }
     }
+    auto total = [](const F2Acc& a, int q) {
+        return q ? (double)a.hi.y + (double)a.lo.y : (double)a.hi.x + (double)a.lo.x;
+    };
+    if constexpr (SPLIT == 1) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (tq[2 * h] < ntgt)
-            store_target(tq[2 * h], accumulate, ke, (double)aph[h].hi.x + (double)aph[h].lo.x,
-                         (double)aex[h].hi.x + (double)aex[h].lo.x, (double)aey[h].hi.x + (double)aey[h].lo.x,
-                         (double)aez[h].hi.x + (double)aez[h].lo.x, phi, E);
-        if (tq[2 * h + 1] < ntgt)
-            store_target(tq[2 * h + 1], accumulate, ke, (double)aph[h].hi.y + (double)aph[h].lo.y,
-                         (double)aex[h].hi.y + (double)aex[h].lo.y, (double)aey[h].hi.y + (double)aey[h].lo.y,
-                         (double)aez[h].hi.y + (double)aez[h].lo.y, phi, E);
+        for (int q = 0; q < 2 * P; ++q) {
+            const int64_t t = first + threadIdx.x + q * kSCT;
+            if (t < ntgt)
+                store_target(t, accumulate, ke, total(aph[q / 2], q & 1), total(aex[q / 2], q & 1),
+                             total(aey[q / 2], q & 1), total(aez[q / 2], q & 1), phi, E);
+        }
+    } else {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2 * P; ++q) {
+            double* o = sm.part + 4 * (threadIdx.x + q * kSCT);
+            o[0] = total(aph[q / 2], q & 1), o[1] = total(aex[q / 2], q & 1);
+            o[2] = total(aey[q / 2], q & 1), o[3] = total(aez[q / 2], q & 1);
+        }
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        cl.sync();
+        // the tile's targets dealt to the blocks
+        for (int i = run * (kTile / SPLIT) + threadIdx.x; i < (run + 1) * (kTile / SPLIT); i += kSCT) {
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int r = 0; r < SPLIT; ++r) {
+                const double2* o = reinterpret_cast<const double2*>(cl.map_shared_rank(sm.part, r)) + 2 * i;
+                const double2 a = o[0], b = o[1];
+                v[0] += a.x, v[1] += a.y, v[2] += b.x, v[3] += b.y;
+            }
+            if (first + i < ntgt) store_target(first + i, accumulate, ke, v[0], v[1], v[2], v[3], phi, E);
+        }
+        cl.sync();  // the other blocks read this block's shared memory
     }
+}
+
+template <int P>
+__global__ void __launch_bounds__(kSCT, 4) k_sc_mixed(const float4* __restrict__ shq, const float4* __restrict__ slo,
+                                                      int64_t nsrc, const double* __restrict__ tgt, int64_t ntgt,
+                                                      int exclude_self, float s2, double ke, int accumulate,
+                                                      double* __restrict__ phi, double* __restrict__ E) {
+    sc_mixed<P, 1>(shq, slo, nsrc, tgt, ntgt, exclude_self, s2, ke, accumulate, phi, E);
+}
+template <int P>
+__global__ void __cluster_dims__(kSCSplit, 1, 1) __launch_bounds__(kSCT, 4)
+    k_sc_mixed_split(const float4* __restrict__ shq, const float4* __restrict__ slo, int64_t nsrc,
+                     const double* __restrict__ tgt, int64_t ntgt, int exclude_self, float s2, double ke,
+                     int accumulate, double* __restrict__ phi, double* __restrict__ E) {
+    sc_mixed<P, kSCSplit>(shq, slo, nsrc, tgt, ntgt, exclude_self, s2, ke, accumulate, phi, E);
 }
 
 // b_i -= phi_sc(c_i) on conductor rows, b_i -= n_i . E_sc(c_i) on interface rows.
@@ -412,12 +389,19 @@ cudaError_t launch_sc_eval(int precision, const double* src, const double* q, co
     if (precision == NEBEM_FP64)
         k_sc_f64<<<blocks, kSCThreads, 0, s>>>(src, q, nsrc, tgt, ntgt, exclude_self, soft * soft, ke, accumulate, phi,
                                                E);
-    else if (ntgt >= (int64_t)152 * 4 * kSC4Tile)  // enough 512-target blocks for several waves
-        k_sc_mixed4<<<(unsigned)((ntgt + kSC4Tile - 1) / kSC4Tile), kSC4Threads, 0, s>>>(
-            hq, lo, nsrc, tgt, ntgt, exclude_self, (float)(soft * soft), ke, accumulate, phi, E);
-    else
-        k_sc_mixed<<<(unsigned)((ntgt + kSC2Tile - 1) / kSC2Tile), kSC2Threads, 0, s>>>(
-            hq, lo, nsrc, tgt, ntgt, exclude_self, (float)(soft * soft), ke, accumulate, phi, E);
+    else {
+        // Sources shared among the blocks of a cluster from kSCSplitFrom on: with 1,100 sources a call takes 13
+        // us against 43 (1,100 targets), 39 against 44 (20,000) and 205 against 178 (200,000, where the blocks'
+        // targets and totals cost more than the idle SMs; 275 against 315 with 2,000 sources).  Two pairs
+        // of targets per thread where that leaves a block for every SM.
+        const bool split = nsrc >= kSCSplitFrom;
+        const int ns = split ? kSCSplit : 1;
+        const bool wide = ntgt * ns >= (int64_t)152 * 2 * kSCT;
+        const int64_t tile = (wide ? 4 : 2) * kSCT;
+        const unsigned grid = (unsigned)((ntgt + tile - 1) / tile * ns);
+        auto* k = split ? (wide ? k_sc_mixed_split<2> : k_sc_mixed_split<1>) : (wide ? k_sc_mixed<2> : k_sc_mixed<1>);
+        k<<<grid, kSCT, 0, s>>>(hq, lo, nsrc, tgt, ntgt, exclude_self, (float)(soft * soft), ke, accumulate, phi, E);
+    }
     return cudaGetLastError();
 }
 
