@@ -112,7 +112,8 @@ __device__ __forceinline__ void node_rinv2(const PairDF2& P, const float4& q0, c
     const float2 r2h = __fadd2_rn(P.d2h, qh);
     const float2 t3 = sub2(qh, sub2(r2h, P.d2h));
     const float2 r2l = __fadd2_rn(P.d2l, __fadd2_rn(lo, t3));
-    y0 = make_float2(rsqrtf(r2h.x), rsqrtf(r2h.y));
+    // (distances beyond 1e-19 m: normal numbers)
+    y0 = make_float2(rsqrt_normal(r2h.x), rsqrt_normal(r2h.y));
     ny0 = __fmul2_rn(y0, m1);
     a = __fmul2_rn(y0, y0);
     nae = __ffma2_rn(ny0, y0, a);  // a - y0^2
@@ -168,7 +169,7 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float 
                                           float2 zh, float2 zl, float2 d2h, float2 d2l, bool far0, bool far1,
                                           MomSum2& S) {
     const float2 m1 = bc2(-1.f);
-    const float2 y0 = make_float2(far0 ? rsqrtf(d2h.x) : 0.f, far1 ? rsqrtf(d2h.y) : 0.f);
+    const float2 y0 = make_float2(far0 ? rsqrt_normal(d2h.x) : 0.f, far1 ? rsqrt_normal(d2h.y) : 0.f);
     // y = y0 + ye: one Newton step in two floats (h = 1 - d2 y0^2)
     const float2 ny0 = __fmul2_rn(y0, m1);
     const float2 a = __fmul2_rn(y0, y0), na = __fmul2_rn(ny0, y0);
@@ -313,7 +314,7 @@ __device__ __forceinline__ void fill_mom_head2(const float4* __restrict__ mom, c
                                                float2& lo) {
     const float2 m1 = bc2(-1.f);
     auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
-    y0 = make_float2(far0 ? rsqrtf(P.d2h.x) : 0.f, far1 ? rsqrtf(P.d2h.y) : 0.f);
+    y0 = make_float2(far0 ? rsqrt_normal(P.d2h.x) : 0.f, far1 ? rsqrt_normal(P.d2h.y) : 0.f);
     const float2 ny0 = __fmul2_rn(y0, m1);
     a = __fmul2_rn(y0, y0);
     const float2 na = __fmul2_rn(ny0, y0);
