@@ -923,53 +923,172 @@ __global__ void k_make_perm_global(const int32_t* __restrict__ piv, int64_t n, i
     }
 }
 
+// Values that CTAs of one launch pass to one another through memory are their own flags: the array is
+// filled with the pattern of all ones (a NaN that no operation produces) and read with relaxed
+// loads until another value is there.
+__device__ __forceinline__ void ld_passed(const float* p, float& v, bool& set) {
+    uint32_t u;
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(u) : "l"(p) : "memory");
+    v = __uint_as_float(u);
+    set = u != 0xffffffffu;
+}
+__device__ __forceinline__ void ld_passed(const double* p, double& v, bool& set) {
+    unsigned long long u;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(u) : "l"(p) : "memory");
+    v = __longlong_as_double((long long)u);
+    set = u != ~0ull;
+}
+__device__ __forceinline__ void st_passed(float* p, float v) {
+    if (v != v) v = __uint_as_float(0x7fc00000u);
+    asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(__float_as_uint(v)) : "memory");
+}
+__device__ __forceinline__ void st_passed(double* p, double v) {
+    if (v != v) v = __longlong_as_double(0x7ff8000000000000ll);
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(__double_as_longlong(v)) : "memory");
+}
+__device__ __forceinline__ void set_unpassed(float& v) { v = __uint_as_float(0xffffffffu); }
+__device__ __forceinline__ void set_unpassed(double& v) { v = __longlong_as_double(-1ll); }
+
+// y = b permuted; z is made ready for the lower sweep's values
 template <typename T>
-__global__ void k_permute(const T* __restrict__ b, const int32_t* __restrict__ perm, int64_t n, T* __restrict__ y) {
+__global__ void k_permute(const T* __restrict__ b, const int32_t* __restrict__ perm, int64_t n, T* __restrict__ y,
+                          T* __restrict__ z) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = b[perm[i]];
+    if (i >= n) return;
+    y[i] = b[perm[i]];
+    set_unpassed(z[i]);
 }
 
 // One triangular sweep in one launch.  Block rows of kTB rows; the CTA with ticket t (taken
 // from an atomic counter, so tickets follow the order in which CTAs start) solves block k =
 // t (lower sweep, unit-diagonal L) or nblk-1-t (upper sweep, U):
 //   x_k = D_k^-1 (rhs_k - sum_c M_kc x_c),  c < k (lower) or c > k (upper),
-// taking the blocks c in sweep order as their solutions are published (flags[c] set with
-// release semantics after x_c is written); when more than one block may be ready, one poll
-// reads the flags of the next blockDim.x blocks and the ready prefix is consumed.  A CTA
-// only waits for blocks of lower tickets, whose CTAs have started, so the waits end.  Each
-// thread owns one row of the block and a quarter of its columns; the matrix values of the
-// next block are loaded before its flag is awaited, so only x_c is read after it.  The
-// four partial sums are added in a fixed order, so the result does not depend on timing.
-// Diagonal block: FP64 sweeps solve it by substitution in one warp (lanes in step with
-// __syncwarp, one synchronisation per column; U's diagonal through reciprocals); FP32
+// taking the blocks c in sweep order as their solutions appear in x, which was filled with the
+// pattern of ld_passed (the lower sweep fills the upper sweep's).  A CTA only waits for
+// blocks of lower tickets, whose CTAs have started, so the waits end.  Each thread owns one
+// row of the block and a quarter of its columns, and every warp waits for its 16 values by
+// itself; the matrix values of the next block are in flight meanwhile.  The four partial sums are
+// added in a fixed order, so the result does not depend on timing.
+// Diagonal block: FP64 sweeps solve it by substitution in one warp (warp_substitute); FP32
 // sweeps (the inner solves of the iterative refinement) invert it in shared memory while
-// the CTA waits, so that the step on the critical path is a 64 x 64 matrix-vector product.  Every wait is bounded: on
-// giving up the CTA records *err, writes NaN for its block and still publishes it.
+// the CTA waits, so that the step on the critical path is a 64 x 64 matrix-vector product.
+// Every wait is bounded: on giving up the CTA records *err and passes NaN for its block.
+// Bound by the chain over the blocks (value to the next CTA, its product, sum and diagonal block): 64
+// rows take 1.1 us in FP32 and 8.5 us in FP64 (3.1 and 15 us with flags that one thread polls
+// and the block barriers around them, and with the substitution in shared memory).
 constexpr int kSvThreads = 256;
 constexpr long long kSvSpinLimit = 1ll << 22;
 
-__device__ __forceinline__ int ld_acquire(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
+// xs = D^-1 xs for the block's w rows by one warp, two rows to a lane, the solved value broadcast
+// by shuffle: L (unit diagonal) downwards, U upwards with the reciprocals of its diagonal.
+// D is zero outside its w x w entries.
+template <typename T>
+__device__ __forceinline__ void warp_substitute(const T (*__restrict__ D)[kTB + 1], const T* __restrict__ dinv,
+                                                T* xs, int w, bool lower) {
+    static_assert(kTB == 64, "two rows per lane");
+    const int lane = threadIdx.x % 32;
+    const bool has0 = lane < w, has1 = lane + 32 < w;
+    T a0 = has0 ? xs[lane] : (T)0, a1 = has1 ? xs[lane + 32] : (T)0;
+    if (lower) {
+        const int m = min(w, 32);
+#pragma unroll 8
+        for (int c = 0; c < m; ++c) {
+            const T d0 = D[lane][c], d1 = D[lane + 32][c];
+            const T xc = __shfl_sync(0xffffffffu, a0, c);
+            if (lane > c) a0 = fma(-d0, xc, a0);
+            a1 = fma(-d1, xc, a1);
+        }
+#pragma unroll 8
+        for (int c = 32; c < w; ++c) {
+            const T d1 = D[lane + 32][c];
+            const T xc = __shfl_sync(0xffffffffu, a1, c - 32);
+            if (lane + 32 > c) a1 = fma(-d1, xc, a1);
+        }
+    } else {
+        const T i0 = has0 ? dinv[lane] : (T)0, i1 = has1 ? dinv[lane + 32] : (T)0;
+#pragma unroll 8
+        for (int c = w - 1; c >= 32; --c) {
+            const T d0 = D[lane][c], d1 = D[lane + 32][c];
+            const T xc = __shfl_sync(0xffffffffu, a1 * i1, c - 32);
+            if (lane + 32 < c) a1 = fma(-d1, xc, a1);
+            a0 = fma(-d0, xc, a0);
+        }
+#pragma unroll 8
+        for (int c = min(w, 32) - 1; c >= 0; --c) {
+            const T d0 = D[lane][c];
+            const T xc = __shfl_sync(0xffffffffu, a0 * i0, c);
+            if (lane < c) a0 = fma(-d0, xc, a0);
+        }
+        a0 *= i0;
+        a1 *= i1;
+    }
+    if (has0) xs[lane] = a0;
+    if (has1) xs[lane + 32] = a1;
 }
-__device__ __forceinline__ void st_release(int* p, int v) {
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+
+// X = D^-1, each warp kTB / warps columns in registers (two rows to a lane), eliminated together.  (9 us
+// with the columns in shared memory and a block barrier per step; every sweep starts with it.)
+template <typename T>
+__device__ __forceinline__ void warp_invert(const T (*__restrict__ D)[kTB + 1], const T* __restrict__ dinv,
+                                            T (*__restrict__ X)[kTB + 1], int w, bool lower) {
+    constexpr int kC = kTB / (kSvThreads / 32);
+    const int lane = threadIdx.x % 32, c0 = threadIdx.x / 32 * kC;
+    T a0[kC], a1[kC];
+#pragma unroll
+    for (int j = 0; j < kC; ++j) {
+        a0[j] = lane == c0 + j && lane < w ? (T)1 : (T)0;
+        a1[j] = lane + 32 == c0 + j && lane + 32 < w ? (T)1 : (T)0;
+    }
+    if (lower) {
+        for (int q = 0; q + 1 < w; ++q) {
+            const T d0 = D[lane][q], d1 = D[lane + 32][q];
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                const T x = __shfl_sync(0xffffffffu, q < 32 ? a0[j] : a1[j], q & 31);
+                if (lane > q) a0[j] = fma(-d0, x, a0[j]);
+                if (lane + 32 > q) a1[j] = fma(-d1, x, a1[j]);
+            }
+        }
+    } else {
+        const T i0 = lane < w ? dinv[lane] : (T)0, i1 = lane + 32 < w ? dinv[lane + 32] : (T)0;
+        for (int q = w - 1; q >= 0; --q) {
+            const T d0 = D[lane][q], d1 = D[lane + 32][q], iq = dinv[q];
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                const T v = __shfl_sync(0xffffffffu, q < 32 ? a0[j] : a1[j], q & 31) * iq;
+                const T x = c0 + j >= q ? v : (T)0;  // X is upper triangular, also beside a zero pivot
+                if (lane < q) a0[j] = fma(-d0, x, a0[j]);
+                if (lane + 32 < q) a1[j] = fma(-d1, x, a1[j]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kC; ++j) {
+            if (lane <= c0 + j) a0[j] *= i0;
+            if (lane + 32 <= c0 + j) a1[j] *= i1;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kC; ++j) {
+        X[lane][c0 + j] = a0[j];
+        X[lane + 32][c0 + j] = a1[j];
+    }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kSvThreads) k_trsv(const T* __restrict__ LU, int64_t n, int64_t nblk, int lower,
-                                                     const T* __restrict__ rhs, T* x, int* flags, int* ticket,
-                                                     int* err, long long limit) {
+                                                     const T* __restrict__ rhs, T* x, T* __restrict__ next,
+                                                     int* ticket, int* err, long long limit) {
     constexpr bool kInv = sizeof(T) == 4;  // explicit inverse of the diagonal block (FP32)
     __shared__ T D[kTB][kTB + 1];
     __shared__ T Xi[kInv ? kTB : 1][kTB + 1];
     __shared__ T part[kSvThreads / kTB][kTB];
     __shared__ T xs[kTB];
-    __shared__ T xo[kInv ? 1 : kTB];
     __shared__ T dinv[kTB];
-    __shared__ int s_t, s_ready, s_ok;
-    if (threadIdx.x == 0) s_t = atomicAdd(ticket, 1);
+    __shared__ int s_t, s_fail;
+    if (threadIdx.x == 0) {
+        s_t = atomicAdd(ticket, 1);
+        s_fail = 0;
+    }
     __syncthreads();
     const int64_t t = s_t;
     const int64_t k = lower ? t : nblk - 1 - t;
@@ -977,106 +1096,58 @@ __global__ void __launch_bounds__(kSvThreads) k_trsv(const T* __restrict__ LU, i
     const int w = (int)(r1 - r0);
     constexpr int kGroups = kSvThreads / kTB, kCols = kTB / kGroups;
     const int row = threadIdx.x % kTB, grp = threadIdx.x / kTB;
-    for (int idx = threadIdx.x; idx < w * w; idx += kSvThreads) {
-        const int r = idx % w, c = idx / w;
-        D[r][c] = LU[(r0 + r) + (r0 + c) * n];
+    if (next && threadIdx.x < w) set_unpassed(next[r0 + threadIdx.x]);
+    for (int idx = threadIdx.x; idx < kTB * kTB; idx += kSvThreads) {
+        const int r = idx % kTB, c = idx / kTB;
+        D[r][c] = (r < w && c < w) ? LU[(r0 + r) + (r0 + c) * n] : (T)0;
     }
     // independent of the other blocks: the block's right-hand side and, for U, the
     // reciprocals of its diagonal
     const T rhs_own = (threadIdx.x < w) ? rhs[r0 + threadIdx.x] : (T)0;
     if (!lower && threadIdx.x < w) dinv[threadIdx.x] = (T)1 / LU[(r0 + threadIdx.x) + (r0 + threadIdx.x) * n];
-    if constexpr (kInv) {
-        // X = D^-1 by forward (L, unit diagonal) or backward (U) substitution of all
-        // columns at once, one block barrier per step
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < kTB * kTB; idx += kSvThreads) {
-            const int r = idx % kTB, c = idx / kTB;
-            Xi[r][c] = (r == c && r < w) ? (T)1 : (T)0;
-        }
-        __syncthreads();
-        if (lower) {
-            for (int q = 0; q + 1 < w; ++q) {
-                const int rows = w - 1 - q;
-                for (int idx = threadIdx.x; idx < rows * (q + 1); idx += kSvThreads) {
-                    const int r = q + 1 + idx % rows, c = idx / rows;
-                    Xi[r][c] -= D[r][q] * Xi[q][c];
-                }
-                __syncthreads();
-            }
-        } else {
-            for (int q = w - 1; q >= 0; --q) {
-                // row q of X is final once scaled by 1 / U[q][q]; then eliminate above
-                const int cols = w - q;
-                for (int c = q + threadIdx.x; c < w; c += kSvThreads) Xi[q][c] *= dinv[q];
-                __syncthreads();
-                for (int idx = threadIdx.x; idx < q * cols; idx += kSvThreads) {
-                    const int r = idx % q, c = q + idx / q;
-                    Xi[r][c] -= D[r][q] * Xi[q][c];
-                }
-                __syncthreads();
-            }
-        }
-    }
+    __syncthreads();
+    if constexpr (kInv) warp_invert<T>(D, dinv, Xi, w, lower);
     T acc = (T)0;
     const int64_t total = lower ? k : nblk - 1 - k;
+    const int lane = threadIdx.x % 32;
     // matrix values of block i (sweep order) for this thread: row `row`, kCols columns
     T mv[kCols];
-    auto load_block = [&](int64_t i) {
+    auto load_block = [&](int64_t i, T (&m)[kCols]) {
         const int64_t c0 = (lower ? i : nblk - 1 - i) * kTB + grp * kCols;
         const T* col = LU + (r0 + row) + c0 * n;
         const int wc = (int)min((int64_t)kCols, n - c0);
 #pragma unroll
-        for (int q = 0; q < kCols; ++q) mv[q] = (row < w && q < wc) ? col[(int64_t)q * n] : (T)0;
+        for (int q = 0; q < kCols; ++q) m[q] = (row < w && q < wc) ? col[(int64_t)q * n] : (T)0;
     };
-    auto use_block = [&](int64_t i) {
+    if (total > 0) load_block(0, mv);
+    long long spins = 0;
+    // block i with the matrix values m, while those of block i + 1 arrive in nx
+    auto step = [&](int64_t i, const T(&m)[kCols], T(&nx)[kCols]) {
+        if (i + 1 < total) load_block(i + 1, nx);
+        // the warp's kCols values of x (the last block of x may be short)
         const int64_t c0 = (lower ? i : nblk - 1 - i) * kTB + grp * kCols;
-        const int wc = (int)min((int64_t)kCols, n - c0);
-#pragma unroll
-        for (int q = 0; q < kCols; ++q)
-            if (q < wc) acc = fma(mv[q], __ldcg(x + c0 + q), acc);
-    };
-    if (total > 0) load_block(0);
-    int64_t done = 0;
-    long long spins = 0;  // used by thread 0
-    bool ok = true;
-    while (done < total) {
-        // one thread waits (bounded) for the next block in sweep order; if more blocks may
-        // be ready, all threads read the flags of the following ones and take the ready prefix
-        if (threadIdx.x == 0) {
-            const int* fp = flags + (lower ? done : nblk - 1 - done);
-            int f = ld_acquire(fp);
-            while (!f && ++spins <= limit) {
-                __nanosleep(32);
-                f = ld_acquire(fp);
-            }
-            s_ok = f != 0;
-            s_ready = kSvThreads;
+        const int q = lane % kCols;
+        T v = (T)0;
+        bool set = true;
+        for (;;) {
+            if (c0 + q < n) ld_passed(x + c0 + q, v, set);
+            if (__all_sync(0xffffffffu, set) || ++spins > limit) break;
+            if (i + 2 < total) __nanosleep(64);  // this block is not the next one's critical path
         }
-        __syncthreads();
-        if (!s_ok) {
-            ok = false;
+        if (!__all_sync(0xffffffffu, set)) return false;
+#pragma unroll
+        for (int j = 0; j < kCols; ++j) acc = fma(m[j], __shfl_sync(0xffffffffu, v, j), acc);
+        return true;
+    };
+    T mw[kCols];
+    for (int64_t i = 0; i < total; i += 2)
+        if (!step(i, mv, mw) || (i + 1 < total && !step(i + 1, mw, mv))) {
+            if (lane == 0) s_fail = 1;
             break;
         }
-        int64_t ready = 1;
-        if (total - done > 1) {
-            const int64_t idx = done + threadIdx.x;
-            if (threadIdx.x > 0 && idx < total && ld_acquire(flags + (lower ? idx : nblk - 1 - idx)) == 0)
-                atomicMin(&s_ready, (int)threadIdx.x);
-            __syncthreads();
-            ready = min((int64_t)s_ready, total - done);
-        }
-        __syncthreads();  // s_ready and s_ok are rewritten by the next poll
-        use_block(done);
-        for (int64_t i = done + 1; i < done + ready; ++i) {
-            load_block(i);
-            use_block(i);
-        }
-        done += ready;
-        if (done < total) load_block(done);  // in flight while the next flag is awaited
-    }
-    if (!ok) atomicExch(err, 1);
     part[grp][row] = acc;
     __syncthreads();
+    const bool ok = s_fail == 0;
     if (threadIdx.x < w) {
         T sum = part[0][threadIdx.x];
 #pragma unroll
@@ -1100,36 +1171,13 @@ __global__ void __launch_bounds__(kSvThreads) k_trsv(const T* __restrict__ LU, i
             T sum = part[0][threadIdx.x];
 #pragma unroll
             for (int g = 1; g < kGroups; ++g) sum += part[g][threadIdx.x];
-            xs[threadIdx.x] = sum;
+            st_passed(x + r0 + threadIdx.x, ok ? sum : (T)NAN);
         }
-    } else {
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            if (lower) {
-                for (int c = 0; c < w; ++c) {
-                    const T xc = xs[c];
-                    for (int r = lane; r < w; r += 32)
-                        if (r > c) xs[r] -= D[r][c] * xc;
-                    __syncwarp();
-                }
-            } else {
-                // every lane scales x_c itself (the same rounded product), the owner lane
-                // keeps it in xo: one warp synchronisation per column
-                for (int c = w - 1; c >= 0; --c) {
-                    const T xc = xs[c] * dinv[c];
-                    if (lane == (c & 31)) xo[c] = xc;
-                    for (int r = lane; r < c; r += 32) xs[r] -= D[r][c] * xc;
-                    __syncwarp();
-                }
-                for (int r = lane; r < w; r += 32) xs[r] = xo[r];
-            }
-        }
+    } else if (threadIdx.x < 32) {
+        warp_substitute<T>(D, dinv, xs, w, lower);
+        for (int r = threadIdx.x; r < w; r += 32) st_passed(x + r0 + r, ok ? xs[r] : (T)NAN);
     }
-    __syncthreads();
-    if (threadIdx.x < w) x[r0 + threadIdx.x] = ok ? xs[threadIdx.x] : (T)NAN;
-    // the block barrier orders the CTA's stores before thread 0's release (cumulative)
-    __syncthreads();
-    if (threadIdx.x == 0) st_release(flags + k, 1);
+    if (threadIdx.x == 0 && !ok) atomicExch(err, 1);
 }
 
 // The same sweep for nr <= kMR right-hand sides at once (columns of rhs and x, leading
@@ -1138,21 +1186,20 @@ __global__ void __launch_bounds__(kSvThreads) k_trsv(const T* __restrict__ LU, i
 // column the arithmetic is k_trsv's, in its order (the fma chain over blocks and columns,
 // the four group sums in order, the diagonal block: FP64 substitution, one warp per column;
 // FP32 explicit inverse), so column j equals k_trsv on that column bit for bit.  Waits,
-// give-up and publication as in k_trsv.  Dynamic shared memory, trsm_smem_bytes<T>():
-//   D[kTB][kTB+1], Xi[kTB][kTB+1] (FP32 only), part[groups][kMR][kTB] (FP64: shared with
-//   the substitution's xo[kMR][kTB]), xs[kMR][kTB] (the block's right-hand sides, then its
-//   solution), dinv[kTB].
+// give-up and passing as in k_trsv.  Dynamic shared memory, trsm_smem_bytes<T>():
+//   D[kTB][kTB+1], Xi[kTB][kTB+1] (FP32 only), part[groups][kMR][kTB], xs[kMR][kTB] (the
+//   block's right-hand sides, then its solution), dinv[kTB], xw[warps][kMR][16] (the passed values).
 constexpr int kMR = 8;
 
 template <typename T>
 __host__ __device__ constexpr size_t trsm_smem_bytes() {
     return sizeof(T) * ((size_t)kTB * (kTB + 1) * (sizeof(T) == 4 ? 2 : 1) + (size_t)(kSvThreads / kTB) * kMR * kTB +
-                        (size_t)kMR * kTB + kTB);
+                        (size_t)kMR * kTB + kTB + (size_t)(kSvThreads / 32) * kMR * (kTB * kTB / kSvThreads));
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kSvThreads) k_trsm(const T* __restrict__ LU, int64_t n, int64_t nblk, int lower,
-                                                     const T* __restrict__ rhs, T* x, int nr, int* flags,
+                                                     const T* __restrict__ rhs, T* x, T* __restrict__ next, int nr,
                                                      int* ticket, int* err, long long limit) {
     constexpr bool kInv = sizeof(T) == 4;
     constexpr int kGroups = kSvThreads / kTB, kCols = kTB / kGroups;
@@ -1160,121 +1207,86 @@ __global__ void __launch_bounds__(kSvThreads) k_trsm(const T* __restrict__ LU, i
     T(*D)[kTB + 1] = reinterpret_cast<T(*)[kTB + 1]>(trsm_sm);
     T(*Xi)[kTB + 1] = D + kTB;  // FP32 only
     T(*part)[kMR][kTB] = reinterpret_cast<T(*)[kMR][kTB]>(reinterpret_cast<T*>(D + (kInv ? 2 : 1) * kTB));
-    T(*xo)[kTB] = part[0];  // FP64 substitution, after the group sums
     T(*xs)[kTB] = reinterpret_cast<T(*)[kTB]>(reinterpret_cast<T*>(part + kGroups));
     T* dinv = reinterpret_cast<T*>(xs + kMR);
-    __shared__ int s_t, s_ready, s_ok;
-    if (threadIdx.x == 0) s_t = atomicAdd(ticket, 1);
+    T(*xw)[kCols] = reinterpret_cast<T(*)[kCols]>(dinv + kTB) + kMR * (threadIdx.x / 32);
+    __shared__ int s_t, s_fail;
+    if (threadIdx.x == 0) {
+        s_t = atomicAdd(ticket, 1);
+        s_fail = 0;
+    }
     __syncthreads();
     const int64_t t = s_t;
     const int64_t k = lower ? t : nblk - 1 - t;
     const int64_t r0 = k * kTB, r1 = min(n, r0 + (int64_t)kTB);
     const int w = (int)(r1 - r0);
     const int row = threadIdx.x % kTB, grp = threadIdx.x / kTB;
-    for (int idx = threadIdx.x; idx < w * w; idx += kSvThreads) {
-        const int r = idx % w, c = idx / w;
-        D[r][c] = LU[(r0 + r) + (r0 + c) * n];
+    for (int idx = threadIdx.x; idx < kTB * kTB; idx += kSvThreads) {
+        const int r = idx % kTB, c = idx / kTB;
+        D[r][c] = (r < w && c < w) ? LU[(r0 + r) + (r0 + c) * n] : (T)0;
     }
     for (int idx = threadIdx.x; idx < w * nr; idx += kSvThreads) {
         const int j = idx / w, r = idx - j * w;
         xs[j][r] = rhs[r0 + r + (int64_t)j * n];
+        if (next) set_unpassed(next[r0 + r + (int64_t)j * n]);
     }
     if (!lower && threadIdx.x < w) dinv[threadIdx.x] = (T)1 / LU[(r0 + threadIdx.x) + (r0 + threadIdx.x) * n];
-    if constexpr (kInv) {
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < kTB * kTB; idx += kSvThreads) {
-            const int r = idx % kTB, c = idx / kTB;
-            Xi[r][c] = (r == c && r < w) ? (T)1 : (T)0;
-        }
-        __syncthreads();
-        if (lower) {
-            for (int q = 0; q + 1 < w; ++q) {
-                const int rows = w - 1 - q;
-                for (int idx = threadIdx.x; idx < rows * (q + 1); idx += kSvThreads) {
-                    const int r = q + 1 + idx % rows, c = idx / rows;
-                    Xi[r][c] -= D[r][q] * Xi[q][c];
-                }
-                __syncthreads();
-            }
-        } else {
-            for (int q = w - 1; q >= 0; --q) {
-                const int cols = w - q;
-                for (int c = q + threadIdx.x; c < w; c += kSvThreads) Xi[q][c] *= dinv[q];
-                __syncthreads();
-                for (int idx = threadIdx.x; idx < q * cols; idx += kSvThreads) {
-                    const int r = idx % q, c = q + idx / q;
-                    Xi[r][c] -= D[r][q] * Xi[q][c];
-                }
-                __syncthreads();
-            }
-        }
-    }
+    __syncthreads();
+    if constexpr (kInv) warp_invert<T>(D, dinv, Xi, w, lower);
     T acc[kMR];
 #pragma unroll
     for (int j = 0; j < kMR; ++j) acc[j] = (T)0;
     const int64_t total = lower ? k : nblk - 1 - k;
+    const int lane = threadIdx.x % 32;
     T mv[kCols];
-    auto load_block = [&](int64_t i) {
+    auto load_block = [&](int64_t i, T (&m)[kCols]) {
         const int64_t c0 = (lower ? i : nblk - 1 - i) * kTB + grp * kCols;
         const T* col = LU + (r0 + row) + c0 * n;
         const int wc = (int)min((int64_t)kCols, n - c0);
 #pragma unroll
-        for (int q = 0; q < kCols; ++q) mv[q] = (row < w && q < wc) ? col[(int64_t)q * n] : (T)0;
+        for (int q = 0; q < kCols; ++q) m[q] = (row < w && q < wc) ? col[(int64_t)q * n] : (T)0;
     };
-    auto use_block = [&](int64_t i) {
-        const int64_t c0 = (lower ? i : nblk - 1 - i) * kTB + grp * kCols;
-        const int wc = (int)min((int64_t)kCols, n - c0);
-#pragma unroll
-        for (int q = 0; q < kCols; ++q)
-            if (q < wc) {
-#pragma unroll
-                for (int j = 0; j < kMR; ++j)
-                    if (j < nr) acc[j] = fma(mv[q], __ldcg(x + c0 + q + (int64_t)j * n), acc[j]);
-            }
-    };
-    if (total > 0) load_block(0);
-    int64_t done = 0;
+    if (total > 0) load_block(0, mv);
     long long spins = 0;
-    bool ok = true;
-    while (done < total) {
-        if (threadIdx.x == 0) {
-            const int* fp = flags + (lower ? done : nblk - 1 - done);
-            int f = ld_acquire(fp);
-            while (!f && ++spins <= limit) {
-                __nanosleep(32);
-                f = ld_acquire(fp);
+    auto step = [&](int64_t i, const T(&m)[kCols], T(&nx)[kCols]) {
+        if (i + 1 < total) load_block(i + 1, nx);
+        // the warp's kCols values of every column of x, two columns per load
+        const int64_t c0 = (lower ? i : nblk - 1 - i) * kTB + grp * kCols;
+        const int q = lane % kCols;
+        for (int j0 = 0; j0 < nr; j0 += 32 / kCols) {
+            const int j = j0 + lane / kCols;
+            T v = (T)0;
+            bool set = true;
+            const bool mine = j < nr && c0 + q < n;
+            for (;;) {
+                if (mine) ld_passed(x + c0 + q + (int64_t)j * n, v, set);
+                if (__all_sync(0xffffffffu, set) || ++spins > limit) break;
+                if (i + 2 < total) __nanosleep(64);
             }
-            s_ok = f != 0;
-            s_ready = kSvThreads;
+            if (!__all_sync(0xffffffffu, set)) return false;
+            xw[j][q] = v;
         }
-        __syncthreads();
-        if (!s_ok) {
-            ok = false;
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < kCols; ++c)
+#pragma unroll
+            for (int j = 0; j < kMR; ++j)
+                if (j < nr) acc[j] = fma(m[c], xw[j][c], acc[j]);
+        __syncwarp();
+        return true;
+    };
+    T mw[kCols];
+    for (int64_t i = 0; i < total; i += 2)
+        if (!step(i, mv, mw) || (i + 1 < total && !step(i + 1, mw, mv))) {
+            if (lane == 0) s_fail = 1;
             break;
         }
-        int64_t ready = 1;
-        if (total - done > 1) {
-            const int64_t idx = done + threadIdx.x;
-            if (threadIdx.x > 0 && idx < total && ld_acquire(flags + (lower ? idx : nblk - 1 - idx)) == 0)
-                atomicMin(&s_ready, (int)threadIdx.x);
-            __syncthreads();
-            ready = min((int64_t)s_ready, total - done);
-        }
-        __syncthreads();
-        use_block(done);
-        for (int64_t i = done + 1; i < done + ready; ++i) {
-            load_block(i);
-            use_block(i);
-        }
-        done += ready;
-        if (done < total) load_block(done);
-    }
-    if (!ok) atomicExch(err, 1);
     // every column's four group sums, in order, subtracted from its right-hand side
 #pragma unroll
     for (int j = 0; j < kMR; ++j)
         if (j < nr) part[grp][j][row] = acc[j];
     __syncthreads();
+    const bool ok = s_fail == 0;
     for (int idx = threadIdx.x; idx < w * nr; idx += kSvThreads) {
         const int j = idx / w, r = idx - j * w;
         T sum = part[0][j][r];
@@ -1306,45 +1318,26 @@ __global__ void __launch_bounds__(kSvThreads) k_trsm(const T* __restrict__ LU, i
             T sum = part[0][j][r];
 #pragma unroll
             for (int g = 1; g < kGroups; ++g) sum += part[g][j][r];
-            xs[j][r] = sum;
+            st_passed(x + r0 + r + (int64_t)j * n, ok ? sum : (T)NAN);
         }
     } else {
-        const int j = threadIdx.x / 32, lane = threadIdx.x % 32;
+        const int j = threadIdx.x / 32;
         if (j < nr) {
-            if (lower) {
-                for (int c = 0; c < w; ++c) {
-                    const T xc = xs[j][c];
-                    for (int r = lane; r < w; r += 32)
-                        if (r > c) xs[j][r] -= D[r][c] * xc;
-                    __syncwarp();
-                }
-            } else {
-                for (int c = w - 1; c >= 0; --c) {
-                    const T xc = xs[j][c] * dinv[c];
-                    if (lane == (c & 31)) xo[j][c] = xc;
-                    for (int r = lane; r < c; r += 32) xs[j][r] -= D[r][c] * xc;
-                    __syncwarp();
-                }
-                for (int r = lane; r < w; r += 32) xs[j][r] = xo[j][r];
-            }
+            warp_substitute<T>(D, dinv, xs[j], w, lower);
+            for (int r = lane; r < w; r += 32) st_passed(x + r0 + r + (int64_t)j * n, ok ? xs[j][r] : (T)NAN);
         }
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < w * nr; idx += kSvThreads) {
-        const int j = idx / w, r = idx - j * w;
-        x[r0 + r + (int64_t)j * n] = ok ? xs[j][r] : (T)NAN;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) st_release(flags + k, 1);
+    if (threadIdx.x == 0 && !ok) atomicExch(err, 1);
 }
 
 template <typename T>
 __global__ void k_permute_m(const T* __restrict__ b, const int32_t* __restrict__ perm, int64_t n, int nr,
-                            T* __restrict__ y) {
+                            T* __restrict__ y, T* __restrict__ z) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * nr) return;
     const int64_t j = idx / n, i = idx - j * n;
     y[idx] = b[perm[i] + j * n];
+    set_unpassed(z[idx]);
 }
 
 template <typename T>
@@ -1353,17 +1346,15 @@ cudaError_t lu_solve(const T* LU, int64_t n, const int32_t* perm, T* b, T* work,
     const int64_t nblk = (n + kTB - 1) / kTB;
     T* y = work;
     T* z = work + n;
-    // flags of both sweeps, their tickets and the error flag (16-byte aligned after z)
-    const uintptr_t fo = ((uintptr_t)(z + n) + 15) & ~(uintptr_t)15;
-    int* flags = reinterpret_cast<int*>(fo);
-    int* tickets = flags + 2 * nblk;
+    // both sweeps' tickets and the error flag (16-byte aligned after z)
+    int* tickets = reinterpret_cast<int*>(((uintptr_t)(z + n) + 15) & ~(uintptr_t)15);
     int* err = tickets + 2;
-    NB_TRY(cudaMemsetAsync(flags, 0, sizeof(int) * (2 * nblk + 3), s));
+    NB_TRY(cudaMemsetAsync(tickets, 0, 3 * sizeof(int), s));
     const unsigned g = (unsigned)((n + 255) / 256);
-    k_permute<T><<<g, 256, 0, s>>>(b, perm, n, y);
+    k_permute<T><<<g, 256, 0, s>>>(b, perm, n, y, z);
     const long long limit = polls > 0 ? polls : kSvSpinLimit;
-    k_trsv<T><<<(unsigned)nblk, kSvThreads, 0, s>>>(LU, n, nblk, 1, y, z, flags, tickets, err, limit);
-    k_trsv<T><<<(unsigned)nblk, kSvThreads, 0, s>>>(LU, n, nblk, 0, z, b, flags + nblk, tickets + 1, err, limit);
+    k_trsv<T><<<(unsigned)nblk, kSvThreads, 0, s>>>(LU, n, nblk, 1, y, z, b, tickets, err, limit);
+    k_trsv<T><<<(unsigned)nblk, kSvThreads, 0, s>>>(LU, n, nblk, 0, z, b, nullptr, tickets + 1, err, limit);
     return cudaGetLastError();
 }
 
@@ -1556,7 +1547,7 @@ cudaError_t lu_factor_f32(float* A, int64_t n, int32_t* piv, int nb, float* work
     return lu_factor<float>(A, n, piv, nb, work, d_info, split, coop, s, polls);
 }
 size_t lu_solve_work_bytes(int64_t n, size_t tsize) {
-    return 2 * tsize * (size_t)n + 16 + sizeof(int) * (size_t)(2 * ((n + kTB - 1) / kTB) + 3) + 256;
+    return 2 * tsize * (size_t)n + 16 + 3 * sizeof(int) + 256;
 }
 
 size_t residual_work_bytes(int64_t n) {
@@ -1585,11 +1576,9 @@ cudaError_t lu_solve_f32(const float* LU, int64_t n, const int32_t* perm, float*
     return lu_solve<float>(LU, n, perm, b, static_cast<float*>(work), s, polls);
 }
 const int* lu_solve_err_flag(const void* work, int64_t n, size_t tsize) {
-    // as laid out by lu_solve: y, z (n values each), then 16-byte aligned flags of both
-    // sweeps (nblk each), the two tickets and the error flag
+    // as laid out by lu_solve: y, z (n values each), then 16-byte aligned the two tickets and the error flag
     const uintptr_t fo = ((uintptr_t)static_cast<const char*>(work) + 2 * tsize * (size_t)n + 15) & ~(uintptr_t)15;
-    const int64_t nblk = (n + kTB - 1) / kTB;
-    return reinterpret_cast<const int*>(fo) + 2 * nblk + 2;
+    return reinterpret_cast<const int*>(fo) + 2;
 }
 cudaError_t gemv_residual(const double* K, int64_t n, const double* x, const double* b, double* r, void* work,
                           cudaStream_t s) {
@@ -1619,17 +1608,16 @@ cudaError_t vec_absmax(const double* a, int64_t n, double* out, cudaStream_t s) 
 
 // ---- several right-hand sides (columns of leading dimension n), kMR per pass
 size_t lu_solve_multi_work_bytes(int64_t n, size_t tsize) {
-    return 2 * tsize * (size_t)n * kMR + 16 + sizeof(int) * (size_t)(2 * ((n + kTB - 1) / kTB) + 3) + 256;
+    return 2 * tsize * (size_t)n * kMR + 16 + 3 * sizeof(int) + 256;
 }
-static int* multi_flags(const void* work, int64_t n, size_t tsize) {
-    // y, z (n x kMR values each), then 16-byte aligned flags of both sweeps, the two
-    // tickets and the error flag
+static int* multi_tickets(const void* work, int64_t n, size_t tsize) {
+    // y, z (n x kMR values each), then the 16-byte aligned tickets of both sweeps and the error flag
     const uintptr_t fo =
         ((uintptr_t)static_cast<const char*>(work) + 2 * tsize * (size_t)n * kMR + 15) & ~(uintptr_t)15;
     return reinterpret_cast<int*>(fo);
 }
 const int* lu_solve_multi_err_flag(const void* work, int64_t n, size_t tsize) {
-    return multi_flags(work, n, tsize) + 2 * ((n + kTB - 1) / kTB) + 2;
+    return multi_tickets(work, n, tsize) + 2;
 }
 template <typename T>
 static cudaError_t lu_solve_multi(const T* LU, int64_t n, const int32_t* perm, T* B, int64_t nrhs, void* work,
@@ -1638,8 +1626,7 @@ static cudaError_t lu_solve_multi(const T* LU, int64_t n, const int32_t* perm, T
     const int64_t nblk = (n + kTB - 1) / kTB;
     T* y = static_cast<T*>(work);
     T* z = y + n * kMR;
-    int* flags = multi_flags(work, n, sizeof(T));
-    int* tickets = flags + 2 * nblk;
+    int* tickets = multi_tickets(work, n, sizeof(T));
     int* err = tickets + 2;
     NB_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
     const long long limit = polls > 0 ? polls : kSvSpinLimit;
@@ -1649,11 +1636,10 @@ static cudaError_t lu_solve_multi(const T* LU, int64_t n, const int32_t* perm, T
     for (int64_t c0 = 0; c0 < nrhs; c0 += kMR) {
         const int nr = (int)std::min<int64_t>(kMR, nrhs - c0);
         T* b = B + c0 * n;
-        NB_TRY(cudaMemsetAsync(flags, 0, sizeof(int) * (2 * nblk + 2), s));
-        k_permute_m<T><<<(unsigned)((n * nr + 255) / 256), 256, 0, s>>>(b, perm, n, nr, y);
-        k_trsm<T><<<(unsigned)nblk, kSvThreads, smem, s>>>(LU, n, nblk, 1, y, z, nr, flags, tickets, err, limit);
-        k_trsm<T><<<(unsigned)nblk, kSvThreads, smem, s>>>(LU, n, nblk, 0, z, b, nr, flags + nblk, tickets + 1, err,
-                                                           limit);
+        NB_TRY(cudaMemsetAsync(tickets, 0, 2 * sizeof(int), s));
+        k_permute_m<T><<<(unsigned)((n * nr + 255) / 256), 256, 0, s>>>(b, perm, n, nr, y, z);
+        k_trsm<T><<<(unsigned)nblk, kSvThreads, smem, s>>>(LU, n, nblk, 1, y, z, b, nr, tickets, err, limit);
+        k_trsm<T><<<(unsigned)nblk, kSvThreads, smem, s>>>(LU, n, nblk, 0, z, b, nullptr, nr, tickets + 1, err, limit);
         NB_TRY(cudaGetLastError());
     }
     return cudaSuccess;
