@@ -52,6 +52,7 @@ constexpr double kErrGammaB = 7e-8;   // FP32 pass: share of B
 constexpr double kErrGammaS = 5e-7;   // FP32 pass: share of S
 constexpr double kGammaL1 = 1e-9;    // two-float, the FP32 pass's rules (truncation ~1e-10 B)
 constexpr double kGammaL2 = 1e-11;   // two-float, fill-grade rules
+constexpr double kMomRatio2 = 40.0;  // level 2: the radius from which the fill's moments are taken (truncation 5e-13 of E)
 
 // What a refinement pass re-evaluates: both phi and E, phi only (its E estimate was within
 // the tolerance, E keeps the FP32 pass's value), or E only.
@@ -146,17 +147,42 @@ __device__ __forceinline__ void df_fma_acc(float ah, float al, float bh, float b
 // Two levels of re-evaluation, both two-float: level 1 takes the pairs from kMomRatio radii on by
 // their moments (mom_pair2) and the nearer ones by the tiers of the FP32 pass (nb_internal.h
 // FarNodes: 3x3 / 6-point, 4x4, 6x6 rules at ratio_a, ratio_b, ratio_near radii; FP64 closed forms
-// nearer); its truncation stays near 1e-10 of B.  Level 2 takes the fill's tiers (truncation below
-// ~3e-12 of each pair, FP64 within kFillRatioC radii).
+// nearer); its truncation stays near 1e-10 of B.  Level 2 takes the pairs from kMomRatio2 radii
+// on by the fill's moments (fill_mom_point2) and the nearer ones by the fill's tiers (truncation
+// below ~3e-12 of each pair, FP64 within kFillRatioC radii).
 //
-// dynamic shared memory per tile of te elements.  Level 1: FillEl (9 float4), the moments, the tier
+// dynamic shared memory per tile of te elements: FillEl (9 float4), the level's moments, the tier
 // radii, and tau as six planes of nimg (padded to even) floats (x, y, z negated: hi, then lo).
-// Level 2: FillEl, the tier-a nodes, tau and image centroids (2 float4 each per image).
 __host__ __device__ constexpr int acc_pad(int nimg) { return (nimg + 1) & ~1; }
+// odd strides (moments in float4, tau in float2): the lanes of the lane path read different elements
+__host__ __device__ constexpr int acc_tau_stride(int nimg) { return 6 * acc_pad(nimg) + 2; }
+__host__ __device__ constexpr int acc_mom_f4(int level) { return (level == 1 ? kMomF4 : kFillMomF4) | 1; }
 __host__ __device__ constexpr int acc_tile_f4(int level, int te, int nimg) {
-    return level == 1 ? te * (9 + kMomF4 + 1) + (te * 6 * acc_pad(nimg) + 3) / 4
-                      : te * (9 + 4 * kFillPairsA + 4 * nimg);
+    return te * (9 + acc_mom_f4(level) + 1) + (te * acc_tau_stride(nimg) + 3) / 4;
 }
+
+// A unit of the lane path (acc_range): kLP points of one leaf.  Per warp the values (sigma, Phi', E') of 32
+// (point, element) pairs, and the chains' results (Sum6) of its points.
+constexpr int kLP = 8;
+// Lists whose units are few take the lane path.  A thread per point cannot end before one thread has taken
+// its leaf, however short the list (0.9 ms at level 1 and 2.4 ms at level 2 for 10,000 elements x 25 copies);
+// with the lane path 20 points take 0.11 and 0.32 ms, 257 take 0.84 and 2.5 (1.7 and 4.0), 500 1.5 and
+// 4.0 (2.1 and 4.9), and from about 1,000 points (50 units per resident block) on both are alike.
+constexpr int64_t kLaneRounds = 32;
+__host__ __device__ __forceinline__ bool lane_path(const SplitPlan& plan, int64_t count, int64_t gb) {
+    return plan.leaf && plan.Gm == 0 && (count + kLP - 1) / kLP * plan.np < kLaneRounds * gb;
+}
+struct LaneScratch {
+    struct Val {  // d: sigma, Phi', E'; for the scales a: |Phi'|, |E'|_1 (level 2), f: |sigma|, |Phi'|, |E'|_1 (level 1)
+        double d[5];
+        union {
+            double a[2];
+            float f[3];
+        };
+    };
+    Val val[kAT / 32][32];
+    double out[kLP][6];
+};
 
 // Sums of an element's nearer pairs (those not taken by moments), two floats each.
 struct NearerSum {
@@ -215,19 +241,164 @@ __device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr,
 // (E: 2.0e-10 B before, 1.7e-11 B now, the largest of 665 refined points).  The FP32 pipe is busy for
 // about two thirds of it; 5 blocks per SM (96 registers) beat 4 by 3 %, 6 are the same.
 //
-// Raw sums (before ke) of the far pairs of one point over the elements [e0, e1) at level 1,
-// with the error scales, of phi and E (M = kBoth), phi only or E only (the other sums stay
-// 0); all threads of the block take part (tiles).
-template <int M>
-__device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
-                                           const float (&pl)[3], int64_t e0, int64_t e1) {
+// Level 2 in the same run: 98 ms with every pair by Gauss nodes, 57 ms by moments; largest errors
+// unchanged (phi 1.1e-15 B, E 1.1e-14 B).
+//
+// An element's sums over its images of one point (before sigma): Phi', and E' in the global frame.
+struct ElemSum {
+    double phi, x, y, z;
+};
+// The far pairs of a point (ph + pl) and element j of a staged tile at level L, of phi and E (M = kBoth),
+// phi only or E only.
+template <int L, int M>
+__device__ __forceinline__ ElemSum acc_element(const AccView& A, int nimg, int np2, int64_t j, const FillEl& F,
+                                               const float4* mom, const float4& hdr, const float* tau,
+                                               const float (&ph)[3], const float (&pl)[3]) {
+    // squared distance from which the moments are taken; never inside the near radius, which
+    // the two classifications of a pair (here and in the near kernel) round differently
+    constexpr double kRatio = L == 1 ? kMomRatio : kMomRatio2;
+    const float mom2 = fmaxf(F.hdr.x * (float)(kRatio * kRatio / (kFillRatioA * kFillRatioA)), hdr.w * 1.0001f);
+    float dh[3], dl[3];
+    df_sub(ph[0], pl[0], F.ch.x, F.cl.x, dh[0], dl[0]);
+    df_sub(ph[1], pl[1], F.ch.y, F.cl.y, dh[1], dl[1]);
+    df_sub(ph[2], pl[2], F.ch.z, F.cl.z, dh[2], dl[2]);
+    float x0h, x0l, y0h, y0l, z0h, z0l;
+    df_dot3(dh, dl, F.exh, F.exl, x0h, x0l);
+    df_dot3(dh, dl, F.eyh, F.eyl, y0h, y0l);
+    df_dot3(dh, dl, F.ezh, F.ezl, z0h, z0l);
+    MomSum2 S{};     // level 1
+    PointSum2 S2{};  // level 2
+    NearerSum nr{};
+    bool any_nearer = false;
+    uint32_t nearer = 0;  // images of the group of 32 at hand whose pair is not taken by moments
+    for (int k = 0; k < np2; k += 2) {
+        auto plane = [&](int q) { return *reinterpret_cast<const float2*>(tau + q * np2 + k); };
+        // X = X0 - tau, two floats
+        auto diff = [&](float ah, float al, int q, float2& h, float2& l) {
+            float2 t;
+            two_sum2(bc2(ah), plane(q), h, t);
+            l = __fadd2_rn(t, __fadd2_rn(bc2(al), plane(q + 3)));
+        };
+        FillPair2 P;
+        float2 &xh = P.xh, &xl = P.xl, &zh = P.zh, &zl = P.zl, yh, yl;
+        diff(x0h, x0l, 0, xh, xl);
+        diff(y0h, y0l, 1, yh, yl);
+        diff(z0h, z0l, 2, zh, zl);
+        float2 px = __fmul2_rn(xh, xh), py = __fmul2_rn(yh, yh), pz = __fmul2_rn(zh, zh);
+        float2 ex = __ffma2_rn(xh, xh, make_float2(-px.x, -px.y)), ey = __ffma2_rn(yh, yh, make_float2(-py.x, -py.y)),
+               ez = __ffma2_rn(zh, zh, make_float2(-pz.x, -pz.y));
+        ex = __ffma2_rn(__fadd2_rn(xh, xh), xl, ex);
+        ey = __ffma2_rn(__fadd2_rn(yh, yh), yl, ey);
+        ez = __ffma2_rn(__fadd2_rn(zh, zh), zl, ez);
+        float2 s, t1, t2, d2h;
+        two_sum2(px, py, s, t1);
+        two_sum2(s, pz, d2h, t2);
+        const float2 d2l = __fadd2_rn(__fadd2_rn(ex, ey), __fadd2_rn(ez, __fadd2_rn(t1, t2)));
+        const bool two = k + 1 < nimg;
+        const bool far0 = d2h.x >= mom2, far1 = two && d2h.y >= mom2;
+        if constexpr (L == 1) {
+            mom_pair2<M != kEOnly, M != kPhiOnly>(mom, F.ch.w, xh, xl, yh, yl, zh, zl, d2h, d2l,
+                                                  far0, far1, S);
+        } else {
+            P.px = px, P.ex = ex, P.pz = pz, P.ez = ez, P.d2h = d2h, P.d2l = d2l;
+            fill_mom_point2(mom, P, yh, yl, far0, far1, S2);
+        }
+        nearer |= ((far0 ? 0u : 1u) | (far1 || !two ? 0u : 2u)) << (k & 31);
+        if ((k & 31) == 30 || k + 2 >= np2) {
+            for (uint32_t m = nearer; m; m &= m - 1) {
+                const int kk = (k & ~31) + __ffs(m) - 1;
+                acc_pair_nodes<M>(A, hdr, (int)F.hdr.w, j, nimg, kk, ph, pl, x0h, x0l, y0h, y0l, z0h, z0l, tau,
+                                  np2, nr);
+            }
+            any_nearer = any_nearer || nearer;
+            nearer = 0;
+        }
+    }
+    // A x (sum over the images) + the other terms as two floats, then FP64, rotated to the global
+    // frame.  A conversion takes the FP64 pipe like an addition does, so each quantity crosses over
+    // once, as two values.
+    ElemSum v{0.0, 0.0, 0.0, 0.0};
+    double lx = 0.0, ly = 0.0, lz = 0.0;
+    const float4 tail = mom[(L == 1 ? kMomF4 : kFillMomF4) - 1];
+    if constexpr (L == 2) {
+        auto area = [&](const float2& h, const float2& l, float nh, float nl) {  // A x + nearer
+            float sh, t, p, e;
+            two_sum(h.x, h.y, sh, t);
+            const float sl = __fadd_rn(t, __fadd_rn(l.x, l.y));
+            two_prod(sh, tail.x, p, e);
+            e = __fmaf_rn(sh, tail.y, __fmaf_rn(sl, tail.x, e));
+            double x = (double)p + (double)e;
+            if (any_nearer) x += (double)nh + (double)nl;
+            return x;
+        };
+        v.phi = area(S2.ph, S2.pl, nr.ph, nr.pl);
+        lx = area(S2.xh, S2.xl, nr.xh, nr.xl);
+        ly = area(S2.yh, S2.yl, nr.yh, nr.yl);
+        lz = area(S2.zh, S2.zl, nr.zh, nr.zl);
+    } else {
+        // sign: -1 where the high parts are kept negated; unit: what c is kept over
+        auto total = [&](float sign, float unit, const float2& h, const float2& l, const float2& c) {
+            float sh, t, p, e;
+            two_sum(h.x, h.y, sh, t);
+            sh *= sign;
+            const float sl = __fmaf_rn(sign, t, __fadd_rn(l.x, l.y));
+            two_prod(sh, tail.z, p, e);
+            e = __fmaf_rn(sh, tail.w, __fmaf_rn(sl, tail.z, e));
+            return (double)p + (double)__fmaf_rn(__fadd_rn(c.x, c.y), unit, e);
+        };
+        const float rho = F.ch.w;
+        if constexpr (M != kEOnly) {
+            v.phi = total(1.f, rho * rho, S.ph, S.pl, S.fc);
+            if (any_nearer) v.phi += (double)nr.ph + (double)nr.pl;
+        }
+        if constexpr (M != kPhiOnly) {
+            lx = total(-1.f, rho, S.xh, S.xl, S.ex);
+            ly = total(-1.f, rho, S.yh, S.yl, S.ey);
+            lz = total(-1.f, rho, S.zh, S.zl, S.ez);
+            if (any_nearer) {
+                lx += (double)nr.xh + (double)nr.xl;
+                ly += (double)nr.yh + (double)nr.yl;
+                lz += (double)nr.zh + (double)nr.zl;
+            }
+        }
+    }
+    if constexpr (M != kPhiOnly) {
+        const Elem& e = A.el[j];
+        v.x = fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0]));
+        v.y = fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1]));
+        v.z = fma(lx, e.ex[2], fma(ly, e.ey[2], lz * e.ez[2]));
+    }
+    return v;
+}
+
+// Raw sums (before ke) over the elements [e0, e1) (at most a leaf) at level L, with the error
+// scales; all threads of the block take part (tiles).
+//   LANES = false: thread per point (ph + pl); returns its sums.
+//   LANES = true: a thread per (point, element): warp w takes the points list[i0 + w kLP / 4 ...] of the
+//   unit's kLP, te elements of 32 / te points at a time, and the ordered chains over the
+//   elements follow from shared memory; the sums go to out[6 per point] in shared memory.
+// Both give a point the same bits.
+template <int L, int M, bool LANES>
+__device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, float4* sm, float (&ph)[3], float (&pl)[3],
+                                          int64_t e0, int64_t e1, const double* __restrict__ pts,
+                                          const int32_t* __restrict__ list, int64_t i0, int64_t count) {
+    constexpr int kMF4 = acc_mom_f4(L);
+    const int np2 = acc_pad(nimg), ts = acc_tau_stride(nimg);
     FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
     float4* s_mom = sm + 9 * te;
-    float4* s_hdr = s_mom + kMomF4 * te;
+    float4* s_hdr = s_mom + kMF4 * te;
     float* s_tau = reinterpret_cast<float*>(s_hdr + te);
-    const int np2 = acc_pad(nimg);
+    LaneScratch* scr = reinterpret_cast<LaneScratch*>(sm + acc_tile_f4(L, te, nimg));
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int kWP = kLP / (kAT / 32);  // points of a warp
+    if constexpr (LANES) {
+        for (int i = lane; i < 6 * kWP; i += 32) scr->out[w * kWP][i] = 0.0;
+        __syncwarp();
+    }
+    const float4* gmom = L == 1 ? A.mom : A.mom2;
+    constexpr int kGM = L == 1 ? kMomF4 : kFillMomF4;
     Sum6 acc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    float bphi = 0.f, bE = 0.f;  // the leaf's error scales
+    float bphi = 0.f, bE = 0.f;  // level 1: the leaf's error scales in FP32
     for (int64_t base = e0; base < e1; base += te) {
         const int cnt = (int)min((int64_t)te, e1 - base);
         __syncthreads();
@@ -236,235 +407,88 @@ __device__ __forceinline__ Sum6 acc_range1(const AccView& A, int nimg, int te, f
             float4* dst = reinterpret_cast<float4*>(s_fe);
             for (int i = threadIdx.x; i < 9 * cnt; i += blockDim.x) dst[i] = src[i];
         }
-        for (int i = threadIdx.x; i < kMomF4 * cnt; i += blockDim.x) s_mom[i] = A.mom[base * kMomF4 + i];
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) s_hdr[i] = A.far[base + i].hdr;
+        for (int i = threadIdx.x; i < kGM * cnt; i += blockDim.x) s_mom[i / kGM * kMF4 + i % kGM] = gmom[base * kGM + i];
+        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {  // (-, tier a, tier b, FP64) squared radii
+            const float4 f = A.fe[base + i].hdr;
+            s_hdr[i] = L == 1 ? A.far[base + i].hdr : make_float4(0.f, f.x, f.y, f.z);
+        }
         for (int i = threadIdx.x; i < cnt * np2; i += blockDim.x) {
             const int jj = i / np2, k = min(i - jj * np2, nimg - 1);
             const float4 h = A.tau[2 * ((base + jj) * nimg + k)], l = A.tau[2 * ((base + jj) * nimg + k) + 1];
-            float* d = s_tau + jj * 6 * np2 + (i - jj * np2);
+            float* d = s_tau + jj * ts + (i - jj * np2);
             d[0] = -h.x, d[np2] = -h.y, d[2 * np2] = -h.z;
             d[3 * np2] = -l.x, d[4 * np2] = -l.y, d[5 * np2] = -l.z;
         }
         __syncthreads();
-        for (int jj = 0; jj < cnt; ++jj) {
-            const FillEl& F = s_fe[jj];
-            const int64_t j = base + jj;
-            const float4 hdr = s_hdr[jj];
-            // squared distance from which the moments are taken; never inside the near radius, which
-            // the two classifications of a pair (here and in the near kernel) round differently
-            const float mom2 = fmaxf(F.hdr.x * (float)(kMomRatio * kMomRatio / (kFillRatioA * kFillRatioA)),
-                                     hdr.w * 1.0001f);
-            float dh[3], dl[3];
-            df_sub(ph[0], pl[0], F.ch.x, F.cl.x, dh[0], dl[0]);
-            df_sub(ph[1], pl[1], F.ch.y, F.cl.y, dh[1], dl[1]);
-            df_sub(ph[2], pl[2], F.ch.z, F.cl.z, dh[2], dl[2]);
-            float x0h, x0l, y0h, y0l, z0h, z0l;
-            df_dot3(dh, dl, F.exh, F.exl, x0h, x0l);
-            df_dot3(dh, dl, F.eyh, F.eyl, y0h, y0l);
-            df_dot3(dh, dl, F.ezh, F.ezl, z0h, z0l);
-            MomSum2 S{};
-            NearerSum nr{};
-            bool any_nearer = false;
-            const float* tau = s_tau + jj * 6 * np2;
-            uint32_t nearer = 0;  // images of the group of 32 at hand whose pair is not taken by moments
-            for (int k = 0; k < np2; k += 2) {
-                auto plane = [&](int q) { return *reinterpret_cast<const float2*>(tau + q * np2 + k); };
-                // X = X0 - tau, two floats
-                auto diff = [&](float ah, float al, int q, float2& h, float2& l) {
-                    float2 t;
-                    two_sum2(bc2(ah), plane(q), h, t);
-                    l = __fadd2_rn(t, __fadd2_rn(bc2(al), plane(q + 3)));
-                };
-                float2 xh, xl, yh, yl, zh, zl;
-                diff(x0h, x0l, 0, xh, xl);
-                diff(y0h, y0l, 1, yh, yl);
-                diff(z0h, z0l, 2, zh, zl);
-                const float2 m1 = bc2(-1.f);
-                float2 px = __fmul2_rn(xh, xh), py = __fmul2_rn(yh, yh), pz = __fmul2_rn(zh, zh);
-                float2 ex = __ffma2_rn(xh, xh, make_float2(-px.x, -px.y)), ey = __ffma2_rn(yh, yh, make_float2(-py.x, -py.y)),
-                       ez = __ffma2_rn(zh, zh, make_float2(-pz.x, -pz.y));
-                ex = __ffma2_rn(__fadd2_rn(xh, xh), xl, ex);
-                ey = __ffma2_rn(__fadd2_rn(yh, yh), yl, ey);
-                ez = __ffma2_rn(__fadd2_rn(zh, zh), zl, ez);
-                float2 s, t1, t2, d2h;
-                two_sum2(px, py, s, t1);
-                two_sum2(s, pz, d2h, t2);
-                const float2 d2l = __fadd2_rn(__fadd2_rn(ex, ey), __fadd2_rn(ez, __fadd2_rn(t1, t2)));
-                const bool two = k + 1 < nimg;
-                const bool far0 = d2h.x >= mom2, far1 = two && d2h.y >= mom2;
-                mom_pair2<M != kEOnly, M != kPhiOnly>(s_mom + kMomF4 * jj, F.ch.w, xh, xl, yh, yl, zh, zl, d2h, d2l, far0,
-                                                      far1, S);
-                nearer |= ((far0 ? 0u : 1u) | (far1 || !two ? 0u : 2u)) << (k & 31);
-                if ((k & 31) == 30 || k + 2 >= np2) {
-                    for (uint32_t m = nearer; m; m &= m - 1) {
-                        const int kk = (k & ~31) + __ffs(m) - 1;
-                        acc_pair_nodes<M>(A, hdr, (int)F.hdr.w, j, nimg, kk, ph, pl, x0h, x0l, y0h, y0l, z0h, z0l, tau,
-                                          np2, nr);
+        const int per = 32 / te;  // points side by side (lanes)
+        const int steps = LANES ? (kWP + per - 1) / per : cnt;
+        for (int t = 0; t < steps; ++t) {
+            const int jj = LANES ? lane % te : t;
+            const int q = t * per + lane / te;  // LANES: the point of the warp's kWP
+            bool valid = true;
+            if constexpr (LANES) {
+                const int64_t i = i0 + w * kWP + q;
+                valid = jj < cnt && q < kWP && i < count;
+                if (valid) load_point_2f(pts, list[i], true, ph[0], ph[1], ph[2], pl[0], pl[1], pl[2]);
+            }
+            double s = 0.0;
+            ElemSum v{0.0, 0.0, 0.0, 0.0};
+            if (valid) {
+                s = A.sigma[base + jj];
+                v = acc_element<L, M>(A, nimg, np2, base + jj, s_fe[jj], s_mom + kMF4 * jj, s_hdr[jj],
+                                      s_tau + jj * ts, ph, pl);
+            }
+            if constexpr (!LANES) {
+                if constexpr (M != kEOnly) {
+                    acc.phi = fma(s, v.phi, acc.phi);
+                    if (L == 1)
+                        bphi = fmaf(fabsf((float)s), fabsf((float)v.phi), bphi);
+                    else
+                        acc.bphi = fma(fabs(s), fabs(v.phi), acc.bphi);
+                }
+                if constexpr (M != kPhiOnly) {
+                    acc.x = fma(s, v.x, acc.x);
+                    acc.y = fma(s, v.y, acc.y);
+                    acc.z = fma(s, v.z, acc.z);
+                    if (L == 1)
+                        bE = fmaf(fabsf((float)s), fabsf((float)v.x) + fabsf((float)v.y) + fabsf((float)v.z), bE);
+                    else
+                        acc.bE = fma(fabs(s), fabs(v.x) + fabs(v.y) + fabs(v.z), acc.bE);
+                }
+                continue;
+            }
+            LaneScratch::Val& o = scr->val[w][lane];
+            o.d[0] = s, o.d[1] = v.phi, o.d[2] = v.x, o.d[3] = v.y, o.d[4] = v.z;
+            if (L == 1) {
+                o.f[0] = fabsf((float)s), o.f[1] = fabsf((float)v.phi);
+                o.f[2] = fabsf((float)v.x) + fabsf((float)v.y) + fabsf((float)v.z);
+            } else {
+                o.a[0] = fabs(v.phi), o.a[1] = fabs(v.x) + fabs(v.y) + fabs(v.z);
+            }
+            __syncwarp();
+            // chain `which` (0 to 5) of a point by one lane, in the order of the elements
+            const int m = min(per, kWP - t * per);
+            for (int c = lane; c < 6 * m; c += 32) {
+                const int qq = c / 6, which = c - 6 * qq;
+                const LaneScratch::Val* r = scr->val[w] + qq * te;
+                double& dst = scr->out[w * kWP + t * per + qq][which];
+                double x = dst;
+                float y = (float)x;
+                const bool scale = which >= 4;
+                for (int e = 0; e < cnt; ++e) {
+                    if (L == 1) {
+                        x = fma(r[e].d[0], r[e].d[scale ? 1 : 1 + which], x);
+                        y = fmaf(r[e].f[0], r[e].f[scale ? which - 3 : 1], y);
+                    } else {
+                        x = fma(scale ? fabs(r[e].d[0]) : r[e].d[0], scale ? r[e].a[which - 4] : r[e].d[1 + which], x);
                     }
-                    any_nearer = any_nearer || nearer;
-                    nearer = 0;
                 }
+                dst = L == 1 && scale ? (double)y : x;
             }
-            // element j: A x (sum over the images) + the other terms as two floats, then FP64:
-            // rotated to the global frame and weighted by sigma_j.  A conversion takes the FP64 pipe
-            // like an addition does, so each quantity crosses over once, as two values; the
-            // error scales stay in FP32.
-            const double s = A.sigma[j];
-            const float4 tail = s_mom[kMomF4 * jj + kMomF4 - 1];
-            // sign: -1 where the high parts are kept negated; unit: what c is kept over
-            auto total = [&](float sign, float unit, const float2& h, const float2& l, const float2& c, float& oh, float& ol) {
-                float sh, t, p, e;
-                two_sum(h.x, h.y, sh, t);
-                sh *= sign;
-                const float sl = __fmaf_rn(sign, t, __fadd_rn(l.x, l.y));
-                two_prod(sh, tail.z, p, e);
-                e = __fmaf_rn(sh, tail.w, __fmaf_rn(sl, tail.z, e));
-                oh = p;
-                ol = __fmaf_rn(__fadd_rn(c.x, c.y), unit, e);
-            };
-            const float rho = F.ch.w;
-            if constexpr (M != kEOnly) {
-                float h, l;
-                total(1.f, rho * rho, S.ph, S.pl, S.fc, h, l);
-                double fphi = (double)h + (double)l;
-                if (any_nearer) fphi += (double)nr.ph + (double)nr.pl;
-                acc.phi = fma(s, fphi, acc.phi);
-                bphi = fmaf(fabsf((float)s), fabsf((float)fphi), bphi);
-            }
-            if constexpr (M != kPhiOnly) {
-                float h, l;
-                total(-1.f, rho, S.xh, S.xl, S.ex, h, l);
-                double lx = (double)h + (double)l;
-                total(-1.f, rho, S.yh, S.yl, S.ey, h, l);
-                double ly = (double)h + (double)l;
-                total(-1.f, rho, S.zh, S.zl, S.ez, h, l);
-                double lz = (double)h + (double)l;
-                if (any_nearer) {
-                    lx += (double)nr.xh + (double)nr.xl;
-                    ly += (double)nr.yh + (double)nr.yl;
-                    lz += (double)nr.zh + (double)nr.zl;
-                }
-                const Elem& e = A.el[j];
-                const double gx = fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0]));
-                const double gy = fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1]));
-                const double gz = fma(lx, e.ex[2], fma(ly, e.ey[2], lz * e.ez[2]));
-                acc.x = fma(s, gx, acc.x);
-                acc.y = fma(s, gy, acc.y);
-                acc.z = fma(s, gz, acc.z);
-                bE = fmaf(fabsf((float)s), fabsf((float)gx) + fabsf((float)gy) + fabsf((float)gz), bE);
-            }
+            __syncwarp();
         }
     }
-    acc.bphi = (double)bphi;
-    acc.bE = (double)bE;
-    return acc;
-}
-
-// Raw sums (before ke) of the far pairs of one point over the elements [e0, e1) at level 2,
-// with the error scales, of phi and E (M = kBoth), phi only or E only (the other sums stay
-// 0); all threads of the block take part (tiles).
-template <int M>
-__device__ __forceinline__ Sum6 acc_range2(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
-                                          const float (&pl)[3], int64_t e0, int64_t e1) {
-    constexpr int kStaged = 4 * kFillPairsA;
-    FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
-    float4* s_na = sm + 9 * te;
-    float4* s_tau = s_na + kStaged * te;
-    float4* s_c = s_tau + 2 * nimg * te;
-    Sum6 acc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t base = e0; base < e1; base += te) {
-        const int cnt = (int)min((int64_t)te, e1 - base);
-        __syncthreads();
-        {
-            const float4* src = reinterpret_cast<const float4*>(A.fe + base);
-            float4* dst = reinterpret_cast<float4*>(s_fe);
-            for (int i = threadIdx.x; i < 9 * cnt; i += blockDim.x) dst[i] = src[i];
-        }
-        for (int e = threadIdx.x; e < cnt * kStaged; e += blockDim.x) {
-            const int jj = e / kStaged, q = e - jj * kStaged;
-            s_na[e] = A.nodes[(base + jj) * kFillNodeRec + q];
-        }
-        for (int i = threadIdx.x; i < 2 * cnt * nimg; i += blockDim.x) {
-            s_tau[i] = A.tau[2 * base * nimg + i];
-            s_c[i] = A.cjk[2 * base * nimg + i];
-        }
-        __syncthreads();
-        for (int jj = 0; jj < cnt; ++jj) {
-            const FillEl& F = s_fe[jj];
-            const int64_t j = base + jj;
-            // squared tier radii, largest first, and the nearest (FP64) radius
-            const float4 hdr = F.hdr;
-            const float near2 = hdr.z;
-            const int na = (int)F.hdr.w;
-            float dh[3], dl[3];
-            df_sub(ph[0], pl[0], F.ch.x, F.cl.x, dh[0], dl[0]);
-            df_sub(ph[1], pl[1], F.ch.y, F.cl.y, dh[1], dl[1]);
-            df_sub(ph[2], pl[2], F.ch.z, F.cl.z, dh[2], dl[2]);
-            float x0h, x0l, y0h, y0l, z0h, z0l;
-            df_dot3(dh, dl, F.exh, F.exl, x0h, x0l);
-            df_dot3(dh, dl, F.eyh, F.eyl, y0h, y0l);
-            df_dot3(dh, dl, F.ezh, F.ezl, z0h, z0l);
-            float2 fph = bc2(0.f), fnph = bc2(0.f);
-            float exh = 0.f, exl = 0.f, eyh = 0.f, eyl = 0.f, ezh = 0.f, ezl = 0.f;
-            for (int k = 0; k < nimg; ++k) {
-                float dx, dy, dz;
-                const float d2 = pair_d2(ph[0], ph[1], ph[2], pl[0], pl[1], pl[2], s_c[2 * (jj * nimg + k)],
-                                         s_c[2 * (jj * nimg + k) + 1], dx, dy, dz);
-                if (!(d2 >= near2)) continue;  // near pair: the level's FP64 kernel
-                const float4 th = s_tau[2 * (jj * nimg + k)], tl = s_tau[2 * (jj * nimg + k) + 1];
-                float xh, xl, yh, yl, zh, zl, d2h, d2l;
-                df_sub(x0h, x0l, th.x, tl.x, xh, xl);
-                df_sub(y0h, y0l, th.y, tl.y, yh, yl);
-                df_sub(z0h, z0l, th.z, tl.z, zh, zl);
-                df_norm2(xh, xl, yh, yl, zh, zl, d2h, d2l);
-                PairDF2 P;
-                P.xh = bc2(xh), P.nxh = bc2(-xh), P.xl = bc2(xl);
-                P.zh = bc2(zh), P.nzh = bc2(-zh), P.zl = bc2(zl);
-                P.d2h = bc2(d2h), P.d2l = bc2(d2l);
-                const float4* nd;
-                int np;
-                if (d2 >= hdr.x) {  // the staged set
-                    nd = s_na + jj * kStaged;
-                    np = na;
-                } else if (d2 >= hdr.y) {
-                    nd = A.nodes + j * kFillNodeRec + kFillOffB;
-                    np = kFillPairsB;
-                } else {
-                    nd = A.nodes + j * kFillNodeRec + kFillOffC;
-                    np = kFillPairsC;
-                }
-                PairSums2 S{bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
-                nodes_acc2<M>(nd, np, P, fph, fnph, S);
-                if constexpr (M == kPhiOnly) continue;
-                float s0h, s0l, sxh, sxl, szh, szl;
-                lanes_to_df(S.s0, S.ns0, 1.f, s0h, s0l);
-                lanes_to_df(S.sx, S.nsx, 0.5f, sxh, sxl);
-                lanes_to_df(S.sz, S.nsz, 0.5f, szh, szl);
-                df_fma_acc(xh, xl, s0h, s0l, sxh, sxl, exh, exl);
-                df_fma_acc(yh, yl, s0h, s0l, 0.f, 0.f, eyh, eyl);
-                df_fma_acc(zh, zl, s0h, s0l, szh, szl, ezh, ezl);
-            }
-            // element j: image sums in FP64, rotated to the global frame, weighted by sigma_j
-            const double s = A.sigma[j];
-            if constexpr (M != kEOnly) {
-                const double fphi = ((double)fph.x - (double)fnph.x) + ((double)fph.y - (double)fnph.y);
-                acc.phi = fma(s, fphi, acc.phi);
-                acc.bphi = fma(fabs(s), fabs(fphi), acc.bphi);
-            }
-            if constexpr (M != kPhiOnly) {
-                const double lx = (double)exh + (double)exl, ly = (double)eyh + (double)eyl,
-                             lz = (double)ezh + (double)ezl;
-                const Elem& e = A.el[j];
-                const double gx = fma(lx, e.ex[0], fma(ly, e.ey[0], lz * e.ez[0]));
-                const double gy = fma(lx, e.ex[1], fma(ly, e.ey[1], lz * e.ez[1]));
-                const double gz = fma(lx, e.ex[2], fma(ly, e.ey[2], lz * e.ez[2]));
-                acc.x = fma(s, gx, acc.x);
-                acc.y = fma(s, gy, acc.y);
-                acc.z = fma(s, gz, acc.z);
-                acc.bE = fma(fabs(s), fabs(gx) + fabs(gy) + fabs(gz), acc.bE);
-            }
-        }
-    }
+    if (L == 1) acc.bphi = (double)bphi, acc.bE = (double)bE;
     return acc;
 }
 
@@ -495,17 +519,15 @@ __device__ __forceinline__ void store_acc(int64_t p, const Sum6& tot, double* __
 
 // The far sums of one point over whole pieces of the summation tree.
 template <int L, int M>
-__device__ __forceinline__ Sum6 acc_sum(const AccView& A, int nimg, int te, float4* sm, const float (&ph)[3],
-                                        const float (&pl)[3], int64_t e0, int64_t e1) {
+__device__ __forceinline__ Sum6 acc_sum(const AccView& A, int nimg, int te, float4* sm, float (&ph)[3],
+                                        float (&pl)[3], int64_t e0, int64_t e1) {
     Sum6 tot{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int64_t c0 = e0; c0 < e1; c0 += kChunkEl) {
         const int64_t c1 = min(c0 + (int64_t)kChunkEl, e1);
         Sum6 ch{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         for (int64_t l = c0; l < c1; l += kLeafEl)
-            if constexpr (L == 1)
-                add_sum(ch, acc_range1<M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
-            else
-                add_sum(ch, acc_range2<M>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1)));
+            add_sum(ch, acc_range<L, M, false>(A, nimg, te, sm, ph, pl, l, min(l + (int64_t)kLeafEl, c1), nullptr,
+                                               nullptr, 0, 0));
         add_sum(tot, ch);
     }
     return tot;
@@ -525,6 +547,7 @@ __global__ void __launch_bounds__(kAT, kATBlocks)
     extern __shared__ float4 sm[];
     const int64_t count = *n_list;
     const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
+    if (lane_path(plan, count, gb)) return;
     const int64_t units = plan.Gm + plan.R * plan.np;
     for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
         const SplitUnit t = split_unit(plan, u, A.n_el);
@@ -539,6 +562,34 @@ __global__ void __launch_bounds__(kAT, kATBlocks)
             store_acc<L, M>(p, tot, phi, E, err, bound);
         else
             part[(t.r * kAT + threadIdx.x) * plan.np + t.piece] = tot;
+    }
+}
+
+// The same for short lists (lane_path): a unit is kLP points of one leaf, a thread takes (point, element)
+// pairs, and the leaf's sums go to the same partial sums.
+template <int L, int M>
+__global__ void __launch_bounds__(kAT, 4)
+    k_eval_acc_lanes(const AccView A, int nimg, int te, const double* __restrict__ pts,
+                     const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
+                     Sum6* __restrict__ part) {
+    extern __shared__ float4 sm[];
+    const int64_t count = *n_list;
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
+    if (!lane_path(plan, count, gb)) return;
+    const int64_t lg = (count + kLP - 1) / kLP;
+    const LaneScratch* scr = reinterpret_cast<LaneScratch*>(sm + acc_tile_f4(L, te, nimg));
+    constexpr int kWP = kLP / (kAT / 32);
+    const int w = threadIdx.x >> 5;
+    for (int64_t u = blockIdx.x; u < lg * plan.np; u += gridDim.x) {
+        const int64_t piece = u / lg, i0 = (u - piece * lg) * kLP;  // consecutive units: the same leaf
+        const int64_t e0 = piece * kLeafEl;
+        float ph[3], pl[3];
+        acc_range<L, M, true>(A, nimg, te, sm, ph, pl, e0, min(e0 + (int64_t)kLeafEl, A.n_el), pts, list, i0, count);
+        for (int c = threadIdx.x & 31; c < 6 * kWP; c += 32) {
+            const int64_t q = i0 + w * kWP + c / 6;
+            if (q < count) reinterpret_cast<double*>(part + q * plan.np + piece)[c % 6] = scr->out[w * kWP + c / 6][c % 6];
+        }
+        __syncwarp();
     }
 }
 
@@ -634,17 +685,26 @@ template <int L, int M>
 cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* pts, int64_t npts, double* phi,
                          double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list, int sms,
                          Sum6* part, cudaStream_t s) {
-    // element tile: a power of two (divides the chunk width), at most 16, within ~40 KB
-    int te = L == 1 ? kLeafEl : 16;
+    // element tile: a power of two (divides the leaf), within ~40 KB
+    int te = kLeafEl;
     while (te > 1 && acc_tile_f4(L, te, img.n) * (int)sizeof(float4) > 40 * 1024) te /= 2;
-    const size_t smem = (size_t)acc_tile_f4(L, te, img.n) * sizeof(float4);
+    const size_t smem = (size_t)acc_tile_f4(L, te, img.n) * sizeof(float4), lane_smem = smem + sizeof(LaneScratch);
     const int64_t gb = kATBlocks * (int64_t)sms, want = (npts + kAT - 1) / kAT;
-    const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
-    cudaError_t e =
-        cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e;
+    // the list's length is known on the device: both kernels are launched unless even the whole input is short
+    if (!lane_path(split_plan(want, gb, A.n_el), npts, gb)) {
+        e = cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
+        k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, gb, part,
+                                                                            phi, E, err, bound);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    e = cudaFuncSetAttribute(k_eval_acc_lanes<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lane_smem);
     if (e != cudaSuccess) return e;
-    k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, gb, part, phi,
-                                                                        E, err, bound);
+    k_eval_acc_lanes<L, M><<<(unsigned)std::min<int64_t>(4 * (int64_t)sms, split_count(npts, kLP) * split_count(A.n_el, kLeafEl)),
+                             kAT, lane_smem, s>>>(A, img.n, te, pts, list, n_list, gb, part);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t left = std::min(want, 2 * gb) * kAT;  // points of the left-over groups, at most

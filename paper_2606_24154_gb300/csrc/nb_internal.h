@@ -169,7 +169,8 @@ struct AccView {
     const FarNodes* far;
     const FillEl* fe;
     const float4* nodes;
-    const float4* mom;  // elem_moments_bytes: planar moments (ElemMom of twofloat.cuh)
+    const float4* mom;   // elem_moments_bytes: planar moments (ElemMom of twofloat.cuh)
+    const float4* mom2;  // fill_moments_bytes: those of the fill (FillMom)
     const float4* tau;
     const float4* cjk;
     const double* sigma;

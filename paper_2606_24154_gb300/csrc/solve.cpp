@@ -391,6 +391,7 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
             A.fe = c->d_fill_el.as<FillEl>();
             A.nodes = c->d_fill_nodes.as<float4>();
             A.mom = c->d_fill_mom.as<float4>();
+            A.mom2 = c->d_fill_phimom.as<float4>();
             A.tau = c->d_fill_tau.as<float4>();
             A.cjk = c->d_cjk.as<float4>();
             A.sigma = c->d_sigma.as<double>();

@@ -383,6 +383,47 @@ __device__ __forceinline__ void fill_mom_phi2(const float4* __restrict__ mom, co
     Sl = __fadd2_rn(Sl, __ffma2_rn(y0, F, lo));
 }
 
+// F, G, F_alpha, F_beta by Horner's rule (qq = q^2)
+__device__ __forceinline__ void fill_mom_poly2(const float4* __restrict__ mom, float2 al1, float2 be1, float2 q,
+                                               float2 qq, float2& F, float2& G, float2& Fa, float2& Fb) {
+    auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
+    F = G = Fa = Fb = bc2(0.f);
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        float2 r = bc2(0.f), ra = bc2(0.f), rg = bc2(0.f);
+#pragma unroll
+        for (int i = 6 - j; i >= 0; --i) {
+            const int o = 8 + fill_mom_off(i, j), k = i + j;
+            const float f0 = (float)(1 + 2 * (k + fill_mom_m0(k)));
+            float2 c = con(o), g;
+            if (fill_mom_terms(k) == 2) {
+                const float2 c1 = __fmul2_rn(con(o + 1), q);
+                c = __fadd2_rn(c, c1);
+                g = __ffma2_rn(c1, bc2(2.f), __fmul2_rn(c, bc2(f0)));
+            } else {
+                g = __fmul2_rn(c, bc2(f0));
+            }
+            if (fill_mom_m0(k) == 1) c = __fmul2_rn(c, q), g = __fmul2_rn(g, q);
+            if (fill_mom_m0(k) == 2) c = __fmul2_rn(c, qq), g = __fmul2_rn(g, qq);
+            if (i == 6 - j) {
+                r = c, rg = g;
+            } else {
+                ra = i == 5 - j ? r : __ffma2_rn(ra, al1, r);
+                r = __ffma2_rn(r, al1, c);
+                rg = __ffma2_rn(rg, al1, g);
+            }
+        }
+        if (j == 6) {
+            F = r, G = rg;
+        } else {
+            Fb = j == 5 ? F : __ffma2_rn(Fb, be1, F);
+            F = __ffma2_rn(F, be1, r);
+            G = __ffma2_rn(G, be1, rg);
+            Fa = j == 5 ? ra : __ffma2_rn(Fa, be1, ra);
+        }
+    }
+}
+
 // (Sh, Sl) += n . E' / A of the lanes that are far; (yh, yl) = the targets' Y
 __device__ __forceinline__ void fill_mom_field2(const float4* __restrict__ mom, const FillRow& R,
                                                 const FillPair2& P, float2 yh, float2 yl, bool far0, bool far1,
@@ -424,41 +465,8 @@ __device__ __forceinline__ void fill_mom_field2(const float4* __restrict__ mom, 
     const float s = mom[kFillMomF4 - 1].z;
     const float2 pr = __fmul2_rn(a, bc2(s)), qq = __fmul2_rn(q, q);
     const float2 al1 = __fmul2_rn(P.xh, pr), be1 = __fmul2_rn(P.zh, pr);
-    float2 F = bc2(0.f), G = bc2(0.f), Fa = bc2(0.f), Fb = bc2(0.f);
-#pragma unroll
-    for (int j = 6; j >= 0; --j) {
-        float2 r = bc2(0.f), ra = bc2(0.f), rg = bc2(0.f);
-#pragma unroll
-        for (int i = 6 - j; i >= 0; --i) {
-            const int o = 8 + fill_mom_off(i, j), k = i + j;
-            const float f0 = (float)(1 + 2 * (k + fill_mom_m0(k)));
-            float2 c = con(o), g;
-            if (fill_mom_terms(k) == 2) {
-                const float2 c1 = __fmul2_rn(con(o + 1), q);
-                c = __fadd2_rn(c, c1);
-                g = __ffma2_rn(c1, bc2(2.f), __fmul2_rn(c, bc2(f0)));
-            } else {
-                g = __fmul2_rn(c, bc2(f0));
-            }
-            if (fill_mom_m0(k) == 1) c = __fmul2_rn(c, q), g = __fmul2_rn(g, q);
-            if (fill_mom_m0(k) == 2) c = __fmul2_rn(c, qq), g = __fmul2_rn(g, qq);
-            if (i == 6 - j) {
-                r = c, rg = g;
-            } else {
-                ra = i == 5 - j ? r : __ffma2_rn(ra, al1, r);
-                r = __ffma2_rn(r, al1, c);
-                rg = __ffma2_rn(rg, al1, g);
-            }
-        }
-        if (j == 6) {
-            F = r, G = rg;
-        } else {
-            Fb = j == 5 ? F : __ffma2_rn(Fb, be1, F);
-            F = __ffma2_rn(F, be1, r);
-            G = __ffma2_rn(G, be1, rg);
-            Fa = j == 5 ? ra : __ffma2_rn(Fa, be1, ra);
-        }
-    }
+    float2 F, G, Fa, Fb;
+    fill_mom_poly2(mom, al1, be1, q, qq, F, G, Fa, Fb);
     // T = N + 5 W N - q H + FP32 part, then y p T
     float2 Th, Tl;
     two_sum2(Nh, W, Th, e1);
@@ -472,6 +480,69 @@ __device__ __forceinline__ void fill_mom_field2(const float4* __restrict__ mom, 
     float2 u;
     two_sum2(Sh, Th, Sh, u);
     Sl = __fadd2_rn(Sl, __fadd2_rn(u, Tl));
+}
+
+// Sums of fill_mom_point2: phi / A and E (local frame) / A, both lanes, two floats each.
+struct PointSum2 {
+    float2 ph, pl, xh, xl, yh, yl, zh, zl;
+};
+// S += Phi' / A and E' / A (the vector) of the lanes that are far: as fill_mom_phi2, and with
+// T = 5 W + 2 q w + G
+//   E'_x / A = y p (X (1 + T) - q (2 a1 X + a2 Z) - s F_alpha),   E'_y / A = y p Y (1 + T),
+// E'_z like E'_x.  About 400 FP32 lane operations.
+__device__ __forceinline__ void fill_mom_point2(const float4* __restrict__ mom, const FillPair2& P, float2 yh, float2 yl,
+                                                bool far0, bool far1, PointSum2& S) {
+    const float2 m1 = bc2(-1.f);
+    auto con = [&](int i) { return lane2(mom[i >> 1], i & 1); };
+    float2 y0, ye, a, al, q, ql, W, wl;
+    fill_mom_head2(mom, P, far0, far1, y0, ye, a, al, q, ql, W, wl);
+    // F, G, F_alpha, F_beta
+    const float s = mom[kFillMomF4 - 1].z;
+    const float2 pr = __fmul2_rn(a, bc2(s)), qq = __fmul2_rn(q, q);
+    const float2 al1 = __fmul2_rn(P.xh, pr), be1 = __fmul2_rn(P.zh, pr);
+    float2 F, G, Fa, Fb;
+    fill_mom_poly2(mom, al1, be1, q, qq, F, G, Fa, Fb);
+    float2 t, u;
+    {  // y (1 + W + F)
+        float2 vh = W, vl = wl;
+        df_times2(y0, ye, vh, vl);
+        two_sum2(S.ph, y0, S.ph, t);
+        two_sum2(S.ph, vh, S.ph, u);
+        vl = __fadd2_rn(vl, __fadd2_rn(ye, __fadd2_rn(t, u)));
+        S.pl = __fadd2_rn(S.pl, __ffma2_rn(y0, F, vl));
+    }
+    // T
+    float2 ch = q, cl = ql, Th, Tl;
+    df_times2(__fmul2_rn(con(6), bc2(-2.f)), __fmul2_rn(con(7), bc2(-2.f)), ch, cl);
+    df_times2(bc2(5.f), bc2(0.f), W, wl);
+    two_sum2(W, ch, Th, t);
+    Tl = __fadd2_rn(__fadd2_rn(wl, cl), __fadd2_rn(t, G));
+    df_times2(y0, ye, a, al);  // y p
+    // component: (c (1 + T) - q g - s f) y p, g = gx X + gz Z (0 without in_plane)
+    auto component = [&](float2 h, float2 l, bool in_plane, int ix, float fx, int iz, float fz, float2 f, float2& Sh,
+                         float2& Sl) {
+        float2 vh = Th, vl = Tl, rh, e, g;
+        df_times2(h, l, vh, vl);
+        two_sum2(h, vh, rh, e);
+        vl = __fadd2_rn(__fadd2_rn(l, vl), e);
+        if (in_plane) {
+            float2 gh = __fmul2_rn(con(ix), bc2(fx)), gl = __fmul2_rn(con(ix + 1), bc2(fx));
+            float2 kh = __fmul2_rn(con(iz), bc2(fz)), kl = __fmul2_rn(con(iz + 1), bc2(fz));
+            df_times2(P.xh, P.xl, gh, gl);
+            df_times2(P.zh, P.zl, kh, kl);
+            two_sum2(gh, kh, g, e);
+            gl = __fadd2_rn(__fadd2_rn(gl, kl), e);
+            df_times2(q, ql, g, gl);
+            two_sum2(rh, __fmul2_rn(g, m1), rh, e);
+            vl = __fadd2_rn(__ffma2_rn(gl, m1, vl), __ffma2_rn(f, bc2(-s), e));
+        }
+        df_times2(a, al, rh, vl);
+        two_sum2(Sh, rh, Sh, e);
+        Sl = __fadd2_rn(Sl, __fadd2_rn(vl, e));
+    };
+    component(P.xh, P.xl, true, 0, 2.f, 2, 1.f, Fa, S.xh, S.xl);
+    component(yh, yl, false, 0, 0.f, 0, 0.f, Fa, S.yh, S.yl);
+    component(P.zh, P.zl, true, 2, 1.f, 4, 2.f, Fb, S.zh, S.zl);
 }
 
 }  // namespace nb
