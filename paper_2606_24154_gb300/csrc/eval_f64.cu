@@ -17,7 +17,7 @@ namespace nb {
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kFillCols = 64;
+constexpr int kFillBlocks = 3;  // resident fill blocks per SM
 constexpr int kF64Blocks = 3;  // resident evaluation blocks per SM (168 registers a thread)
 
 // Block u takes unit u of `plan`: whole groups of points, then element pieces of the left-over
@@ -58,8 +58,9 @@ __global__ void __launch_bounds__(256) k_f64_reduce(const double* __restrict__ p
 // 0.619e12 a second).  Conductor rows form the potential only and interface rows the
 // field only; the row's normal is rotated into the column's frame once per (row, column), so that
 // an image of an interface row adds three products.
-__global__ void __launch_bounds__(kThreads, 3) k_fill_f64(const Elem* __restrict__ el, const double* __restrict__ diag_in,
-                                                       int64_t n, const ImageTable img, double* __restrict__ K) {
+__global__ void __launch_bounds__(kThreads, kFillBlocks) k_fill_f64(const Elem* __restrict__ el, const double* __restrict__ diag_in,
+                                                       int64_t n, const ImageTable img, int cols,
+                                                       double* __restrict__ K) {
     __shared__ Tile64 s_t;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = i < n;
@@ -77,8 +78,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_fill_f64(const Elem* __restrict
         diag = diag_in[i];  // (eps_a + eps_b) / (2 eps0 (eps_b - eps_a)) on interface rows, else 0
     }
     const double ke = 1.0 / (4.0 * kPi * kEps0);
-    const int64_t j0 = (int64_t)blockIdx.y * kFillCols;
-    const int64_t j1 = min(n, j0 + kFillCols);
+    const int64_t j0 = (int64_t)blockIdx.y * cols;
+    const int64_t j1 = min(n, j0 + cols);
     for (int64_t base = j0; base < j1; base += kTile64) {
         const int cnt = (int)min((int64_t)kTile64, j1 - base);
         load_tile64(s_t, el, base, cnt, img);
@@ -149,11 +150,24 @@ cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, c
     return cudaGetLastError();
 }
 
+cudaError_t fill_cols(int64_t n, int rows, int per_sm, int* cols) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    *cols = 64;
+    while (*cols > 2 && (n + rows - 1) / rows * ((n + *cols - 1) / *cols) < 2 * (int64_t)per_sm * sms) *cols /= 2;
+    return cudaSuccess;
+}
+
 cudaError_t launch_fill_f64(const Elem* el, const double* diag, int64_t n, const ImageTable& img, double* K,
                             cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    dim3 grid((unsigned)((n + kThreads - 1) / kThreads), (unsigned)((n + kFillCols - 1) / kFillCols));
-    k_fill_f64<<<grid, kThreads, 0, s>>>(el, diag, n, img, K);
+    int cols = 0;
+    const cudaError_t e = fill_cols(n, kThreads, kFillBlocks, &cols);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)((n + kThreads - 1) / kThreads), (unsigned)((n + cols - 1) / cols));
+    k_fill_f64<<<grid, kThreads, 0, s>>>(el, diag, n, img, cols, K);
     return cudaGetLastError();
 }
 

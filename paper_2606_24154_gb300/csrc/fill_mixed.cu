@@ -36,7 +36,7 @@ namespace nb {
 namespace {
 
 constexpr int kFT = 128;       // threads per block (one row each)
-constexpr int kFillCols = 64;  // columns per block (grid.y)
+constexpr int kFillBlocks = 4;  // resident far blocks per SM
 
 // Phi' nodes: S += w / r (sh = hi sum, nl = -lo sum), two nodes per step
 __device__ __forceinline__ void nodes_phi2(const float4* __restrict__ nd, int pairs, const PairDF2& P, float2& sh,
@@ -146,13 +146,13 @@ __device__ __noinline__ void fill_pair_nodes(const float4* __restrict__ nd, cons
     nodes_nE2(nd + (b ? kFillOffB : kFillOffC), b ? kFillPairsB : kFillPairsC, P, Nn, sh, snl);
 }
 
-// Far pairs of a block's 128 rows and kFillCols columns: the moments from 32 radii on (interface rows:
+// Far pairs of a block's 128 rows and `cols` columns: the moments from 32 radii on (interface rows:
 // 52), nodes nearer.  9,996 elements x 25 copies (18 % interface rows) took 71 ms with nodes
 // for every pair and 35 ms so; bound by the FP32 pipe.
-__global__ void __launch_bounds__(kFT, 4)
+__global__ void __launch_bounds__(kFT, kFillBlocks)
     k_fill_far(const FillEl* __restrict__ fe, const float4* __restrict__ nodes, const float4* __restrict__ mom,
                const float4* __restrict__ tau, const float4* __restrict__ cjk, const double* __restrict__ diag_in,
-               int64_t n, int nimg, int te, double* __restrict__ K) {
+               int64_t n, int nimg, int te, int cols, double* __restrict__ K) {
     extern __shared__ float4 sm[];
     FillEl* s_fe = reinterpret_cast<FillEl*>(sm);
     float4* s_mom = sm + 9 * te;
@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(kFT, 4)
         iface = diag != 0.0;  // interface rows carry the nonzero diagonal term
     }
     const double ke = 1.0 / (4.0 * kPi * kEps0);
-    const int64_t j0 = (int64_t)blockIdx.y * kFillCols;
-    const int64_t j1 = min(n, j0 + kFillCols);
+    const int64_t j0 = (int64_t)blockIdx.y * cols;
+    const int64_t j1 = min(n, j0 + cols);
     for (int64_t base = j0; base < j1; base += te) {
         const int cnt = (int)min((int64_t)te, j1 - base);
         __syncthreads();
@@ -406,8 +406,11 @@ cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* no
     const size_t smem = (size_t)fill_tile_f4(te, img.n) * sizeof(float4);
     cudaError_t e = cudaFuncSetAttribute(k_fill_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 g1((unsigned)((n + kFT - 1) / kFT), (unsigned)((n + kFillCols - 1) / kFillCols));
-    k_fill_far<<<g1, kFT, smem, s>>>(fe, nodes, mom, tau, cjk, diag, n, img.n, te, K);
+    int cols = 0;
+    e = fill_cols(n, kFT, kFillBlocks, &cols);
+    if (e != cudaSuccess) return e;
+    dim3 g1((unsigned)((n + kFT - 1) / kFT), (unsigned)((n + cols - 1) / cols));
+    k_fill_far<<<g1, kFT, smem, s>>>(fe, nodes, mom, tau, cjk, diag, n, img.n, te, cols, K);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_fill_near<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(el, fe, cjk, n, img, grid, cell_start, cell_items, K);
