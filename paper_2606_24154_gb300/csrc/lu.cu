@@ -12,6 +12,7 @@
 // A22 -= L21 U12 runs on the tensor cores in both precisions (lu_tc.cu, lu_tc64.cu).
 // Templated on the element type: double (FP64 solves) and float (mixed solves, the
 // FP64 iterative refinement lives in the caller).
+#include <cooperative_groups.h>
 #include <algorithm>
 #include <climits>
 #include <vector>
@@ -338,10 +339,16 @@ __device__ __forceinline__ void warp_best(long long& key, int& idx) {
     key = ((long long)mh << 32) | ml;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kCoopThreads, 1)
-    k_panel_coop(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
-                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch<T>* cs, unsigned int bar_base, long long limit) {
+// CL: the grid is one cluster of kPanelCluster CTAs.  The slots are pushed into every CTA's shared memory, the
+// rows are read from their holders' (distributed shared memory), and the cluster barrier, which needs no
+// bound, takes the place of the counter: 2.2 us a column in FP64 (up to 1,536 rows), 1.7 to 2.1 in FP32 (up to 4,096).
+constexpr int kPanelCluster = 16;
+
+template <typename T, bool CL>
+__device__ __forceinline__ void panel(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R,
+                                      int32_t* __restrict__ piv, int* __restrict__ info, int* __restrict__ tmo,
+                                      CoopScratch<T>* cs, unsigned int bar_base, long long limit) {
+    namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ld_acquire_i(&cs->err)) return;  // an earlier panel gave up: leave the matrix as it is
     const int w = (int)(k1 - k0);
@@ -351,6 +358,8 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
     __shared__ long long wk[2][kWarps];
     __shared__ int wi[2][kWarps];
     __shared__ int s_fail;
+    __shared__ CoopSlot c_slot[2][CL ? kPanelCluster : 1];  // CL: every CTA's slots, own candidate, own row j
+    __shared__ T c_cand[2][CL ? 64 : 1], c_srow[2][CL ? 64 : 1];
     const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int64_t rb0 = k0 + (int64_t)b * R;
     const int nr = (int)max((int64_t)0, min((int64_t)R, n - rb0));
@@ -404,12 +413,18 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         if (tid < 32) {
             const int mine = bidx != INT_MAX ? (int)(bidx - rb0) : -1;
             const bool own = j >= rb0 && j < rb0 + nr;
+            T* cand = CL ? c_cand[par] : cs->cand[par][b];
+            T* srow = CL ? c_srow[par] : cs->srow[par];
             for (int c = lane; c < w; c += 32) {
-                cs->cand[par][b][c] = mine >= 0 ? S[c * R + mine] : (T)0;
-                if (own) cs->srow[par][c] = S[c * R + (int)(j - rb0)];
+                cand[c] = mine >= 0 ? S[c * R + mine] : (T)0;
+                if (own) srow[c] = S[c * R + (int)(j - rb0)];
+            }
+            if constexpr (CL) {
+                if (lane < G)
+                    *cg::this_cluster().map_shared_rank(&c_slot[par][b], lane) = CoopSlot{best, bidx, 0};
             }
             __syncwarp();
-            if (lane == 0) {
+            if (!CL && lane == 0) {
                 __stcg(reinterpret_cast<int4*>(&cs->slot[par][b]),
                        make_int4((int)best, (int)(best >> 32), bidx, 0));
                 // the barrier: the release half publishes the warp's stores (cumulative over the
@@ -428,17 +443,23 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
                 }
             }
         }
-        __syncthreads();
+        if constexpr (CL)
+            cg::this_cluster().sync();
+        else
+            __syncthreads();
         // (c) every CTA's candidate
         best = -1;
         bidx = INT_MAX;
-        if (tid < G) {
+        if (CL && tid < G) {
+            best = c_slot[par][tid].key;
+            bidx = c_slot[par][tid].idx;
+        } else if (!CL && tid < G) {
             const int4 q = __ldcg(reinterpret_cast<const int4*>(&cs->slot[par][tid]));
             best = ((long long)q.y << 32) | (unsigned int)q.x;
             bidx = q.z;
         }
         block_best(1, best, bidx);
-        if (s_fail) {
+        if (!CL && s_fail) {
             if (tid == 0) {
                 atomicExch(&cs->err, 1);
                 atomicExch(tmo, 1);
@@ -449,10 +470,18 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         const bool any = (int64_t)bidx >= j && (int64_t)bidx < n;
         const int64_t p = any ? (int64_t)bidx : j;
         if (tid < w) {
-            const T v = __ldcg(any ? &cs->cand[par][(int)((p - k0) / R)][tid] : &cs->srow[par][tid]);
+            auto row_j = [&]() {
+                if constexpr (CL) return *cg::this_cluster().map_shared_rank(&c_srow[par][tid], (int)((j - k0) / R));
+                return __ldcg(&cs->srow[par][tid]);
+            };
+            auto row_p = [&]() {
+                if constexpr (CL) return *cg::this_cluster().map_shared_rank(&c_cand[par][tid], (int)((p - k0) / R));
+                return __ldcg(&cs->cand[par][(int)((p - k0) / R)][tid]);
+            };
+            const T v = any ? row_p() : row_j();
             prow[tid] = v;
             if (j >= rb0 && j < rb0 + nr) S[tid * R + (int)(j - rb0)] = v;
-            if (p != j && p >= rb0 && p < rb0 + nr) S[tid * R + (int)(p - rb0)] = __ldcg(&cs->srow[par][tid]);
+            if (p != j && p >= rb0 && p < rb0 + nr) S[tid * R + (int)(p - rb0)] = row_j();
             // a zero pivot leaves its column unscaled and skips its update, as in k_panel_col
             if (tid == jj) sinv[jj] = v != (T)0 ? (T)1 / v : (T)1;
         }
@@ -468,7 +497,25 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
         const T v = S[c * R + r];
         A[(rb0 + r) + (k0 + c) * n] = rb0 + r > k0 + c ? v * sinv[c] : v;
     }
+    if constexpr (CL) cg::this_cluster().sync();  // the others may still read this CTA's last rows
 }
+template <typename T>
+__global__ void __launch_bounds__(kCoopThreads, 1)
+    k_panel_coop(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
+                 int* __restrict__ info, int* __restrict__ tmo, CoopScratch<T>* cs, unsigned int bar_base,
+                 long long limit) {
+    panel<T, false>(A, n, k0, k1, R, piv, info, tmo, cs, bar_base, limit);
+}
+template <typename T>
+__global__ void __launch_bounds__(kCoopThreads, 1)
+    k_panel_cluster(T* __restrict__ A, int64_t n, int64_t k0, int64_t k1, int R, int32_t* __restrict__ piv,
+                    int* __restrict__ info, CoopScratch<T>* cs) {
+    panel<T, true>(A, n, k0, k1, R, piv, info, nullptr, cs, 0, 0);
+}
+// rows a CTA of the cluster takes at most: above, the update of one CTA's rows takes longer than the grid
+// barrier that the cluster saves
+template <typename T>
+constexpr int64_t kClusterRows = sizeof(T) == 8 ? 96 : 256;
 
 // Apply the row swaps of panel rows [k0, k1) to columns outside the panel.
 // The row swaps of panel rows [k0, k1) (LAPACK order: row r with piv[r]) composed into one
@@ -586,30 +633,36 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_trtri_unit_lower(const T* __
 // with Linv_i (nbk blocks of 64 x 64, ld 64) from k_trtri_unit_lower and L_ij read from A.
 // One CTA per kTrsmCols columns holds its tile of the block row in shared memory (all nbk
 // blocks), staging one 64 x 64 block of L (or Linv) at a time; thread t owns row t % 64 and
-// columns 8 (t / 64) .. + 7 of the current 64-row block.  Dynamic shared memory:
+// kTrsmPer columns of the current 64-row block.  Dynamic shared memory:
 // trsm_block_smem<T>(nbk).
-constexpr int kTrsmCols = 32;
+// FP64 takes 8 columns per CTA: 64 x 64 x 8 products already hold one SM's FP64 pipe for 8 us, and
+// 32 columns left most SMs idle (43 us a block row at n = 6145, 36 at 384; 8 columns: 23 and 10).
+template <typename T>
+constexpr int kTrsmPer = sizeof(T) == 8 ? 2 : 8;  // columns per thread
+template <typename T>
+constexpr int kTrsmCols = 4 * kTrsmPer<T>;
 
 template <typename T>
 __host__ __device__ constexpr size_t trsm_block_smem(int nbk) {
-    return sizeof(T) * ((size_t)64 * nbk * (kTrsmCols + 1) + (size_t)64 * 65);
+    return sizeof(T) * ((size_t)64 * nbk * (kTrsmCols<T> + 1) + (size_t)64 * 65);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_trsm_block(T* __restrict__ A, int64_t n, int64_t K0, int nbk,
                                                     const T* __restrict__ Linv, int64_t c0, int64_t c1) {
+    constexpr int kP = kTrsmPer<T>, kC = kTrsmCols<T>;
     extern __shared__ __align__(16) unsigned char trsm_blk_sm[];
-    T(*X)[kTrsmCols + 1] = reinterpret_cast<T(*)[kTrsmCols + 1]>(trsm_blk_sm);
-    T(*L)[65] = reinterpret_cast<T(*)[65]>(trsm_blk_sm + sizeof(T) * 64 * nbk * (kTrsmCols + 1));
-    const int64_t cb = c0 + (int64_t)blockIdx.x * kTrsmCols;
-    const int wc = (int)min((int64_t)kTrsmCols, c1 - cb);
+    T(*X)[kC + 1] = reinterpret_cast<T(*)[kC + 1]>(trsm_blk_sm);
+    T(*L)[65] = reinterpret_cast<T(*)[65]>(trsm_blk_sm + sizeof(T) * 64 * nbk * (kC + 1));
+    const int64_t cb = c0 + (int64_t)blockIdx.x * kC;
+    const int wc = (int)min((int64_t)kC, c1 - cb);
     const int rows = 64 * nbk;
     const int r = threadIdx.x % 64, g = threadIdx.x / 64;
-    for (int idx = threadIdx.x; idx < rows * kTrsmCols; idx += 256) {
+    for (int idx = threadIdx.x; idx < rows * kC; idx += 256) {
         const int rr = idx % rows, cc = idx / rows;
         X[rr][cc] = cc < wc ? A[(K0 + rr) + (cb + cc) * n] : (T)0;
     }
-    T acc[8];
+    T acc[kP];
     for (int i = 0; i < nbk; ++i) {
         // X_i -= L_ij X_j, j < i
         for (int j = 0; j < i; ++j) {
@@ -620,14 +673,14 @@ __global__ void __launch_bounds__(256) k_trsm_block(T* __restrict__ A, int64_t n
             }
             __syncthreads();
 #pragma unroll
-            for (int c = 0; c < 8; ++c) acc[c] = (T)0;
+            for (int c = 0; c < kP; ++c) acc[c] = (T)0;
             for (int q = 0; q < 64; ++q) {
                 const T l = L[r][q];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) acc[c] = fma(l, X[64 * j + q][8 * g + c], acc[c]);
+                for (int c = 0; c < kP; ++c) acc[c] = fma(l, X[64 * j + q][kP * g + c], acc[c]);
             }
 #pragma unroll
-            for (int c = 0; c < 8; ++c) X[64 * i + r][8 * g + c] -= acc[c];
+            for (int c = 0; c < kP; ++c) X[64 * i + r][kP * g + c] -= acc[c];
         }
         // X_i = Linv_i X_i
         __syncthreads();
@@ -637,18 +690,18 @@ __global__ void __launch_bounds__(256) k_trsm_block(T* __restrict__ A, int64_t n
         }
         __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = (T)0;
-        for (int q = 0; q < 64; ++q) {
+        for (int c = 0; c < kP; ++c) acc[c] = (T)0;
+        for (int q = 0; q <= (r | 31); ++q) {  // Linv is lower triangular: the warp's last row
             const T l = L[r][q];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) acc[c] = fma(l, X[64 * i + q][8 * g + c], acc[c]);
+            for (int c = 0; c < kP; ++c) acc[c] = fma(l, X[64 * i + q][kP * g + c], acc[c]);
         }
         __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 8; ++c) X[64 * i + r][8 * g + c] = acc[c];
+        for (int c = 0; c < kP; ++c) X[64 * i + r][kP * g + c] = acc[c];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < rows * kTrsmCols; idx += 256) {
+    for (int idx = threadIdx.x; idx < rows * kC; idx += 256) {
         const int rr = idx % rows, cc = idx / rows;
         if (cc < wc) A[(K0 + rr) + (cb + cc) * n] = X[rr][cc];
     }
@@ -779,6 +832,26 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
         }
         cudaGetLastError();  // a refused attribute or query leaves the per-column path
     }
+    // panels of few rows in one cluster, where the device can hold it
+    cudaLaunchAttribute cl_attr{};
+    cl_attr.id = cudaLaunchAttributeClusterDimension;
+    cl_attr.val.clusterDim = {kPanelCluster, 1, 1};
+    cudaLaunchConfig_t cl{};
+    cl.gridDim = dim3(kPanelCluster);
+    cl.blockDim = dim3(kCoopThreads);
+    cl.dynamicSmemBytes = (size_t)kClusterRows<T> * 64 * sizeof(T);
+    cl.stream = s;
+    cl.attrs = &cl_attr;
+    cl.numAttrs = 1;
+    int clusters = 0;
+    if (gmax > 0 &&
+        (cudaFuncSetAttribute(k_panel_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+         cudaFuncSetAttribute(k_panel_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)cl.dynamicSmemBytes) != cudaSuccess ||
+         cudaOccupancyMaxActiveClusters(&clusters, k_panel_cluster<T>, &cl) != cudaSuccess)) {
+        clusters = 0;
+        cudaGetLastError();
+    }
     unsigned int arrivals = 0;
     // FP32 with the bulk tensor-core path: two-level blocking.  Super-panels of kSuperPanels
     // panels; inside one, each panel's U12 and update stop at the super-panel's last column;
@@ -799,8 +872,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
     auto trsm_block = [&](int64_t r0, int nbk, const T* inv, int64_t c0, int64_t c1) -> cudaError_t {
         const int smem = (int)trsm_block_smem<T>(nbk);
         NB_TRY(cudaFuncSetAttribute(k_trsm_block<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        k_trsm_block<T><<<(unsigned)((c1 - c0 + kTrsmCols - 1) / kTrsmCols), 256, smem, s>>>(A, n, r0, nbk, inv, c0,
-                                                                                            c1);
+        k_trsm_block<T><<<(unsigned)((c1 - c0 + kTrsmCols<T> - 1) / kTrsmCols<T>), 256, smem, s>>>(A, n, r0, nbk, inv,
+                                                                                                  c0, c1);
         return cudaGetLastError();
     };
     for (int64_t K0 = 0; K0 < n; K0 += sp) {
@@ -809,7 +882,11 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
         for (int64_t k0 = K0; k0 < K1; k0 += nb) {
             const int64_t k1 = std::min<int64_t>(n, k0 + nb);
             const int w = (int)(k1 - k0);
-            if (gmax > 0) {
+            if (clusters > 0 && n - k0 <= kClusterRows<T> * kPanelCluster) {
+                const int R = (int)((n - k0 + kPanelCluster - 1) / kPanelCluster);
+                cl.dynamicSmemBytes = (size_t)R * w * sizeof(T);
+                NB_TRY(cudaLaunchKernelEx(&cl, k_panel_cluster<T>, A, n, k0, k1, R, piv, d_info, cs));
+            } else if (gmax > 0) {
                 const int64_t rows = n - k0;
                 const int R = (int)std::max<int64_t>(kCoopMinRows<T>, (rows + gmax - 1) / gmax);
                 const int G = (int)((rows + R - 1) / R);
