@@ -788,6 +788,34 @@ constexpr int kSuperPanels = 4;  // panels per super-panel of the two-level FP32
 
 // work layout: [0, 4 nb*nb) unit-lower inverses; then nb*n U12 staging;
 // then kPivBlocks doubles + kPivBlocks int64 for the pivot search and one int ticket.
+// The stream on which the FP64 factorisation takes the next panel while the rest of the trailing
+// update runs.  A panel is bound by latency and leaves the SMs nearly idle: with the update of the
+// panel's columns first, the panel then beside the other columns' update (its CTAs at the higher priority,
+// beside the update's in registers and shared memory up to 8,000 rows), the LU of 6,145 rows takes 40.2 ms
+// instead of 44.4 (8,192: 65.0 and 72.6, 12,000: 151 and 164).  The two share the FP64 pipe: beside the
+// update a panel takes 310 us instead of 206.  Where kAheadFrom rows or more are left: below, the second
+// update launch and the events cost more (1,024 rows: 4.00 and 3.88 ms; 2,500: 11.5 and 11.4; 3,000: 14.1 and 14.3).
+constexpr int64_t kAheadFrom = 2048;
+struct Ahead {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t ready = nullptr, done = nullptr;
+    cudaError_t init() {
+        int lo = 0, hi = 0;
+        cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&stream, cudaStreamNonBlocking, hi);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+        return e;
+    }
+    bool joined = true;  // the caller's stream waits for all that was queued here
+    ~Ahead() {
+        if (!joined) cudaStreamSynchronize(stream);
+        if (done) cudaEventDestroy(done);
+        if (ready) cudaEventDestroy(ready);
+        if (stream) cudaStreamDestroy(stream);
+    }
+};
+
 template <typename T>
 cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_info, void* split, void* coop,
                       cudaStream_t s, long long polls) {
@@ -826,6 +854,9 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_coop<T>, kCoopThreads, (size_t)smem0) ==
                     cudaSuccess &&
                 per_sm >= 1) {
+                // beside another kernel's CTA on an SM (Ahead) only if the SM's carve-out has room for both
+                NB_TRY(cudaFuncSetAttribute(k_panel_coop<T>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                            cudaSharedmemCarveoutMaxShared));
                 gmax = g;
                 NB_TRY(cudaMemsetAsync(cs, 0, sizeof(CoopScratch<T>), s));
             }
@@ -848,6 +879,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
         (cudaFuncSetAttribute(k_panel_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
          cudaFuncSetAttribute(k_panel_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)cl.dynamicSmemBytes) != cudaSuccess ||
+         cudaFuncSetAttribute(k_panel_cluster<T>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
          cudaOccupancyMaxActiveClusters(&clusters, k_panel_cluster<T>, &cl) != cudaSuccess)) {
         clusters = 0;
         cudaGetLastError();
@@ -876,43 +909,54 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                                                                                                   c0, c1);
         return cudaGetLastError();
     };
+    // the panel [k0, k1) and the permutation of its swaps, on stream st
+    auto panel_step = [&](int64_t k0, int64_t k1, cudaStream_t st) -> cudaError_t {
+        const int w = (int)(k1 - k0);
+        if (clusters > 0 && n - k0 <= kClusterRows<T> * kPanelCluster) {
+            const int R = (int)((n - k0 + kPanelCluster - 1) / kPanelCluster);
+            cl.dynamicSmemBytes = (size_t)R * w * sizeof(T);
+            cl.stream = st;
+            NB_TRY(cudaLaunchKernelEx(&cl, k_panel_cluster<T>, A, n, k0, k1, R, piv, d_info, cs));
+        } else if (gmax > 0) {
+            const int64_t rows = n - k0;
+            const int R = (int)std::max<int64_t>(kCoopMinRows<T>, (rows + gmax - 1) / gmax);
+            const int G = (int)((rows + R - 1) / R);
+            T* Af = A;
+            int64_t nn = n, kk0 = k0, kk1 = k1;
+            int RR = R;
+            int* tmo = d_info + 1;
+            unsigned int base = arrivals;
+            arrivals += (unsigned int)G * (unsigned int)w;
+            long long lim = polls > 0 ? polls : kCoopSpinLimit;
+            void* args[] = {&Af, &nn, &kk0, &kk1, &RR, &piv, &d_info, &tmo, &cs, &base, &lim};
+            NB_TRY(cudaLaunchCooperativeKernel((const void*)k_panel_coop<T>, dim3((unsigned)G), dim3(kCoopThreads),
+                                               args, (size_t)R * w * sizeof(T), st));
+        } else {
+            // columns k0..k1-1: update by the previous column + pivot of this one; then the
+            // last column's scaling of the rows below the panel
+            for (int64_t j = k0; j <= k1; ++j) {
+                if (j == n) break;
+                const int64_t rows = n - j;
+                const int pb = (int)std::min<int64_t>(kPivBlocks, (rows + kPivThreads - 1) / kPivThreads);
+                k_panel_col<T><<<pb, kPivThreads, 0, st>>>(A, n, j, k0, k1, j < k1 ? 1 : 0, pval, pidx, ticket,
+                                                          piv, d_info);
+            }
+        }
+        k_swap_perm<<<1, kSwapMax, 0, st>>>(piv, n, k0, k1, swap_perm);
+        return cudaGetLastError();
+    };
+    Ahead ahead;
+    const bool look = sizeof(T) == 8 && split && nb == 64 && n - nb >= kAheadFrom;
+    if (look) NB_TRY(ahead.init());
+    bool panel_done = false;  // taken ahead
     for (int64_t K0 = 0; K0 < n; K0 += sp) {
         const int64_t K1 = std::min<int64_t>(n, K0 + sp);
         const int64_t e1 = super ? K1 : n;  // last column (exclusive) the panels' updates reach
         for (int64_t k0 = K0; k0 < K1; k0 += nb) {
             const int64_t k1 = std::min<int64_t>(n, k0 + nb);
             const int w = (int)(k1 - k0);
-            if (clusters > 0 && n - k0 <= kClusterRows<T> * kPanelCluster) {
-                const int R = (int)((n - k0 + kPanelCluster - 1) / kPanelCluster);
-                cl.dynamicSmemBytes = (size_t)R * w * sizeof(T);
-                NB_TRY(cudaLaunchKernelEx(&cl, k_panel_cluster<T>, A, n, k0, k1, R, piv, d_info, cs));
-            } else if (gmax > 0) {
-                const int64_t rows = n - k0;
-                const int R = (int)std::max<int64_t>(kCoopMinRows<T>, (rows + gmax - 1) / gmax);
-                const int G = (int)((rows + R - 1) / R);
-                T* Af = A;
-                int64_t nn = n, kk0 = k0, kk1 = k1;
-                int RR = R;
-                int* tmo = d_info + 1;
-                unsigned int base = arrivals;
-                arrivals += (unsigned int)G * (unsigned int)w;
-                long long lim = polls > 0 ? polls : kCoopSpinLimit;
-                void* args[] = {&Af, &nn, &kk0, &kk1, &RR, &piv, &d_info, &tmo, &cs, &base, &lim};
-                NB_TRY(cudaLaunchCooperativeKernel((const void*)k_panel_coop<T>, dim3((unsigned)G), dim3(kCoopThreads),
-                                                   args, (size_t)R * w * sizeof(T), s));
-            } else {
-                // columns k0..k1-1: update by the previous column + pivot of this one; then the
-                // last column's scaling of the rows below the panel
-                for (int64_t j = k0; j <= k1; ++j) {
-                    if (j == n) break;
-                    const int64_t rows = n - j;
-                    const int pb = (int)std::min<int64_t>(kPivBlocks, (rows + kPivThreads - 1) / kPivThreads);
-                    k_panel_col<T><<<pb, kPivThreads, 0, s>>>(A, n, j, k0, k1, j < k1 ? 1 : 0, pval, pidx, ticket,
-                                                              piv, d_info);
-                }
-            }
-            NB_TRY(cudaGetLastError());
-            k_swap_perm<<<1, kSwapMax, 0, s>>>(piv, n, k0, k1, swap_perm);
+            if (!panel_done) NB_TRY(panel_step(k0, k1, s));
+            panel_done = false;
             k_laswp<T><<<(unsigned)((n + kSwapThreads - 1) / kSwapThreads), kSwapThreads, swap_smem, s>>>(A, n, k0,
                                                                                                     k1, swap_perm);
             const bool tc64 = sizeof(T) == 8 && split;  // FP64 with the tensor-core update
@@ -938,8 +982,22 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                         continue;
                     }
                 } else if (tc64) {
-                    NB_TRY(tc_update_f64(m, mc, w, A + k1 + k0 * n, n, A + k0 + k1 * n, n, A + k1 + k1 * n, n, split,
-                                         d_info + 1, s));
+                    T* C = A + k1 + k1 * n;
+                    NB_TRY(tc_split_f64(m, mc, w, A + k1 + k0 * n, n, A + k0 + k1 * n, n, split, s));
+                    if (look && m >= kAheadFrom) {
+                        NB_TRY(tc_apply_f64(m, mc, 0, nb, C, n, split, d_info + 1, s));
+                        NB_TRY(cudaEventRecord(ahead.ready, s));
+                        NB_TRY(cudaStreamWaitEvent(ahead.stream, ahead.ready, 0));
+                        ahead.joined = false;
+                        NB_TRY(panel_step(k1, k1 + nb, ahead.stream));
+                        NB_TRY(cudaEventRecord(ahead.done, ahead.stream));
+                        NB_TRY(tc_apply_f64(m, mc, nb, mc, C, n, split, d_info + 1, s));
+                        NB_TRY(cudaStreamWaitEvent(s, ahead.done, 0));
+                        ahead.joined = true;
+                        panel_done = true;
+                    } else {
+                        NB_TRY(tc_apply_f64(m, mc, 0, mc, C, n, split, d_info + 1, s));
+                    }
                     continue;
                 }
                 NB_TRY(gemm<T>(m, mc, w, (T)-1, A + k1 + k0 * n, n, A + k0 + k1 * n, n, (T)1, A + k1 + k1 * n, n, s));

@@ -27,7 +27,7 @@
 // the same time, and share a CTA in turn.  Every wait is bounded.
 //
 // Measured, LU of a random matrix of order 6145: the updates 142 ms on the FP64 pipe, 15 ms here; the
-// whole factorisation 234 -> 62 ms (16384: 2717 -> 389 ms), |P A - L U| / |A| 3.4e-14 -> 2.7e-14.
+// whole factorisation 234 -> 40 ms, |P A - L U| / |A| 3.4e-14 -> 2.7e-14.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -196,10 +196,11 @@ __device__ __forceinline__ double take_off(double c, const uint32_t (&a)[kDig], 
     return c - scalbn(t, max(-3000, e - 2100));
 }
 
-__global__ void __launch_bounds__(kDThreads, 1)
+// (bounds: 168 registers, so that a CTA of the next panel fits beside this one)
+__global__ void __launch_bounds__(384, 1)
     k_tc_update_f64(int64_t M, int64_t N, const unsigned char* __restrict__ da, const unsigned char* __restrict__ db,
                     const int* __restrict__ ea, const int* __restrict__ eb, double* __restrict__ C, int64_t ldc,
-                    int tpc, int* __restrict__ err) {
+                    int64_t tile0, int64_t tile1, int tpc, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem;
     unsigned char* sB = smem + kDTileA;
@@ -208,9 +209,8 @@ __global__ void __launch_bounds__(kDThreads, 1)
     uint64_t* barM = barA + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(barA + 3);
 
-    const int64_t tiles_n = (N + kDN - 1) / kDN;
-    const int64_t t0 = (int64_t)blockIdx.y * tpc;
-    const int nt = (int)min((int64_t)tpc, tiles_n - t0);
+    const int64_t t0 = tile0 + (int64_t)blockIdx.y * tpc;  // column tiles [tile0, tile1)
+    const int nt = (int)min((int64_t)tpc, tile1 - t0);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto load_b = [&](int t) {
         mbar_expect(barB, kDTileB);
@@ -326,29 +326,51 @@ size_t tc64_work_bytes(int64_t M, int64_t N) {
     return (size_t)(m / kDM) * kDTileA + (size_t)(n / kDN) * kDTileB + sizeof(int) * (size_t)(m + n + kDK) + 256;
 }
 
-cudaError_t tc_update_f64(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B, int64_t ldb,
-                          double* C, int64_t ldc, void* work, int* err, cudaStream_t s) {
+namespace {
+struct Tables64 {
+    unsigned char *da, *db;
+    int *ea, *eb, *g;
+};
+Tables64 tables64(int64_t M, int64_t N, void* work) {
+    const int64_t m = pad_to(M, kDM), n = pad_to(N, kDN);
+    Tables64 t;
+    t.da = static_cast<unsigned char*>(work);
+    t.db = t.da + (size_t)(m / kDM) * kDTileA;
+    t.ea = reinterpret_cast<int*>(t.db + (size_t)(n / kDN) * kDTileB);
+    t.eb = t.ea + m;
+    t.g = t.eb + n;
+    return t;
+}
+}  // namespace
+
+cudaError_t tc_split_f64(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B, int64_t ldb,
+                         void* work, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     if (K > kDK || !work) return cudaErrorInvalidValue;
     const int64_t m = pad_to(M, kDM), n = pad_to(N, kDN);
-    unsigned char* da = static_cast<unsigned char*>(work);
-    unsigned char* db = da + (size_t)(m / kDM) * kDTileA;
-    int* ea = reinterpret_cast<int*>(db + (size_t)(n / kDN) * kDTileB);
-    int* eb = ea + m;
-    int* g = eb + n;
-    cudaError_t e = cudaMemsetAsync(g, 0, sizeof(int) * kDK, s);
+    const Tables64 t = tables64(M, N, work);
+    cudaError_t e = cudaMemsetAsync(t.g, 0, sizeof(int) * kDK, s);
     if (e != cudaSuccess) return e;
-    k_row_exps<<<(unsigned)std::min<int64_t>((N + 15) / 16, 304), 256, 0, s>>>(B, ldb, (int)K, N, g);
-    k_split_digits<<<(unsigned)(m / 32 + n / 32), 256, 0, s>>>(A, lda, B, ldb, M, N, (int)K, g, m / 32, da, db, ea,
-                                                               eb);
+    k_row_exps<<<(unsigned)std::min<int64_t>((N + 15) / 16, 304), 256, 0, s>>>(B, ldb, (int)K, N, t.g);
+    k_split_digits<<<(unsigned)(m / 32 + n / 32), 256, 0, s>>>(A, lda, B, ldb, M, N, (int)K, t.g, m / 32, t.da, t.db,
+                                                               t.ea, t.eb);
+    return cudaGetLastError();
+}
+
+cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t c0, int64_t c1, double* C, int64_t ldc, void* work, int* err,
+                         cudaStream_t s) {
+    c1 = std::min(c1, N);
+    if (M <= 0 || c0 >= c1) return cudaSuccess;
+    if (c0 % kDN || !work) return cudaErrorInvalidValue;
+    const Tables64 t = tables64(M, N, work);
     // set for the current device on every call (an attribute is per device)
-    e = cudaFuncSetAttribute(k_tc_update_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_tc_update_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
     if (e != cudaSuccess) return e;
     // column tiles per CTA: about three CTAs per SM in all, at most 8 tiles each
-    const int64_t tiles_m = m / kDM, tiles_n = n / kDN;
+    const int64_t tiles_m = pad_to(M, kDM) / kDM, tile0 = c0 / kDN, tile1 = (c1 + kDN - 1) / kDN, tiles_n = tile1 - tile0;
     const int64_t tpc = std::max<int64_t>(1, std::min<int64_t>(8, tiles_m * tiles_n / (3 * 152)));
     dim3 grid((unsigned)tiles_m, (unsigned)((tiles_n + tpc - 1) / tpc));
-    k_tc_update_f64<<<grid, kDThreads, kDSmem, s>>>(M, N, da, db, ea, eb, C, ldc, (int)tpc, err);
+    k_tc_update_f64<<<grid, kDThreads, kDSmem, s>>>(M, N, t.da, t.db, t.ea, t.eb, C, ldc, tile0, tile1, (int)tpc, err);
     return cudaGetLastError();
 }
 

@@ -34,3 +34,26 @@ def test_factors(n, single):
     assert np.abs(L).max() <= 1 + 4 * u
     bound = 4 * max(n, 8) * u * (np.abs(L) @ np.abs(U))
     assert (np.abs(A[perm].astype(np.float64) - L @ U) <= bound).all()
+
+
+@pytest.mark.parametrize("n", [2111, 2112, 2240, 3001])
+def test_panels_ahead(n):
+    """Sizes where the first panels are taken beside the trailing update: the first whole step, one row less,
+    and a partial last panel; backward error 4 n u of |A| |x|."""
+    import torch
+
+    from paper_2606_24154_gb300 import build, nebem as N
+    build.build()
+    gen = np.random.default_rng(n)
+    A = gen.normal(size=(n, n)) + 8 * np.sqrt(n) * np.eye(n)[gen.permutation(n)]
+    b = gen.normal(size=n)
+    dA = torch.tensor(A.T.copy(), device="cuda")
+    piv = torch.empty(n, dtype=torch.int32, device="cuda")
+    x = torch.tensor(b, device="cuda")
+    ctx = N.Context()
+    N.nebem_lu_factor_device(ctx.h, dA.data_ptr(), n, piv.data_ptr())
+    N.nebem_lu_solve_device(ctx.h, dA.data_ptr(), n, piv.data_ptr(), x.data_ptr())
+    torch.cuda.synchronize()
+    ctx.close()
+    x = x.cpu().numpy()
+    assert (np.abs(A @ x - b) <= 4 * n * 1.2e-16 * (np.abs(A) @ np.abs(x) + np.abs(b))).all()
