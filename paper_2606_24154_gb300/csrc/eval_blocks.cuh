@@ -293,6 +293,10 @@ __device__ __forceinline__ Sum4 far_range(const GeomView& g, float phx, float ph
 #pragma unroll
             for (int i = 0; i < 2 * kPairs0; ++i) q[i] = s_f[jj][i];
             float2 lphi = make_float2(0.f, 0.f), lx = lphi, ly = lphi, lz = lphi;
+            // four images per round, so that one's distance test overlaps another's roots (1e6 points of the
+            // 9,996-element cell x 25 copies: 610 ms, 592 so; two images 602, eight blocks of 64
+            // registers per SM instead of six of 80 594 alone and 604 with it)
+#pragma unroll 4
             for (int k = 0; k < nimg; ++k) {
                 float dx, dy, dz;
                 const float d2 = pair_d2(phx, phy, phz, plx, ply, plz, s_c[jj * nimg + k][0], s_c[jj * nimg + k][1],

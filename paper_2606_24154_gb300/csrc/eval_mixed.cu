@@ -14,8 +14,8 @@ constexpr int kFarBlocks = 6;  // resident far blocks per SM (80 registers a thr
 // left-over groups).  Bound by the FP32 pipe where every SM has its six
 // blocks; a thread's own chain of pairs takes as long on an idle SM as on a full one, so few
 // points are spread over element pieces (see split_plan): 257 points of the 9,996-element
-// cell x 25 copies took 71.2 ms in 3 blocks and take 0.64 ms in 939; 20,000 points 69 and 15 ms,
-// 200,000 points 162 and 126 ms, 1e6 points 644 and 610 ms (with binning and near pairs).
+// cell x 25 copies took 71.2 ms in 3 blocks and take 0.63 ms in 939; 20,000 points 69 and 15 ms,
+// 200,000 points 162 and 122 ms, 1e6 points 644 and 592 ms (with binning and near pairs).
 __global__ void __launch_bounds__(kEvalThreads, kFarBlocks)
     k_eval_far(const GeomView g, const double* __restrict__ pts, const int32_t* __restrict__ order, int64_t npts,
                const SplitPlan plan, SumB* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
