@@ -39,6 +39,153 @@ __global__ void __launch_bounds__(kEvalThreads, kFarBlocks)
     }
 }
 
+// The same for few points: a unit is kFL points of one leaf (at most 32 elements), and a thread takes
+// (point, element) pairs, two points of its element at a time, so that a launch does not end with
+// threads that walk a whole leaf.  The chains over the elements follow from shared memory, a lane per
+// quantity, with far_range's operations in its order (FP32 groups of kGroup elements within its tiles,
+// the scales in FP32): the same bits.  Shared memory per tile of te elements in odd strides of float4, since
+// the lanes read different elements.  10,000 elements x 25 copies: 5 points 0.33 ms by k_eval_far and
+// 0.03 ms here, 64 points 0.49 and 0.13, 257 points 0.66 and 0.42.  The lanes of a warp take different tiers more
+// often than neighbouring points do, so a point costs twice as much, and calls that share the GPU with
+// others lose where k_eval_far's groups are full (257 points in several streams: 0.91 and 0.93 ms for the
+// whole refined call): kFarLaneRounds units per resident block of k_eval_far, about 70 points.
+constexpr int kFL = 8;                       // points of a unit
+constexpr int kFLCentres = 1792;             // float4 of image centroids
+constexpr int64_t kFarLaneRounds = 3;
+__global__ void __launch_bounds__(kEvalThreads, 4)
+    k_eval_far_lanes(const GeomView g, const double* __restrict__ pts, const int32_t* __restrict__ order, int64_t npts,
+                     int64_t np, int te, SumB* __restrict__ part) {
+    constexpr int kWarps = kEvalThreads / 32, kWP = kFL / kWarps, kF = 2 * kPairs0, kA = 2 * kPairsA;
+    __shared__ float4 s_f[32][kF + 1], s_a[32][kA + 1], s_hdr[32], s_c[kFLCentres];
+    __shared__ float2 s_sig[32];
+    __shared__ int s_na[32];
+    __shared__ float s_val[kWarps][kWP][32][7];  // sigma hi, lo, Phi', E'
+    __shared__ float s_g[kFL][8];           // chains: the group's four sums, the four scales
+    __shared__ double s_sum[kFL][4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nimg = g.nimg, st = 2 * nimg + 1;
+    const int64_t groups = (npts + kFL - 1) / kFL;
+    const int64_t piece = blockIdx.x / groups, i0 = (blockIdx.x - piece * groups) * kFL;
+    const int64_t e0 = piece * kLeafEl, e1 = min(e0 + (int64_t)kLeafEl, g.n_el);
+    for (int c = lane; c < 8 * kWP; c += 32) s_g[w * kWP][c] = 0.f;
+    for (int c = lane; c < 4 * kWP; c += 32) s_sum[w * kWP][c] = 0.0;
+    __syncwarp();
+    for (int64_t base = e0; base < e1; base += te) {
+        const int cnt = (int)min((int64_t)te, e1 - base);
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt * kA; i += kEvalThreads) s_a[i / kA][i % kA] = g.far[base + i / kA].a[i % kA];
+        for (int i = threadIdx.x; i < cnt * kF; i += kEvalThreads) s_f[i / kF][i % kF] = g.far[base + i / kF].f[i % kF];
+        for (int i = threadIdx.x; i < cnt; i += kEvalThreads) {
+            s_hdr[i] = g.far[base + i].hdr;
+            s_na[i] = g.far[base + i].n_a;
+            const double sd = fma(g.sigma[base + i], (double)g.far[base + i].wcorr, g.sigma[base + i]);
+            const float sh = __double2float_rn(sd);
+            s_sig[i] = make_float2(sh, __double2float_rn(sd - (double)sh));
+        }
+        for (int i = threadIdx.x; i < 2 * cnt * nimg; i += kEvalThreads)
+            s_c[i / (2 * nimg) * st + i % (2 * nimg)] = g.cjk[2 * base * nimg + i];
+        __syncthreads();
+        // te = 32: a thread takes its element with the warp's two points; else 32 / te >= kWP points side by side
+        static_assert(kWP == 2, "points of a warp");
+        const int jj = lane % te;
+        bool valid[kWP];
+        float ph[kWP][6];
+#pragma unroll
+        for (int u = 0; u < kWP; ++u) {
+            const int q = te == 32 ? u : lane / te;
+            const int64_t i = i0 + w * kWP + q;
+            valid[u] = jj < cnt && q < kWP && i < npts && (te == 32 || u == 0);
+            load_point_2f(pts, valid[u] ? (int64_t)order[i] : 0, valid[u], ph[u][0], ph[u][1], ph[u][2], ph[u][3],
+                          ph[u][4], ph[u][5]);
+        }
+        if (valid[0]) {
+            const float4 hdr = s_hdr[jj];
+            const bool rect = s_na[jj] == kPairsA;
+            const FarNodes* fj = g.far + base + jj;
+            const float4* cj = s_c + jj * st;
+            float4 f0[kF];
+#pragma unroll
+            for (int i = 0; i < kF; ++i) f0[i] = s_f[jj][i];
+            float2 lphi[kWP], lx[kWP], ly[kWP], lz[kWP];
+#pragma unroll
+            for (int u = 0; u < kWP; ++u) lphi[u] = lx[u] = ly[u] = lz[u] = make_float2(0.f, 0.f);
+            for (int k = 0; k < nimg; ++k) {
+                const float4 ch = cj[2 * k], cl = cj[2 * k + 1];
+#pragma unroll
+                for (int u = 0; u < kWP; ++u) {
+                    if (!valid[u]) continue;
+                    float dx, dy, dz;
+                    const float d2 =
+                        pair_d2(ph[u][0], ph[u][1], ph[u][2], ph[u][3], ph[u][4], ph[u][5], ch, cl, dx, dy, dz);
+                    const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy), DZ = make_float2(dz, dz);
+                    if (d2 >= hdr.x) {
+                        pairs0_reg(f0, DX, DY, DZ, lphi[u], lx[u], ly[u], lz[u]);
+                    } else if (d2 >= hdr.y) {
+                        if (rect)
+                            node_pairs<kPairsA>(s_a[jj], DX, DY, DZ, lphi[u], lx[u], ly[u], lz[u]);
+                        else
+                            node_pairs<3>(s_a[jj], DX, DY, DZ, lphi[u], lx[u], ly[u], lz[u]);
+                    } else if (d2 >= hdr.z) {
+                        node_pairs<kPairsB>(fj->b, DX, DY, DZ, lphi[u], lx[u], ly[u], lz[u]);
+                    } else if (d2 >= hdr.w) {
+                        node_pairs<kPairsC>(fj->c, DX, DY, DZ, lphi[u], lx[u], ly[u], lz[u]);
+                    }
+                    // nearer pairs: k_eval_near
+                }
+            }
+            const float2 sg = s_sig[jj];
+#pragma unroll
+            for (int u = 0; u < kWP; ++u) {
+                float* o = s_val[w][u][lane];
+                o[0] = sg.x, o[1] = sg.y;
+                o[2] = lphi[u].x + lphi[u].y, o[3] = lx[u].x + lx[u].y;
+                o[4] = ly[u].x + ly[u].y, o[5] = lz[u].x + lz[u].y;
+            }
+        }
+        __syncwarp();
+        // chain c of a point: 0-3 phi and E, 4-7 the scales
+        for (int l = lane; l < 8 * kWP; l += 32) {
+            const int q = l / 8, c = l % 8, pt = w * kWP + q;
+            const float(*r)[7] = te == 32 ? s_val[w][q] : s_val[w][0] + q * te;
+            float x = s_g[pt][c];
+            double sum = c < 4 ? s_sum[pt][c] : 0.0;
+            for (int e = 0; e < cnt; ++e) {
+                const float s = r[e][0];
+                if (c < 4) {
+                    const float f = r[e][2 + c];
+                    x = fmaf(s, f, fmaf(r[e][1], f, x));
+                    const int in_tile = ((int)(base - e0) + e) & (g.tile_el - 1);  // a power of two
+                    if (in_tile % kGroup == kGroup - 1 || in_tile == g.tile_el - 1 || base + e == e1 - 1) {
+                        sum += (double)x;
+                        x = 0.f;
+                    }
+                } else {
+                    const float a = c & 1 ? fabsf(r[e][3]) + fabsf(r[e][4]) + fabsf(r[e][5]) : fabsf(r[e][2]);
+                    const float b = fabsf(s) * a;
+                    if (c < 6) {
+                        x += b;
+                    } else {
+                        const float v = b * kScaleSq;
+                        x = fmaf(v, v, x);
+                    }
+                }
+            }
+            s_g[pt][c] = x;
+            if (c < 4) s_sum[pt][c] = sum;
+        }
+        __syncwarp();
+    }
+    for (int l = lane; l < 8 * kWP; l += 32) {
+        const int pt = w * kWP + l / 8, c = l % 8;
+        const int64_t i = i0 + pt;
+        if (i >= npts) continue;
+        SumB* o = part + i * np + piece;
+        if (c < 4)
+            reinterpret_cast<double*>(&o->s)[c] = s_sum[pt][c];
+        else
+            reinterpret_cast<float*>(&o->b)[c - 4] = s_g[pt][c];
+    }
+}
+
 // the left-over groups' points: their pieces added along the summation tree, a warp per point
 __global__ void __launch_bounds__(256) k_far_reduce(const double* __restrict__ pts, const int32_t* __restrict__ order,
                                                     int64_t npts, const SplitPlan plan,
@@ -272,8 +419,16 @@ cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4*
     const int64_t gb = kFarBlocks * (int64_t)sms;
     const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
     const int64_t units = plan.Gm + plan.R * plan.np;
-    k_eval_far<<<(unsigned)units, kEvalThreads, 0, s>>>(g, pts, ms.order, npts, plan, static_cast<SumB*>(part), phi, E,
-                                                        ms.bound);
+    const int64_t lane_units = (npts + kFL - 1) / kFL * plan.np;
+    if (plan.leaf && plan.Gm == 0 && lane_units < kFarLaneRounds * gb) {
+        int te = 32;
+        while (te > 1 && te * (2 * img.n + 1) > kFLCentres) te /= 2;
+        k_eval_far_lanes<<<(unsigned)lane_units, kEvalThreads, 0, s>>>(g, pts, ms.order, npts, plan.np, te,
+                                                                       static_cast<SumB*>(part));
+    } else {
+        k_eval_far<<<(unsigned)units, kEvalThreads, 0, s>>>(g, pts, ms.order, npts, plan, static_cast<SumB*>(part), phi,
+                                                            E, ms.bound);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (plan.R > 0)

@@ -42,3 +42,26 @@ def test_short_lists(half, tol):
     assert (np.abs(phi[:505] - rp) <= scale * np.abs(rp)).all()  # one sign: the sum is its magnitudes'
     # |E|: the magnitudes' sum is at most phi's over the distance, 0.05 size
     assert (np.linalg.norm(E[:505] - rE, axis=1) <= scale * np.abs(rp) / (0.05 * size)).all()
+
+
+@pytest.mark.parametrize("half", [0, 1, 5])
+@pytest.mark.parametrize("per_edge", [3, 7])
+def test_short_lists_fp32_pass(half, per_edge):
+    """The FP32 pass of few points (a thread per point and element) and of many: the same bits, estimates included;
+    tiles of 16 and 4 elements with whole and partial groups, a last leaf of 22 and of 6 elements."""
+    from paper_2606_24154_gb300 import build, nebem as N
+    build.build()
+    g = I.cube(n_per_edge=per_edge)
+    gen = np.random.default_rng(half)
+    size = np.abs(g.elements["v"]).max()
+    ctx = N.Context(mixed_point_tol=0.0)
+    lattice = np.array([6 * size, 0, 0, 0, 6 * size, 0]) if half else None
+    N.nebem_set_geometry(ctx.h, g.elements, lattice, -half, half)
+    ctx.n = g.elements.size
+    ctx.set_sigma(gen.normal(size=ctx.n) * 1e-9)
+    pts = gen.uniform(-2.5 * size, 2.5 * size, (12000, 3))
+    phi, E, err, _ = ctx.eval_err(pts)
+    for a, b in ((0, 1), (3, 10), (11, 19), (100, 133), (5, 505)):
+        p, e, r, _ = ctx.eval_err(pts[a:b])
+        assert np.array_equal(p, phi[a:b]) and np.array_equal(e, E[a:b]) and np.array_equal(r, err[a:b])
+    ctx.close()
