@@ -26,106 +26,6 @@ namespace {
 constexpr int kPivBlocks = 256;
 constexpr int kPivThreads = 256;
 
-template <typename T>
-__global__ void k_pivot_partial(const T* __restrict__ A, int64_t n, int64_t j, double* __restrict__ pval,
-                                int64_t* __restrict__ pidx) {
-    double best = -1.0;
-    int64_t bidx = INT64_MAX;
-    for (int64_t i = j + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = fabs((double)A[i + j * n]);
-        if (v > best || (v == best && i < bidx)) {
-            best = v;
-            bidx = i;
-        }
-    }
-    __shared__ double sv[kPivThreads];
-    __shared__ int64_t si[kPivThreads];
-    sv[threadIdx.x] = best;
-    si[threadIdx.x] = bidx;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const double v = sv[threadIdx.x + s];
-            const int64_t ix = si[threadIdx.x + s];
-            if (v > sv[threadIdx.x] || (v == sv[threadIdx.x] && ix < si[threadIdx.x])) {
-                sv[threadIdx.x] = v;
-                si[threadIdx.x] = ix;
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        pval[blockIdx.x] = sv[0];
-        pidx[blockIdx.x] = si[0];
-    }
-}
-
-// Final pivot reduction + row swap inside the panel columns [k0, k1).
-template <typename T>
-__global__ void k_pivot_swap(T* __restrict__ A, int64_t n, int64_t j, int64_t k0, int64_t k1,
-                             const double* __restrict__ pval, const int64_t* __restrict__ pidx, int nparts,
-                             int32_t* __restrict__ piv, int* __restrict__ info) {
-    __shared__ double sv[kPivThreads];
-    __shared__ int64_t si[kPivThreads];
-    double best = -1.0;
-    int64_t bidx = INT64_MAX;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x) {
-        const double v = pval[b];
-        const int64_t ix = pidx[b];
-        if (v > best || (v == best && ix < bidx)) {
-            best = v;
-            bidx = ix;
-        }
-    }
-    sv[threadIdx.x] = best;
-    si[threadIdx.x] = bidx;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const double v = sv[threadIdx.x + s];
-            const int64_t ix = si[threadIdx.x + s];
-            if (v > sv[threadIdx.x] || (v == sv[threadIdx.x] && ix < si[threadIdx.x])) {
-                sv[threadIdx.x] = v;
-                si[threadIdx.x] = ix;
-            }
-        }
-        __syncthreads();
-    }
-    // a column without a valid maximum (all NaN) keeps its own row: the factorisation is
-    // then reported singular through info and no out-of-range row is ever swapped
-    const int64_t p = (si[0] >= j && si[0] < n) ? si[0] : j;
-    if (threadIdx.x == 0) {
-        piv[j] = (int32_t)p;
-        if (!(sv[0] > 0.0) && *info == 0) *info = (int)(j + 1);
-    }
-    if (p != j) {
-        for (int64_t c = k0 + threadIdx.x; c < k1; c += blockDim.x) {
-            const T a = A[j + c * n];
-            A[j + c * n] = A[p + c * n];
-            A[p + c * n] = a;
-        }
-    }
-}
-
-// Scale column j below the diagonal and apply the rank-1 update to panel columns (j, k1).
-template <typename T>
-__global__ void k_scale_update(T* __restrict__ A, int64_t n, int64_t j, int64_t k1) {
-    extern __shared__ unsigned char smem_raw[];
-    T* urow = reinterpret_cast<T*>(smem_raw);
-    const int w = (int)(k1 - j - 1);
-    for (int c = threadIdx.x; c < w; c += blockDim.x) urow[c] = A[j + (j + 1 + c) * n];
-    __syncthreads();
-    const T d = A[j + j * n];
-    if (d == (T)0) return;
-    const T inv = (T)1 / d;
-    for (int64_t i = j + 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const T l = A[i + j * n] * inv;
-        A[i + j * n] = l;
-        for (int c = 0; c < w; ++c) A[i + (j + 1 + c) * n] -= l * urow[c];
-    }
-}
-
 // One launch per panel column j, fusing what would otherwise be three launches:
 //   (a) for j > k0: scale column j-1 below its diagonal and apply its rank-1 update to
 //       the panel columns (j-1, k1), each thread for its own rows i >= j;
