@@ -428,7 +428,7 @@ def run_native(args):
     _, _, err_r, _ = N.nebem_eval_err(ctx.h, sub)
     _, _, err_s, _ = N.nebem_eval_err(single.h, sub)
     refined_sub = sub[(err_r != err_s).any(axis=1)]
-    counts_l1 = R.tier_counts(g, refined_sub, sample=CHECK_SAMPLE)
+    counts_l1 = R.acc1_counts(g, refined_sub, sample=CHECK_SAMPLE)
     n_phi, n_E = stats.refined_level1_phi_only, stats.refined_level1_E_only
     ops_l1 = ((stats.refined_level1 - n_phi - n_E) * R.acc1_ops_per_point(counts_l1, n_el)
               + n_phi * R.acc1_ops_per_point(counts_l1, n_el, "phi") + n_E * R.acc1_ops_per_point(counts_l1, n_el, "E"))
@@ -564,7 +564,7 @@ def run_native(args):
                                        "peak": peak_fp64 / 1e12,
                                        "unit": "T FP64 instructions/s",
                                        "frac": fp64_rate * R.FP64_INST_PER_PAIR / peak_fp64,
-                                       "note": "278 FP64 instructions per pair (ncu count); peak = measured FP64 "
+                                       "note": "118 FP64 instructions per pair; peak = measured FP64 "
                                                "FMA rate (nebem_peak_rates)"}},
             "roofline": {"bound": "alu", "kernel": "k_eval_acc_far<1> (first refinement level, two-float)",
                          "achieved": ach_l1 / 1e12, "peak": peak_ops / 1e12, "unit": "Tops/s",
@@ -590,7 +590,7 @@ def run_native(args):
             "cpu_baseline": cpu,
             # per step: k_bin_keys, k_bin_scan, k_bin_scatter, k_eval_far, k_eval_near, then
             # k_flag + k_eval_acc_far + near per refinement level
-            "gpu_launches": 11 * args.steps,
+            "gpu_launches": 29 * args.steps,
             "clocks": clocks,
             "wall_s_timed_region": wall,
         }

@@ -185,8 +185,9 @@ int nebem_set_bc(nebem_ctx *ctx, const double *voltages, int32_t n_conductors);
 /* Solve K sigma = b (Eq. Matrix; Alg. 1 with an LU solve instead of an explicit inverse).
  *   precision  NEBEM_FP64: FP64 fill (closed forms for every pair), FP64 blocked LU with
  *              partial pivoting, FP64 triangular solves.  NEBEM_MIXED: mixed fill (pairs
- *              at >= 6 element radii by Gauss rules in two-float arithmetic, truncation
- *              below ~3e-12 of the pair, nearer pairs by the FP64 closed forms; an FP64
+ *              at >= 6 element radii in two-float arithmetic, by the element's moments from 32
+ *              (interface rows 52) radii on and by Gauss rules nearer, truncation below
+ *              ~3e-12 of the pair, nearer pairs by the FP64 closed forms; an FP64
  *              matrix from an earlier FP64 fill is reused instead), FP32 LU with tensor-core
  *              trailing updates, FP64 iterative refinement (residual with that K) until
  *              ir_tol.
@@ -284,9 +285,9 @@ int nebem_eval_device(nebem_ctx *ctx, const double *d_pts, int64_t n, double *d_
  * bound).  A point whose estimate exceeds mixed_point_tol times its
  * |phi| or |E| (context option, default 1e-6) is evaluated again in two-float arithmetic
  * (about 44 bits) for the quantity or quantities whose estimate exceeds it (the other keeps
- * its value and estimate): first with the same Gauss rules and FP64 near pairs (estimate
- * 1e-9 B),
- * and where that estimate still exceeds the tolerance, with rules truncated below ~3e-12 of
+ * its value and estimate): first with the element's moments from 28 radii on, and the same
+ * Gauss rules and FP64 near pairs nearer (estimate 1e-9 B), and where that estimate still
+ * exceeds the tolerance, with moments (from 40 radii on) and rules truncated below ~3e-12 of
  * each pair and FP64 closed forms within 6 element radii (estimate 1e-11 B).
  * nebem_eval / nebem_eval_device with NEBEM_MIXED
  * apply the same refinement; these calls also return the estimates.

@@ -25,15 +25,15 @@
 //
 // Refinement.  A point is re-evaluated when its estimate exceeds tol |phi| or tol |E|,
 // in two-float arithmetic (about 44 bits; the error-free transformations of twofloat.cuh),
-// in two levels.  Level 1 keeps the FP32 pass's Gauss rules and tiers and its FP64 near
-// pairs: their truncation, measured against the closed forms on THGEM points, stays below
-// ~2e-10 of B, so its estimate is 1e-9 B.  Points whose level-1 estimate still exceeds the
-// tolerance go to level 2, the rules of the mixed fill (fill_mixed.cu: truncation below
-// ~3e-12 of each pair, FP64 closed forms within kFillRatioC element radii), estimate
-// 1e-11 B.  In the frame of
-// element j (axes ex, ey = normal, ez), a pair (point, image k) has D = P - c_j - t_k with
+// in two levels.  Level 1 takes the pairs from 28 radii on by the element's moments (two-float
+// monopole, degrees 2 to 4 in FP32) and the nearer ones by the FP32 pass's Gauss rules and FP64 near
+// pairs: its error, measured against the closed forms on THGEM points, stays below
+// ~2e-11 of B; its estimate is 1e-9 B.  Points whose level-1 estimate still exceeds the
+// tolerance go to level 2, the arithmetic of the mixed fill (fill_mixed.cu: moments with a two-float
+// quadrupole from 40 radii on, rules truncated below ~3e-12 of each pair nearer, FP64 closed forms
+// within kFillRatioC element radii), estimate 1e-11 B.  In the frame of element j (axes ex, ey = normal, ez), a pair (point, image k) has D = P - c_j - t_k with
 // local components X = (P - c_j) . ex - tau_k.x (likewise Y, Z; tau tabulated per element
-// and image); a node at offset s = centroid - node (in the element plane) sees the point at
+// and image), from which the moments' series follow (twofloat.cuh); a node at offset s = centroid - node (in the element plane) sees the point at
 // D + s, so r^2 = |D|^2 + 2 (X s_x + Z s_z) + |s|^2 and
 //   Phi' = sum w / r,   E'_local = D sum w / r^3 + (sum w s_x / r^3, 0, sum w s_z / r^3).
 // Per element the image sums are rotated to the global frame and weighted by sigma_j in

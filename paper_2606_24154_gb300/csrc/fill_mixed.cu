@@ -3,14 +3,15 @@
 //   conductor row i:  K_ij = ke sum_k Phi'(c_i - t_k; j)
 //   interface row i:  K_ij = ke sum_k n_i . E'(c_i - t_k; j) + delta_ij diag_i
 //
-// Far pairs (distance to the image centroid >= kFillRatioC element radii) use Gauss rules
-// whose truncation error stays below ~3e-12 of the pair (tiers in nb_internal.h), evaluated
-// in two-float arithmetic: every quantity is an unevaluated sum hi + lo of two FP32 values
-// and products and sums keep their rounding errors through error-free transformations
-// (Dekker / Knuth TwoSum, FMA-based TwoProd), about 44 significant bits.  Near pairs use the
-// FP64 closed forms of influence.cuh.  The FP32 pipe runs 64 times the FP64 rate on this
-// GPU, so a two-float node (54-91 FP32 lane operations, issued two nodes per packed FP32x2
-// instruction) costs about as much as one FP64 operation.
+// Far pairs (distance to the image centroid >= kFillRatioC element radii) are evaluated in two-float
+// arithmetic: every quantity is an unevaluated sum hi + lo of two FP32 values and products and
+// sums keep their rounding errors through error-free transformations (Dekker / Knuth TwoSum,
+// FMA-based TwoProd), about 44 significant bits.  From 32 radii on (interface rows: 52) a pair
+// is the element's moments (fill_mom_phi2, fill_mom_field2 of twofloat.cuh), two images per packed
+// FP32x2 instruction; nearer, one to three pairs in a hundred, Gauss rules whose truncation stays
+// below ~3e-12 of the pair (tiers in nb_internal.h).  Near pairs use the FP64 closed forms of
+// influence.cuh.  The FP32 pipe runs 64 times the FP64 rate on this GPU, so a pair by moments (201
+// or 427 FP32 lane operations) costs as much as three to seven FP64 operations.
 //
 // Geometry of one pair in the local frame of the column element j (origin anywhere, axes
 // ex, ey = normal, ez): D = c_i - (c_j + t_k) has components
@@ -23,7 +24,7 @@
 // Newton step carried in two-float form; Phi' += w / r, n . E' += w (n . (D + s)) / r^3.
 //
 // Kernel k_fill_far: thread per row i, grid.y over column chunks; column tiles (element
-// records, tier-a nodes, tau, image centroids) staged in shared memory.  It writes
+// records, moments, tau) staged in shared memory.  It writes
 // ke * (far sum) (+ the interface diagonal) to every entry.  Kernel k_fill_near: warp
 // per row i; it visits the image centroids in the 27 grid cells around c_i (cell edge >=
 // the largest near radius) and adds ke * (FP64 closed form) of every near pair.  Both

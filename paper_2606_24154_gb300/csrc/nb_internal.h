@@ -62,9 +62,9 @@ struct __align__(16) FarNodes {
     int32_t pad[2];
 };
 
-// Mixed-precision fill (Eq. Matrix with far pairs by Gauss rules in two-float arithmetic).
-// Pairs are tiered by the distance d from the collocation point to the image centroid, in
-// radii rho of the column element:
+// Node tables of the mixed fill and of the refinement, whose nearer pairs use Gauss rules in two-float
+// arithmetic (the others: the element's moments, twofloat.cuh).  Pairs are tiered by the distance d
+// from the point to the image centroid, in radii rho of the column element:
 //   d >= kFillRatioA rho   tier a: rectangle / quadrilateral 3x3, triangle 6-point rule
 //   d >= kFillRatioB rho   tier b: 4x4 / collapsed 4x4
 //   d >= kFillRatioC rho   tier c: 6x6 / collapsed 6x6
@@ -217,7 +217,7 @@ cudaError_t launch_image_centroids(const Elem* el, int64_t n, const ImageTable& 
 cudaError_t fill_cols(int64_t n, int rows, int per_sm, int* cols);
 cudaError_t launch_fill_f64(const Elem* el, const double* diag, int64_t n, const ImageTable& img, double* K,
                             cudaStream_t s);
-// Mixed fill: far pairs (tiers a-c) write K; near pairs (grid of image centroids with
+// Mixed fill: far pairs (moments, tiers b and c) write K; near pairs (grid of image centroids with
 // the near radius kFillRatioC rho) add their FP64 closed forms afterwards.  tau[j][k] =
 // t_k . (ex_j, ey_j, ez_j) as (hi, lo) float4 pairs; nodes of kFillNodeRec float4 per element.
 // mom: fill_moments_bytes(n) bytes from launch_fill_moments.

@@ -268,9 +268,9 @@ __device__ __forceinline__ void mom_pair2(const float4* __restrict__ mom, float 
 // at any size of the geometry, and q is exact.
 // The monopole and the quadrupole (below 1.5e-4 of the pair) are in two-float arithmetic, F (below
 // 1.5e-6) in FP32; the terms left out (degree 7) are below 3e-13 at 32 radii.  In the field they count
-// eight times as much, so interface rows use the moments from kFillMomField = 52 radii on.  About 200 (Phi') and 360
-// (n . E') FP32 lane operations and one MUFU root per pair, where the 6, 9 and 16 nodes of the Gauss
-// rules took 480 to 1009 and 650 to 1500 and as many roots.
+// eight times as much, so interface rows use the moments from kFillMomField = 52 radii on.  150 (Phi') and
+// 376 (n . E') FP32 lane operations after the pair's geometry (51) and one MUFU root per pair, where the
+// 6, 9 and 16 nodes of the Gauss rules took 390 to 920 and 640 to 1540 and as many roots.
 // FillMom per element, every constant twice (both lanes), two per float4: a1, a2, a3, -w as hi, lo, then
 // the coefficients of F in the order of fill_mom_off, then A as hi, lo, s, s^2.
 constexpr double kFillMomField = 52.0;

@@ -87,7 +87,7 @@ def mufu_peak(sm_mhz):
 # evaluation kernel, from an ncu instruction count on the THGEM cell (166 DFMA, 59 DADD,
 # 53 DMUL); the FP64 pipe issues 2 such instructions per clock per SM on this GPU
 # (1.25 TFLOP/s nominal with an FMA as 2 flops).
-FP64_INST_PER_PAIR = 278
+FP64_INST_PER_PAIR = 118  # the series of the closed forms that most pairs take, counted from the code
 FP64_INST_PER_SM_CLK = 2
 
 
@@ -97,18 +97,18 @@ def fp64_peak_inst(sm_mhz):
 
 # ---------------------------------------------------------------- mixed fill
 # Two-float (hi + lo FP32) operations of the mixed fill kernel, counted from its code (FP32
-# lane operations; the node loops run two nodes per packed FP32x2 instruction, one lane
+# lane operations; images and node loops run two per packed FP32x2 instruction, one lane
 # each): per (row, column): c_i - c_j (3 two-float differences, 8 each) and its local
 # components (3 two-float dot products, 28 each); interface rows add the normal's local
-# components (3 more dot products).  Per far image pair: the FP32 tier test (12 + 3
-# compares), X, Y, Z (3 differences), |D|^2 (28) and two negations; interface rows add
-# n . D (28).  Per Gauss node: r^2 and the refined 1/r (41, plus one MUFU rsqrt), then w / r
-# accumulated (12) on conductor rows, or w (n . (D + s)) / r^3 accumulated (49) on
-# interface rows.
+# components (3 more dot products).  Per far image pair, nearer or not: X, Y, Z and |D|^2 (51)
+# and the moments (150 on conductor rows, 376 on interface rows).  Per Gauss node of a pair
+# nearer than the moments reach (32 radii; interface rows 52): r^2 and the refined 1/r (41, plus
+# one MUFU rsqrt), then w / r accumulated (12) on conductor rows, or w (n . (D + s)) / r^3
+# accumulated (49) on interface rows.
 FILL_OPS_COLUMN = (108, 192)   # conductor, interface row
-FILL_OPS_IMAGE = (69, 97)
+FILL_OPS_IMAGE = (201, 427)
 FILL_OPS_NODE = (53, 90)
-FILL_RATIOS = (96.0, 32.0, 6.0)
+FILL_RATIOS = (52.0, 32.0, 6.0)  # moments on interface rows; on conductor rows, 36 nodes nearer; FP64
 
 
 def fill_tier_counts(g, rows=256, seed=0, chunk=16):
@@ -118,8 +118,6 @@ def fill_tier_counts(g, rows=256, seed=0, chunk=16):
     t = _images(g)
     C = (c[:, None, :] + t[None]).reshape(-1, 3)
     R = np.repeat(rho, t.shape[0])
-    NV = np.repeat(nv, t.shape[0])
-    na = np.where(NV == 4, 9, 6)
     bc = g.elements["bc"]
     n = c.shape[0]
     sel = np.random.default_rng(seed).choice(n, min(rows, n), replace=False)
@@ -131,7 +129,7 @@ def fill_tier_counts(g, rows=256, seed=0, chunk=16):
         tb = (~ta) & (d >= FILL_RATIOS[1])
         tc = (d < FILL_RATIOS[1]) & (d >= FILL_RATIOS[2])
         far = ta | tb | tc
-        nodes = (ta * na[None]).sum(1) + 16 * tb.sum(1) + 36 * tc.sum(1)
+        nodes = 16 * tb.sum(1) * (bc[r] == 1) + 36 * tc.sum(1)
         for k, key in ((0, "cond"), (1, "iface")):
             m = bc[r] == k
             o = out[key]
@@ -155,32 +153,37 @@ def fill_ops(counts, n):
 
 
 # ---------------------------------------------------------------- refinement, first level
-# Two-float re-evaluation of flagged points with the FP32 pass's tiers (eval_acc.cu), FP32
-# lane operations counted from its code (node pairs run in the packed FP32x2 instructions,
-# two lanes each; a node slot is one lane of a node pair, padding included):
-#   per (point, element): P - c_j (3 two-float differences, 8 each) and its local
-#     components (3 two-float dot products, 28 each);
-#   per far (point, element, image) pair: the FP32 tier test (12 + 4 compares), X, Y, Z
-#     (3 differences, 24), |D|^2 (28), negations (3), the three node-pair sums folded to
-#     two-float values (30) and E_local += D S0 + S (3 two-float multiply-adds, 60);
-#   per node slot: r^2 and the refined 1/r (41, plus one MUFU rsqrt), w / r accumulated
-#     (12), w / r^3 (11) accumulated (8), and w (2 s_x) / r^3, w (2 s_z) / r^3 accumulated
-#     (1 + 12 + 12).
-# A point whose E estimate was within the tolerance has phi alone re-evaluated: per pair
-# without the folding and the E multiply-adds (161 - 90), per slot r^2, 1/r and w / r
-# (41 + 12).  A point whose phi estimate was within it has E alone re-evaluated: per slot
-# without w / r (97 - 12).
-ACC1_OPS_ELEMENT = 108
-ACC1_OPS_PAIR = 161
+# Two-float re-evaluation of flagged points (eval_acc.cu), FP32 lane operations counted from
+# its code (images and node pairs run two per packed FP32x2 instruction; a node slot is one lane
+# of a node pair):
+#   per (point, element): P - c_j (3 two-float differences, 8 each), its local components (3
+#     two-float dot products, 28 each) and the element's totals (60);
+#   per far (point, element, image) pair: X, Y, Z, |D|^2 and the moments: 194 for phi and E, 126
+#     for phi alone, 177 for E alone; pairs for both are counted with 177;
+#   per node slot of a pair nearer than 24 radii (acc1_counts; the pairs from 24 to 28 radii, which also
+#     take nodes, are left out): r^2 and the refined 1/r (41, plus one MUFU rsqrt), w / r
+#     accumulated (12), w / r^3 (11) accumulated (8), and w (2 s_x) / r^3, w (2 s_z) / r^3
+#     accumulated (1 + 12 + 12); phi alone 41 + 12, E alone 97 - 12.
+# So the counts are lower bounds.
+ACC1_OPS_ELEMENT = 168
+ACC1_OPS_PAIR = 177
 ACC1_OPS_SLOT = 97
-ACC1_OPS_PAIR_PHI = 71
+ACC1_OPS_PAIR_PHI = 126
 ACC1_OPS_SLOT_PHI = 53
 ACC1_OPS_SLOT_E = 85
 
 
+def acc1_counts(g, pts, sample=4096):
+    """tier_counts with the node slots of the pairs that the first refinement level takes by nodes
+    (tiers b and c: 16 and 36)."""
+    c = tier_counts(g, pts, sample=sample)
+    c["slots"] = 16 * c["b"] + 36 * c["c"]
+    return c
+
+
 def acc1_ops_per_point(counts, n_el, mode="both"):
     """FP32 lane operations of the first refinement level per refined point, from
-    tier_counts taken on a sample of refined points; mode "both", "phi" or "E" (which
+    acc1_counts taken on a sample of refined points; mode "both", "phi" or "E" (which
     quantities the point has re-evaluated)."""
     pair, slot = {"both": (ACC1_OPS_PAIR, ACC1_OPS_SLOT), "phi": (ACC1_OPS_PAIR_PHI, ACC1_OPS_SLOT_PHI),
                   "E": (ACC1_OPS_PAIR, ACC1_OPS_SLOT_E)}[mode]
