@@ -237,11 +237,11 @@ __device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr,
 }
 
 // Level 1, 1e6 points of the 9,996-element cell x 25 copies (320,000 of them refined): 1,490 ms with
-// every pair by Gauss nodes in two-float arithmetic, 629 ms so, with an error 10 to 25 times smaller
+// every pair by Gauss nodes in two-float arithmetic, 612 ms so (540 with the units dealt as below), with an error 10 to 25 times smaller
 // (E: 2.0e-10 B before, 1.7e-11 B now, the largest of 665 refined points).  The FP32 pipe is busy for
 // about two thirds of it; 5 blocks per SM (96 registers) beat 4 by 3 %, 6 are the same.
 //
-// Level 2 in the same run: 98 ms with every pair by Gauss nodes, 57 ms by moments; largest errors
+// Level 2 in the same run: 98 ms with every pair by Gauss nodes, 57 ms by moments (51); largest errors
 // unchanged (phi 1.1e-15 B, E 1.1e-14 B).
 //
 // An element's sums over its images of one point (before sigma): Phi', and E' in the global frame.
@@ -536,12 +536,14 @@ __device__ __forceinline__ Sum6 acc_sum(const AccView& A, int nimg, int te, floa
 // Far part of every listed point at level L, thread per point, kAT points (a group) per
 // block pass.  The ceil(*n_list / kAT) groups are dealt by split_plan: whole groups, then the
 // pieces of the left-over groups, whose Sum6 go to part[(i - Gm kAT) np + piece] of list entry
-// i for k_acc_reduce.  A point gets the same bits whichever way it is taken.  M: which
+// i for k_acc_reduce.  The resident blocks take the units in turn as they finish (*next): dealt round
+// robin, 15 of 20 warps per SM were there on average, since units near the points take longer (1e6
+// points: level 1 612 ms, level 2 57; in turn 540 and 51).  A point gets the same bits whichever way it is taken.  M: which
 // quantities the pass re-evaluates (kBoth, kPhiOnly, kEOnly).
 template <int L, int M>
 __global__ void __launch_bounds__(kAT, kATBlocks)
     k_eval_acc_far(const AccView A, int nimg, int te, const double* __restrict__ pts,
-                   const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
+                   const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int32_t* next, int64_t gb,
                    Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
                    double* __restrict__ err, float4* __restrict__ bound) {
     extern __shared__ float4 sm[];
@@ -549,7 +551,13 @@ __global__ void __launch_bounds__(kAT, kATBlocks)
     const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
     if (lane_path(plan, count, gb)) return;
     const int64_t units = plan.Gm + plan.R * plan.np;
-    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+    __shared__ int s_unit;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_unit = atomicAdd(next, 1);
+        __syncthreads();
+        const int64_t u = s_unit;
+        if (u >= units) break;
         const SplitUnit t = split_unit(plan, u, A.n_el);
         const int64_t i = t.group * kAT + threadIdx.x;
         const bool active = i < count;
@@ -683,8 +691,8 @@ __global__ void __launch_bounds__(256)
 
 template <int L, int M>
 cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* pts, int64_t npts, double* phi,
-                         double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list, int sms,
-                         Sum6* part, cudaStream_t s) {
+                         double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list,
+                         int32_t* next, int sms, Sum6* part, cudaStream_t s) {
     // element tile: a power of two (divides the leaf), within ~40 KB
     int te = kLeafEl;
     while (te > 1 && acc_tile_f4(L, te, img.n) * (int)sizeof(float4) > 40 * 1024) te /= 2;
@@ -696,8 +704,8 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
         e = cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
-        k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, gb, part,
-                                                                            phi, E, err, bound);
+        k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, next, gb,
+                                                                            part, phi, E, err, bound);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -780,8 +788,9 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
     if (npts == 0) return cudaSuccess;
     if (npts > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
     const bool refine = tol > 0.0 && (phi || E);
-    // counts: [0] level 1, both quantities; [1] level 2; [2] level 1, phi only; [3] level 1, E only
-    cudaError_t e = cudaMemsetAsync(ms.n_list, 0, 4 * sizeof(int32_t), s);
+    // counts: [0] level 1, both quantities; [1] level 2; [2] level 1, phi only; [3] level 1, E only;
+    // [4] to [7] the next unit of the passes
+    cudaError_t e = cudaMemsetAsync(ms.n_list, 0, kRefineCounts * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
     const unsigned fb = (unsigned)((npts + 255) / 256);
     k_flag<<<fb, 256, 0, s>>>(phi, E, ms.bound, ms.order, npts, nullptr, em.gamma_r, em.gamma_b, em.gamma_s, tol,
@@ -797,12 +806,14 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && refine)
-        e = launch_level<1, kBoth>(A, img, pts, npts, phi, E, err, ms.bound, ms.list, ms.n_list, sms, part, s);
+        e = launch_level<1, kBoth>(A, img, pts, npts, phi, E, err, ms.bound, ms.list, ms.n_list, ms.n_list + 4, sms, part,
+                                    s);
     if (e == cudaSuccess && refine)
-        e = launch_level<1, kPhiOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_p, ms.n_list + 2, sms, part,
-                                      s);
+        e = launch_level<1, kPhiOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_p, ms.n_list + 2, ms.n_list + 5, sms,
+                                      part, s);
     if (e == cudaSuccess && refine)
-        e = launch_level<1, kEOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_e, ms.n_list + 3, sms, part, s);
+        e = launch_level<1, kEOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_e, ms.n_list + 3, ms.n_list + 6, sms,
+                                    part, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], s);
     if (e == cudaSuccess && refine) {
         // level 2 on the points whose level-1 estimate still exceeds the tolerance (a quantity
@@ -814,7 +825,8 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
                                       ms.list2, ms.n_list + 1);
         e = cudaGetLastError();
         if (e == cudaSuccess)
-            e = launch_level<2, kBoth>(A, img, pts, npts, phi, E, err, nullptr, ms.list2, ms.n_list + 1, sms, part, s);
+            e = launch_level<2, kBoth>(A, img, pts, npts, phi, E, err, nullptr, ms.list2, ms.n_list + 1, ms.n_list + 7, sms,
+                                    part, s);
     }
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], s);
     return e;

@@ -137,6 +137,7 @@ cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, c
 // Scratch of one mixed evaluation of npts points: binning (bin counts, keys, the binned
 // order), the FP32 pass's error scales ke * (B_phi, B_E, S_phi, S_E) per point, and the
 // list and count of the points the refinement re-evaluates.
+constexpr int kRefineCounts = 8;
 struct MixedScratch {
     int32_t* count;  // kBins
     int32_t* key;    // npts
@@ -146,7 +147,7 @@ struct MixedScratch {
     int32_t* list2;  // npts: points of the second level
     int32_t* list_p; // npts: points of the first level, phi only
     int32_t* list_e; // npts: points of the first level, E only
-    int32_t* n_list; // 4: the lengths of list, list2, list_p, list_e
+    int32_t* n_list; // kRefineCounts: the lengths of list, list2, list_p, list_e; the passes' next units
     int32_t* bin_sums;  // block sums of the bin scan
 };
 MixedScratch mixed_scratch(void* base, int64_t npts);

@@ -183,7 +183,7 @@ struct Server {
         ms.list2 = d_list2.as<int32_t>() + r->offset;
         ms.list_p = d_list_p.as<int32_t>() + r->offset;
         ms.list_e = d_list_e.as<int32_t>() + r->offset;
-        ms.n_list = d_nlist.as<int32_t>() + 4 * r->slot;
+        ms.n_list = d_nlist.as<int32_t>() + kRefineCounts * r->slot;
         // the refine stream runs one request at a time, so one partial-sum area serves them all
         void* part = d_rpart.ptr;
         CK(launch_eval_refine(A, c->img, d_pts.as<double>() + 3 * r->offset, r->n,
@@ -423,7 +423,7 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         (e = s->d_list_p.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_list_e.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_rpart.ensure(refine_part_bytes(cap, cs[0]->props.multiProcessorCount, max_el))) != cudaSuccess ||
-        (e = s->d_nlist.ensure(4 * sizeof(int32_t) * o.max_requests)) != cudaSuccess ||
+        (e = s->d_nlist.ensure(kRefineCounts * sizeof(int32_t) * o.max_requests)) != cudaSuccess ||
         (e = s->d_pcount.ensure(sizeof(int) * kPartialBlocks)) != cudaSuccess)
         return bail(cuda_fail(e, "server device buffers"));
     if ((e = cudaHostAlloc(&s->h_ring, sizeof(WorkItem) * s->ring_cap, cudaHostAllocMapped)) != cudaSuccess ||
