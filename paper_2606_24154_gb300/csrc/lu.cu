@@ -268,7 +268,12 @@ __device__ __forceinline__ void panel(T* __restrict__ A, int64_t n, int64_t k0, 
         const int r = idx % nr, c = idx / nr;
         S[c * R + r] = A[(rb0 + r) + (k0 + c) * n];
     }
-    __syncthreads();
+    // CL: the first column's slots go to the other CTAs' shared memory, which may be touched only once those
+    // CTAs run (one that holds no rows gets here at once)
+    if constexpr (CL)
+        cg::this_cluster().sync();
+    else
+        __syncthreads();
     // thread -> row and group of columns: `step` rows at a time, `groups` column groups
     const int step = R <= kCoopThreads / 2 ? (R + 31) & ~31 : kCoopThreads;
     const int groups = kCoopThreads / step, grp = tid / step, row0 = tid - grp * step;
