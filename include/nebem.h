@@ -442,9 +442,11 @@ int nebem_step(nebem_ctx *ctx, int32_t steps, double mu, double dt, int32_t prec
  *          diagonal) and U.
  *   d_piv  device int32[n]; row k was swapped with row d_piv[k] at step k.
  * Runs on `stream` (NULL = the context stream) and synchronises it before returning.
- * The trailing updates are formed exactly from integer digits on the tensor cores and
- * rounded to FP64 once per panel; each panel is one cooperative launch (all CTAs resident,
- * one bounded grid barrier per column) when the device supports it.
+ * The trailing updates are formed from integer digits on the tensor cores and rounded to FP64 once
+ * per panel; the elements that are too small beside their row and column for the digits, by FP64
+ * fmas (elementwise backward error as with fmas throughout: |P A - L U| <= c n u |L| |U| per
+ * element).  Each panel is one cooperative launch (all CTAs resident, one bounded grid barrier per
+ * column) or one cluster, when the device supports it.
  * Allocates its work buffer (about (lu_block + 257) * n doubles and 1.1 MB) on the context's
  * device for the duration of the call.  An exact zero pivot (the whole remaining column is zero)
  * does not stop the factorisation: that column is left unscaled, the remaining columns

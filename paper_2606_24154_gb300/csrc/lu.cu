@@ -887,21 +887,22 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
                         continue;
                     }
                 } else if (tc64) {
+                    const T *L21 = A + k1 + k0 * n, *U12 = A + k0 + k1 * n;
                     T* C = A + k1 + k1 * n;
-                    NB_TRY(tc_split_f64(m, mc, w, A + k1 + k0 * n, n, A + k0 + k1 * n, n, split, s));
+                    NB_TRY(tc_split_f64(m, mc, w, L21, n, U12, n, split, s));
                     if (look && m >= kAheadFrom) {
-                        NB_TRY(tc_apply_f64(m, mc, 0, nb, C, n, split, d_info + 1, s));
+                        NB_TRY(tc_apply_f64(m, mc, w, 0, nb, L21, n, U12, n, C, n, split, d_info + 1, s));
                         NB_TRY(cudaEventRecord(ahead.ready, s));
                         NB_TRY(cudaStreamWaitEvent(ahead.stream, ahead.ready, 0));
                         ahead.joined = false;
                         NB_TRY(panel_step(k1, k1 + nb, ahead.stream));
                         NB_TRY(cudaEventRecord(ahead.done, ahead.stream));
-                        NB_TRY(tc_apply_f64(m, mc, nb, mc, C, n, split, d_info + 1, s));
+                        NB_TRY(tc_apply_f64(m, mc, w, nb, mc, L21, n, U12, n, C, n, split, d_info + 1, s));
                         NB_TRY(cudaStreamWaitEvent(s, ahead.done, 0));
                         ahead.joined = true;
                         panel_done = true;
                     } else {
-                        NB_TRY(tc_apply_f64(m, mc, 0, mc, C, n, split, d_info + 1, s));
+                        NB_TRY(tc_apply_f64(m, mc, w, 0, mc, L21, n, U12, n, C, n, split, d_info + 1, s));
                     }
                     continue;
                 }

@@ -2,33 +2,42 @@
 // C[M x N] -= A[M x K] B[K x N], K <= 64, column-major FP64, the update that follows each panel
 // (Sec. 4.1 / Alg. 1; almost all of the 2/3 n^3 operations).
 //
-// The FP64 pipe does two multiply-adds per SM and clock (1.24 TFLOP/s on 152 SMs).  Here the
-// product is formed exactly from integer digits on the FP16 tensor pipe, after the error-free
-// splitting of Ozaki, Ogita, Oishi and Rump ("Error-free transformations of matrix multiplication
-// by using fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
+// The FP64 pipe does two multiply-adds per SM and clock (1.24 TFLOP/s on 152 SMs).  Here most elements of
+// the product are formed from integer digits on the BF16 tensor pipe, after the splitting of Ozaki, Ogita,
+// Oishi and Rump ("Error-free transformations of matrix multiplication by using fast routines of matrix
+// multiplication", Numer. Algorithms 59, 2012), and the others by a chain of FP64 fmas:
 //   - Scaling.  g_k = exponent of the largest |B_kj| of row k; A_ik 2^g_k is scaled per row and
-//     B_kj 2^-g_k per column, both by powers of two, to 62-bit fixed point.  With g_k the split is
-//     unchanged when rows or columns of the factored matrix are scaled (conductor rows and interface
-//     rows differ by a factor of 1e6), which a split by rows and columns alone is not.
-//   - Digits.  Eight balanced base-256 digits (-128 .. 127) per number, exact in FP16: 64 bits,
-//     where an FP64 number has 53.
+//     B_kj 2^-g_k per column, both by powers of two, to 63-bit fixed point.  With g_k the split is unchanged
+//     when rows of the factored matrix are scaled, or dense columns (conductor rows and interface rows
+//     differ by a factor of 1e6).
+//   - Digits.  Eight balanced base-256 digits (-128 .. 128) per number, digit s held as digit x 256^-s, exact
+//     in BF16: 64 bits, where an FP64 number has 53.  An entry more than 10 binary places below the largest
+//     of its (scaled) row or column loses its last bits: at most 2^-64 of the scale.
 //   - Products.  The 36 digit products s + t <= 7 accumulate by d = s + t in eight FP32 accumulators:
-//     |sum| <= 8 terms x 64 x 2^14 = 2^23, so every partial sum is an integer that FP32 holds exactly.
-//     The products left out are below 2^-53 of (row scale x column scale) in the worst case and
-//     about 2^-59 for digits of random sign.
-//   - Epilogue.  The eight integers are joined to one 64-bit integer, rounded once to FP64 and
+//     |sum| <= 8 terms x 64 x 2^14 = 2^23 units, so every partial sum is an integer that FP32 holds exactly.
+//     The seven of s + t = 8 (below 2^15 of the units of d = 7) go to the accumulator of d = 7 first, where
+//     they are kept to a unit at worst.  The 21 products left out are below 2^-63 of
+//     row scale x column scale.
+//   - Epilogue.  The eight sums are joined to one integer, cut to 62 bits, rounded once to FP64 and
 //     subtracted from C by one fma: two FP64 instructions per element instead of 64.
-// Against 64 fmas in a row, whose roundings add up, the result is the more accurate one.
+//   - Elements that are small beside their row and column.  All errors above stay within 2^-57 of row scale x
+//     column scale (64 terms with two entries off by 2^-64 each).  The chain's bound is 64 x 2^-53 of
+//     |C_ij| + sum_k |A_ik B_kj|.  So where |C_ij| or the result's own sum reaches 2^-10 of row scale x column
+//     scale, the digits keep the chain's bound element by element (their largest error there is a sixth of the
+//     chain's).  The other elements (take_off: false), those of rows or columns that are not finite and those
+//     at the ends of the exponent range are formed by fmas.  Random matrices: 5 in 100,000 elements; THGEM
+//     cells of 4,632, 2,100 and 828 elements: 0.04, 0.13 and 0.7 %; two groups of rows and columns coupled by
+//     1e-4 or less: the coupled half, which then costs what it costs on the FP64 pipe.
 //
 // One CTA per SM (192 KB of shared memory): the A digits of 128 rows (128 KB) once, then the
-// B digits of 64 columns (64 KB) tile by tile; 144 MMAs (M 128, N 64, K 16) per tile into the whole of
+// B digits of 64 columns (64 KB) tile by tile; 172 MMAs (M 128, N 64, K 16) per tile into the whole of
 // tensor memory (8 x 64 columns).  The next tile's B digits are copied while the epilogue runs.
 // The epilogue's FP64 and conversion instructions and the MMAs' shared-memory reads take about
 // the same time, and share a CTA in turn.  Every wait is bounded.
 //
-// Measured, LU of a random matrix of order 6145: the updates 142 ms on the FP64 pipe, 15 ms here; the
-// whole factorisation 234 -> 40 ms, |P A - L U| / |A| 3.4e-14 -> 2.7e-14.
-#include <cuda_fp16.h>
+// Measured, LU of a random matrix of order 6145: 234 ms with the updates (142 ms) on the FP64 pipe, 41.4 ms so;
+// with every second row and column in a group coupled by 1e-4 or 1e-12, 234 and 210 ms; one in 32, 234 and 73 ms.
+#include <cuda_bf16.h>
 
 #include <algorithm>
 
@@ -41,17 +50,19 @@ namespace {
 
 constexpr int kDM = 128, kDN = 64, kDK = 64, kDig = 8;
 constexpr int kDThreads = 256;
-constexpr uint32_t kDLbo = 128;                       // next core matrix (8 rows x 8 halves) along K
+constexpr uint32_t kDLbo = 128;                       // next core matrix (8 rows x 8 values) along K
 constexpr uint32_t kDSbo = (kDK / 8) * 128;           // next 8-row group
 constexpr uint32_t kDPlaneA = kDM * kDK * 2;          // 16 KB: one digit of the A tile
 constexpr uint32_t kDPlaneB = kDN * kDK * 2;          // 8 KB
 constexpr uint32_t kDTileA = kDig * kDPlaneA, kDTileB = kDig * kDPlaneB;
 constexpr uint32_t kDSmem = kDTileA + kDTileB + 64;
 constexpr int kNonFinite = 1 << 24;                   // exponent mark of a row or column with Inf or NaN
+constexpr int kZeroMark = -16384;                     // of a row or column of zeros: below every exponent
+constexpr int kFixed = 10;                            // binary places that the largest mantissa (53 bits) is raised by
 
-// instruction descriptor, kind::f16: D = F32 (bits 4-5 = 1), A = B = F16 (0), both K-major, N >> 3 at
-// bits 17-22, M >> 4 at bits 24-28
-constexpr uint32_t kDIdesc = (1u << 4) | ((uint32_t)(kDN >> 3) << 17) | ((uint32_t)(kDM >> 4) << 24);
+// instruction descriptor, kind::f16: D = F32 (bits 4-5 = 1), A = B = BF16 (1 at bits 7-9 and 10-12), both
+// K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
+constexpr uint32_t kDIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kDN >> 3) << 17) | ((uint32_t)(kDM >> 4) << 24);
 
 __device__ __forceinline__ uint64_t digit_desc(uint32_t saddr) {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kDLbo >> 4) << 16) | ((uint64_t)(kDSbo >> 4) << 32) |
@@ -74,8 +85,8 @@ __global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ B, 
     if (k < K) atomicMax(&g[k], e);
 }
 
-// x 2^shift as a 62-bit fixed-point number: mantissa m (53 bits) shifted by sh = 9 - (top - e)
-__device__ __forceinline__ long long fixed62(unsigned long long bits, int sh) {
+// x 2^shift as a 63-bit fixed-point number: mantissa m (53 bits) shifted by sh = kFixed - (top - e)
+__device__ __forceinline__ long long fixed63(unsigned long long bits, int sh) {
     const unsigned long long mag = bits & ~(1ull << 63);
     unsigned long long m = mag & ((1ull << 52) - 1);
     if (mag >> 52) m |= 1ull << 52;
@@ -86,20 +97,27 @@ __device__ __forceinline__ long long fixed62(unsigned long long bits, int sh) {
     return (bits >> 63) ? -(long long)m : (long long)m;
 }
 
-// eight numbers (consecutive k) to eight digit planes, 16 bytes each
+// 256^d, d <= 8
+__host__ __device__ constexpr float pow256(int d) {
+    float p = 1.f;
+    for (int i = 0; i < d; ++i) p *= 256.f;
+    return p;
+}
+
+// eight numbers (consecutive k) to eight digit planes (digit s x 256^-s), 16 bytes each
 __device__ __forceinline__ void store_digits(const unsigned long long (&v)[8], const int (&sh)[8],
                                              unsigned char* __restrict__ dst, uint32_t plane) {
     long long x[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) x[q] = fixed62(v[q], sh[q]);
+    for (int q = 0; q < 8; ++q) x[q] = fixed63(v[q], sh[q]);
 #pragma unroll
     for (int s = kDig - 1; s >= 0; --s) {
-        alignas(16) __half h[8];
+        alignas(16) __nv_bfloat16 h[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int d = s ? (int)(signed char)(x[q] & 255) : (int)x[q];
             x[q] = (x[q] - d) >> 8;
-            h[q] = __int2half_rn(d);
+            h[q] = __float2bfloat16_rn((float)d * (1.f / pow256(s)));
         }
         *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = *reinterpret_cast<const uint4*>(h);
     }
@@ -115,7 +133,7 @@ __global__ void __launch_bounds__(256) k_split_digits(const double* __restrict__
                                                       int* __restrict__ ea, int* __restrict__ eb) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long v[8];
-    int sh[8], top = 0;
+    int sh[8], top = kZeroMark;
     if ((int64_t)blockIdx.x < blocks_a) {
         __shared__ int s_top[8][32];
         const int64_t row = (int64_t)blockIdx.x * 32 + lane;
@@ -136,7 +154,7 @@ __global__ void __launch_bounds__(256) k_split_digits(const double* __restrict__
         for (int w = 0; w < 8; ++w) top = max(top, s_top[w][lane]);
         if (warp == 0) ea[row] = top;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) sh[q] = top >= kNonFinite ? -64 : 9 - (top - sh[q]);
+        for (int q = 0; q < 8; ++q) sh[q] = top >= kNonFinite ? -64 : kFixed - (top - sh[q]);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             if (!(v[q] << 1)) sh[q] = 0;
@@ -146,7 +164,6 @@ __global__ void __launch_bounds__(256) k_split_digits(const double* __restrict__
     } else {
         const int64_t col = ((int64_t)blockIdx.x - blocks_a) * 32 + warp * 4 + lane / 8;
         const int kg = lane % 8;
-        top = -8192;  // a zero column's mark: below every exponent
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int k = 8 * kg + q;
@@ -162,7 +179,7 @@ __global__ void __launch_bounds__(256) k_split_digits(const double* __restrict__
         for (int o = 1; o < 8; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
         if (kg == 0) eb[col] = top;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) sh[q] = top >= kNonFinite ? -64 : 9 - (top - sh[q]);
+        for (int q = 0; q < 8; ++q) sh[q] = top >= kNonFinite ? -64 : kFixed - (top - sh[q]);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             if (!(v[q] << 1)) sh[q] = 0;
@@ -179,28 +196,68 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8]) {
                  : "r"(addr));
 }
 
-// c - (sum of acc_d 256^(7-d)) 2^(56 + e0), the eight sums given as exact FP32 integers, e = the
-// exponents of row and column added up.
-__device__ __forceinline__ double take_off(double c, const uint32_t (&a)[kDig], int e) {
+// c -= T 2^(e - 2114), T = sum of acc_d 256^(7 - d) for the eight sums (integers; the last one with a
+// fraction) of e = the exponents of row and column added up, row scale x column scale = 2^(e - 2044).
+// false, and c as it was, where neither c nor the product reaches 2^-10 of the scale, or a power of two needed
+// here is outside the normal range (also: a row or column that is not finite).
+__device__ __forceinline__ bool take_off(double& c, const uint32_t (&a)[kDig], int e) {
     int i[kDig];
 #pragma unroll
-    for (int d = 0; d < kDig; ++d) i[d] = __float2int_rn(__uint_as_float(a[d]));
+    for (int d = 0; d < kDig; ++d) i[d] = __float2int_rn(__uint_as_float(a[d]) * pow256(d));
+    // T = 2^32 H + L, |H| < 2^44.1, |L| < 2^46.5
     const long long H = (long long)((i[0] << 8) + i[1]) * 65536 + ((i[2] << 8) + i[3]);
     const long long L = (long long)((i[4] << 8) + i[5]) * 65536 + ((i[6] << 8) + i[7]);
-    // |H| < 2^42.2 (top digits <= 65); the low part rounded to nearest: cut off, it would lean every
-    // element of every update the same way (the residual of n = 6145 was 2.4 times the chain's)
-    const double t = (double)((H << 20) + ((L + 2048) >> 12));  // units of 2^68 of the digit product
-    const int x = e - 2100 + 1023;
-    if (x > 0 && x < 2047) return __fma_rn(-t, __longlong_as_double((long long)x << 52), c);
-    if (e >= kNonFinite / 2) return __longlong_as_double(0x7ff8000000000000ll);
-    return c - scalbn(t, max(-3000, e - 2100));
+    const long long mag = H < 0 ? -H : H;
+    const int ec = (__double2hiint(c) >> 20) & 0x7ff;
+    if (e <= 1091 || e >= 3122 || (mag < (1ll << 28) && ec < e - 1031)) return false;
+    // t = T 2^-s of at most 62 bits, rounded to nearest (cut off, it would lean every element of every
+    // update the same way); |t| >= 2^60 where s > 0
+    const int s = max(0, 35 - __clzll(mag));
+    const long long t = (H << (32 - s)) + ((L + ((1ll << s) >> 1)) >> s);
+    c = __fma_rn(-(double)t, __longlong_as_double((long long)(e - 2114 + 1023 + s) << 52), c);
+    return true;
 }
 
-// (bounds: 168 registers, so that a CTA of the next panel fits beside this one)
+// The elements of the warp's 32 rows (from row0) and 32 columns (from n0) whose bits are set in the lanes'
+// masks: C_ij -= sum_k A_ik B_kj by fmas.  Few rows of a column: the 64 terms of one element side by side
+// (seven FP64 instructions); from kRedoRows on a chain per row (64 for all of them).
+constexpr int kRedoRows = 9;
+__device__ __noinline__ void redo(unsigned mask, int64_t row0, int64_t n0, int K, const double* __restrict__ A,
+                                  int64_t lda, const double* __restrict__ B, int64_t ldb, double* C, int64_t ldc) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned any = __reduce_or_sync(0xffffffffu, mask); any; any &= any - 1) {
+        const int j = __ffs(any) - 1;
+        const double* b = B + (n0 + j) * ldb;
+        double* c = C + row0 + (n0 + j) * ldc;
+        unsigned who = __ballot_sync(0xffffffffu, (mask >> j) & 1u);
+        if (__popc(who) >= kRedoRows) {
+            if ((who >> lane) & 1u) {
+                double acc = 0.0;
+#pragma unroll 8
+                for (int k = 0; k < K; ++k) acc = __fma_rn(A[row0 + lane + (int64_t)k * lda], b[k], acc);
+                c[lane] = __dsub_rn(c[lane], acc);
+            }
+            continue;
+        }
+        const double b0 = lane < K ? b[lane] : 0.0, b1 = lane + 32 < K ? b[lane + 32] : 0.0;
+        for (; who; who &= who - 1) {
+            const int r = __ffs(who) - 1;
+            double v = lane < K ? __dmul_rn(A[row0 + r + (int64_t)lane * lda], b0) : 0.0;
+            if (lane + 32 < K) v = __fma_rn(A[row0 + r + (int64_t)(lane + 32) * lda], b1, v);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (lane == r) c[lane] = __dsub_rn(c[lane], v);
+        }
+    }
+}
+
+// (launched with kDThreads; bounds of 384 threads: 168 registers, so that a CTA of the next panel fits beside)
 __global__ void __launch_bounds__(384, 1)
-    k_tc_update_f64(int64_t M, int64_t N, const unsigned char* __restrict__ da, const unsigned char* __restrict__ db,
-                    const int* __restrict__ ea, const int* __restrict__ eb, double* __restrict__ C, int64_t ldc,
-                    int64_t tile0, int64_t tile1, int tpc, int* __restrict__ err) {
+    k_tc_update_f64(int64_t M, int64_t N, int K, const double* __restrict__ A, int64_t lda,
+                    const double* __restrict__ B, int64_t ldb, const unsigned char* __restrict__ da,
+                    const unsigned char* __restrict__ db, const int* __restrict__ ea, const int* __restrict__ eb,
+                    double* __restrict__ C, int64_t ldc, int64_t tile0, int64_t tile1, int tpc,
+                    int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* sA = smem;
     unsigned char* sB = smem + kDTileA;
@@ -248,17 +305,21 @@ __global__ void __launch_bounds__(384, 1)
         ++used_b;
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (tid == 0) {
-            for (int d = 0; d < kDig; ++d)
-                for (int s = 0; s <= d; ++s)
+            bool first = true;
+            for (int d = kDig; d >= 0; --d) {  // d = 8 before d = 7, into the same sums
+                if (d < kDig - 1) first = true;
+                for (int s = max(0, d - kDig + 1); s <= min(d, kDig - 1); ++s)
                     for (int ks = 0; ks < kDK / 16; ++ks) {
                         const uint64_t ad = digit_desc(smem_u32(sA + s * kDPlaneA) + (uint32_t)ks * 2u * kDLbo);
                         const uint64_t bd = digit_desc(smem_u32(sB + (d - s) * kDPlaneB) + (uint32_t)ks * 2u * kDLbo);
                         asm volatile(
                             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
-                                tmem + (uint32_t)(d * kDN)),
-                            "l"(ad), "l"(bd), "r"(kDIdesc), "r"((s | ks) ? 1u : 0u));
+                                tmem + (uint32_t)(min(d, kDig - 1) * kDN)),
+                            "l"(ad), "l"(bd), "r"(kDIdesc), "r"(first ? 0u : 1u));
+                        first = false;
                     }
+            }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                 smem_u32(barM)));
         }
@@ -279,6 +340,7 @@ __global__ void __launch_bounds__(384, 1)
             if (tid == 0) load_b(t + 1);  // the MMAs have read B
             ++loads;
         }
+        unsigned again = 0;  // columns of this thread's row that the digits are too coarse for
 #pragma unroll
         for (int cb = 0; cb < kDN / 2; cb += 8) {
             uint32_t v[kDig][8];
@@ -295,12 +357,18 @@ __global__ void __launch_bounds__(384, 1)
                 uint32_t a[kDig];
 #pragma unroll
                 for (int d = 0; d < kDig; ++d) a[d] = v[d][j];
-                if (row < M && n0 + cb + j < N)
-                    C[row + (n0 + cb + j) * ldc] = take_off(c[cb + j], a, er + eb[n0 + cb + j]);
+                const int e = er + eb[n0 + cb + j];  // (padded to whole tiles)
+                if (row < M && n0 + cb + j < N && e > kZeroMark / 2) {
+                    if (take_off(c[cb + j], a, e))
+                        C[row + (n0 + cb + j) * ldc] = c[cb + j];
+                    else
+                        again |= 1u << (cb + j);
+                }
             }
         }
         // the next tile's MMAs overwrite the accumulators: every warp's reads come first
         asm volatile("tcgen05.fence::before_thread_sync;");
+        if (__any_sync(0xffffffffu, again)) redo(again, row - lane, n0, K, A, lda, B, ldb, C, ldc);
     }
     if (!ok) {
         if (tid == 0) {
@@ -357,8 +425,8 @@ cudaError_t tc_split_f64(int64_t M, int64_t N, int64_t K, const double* A, int64
     return cudaGetLastError();
 }
 
-cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t c0, int64_t c1, double* C, int64_t ldc, void* work, int* err,
-                         cudaStream_t s) {
+cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t K, int64_t c0, int64_t c1, const double* A, int64_t lda,
+                         const double* B, int64_t ldb, double* C, int64_t ldc, void* work, int* err, cudaStream_t s) {
     c1 = std::min(c1, N);
     if (M <= 0 || c0 >= c1) return cudaSuccess;
     if (c0 % kDN || !work) return cudaErrorInvalidValue;
@@ -370,7 +438,8 @@ cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t c0, int64_t c1, double* C
     const int64_t tiles_m = pad_to(M, kDM) / kDM, tile0 = c0 / kDN, tile1 = (c1 + kDN - 1) / kDN, tiles_n = tile1 - tile0;
     const int64_t tpc = std::max<int64_t>(1, std::min<int64_t>(8, tiles_m * tiles_n / (3 * 152)));
     dim3 grid((unsigned)tiles_m, (unsigned)((tiles_n + tpc - 1) / tpc));
-    k_tc_update_f64<<<grid, kDThreads, kDSmem, s>>>(M, N, t.da, t.db, t.ea, t.eb, C, ldc, tile0, tile1, (int)tpc, err);
+    k_tc_update_f64<<<grid, kDThreads, kDSmem, s>>>(M, N, (int)K, A, lda, B, ldb, t.da, t.db, t.ea, t.eb, C, ldc, tile0,
+                                                    tile1, (int)tpc, err);
     return cudaGetLastError();
 }
 

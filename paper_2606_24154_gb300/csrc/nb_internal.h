@@ -244,15 +244,15 @@ cudaError_t tc_update_f32_k(int64_t M, int64_t N, int64_t K, const float* A, int
                             int64_t ldb, float* C, int64_t ldc, void* split, int* err, cudaStream_t s);
 size_t tc_split_bytes(int64_t M, int64_t N, int kc);
 
-// FP64 through exact digit products on the FP16 tensor pipe (lu_tc64.cu); work: tc64_work_bytes(M, N)
-// bytes, 256-byte aligned; *err is set if a bounded wait gave up.
+// FP64 through integer digits on the tensor pipe, with FP64 fmas for the elements that the digits are too coarse
+// for (lu_tc64.cu); work: tc64_work_bytes(M, N) bytes, 256-byte aligned; *err is set if a bounded wait gave up.
 size_t tc64_work_bytes(int64_t M, int64_t N);
 // C[M x N] -= A[M x K] B[K x N] in two steps: the digits of A and B (K <= 64) to work (tc64_work_bytes), then the
-// columns [c0, c1) of C (c0 a multiple of 64)
+// columns [c0, c1) of C (c0 a multiple of 64) from them and from A and B themselves
 cudaError_t tc_split_f64(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B, int64_t ldb,
                          void* work, cudaStream_t s);
-cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t c0, int64_t c1, double* C, int64_t ldc, void* work, int* err,
-                         cudaStream_t s);
+cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t K, int64_t c0, int64_t c1, const double* A, int64_t lda,
+                         const double* B, int64_t ldb, double* C, int64_t ldc, void* work, int* err, cudaStream_t s);
 
 // Dense LU (column-major, lda = n).  d_info: two ints (first zero pivot, tensor-core timeout).  Scratch: pivots int32[n], work as documented in lu.cu.
 // lu_factor_f64: work of lu_work_bytes_f64(n, nb) bytes (256-byte aligned); lu_factor_f64_small: work
