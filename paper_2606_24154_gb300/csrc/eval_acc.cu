@@ -173,12 +173,8 @@ __host__ __device__ __forceinline__ bool lane_path(const SplitPlan& plan, int64_
     return plan.leaf && plan.Gm == 0 && (count + kLP - 1) / kLP * plan.np < kLaneRounds * gb;
 }
 struct LaneScratch {
-    struct Val {  // d: sigma, Phi', E'; for the scales a: |Phi'|, |E'|_1 (level 2), f: |sigma|, |Phi'|, |E'|_1 (level 1)
-        double d[5];
-        union {
-            double a[2];
-            float f[3];
-        };
+    struct Val {  // d: sigma, Phi', E'; for the scales a: |Phi'|, |E'|_1
+        double d[5], a[2];
     };
     Val val[kAT / 32][32];
     double out[kLP][6];
@@ -398,7 +394,6 @@ __device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, fl
     const float4* gmom = L == 1 ? A.mom : A.mom2;
     constexpr int kGM = L == 1 ? kMomF4 : kFillMomF4;
     Sum6 acc{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    float bphi = 0.f, bE = 0.f;  // level 1: the leaf's error scales in FP32
     for (int64_t base = e0; base < e1; base += te) {
         const int cnt = (int)min((int64_t)te, e1 - base);
         __syncthreads();
@@ -441,30 +436,19 @@ __device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, fl
             if constexpr (!LANES) {
                 if constexpr (M != kEOnly) {
                     acc.phi = fma(s, v.phi, acc.phi);
-                    if (L == 1)
-                        bphi = fmaf(fabsf((float)s), fabsf((float)v.phi), bphi);
-                    else
-                        acc.bphi = fma(fabs(s), fabs(v.phi), acc.bphi);
+                    acc.bphi = fma(fabs(s), fabs(v.phi), acc.bphi);
                 }
                 if constexpr (M != kPhiOnly) {
                     acc.x = fma(s, v.x, acc.x);
                     acc.y = fma(s, v.y, acc.y);
                     acc.z = fma(s, v.z, acc.z);
-                    if (L == 1)
-                        bE = fmaf(fabsf((float)s), fabsf((float)v.x) + fabsf((float)v.y) + fabsf((float)v.z), bE);
-                    else
-                        acc.bE = fma(fabs(s), fabs(v.x) + fabs(v.y) + fabs(v.z), acc.bE);
+                    acc.bE = fma(fabs(s), fabs(v.x) + fabs(v.y) + fabs(v.z), acc.bE);
                 }
                 continue;
             }
             LaneScratch::Val& o = scr->val[w][lane];
             o.d[0] = s, o.d[1] = v.phi, o.d[2] = v.x, o.d[3] = v.y, o.d[4] = v.z;
-            if (L == 1) {
-                o.f[0] = fabsf((float)s), o.f[1] = fabsf((float)v.phi);
-                o.f[2] = fabsf((float)v.x) + fabsf((float)v.y) + fabsf((float)v.z);
-            } else {
-                o.a[0] = fabs(v.phi), o.a[1] = fabs(v.x) + fabs(v.y) + fabs(v.z);
-            }
+            o.a[0] = fabs(v.phi), o.a[1] = fabs(v.x) + fabs(v.y) + fabs(v.z);
             __syncwarp();
             // chain `which` (0 to 5) of a point by one lane, in the order of the elements
             const int m = min(per, kWP - t * per);
@@ -473,22 +457,14 @@ __device__ __forceinline__ Sum6 acc_range(const AccView& A, int nimg, int te, fl
                 const LaneScratch::Val* r = scr->val[w] + qq * te;
                 double& dst = scr->out[w * kWP + t * per + qq][which];
                 double x = dst;
-                float y = (float)x;
                 const bool scale = which >= 4;
-                for (int e = 0; e < cnt; ++e) {
-                    if (L == 1) {
-                        x = fma(r[e].d[0], r[e].d[scale ? 1 : 1 + which], x);
-                        y = fmaf(r[e].f[0], r[e].f[scale ? which - 3 : 1], y);
-                    } else {
-                        x = fma(scale ? fabs(r[e].d[0]) : r[e].d[0], scale ? r[e].a[which - 4] : r[e].d[1 + which], x);
-                    }
-                }
-                dst = L == 1 && scale ? (double)y : x;
+                for (int e = 0; e < cnt; ++e)
+                    x = fma(scale ? fabs(r[e].d[0]) : r[e].d[0], scale ? r[e].a[which - 4] : r[e].d[1 + which], x);
+                dst = x;
             }
             __syncwarp();
         }
     }
-    if (L == 1) acc.bphi = (double)bphi, acc.bE = (double)bE;
     return acc;
 }
 
