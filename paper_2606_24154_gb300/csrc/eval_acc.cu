@@ -670,14 +670,16 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
                          double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list,
                          int32_t* next, int sms, Sum6* part, cudaStream_t s) {
     // element tile: a power of two (divides the leaf), within ~40 KB
+    constexpr int kSmem = 40 * 1024;
     int te = kLeafEl;
-    while (te > 1 && acc_tile_f4(L, te, img.n) * (int)sizeof(float4) > 40 * 1024) te /= 2;
+    while (te > 1 && acc_tile_f4(L, te, img.n) * (int)sizeof(float4) > kSmem) te /= 2;
     const size_t smem = (size_t)acc_tile_f4(L, te, img.n) * sizeof(float4), lane_smem = smem + sizeof(LaneScratch);
     const int64_t gb = kATBlocks * (int64_t)sms, want = (npts + kAT - 1) / kAT;
     cudaError_t e;
     // the list's length is known on the device: both kernels are launched unless even the whole input is short
     if (!lane_path(split_plan(want, gb, A.n_el), npts, gb)) {
-        e = cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // one value whatever the tile: another thread's call may be between this and its launch
+        e = cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
         const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
         k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, next, gb,
@@ -685,7 +687,8 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(k_eval_acc_lanes<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lane_smem);
+    e = cudaFuncSetAttribute(k_eval_acc_lanes<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmem + (int)sizeof(LaneScratch));
     if (e != cudaSuccess) return e;
     k_eval_acc_lanes<L, M><<<(unsigned)std::min<int64_t>(4 * (int64_t)sms, split_count(npts, kLP) * split_count(A.n_el, kLeafEl)),
                              kAT, lane_smem, s>>>(A, img.n, te, pts, list, n_list, gb, part);

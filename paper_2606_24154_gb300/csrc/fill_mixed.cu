@@ -402,10 +402,12 @@ cudaError_t launch_fill_mixed(const Elem* el, const FillEl* fe, const float4* no
                               const int32_t* cell_items, double* K, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     // column tile: as many elements as fit in ~40 KB (four blocks per SM), at most 16
+    constexpr int kSmem = 40 * 1024;
     int te = 16;
-    while (te > 1 && fill_tile_f4(te, img.n) * (int)sizeof(float4) > 40 * 1024) --te;
+    while (te > 1 && fill_tile_f4(te, img.n) * (int)sizeof(float4) > kSmem) --te;
     const size_t smem = (size_t)fill_tile_f4(te, img.n) * sizeof(float4);
-    cudaError_t e = cudaFuncSetAttribute(k_fill_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // one value whatever the tile: another thread's call may be between this and its launch
+    cudaError_t e = cudaFuncSetAttribute(k_fill_far, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
     int cols = 0;
     e = fill_cols(n, kFT, kFillBlocks, &cols);

@@ -181,6 +181,9 @@ __global__ void __launch_bounds__(kPivThreads, 2) k_panel_col(T* __restrict__ A,
 constexpr int kCoopThreads = 256;
 constexpr int kCoopMaxG = kCoopThreads;  // one reading thread per CTA of the grid
 constexpr long long kCoopSpinLimit = 1ll << 22;
+// The kernels' shared-memory limits are set to one value each, whatever the call's size: a limit belongs to the
+// function, and another thread's call of another size may be between its setting and its launches.
+constexpr int kCoopSmemMax = 200 * 1024;
 
 // A magnitude as it is compared: its bits (non-negative numbers order as their bits, and integer
 // compares leave the FP64 pipe alone).  NaN never wins: -1.
@@ -753,8 +756,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
             const int64_t R0 = std::max<int64_t>(kCoopMinRows<T>, (n + g - 1) / g);
             const int64_t smem0 = R0 * 64 * (int64_t)sizeof(T);
             int per_sm = 0;
-            if (smem0 <= 200 * 1024 &&
-                cudaFuncSetAttribute(k_panel_coop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) ==
+            if (smem0 <= kCoopSmemMax &&
+                cudaFuncSetAttribute(k_panel_coop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoopSmemMax) ==
                     cudaSuccess &&
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_coop<T>, kCoopThreads, (size_t)smem0) ==
                     cudaSuccess &&
@@ -809,7 +812,8 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
     };
     auto trsm_block = [&](int64_t r0, int nbk, const T* inv, int64_t c0, int64_t c1) -> cudaError_t {
         const int smem = (int)trsm_block_smem<T>(nbk);
-        NB_TRY(cudaFuncSetAttribute(k_trsm_block<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        NB_TRY(cudaFuncSetAttribute(k_trsm_block<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)trsm_block_smem<T>(kSuperPanels)));
         k_trsm_block<T><<<(unsigned)((c1 - c0 + kTrsmCols<T> - 1) / kTrsmCols<T>), 256, smem, s>>>(A, n, r0, nbk, inv,
                                                                                                   c0, c1);
         return cudaGetLastError();
