@@ -109,8 +109,9 @@ typedef struct nebem_options {
     double sc_near;          /* space charge: pairs closer than this (m) form the FP32
                                 difference from exact two-float coordinates (default 1e-4) */
     int32_t lu_block;        /* LU panel width, 32 or 64 (default 64) */
-    int32_t wait_polls;      /* poll limit of the software waits on the device (the FP32
-                                panel's grid barrier, the triangular sweeps' block flags);
+    int32_t wait_polls;      /* poll limit of the software waits on the device (in
+                                nebem_solve, the factorisation panels' grid barrier; the
+                                triangular sweeps' waits for the blocks before);
                                 0 = 4,194,304 polls (about 0.1-0.3 s).  A wait that runs out
                                 gives NEBEM_TIMEOUT (see nebem_solve); default 0 */
     double mixed_point_tol;  /* mixed eval: a point whose estimated error exceeds this fraction

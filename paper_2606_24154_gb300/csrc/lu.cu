@@ -1571,12 +1571,13 @@ static size_t coop64_offset(int64_t n, int nb) {
     return (digits_offset(n, nb) + tc64_work_bytes(n, n) + 255) & ~(size_t)255;
 }
 size_t lu_work_bytes_f64(int64_t n, int nb) { return coop64_offset(n, nb) + sizeof(CoopScratch<double>); }
-cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, void* work, int* d_info, cudaStream_t s) {
+cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, void* work, int* d_info, cudaStream_t s,
+                          long long polls) {
     // work: panel staging, then the digits of the tensor-core update, then the cooperative
     // panel's candidates and barrier
     char* w = static_cast<char*>(work);
     return lu_factor<double>(A, n, piv, nb, reinterpret_cast<double*>(w), d_info, w + digits_offset(n, nb),
-                             w + coop64_offset(n, nb), s, 0);
+                             w + coop64_offset(n, nb), s, polls);
 }
 static size_t split_offset(int64_t n, int nb) { return (sizeof(float) * lu_work_elems(n, nb) + 255) & ~(size_t)255; }
 static size_t coop_offset(int64_t n, int nb) {

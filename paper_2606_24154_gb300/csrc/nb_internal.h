@@ -255,14 +255,15 @@ cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t K, int64_t c0, int64_t c1
                          const double* B, int64_t ldb, double* C, int64_t ldc, void* work, int* err, cudaStream_t s);
 
 // Dense LU (column-major, lda = n).  d_info: two ints (first zero pivot, tensor-core timeout).  Scratch: pivots int32[n], work as documented in lu.cu.
-// lu_factor_f64: work of lu_work_bytes_f64(n, nb) bytes (256-byte aligned); lu_factor_f64_small: work
-// of lu_work_elems(n, nb) doubles, a launch per panel column and FP64-pipe updates.
-cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, void* work, int* d_info, cudaStream_t s);
+// lu_factor_f64_small: work of lu_work_elems(n, nb) doubles, a launch per panel column and FP64-pipe updates.
 cudaError_t lu_factor_f64_small(double* A, int64_t n, int32_t* piv, int nb, double* work, int* d_info,
                                 cudaStream_t s);
 size_t lu_work_bytes_f64(int64_t n, int nb);
+// lu_factor_f64: work of lu_work_bytes_f64(n, nb) bytes (256-byte aligned).
 // polls > 0: poll limit of the software waits (the cooperative panel's grid barrier, the
-// triangular sweeps' block flags); 0 = their defaults
+// triangular sweeps' passed values); 0 = their defaults
+cudaError_t lu_factor_f64(double* A, int64_t n, int32_t* piv, int nb, void* work, int* d_info, cudaStream_t s,
+                          long long polls = 0);
 cudaError_t lu_factor_f32(float* A, int64_t n, int32_t* piv, int nb, float* work, int* d_info,
                           cudaStream_t s, long long polls = 0);
 size_t lu_work_elems(int64_t n, int nb);

@@ -99,7 +99,7 @@ int ensure_factors(Ctx* c, int precision, double* ms) {
         CK(cudaEventRecord(c->ev0, c->stream));
         CK(cudaMemcpyAsync(c->d_LU64.ptr, c->d_K.ptr, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, c->stream));
         CK(lu_factor_f64(c->d_LU64.as<double>(), n, c->d_piv64.as<int32_t>(), nb, c->d_work.ptr,
-                         c->d_small.as<int>(), c->stream));
+                         c->d_small.as<int>(), c->stream, c->opt.wait_polls));
         int rc = elapsed_ms(c, ms);
         if (rc) return rc;
         int h2[2] = {0, 0};
