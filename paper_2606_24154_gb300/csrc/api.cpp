@@ -514,9 +514,9 @@ int nebem_lu_factor_device(nebem_ctx* ctx, double* d_A, int64_t n, int32_t* d_pi
     cudaStream_t s = stream ? (cudaStream_t)stream : c->stream;
     const int nb = c->opt.lu_block;
     DevBuf work, info;
-    CK(work.ensure(lu_work_bytes_f64(n, nb)));
     CK(info.ensure(2 * sizeof(int)));
-    CK(lu_factor_f64(d_A, n, d_piv, nb, work.ptr, info.as<int>(), s));
+    const int rc = factor_f64(c, d_A, n, d_piv, work, info.as<int>(), s, 0);
+    if (rc) return rc;
     int h2[2] = {0, 0};
     CK(cudaMemcpyAsync(h2, info.ptr, sizeof(h2), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

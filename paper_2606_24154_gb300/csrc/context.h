@@ -136,6 +136,8 @@ int ensure_fill(Ctx* c, int precision, double* ms);
 int ensure_factors(Ctx* c, int precision, double* ms);
 int build_rhs(Ctx* c);
 int solve_with_factors(Ctx* c, int precision, nebem_solve_info* info);
+// FP64 factorisation in place with work space in `work` (grown; less of it where the device has no room)
+int factor_f64(Ctx* c, double* A, int64_t n, int32_t* piv, DevBuf& work, int* d_info, cudaStream_t s, long long polls);
 // k weighting-field solutions (unit potential on readout[j], 0 on the other conductors, no
 // known charges) into c->d_wX (n x k, column-major) with the retained factors
 int weighting_solve(Ctx* c, const int32_t* readout, int k, int precision, nebem_solve_info* info);

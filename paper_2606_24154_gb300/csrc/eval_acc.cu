@@ -520,11 +520,11 @@ template <int L, int M>
 __global__ void __launch_bounds__(kAT, kATBlocks)
     k_eval_acc_far(const AccView A, int nimg, int te, const double* __restrict__ pts,
                    const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int32_t* next, int64_t gb,
-                   Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
+                   int64_t cap, Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
                    double* __restrict__ err, float4* __restrict__ bound) {
     extern __shared__ float4 sm[];
     const int64_t count = *n_list;
-    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el, cap);
     if (lane_path(plan, count, gb)) return;
     const int64_t units = plan.Gm + plan.R * plan.np;
     __shared__ int s_unit;
@@ -555,10 +555,10 @@ template <int L, int M>
 __global__ void __launch_bounds__(kAT, 4)
     k_eval_acc_lanes(const AccView A, int nimg, int te, const double* __restrict__ pts,
                      const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
-                     Sum6* __restrict__ part) {
+                     int64_t cap, Sum6* __restrict__ part) {
     extern __shared__ float4 sm[];
     const int64_t count = *n_list;
-    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el);
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, A.n_el, cap);
     if (!lane_path(plan, count, gb)) return;
     const int64_t lg = (count + kLP - 1) / kLP;
     const LaneScratch* scr = reinterpret_cast<LaneScratch*>(sm + acc_tile_f4(L, te, nimg));
@@ -582,10 +582,10 @@ __global__ void __launch_bounds__(kAT, 4)
 template <int L, int M>
 __global__ void __launch_bounds__(256)
     k_acc_reduce(int64_t n_el, const int32_t* __restrict__ list, const int32_t* __restrict__ n_list, int64_t gb,
-                 const Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
+                 int64_t cap, const Sum6* __restrict__ part, double* __restrict__ phi, double* __restrict__ E,
                  double* __restrict__ err, float4* __restrict__ bound) {
     const int64_t count = *n_list;
-    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, n_el);
+    const SplitPlan plan = split_plan((count + kAT - 1) / kAT, gb, n_el, cap);
     const int64_t first = plan.Gm * kAT, warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; first + w < count; w += warps) {
         const Sum6 tot = split_reduce(part + w * plan.np, plan.np, plan.leaf);
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(256)
 template <int L, int M>
 cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* pts, int64_t npts, double* phi,
                          double* E, double* err, float4* bound, const int32_t* list, const int32_t* n_list,
-                         int32_t* next, int sms, Sum6* part, cudaStream_t s) {
+                         int32_t* next, int sms, Sum6* part, int64_t cap, cudaStream_t s) {
     // element tile: a power of two (divides the leaf), within ~40 KB
     constexpr int kSmem = 40 * 1024;
     int te = kLeafEl;
@@ -677,13 +677,13 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
     const int64_t gb = kATBlocks * (int64_t)sms, want = (npts + kAT - 1) / kAT;
     cudaError_t e;
     // the list's length is known on the device: both kernels are launched unless even the whole input is short
-    if (!lane_path(split_plan(want, gb, A.n_el), npts, gb)) {
+    if (!lane_path(split_plan(want, gb, A.n_el, cap), npts, gb)) {
         // one value whatever the tile: another thread's call may be between this and its launch
         e = cudaFuncSetAttribute(k_eval_acc_far<L, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
         const int64_t most = want * split_count(A.n_el, kLeafEl);  // units of the longest list
         k_eval_acc_far<L, M><<<(unsigned)std::min(gb, most), kAT, smem, s>>>(A, img.n, te, pts, list, n_list, next, gb,
-                                                                            part, phi, E, err, bound);
+                                                                            cap, part, phi, E, err, bound);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -691,12 +691,12 @@ cudaError_t launch_level(const AccView& A, const ImageTable& img, const double* 
                              kSmem + (int)sizeof(LaneScratch));
     if (e != cudaSuccess) return e;
     k_eval_acc_lanes<L, M><<<(unsigned)std::min<int64_t>(4 * (int64_t)sms, split_count(npts, kLP) * split_count(A.n_el, kLeafEl)),
-                             kAT, lane_smem, s>>>(A, img.n, te, pts, list, n_list, gb, part);
+                             kAT, lane_smem, s>>>(A, img.n, te, pts, list, n_list, gb, cap, part);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t left = std::min(want, 2 * gb) * kAT;  // points of the left-over groups, at most
     k_acc_reduce<L, M><<<(unsigned)std::min<int64_t>((left + 7) / 8, 8 * (int64_t)sms), 256, 0, s>>>(
-        A.n_el, list, n_list, gb, part, phi, E, err, bound);
+        A.n_el, list, n_list, gb, cap, part, phi, E, err, bound);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the FP64 near pairs, added to the quantities this pass re-evaluated only
@@ -756,14 +756,16 @@ cudaError_t launch_elem_moments(const FillEl* fe, const float4* nodes, int64_t n
 ErrModel default_err_model() { return ErrModel{kErrGammaR, kErrGammaB, kErrGammaS}; }
 
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el) {
-    return sizeof(Sum6) * (size_t)split_parts((npts + kAT - 1) / kAT, kATBlocks * (int64_t)sms, n_el);
+    static_assert(kAT == kEvalThreads, "points of a group");
+    return split_part_bytes<Sum6>(npts, kATBlocks * (int64_t)sms, n_el);
 }
 
 cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const double* pts, int64_t npts,
                                double* phi, double* E, double* err, double tol, const ErrModel& em,
-                               const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part_buf) {
+                               const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part_buf,
+                               size_t part_bytes) {
     Sum6* part = static_cast<Sum6*>(part_buf);
-    if (!part) return cudaErrorInvalidValue;
+    const int64_t cap = (int64_t)(part_bytes / sizeof(Sum6));
     if (npts == 0) return cudaSuccess;
     if (npts > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
     const bool refine = tol > 0.0 && (phi || E);
@@ -786,13 +788,13 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
     }
     if (e == cudaSuccess && refine)
         e = launch_level<1, kBoth>(A, img, pts, npts, phi, E, err, ms.bound, ms.list, ms.n_list, ms.n_list + 4, sms, part,
-                                    s);
+                                    cap, s);
     if (e == cudaSuccess && refine)
         e = launch_level<1, kPhiOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_p, ms.n_list + 2, ms.n_list + 5, sms,
-                                      part, s);
+                                      part, cap, s);
     if (e == cudaSuccess && refine)
         e = launch_level<1, kEOnly>(A, img, pts, npts, phi, E, err, ms.bound, ms.list_e, ms.n_list + 3, ms.n_list + 6, sms,
-                                    part, s);
+                                    part, cap, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], s);
     if (e == cudaSuccess && refine) {
         // level 2 on the points whose level-1 estimate still exceeds the tolerance (a quantity
@@ -805,7 +807,7 @@ cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const do
         e = cudaGetLastError();
         if (e == cudaSuccess)
             e = launch_level<2, kBoth>(A, img, pts, npts, phi, E, err, nullptr, ms.list2, ms.n_list + 1, ms.n_list + 7, sms,
-                                    part, s);
+                                    part, cap, s);
     }
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], s);
     return e;

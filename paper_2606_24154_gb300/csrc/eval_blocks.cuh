@@ -70,7 +70,9 @@ static_assert(kChunkEl % kLeafEl == 0 && kLeafEl % kTileMax == 0 && kLeafEl % kT
 // 0.29 us a pair whatever else the SM does, so a launch cannot end before its longest piece:
 // 250,000 pairs (72 ms) for a whole point of a 10,000-element cell with 25 copies, 1.9 ms for a
 // chunk, 0.23 ms for a leaf.  The leaves cost eight times the chunks' partial sums (48 B per
-// point and piece), which is why they are kept for launches that are short of pieces.
+// point and piece), which is why they are kept for launches that are short of pieces.  Where the pieces' sums
+// do not fit in the `cap` sums that the caller has room for, more groups are taken whole: the same bits, with a
+// longer last round.
 constexpr int kSplitRounds = 4;
 struct SplitPlan {
     int64_t Gm, R, np;
@@ -80,13 +82,17 @@ struct SplitPlan {
 __host__ __device__ __forceinline__ int64_t split_count(int64_t n_el, int64_t len) {
     return n_el > 0 ? (n_el + len - 1) / len : 1;
 }
-__host__ __device__ __forceinline__ SplitPlan split_plan(int64_t G, int64_t gb, int64_t n_el) {
+__host__ __device__ __forceinline__ SplitPlan split_plan(int64_t G, int64_t gb, int64_t n_el, int64_t cap) {
     SplitPlan s;
     s.Gm = G >= 2 * gb ? (G / gb - 1) * gb : 0;
     s.R = G - s.Gm;
-    const int64_t nch = split_count(n_el, kChunkEl);
-    s.leaf = s.R * nch < kSplitRounds * gb;
-    s.np = s.leaf ? split_count(n_el, kLeafEl) : nch;
+    const int64_t nch = split_count(n_el, kChunkEl), nleaf = split_count(n_el, kLeafEl);
+    s.leaf = s.R * nch < kSplitRounds * gb && s.R * nleaf * kEvalThreads <= cap;
+    s.np = s.leaf ? nleaf : nch;
+    if (s.R * s.np * kEvalThreads > cap) {
+        s.R = cap / (s.np * kEvalThreads);
+        s.Gm = G - s.R;
+    }
     return s;
 }
 // partial sums (one per point and piece) of the largest left-over part of up to G groups
@@ -96,6 +102,12 @@ inline int64_t split_parts(int64_t G, int64_t gb, int64_t n_el) {
     const int64_t rl = (kSplitRounds * gb + nch - 1) / nch;          // the most that go by leaves
     const int64_t a = r * nch, b = (r < rl ? r : rl) * nleaf;
     return (a > b ? a : b) * kEvalThreads;
+}
+// bytes of that many sums of type T, at most kPartMax
+template <class T>
+inline size_t split_part_bytes(int64_t npts, int64_t gb, int64_t n_el) {
+    const size_t b = sizeof(T) * (size_t)split_parts((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
+    return b < kPartMax ? b : kPartMax;
 }
 // The piece that unit u (< Gm + R np) stands for: its group and element range.
 struct SplitUnit {

@@ -130,17 +130,18 @@ __global__ void k_element_influence(const Elem* __restrict__ el, int64_t n_el, c
 }  // namespace
 
 size_t f64_part_bytes(int64_t npts, int sms, int64_t n_el) {
-    const int64_t G = (npts + kEvalThreads - 1) / kEvalThreads, gb = kF64Blocks * (int64_t)sms;
-    const SplitPlan plan = split_plan(G, gb, n_el);
+    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, kF64Blocks * (int64_t)sms, n_el,
+                                      (int64_t)(kPartMax / sizeof(Sum4)));
     return sizeof(Sum4) * (size_t)(plan.R * plan.np * kEvalThreads);
 }
 
 cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
                             const double* pts, int64_t npts, double* phi, double* E, int sms, void* part,
-                            cudaStream_t s) {
+                            size_t part_bytes, cudaStream_t s) {
     if (npts == 0) return cudaSuccess;
     const int64_t gb = kF64Blocks * (int64_t)sms;
-    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
+    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el,
+                                      (int64_t)(part_bytes / sizeof(Sum4)));
     const int64_t units = plan.Gm + plan.R * plan.np;
     k_eval_f64<<<(unsigned)units, kEvalThreads, 0, s>>>(el, sigma, n_el, img, pts, npts, plan,
                                                         static_cast<Sum4*>(part), phi, E);

@@ -399,13 +399,13 @@ size_t eval_mixed_scratch_bytes(int64_t npts) {
 }
 
 size_t far_part_bytes(int64_t npts, int sms, int64_t n_el) {
-    return sizeof(SumB) * (size_t)split_parts((npts + kEvalThreads - 1) / kEvalThreads, kFarBlocks * (int64_t)sms, n_el);
+    return split_part_bytes<SumB>(npts, kFarBlocks * (int64_t)sms, n_el);
 }
 
 cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4* cjk, const double* sigma,
                               int64_t n_el, const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
                               const int32_t* cell_items, const double* pts, int64_t npts, double* phi, double* E,
-                              const MixedScratch& ms, int sms, void* part, cudaStream_t s) {
+                              const MixedScratch& ms, int sms, void* part, size_t part_bytes, cudaStream_t s) {
     if (npts == 0) return cudaSuccess;
     if (npts > (int64_t)INT32_MAX) return cudaErrorInvalidValue;
     const GeomView g = make_view(el, far, cjk, sigma, n_el, img, grid, cell_start, cell_items);
@@ -417,7 +417,8 @@ cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4*
     k_bin_scan<<<kScanBlocks, 1024, 0, s>>>(ms.count, ms.bin_sums);
     k_bin_scatter<<<pblocks, 256, 0, s>>>(ms.key, npts, ms.count, ms.order);
     const int64_t gb = kFarBlocks * (int64_t)sms;
-    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el);
+    const SplitPlan plan = split_plan((npts + kEvalThreads - 1) / kEvalThreads, gb, n_el,
+                                      (int64_t)(part_bytes / sizeof(SumB)));
     const int64_t units = plan.Gm + plan.R * plan.np;
     const int64_t lane_units = (npts + kFL - 1) / kFL * plan.np;
     if (plan.leaf && plan.Gm == 0 && lane_units < kFarLaneRounds * gb) {

@@ -129,11 +129,15 @@ GeomView make_view(const Elem* el, const FarNodes* far, const float4* cjk, const
 
 // ------------------------------------------------------------------ launchers (.cu)
 // Each returns cudaSuccess or the launch error.
-// FP64 evaluation; part: f64_part_bytes(npts, sms, n_el) bytes of device scratch (NULL when 0)
+// The evaluations split points over pieces of the elements, whose partial sums (`part`) are at most this much
+// (10,000 elements take 450 MB, 40,000 would take 1.8 GB).  Every launcher takes less, down to none (NULL),
+// and gives the same bits: what has no room is summed whole.
+constexpr size_t kPartMax = (size_t)512 << 20;
+// FP64 evaluation; part: f64_part_bytes(npts, sms, n_el) bytes of device scratch
 size_t f64_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
                             const double* pts, int64_t npts, double* phi, double* E, int sms, void* part,
-                            cudaStream_t s);
+                            size_t part_bytes, cudaStream_t s);
 // Scratch of one mixed evaluation of npts points: binning (bin counts, keys, the binned
 // order), the FP32 pass's error scales ke * (B_phi, B_E, S_phi, S_E) per point, and the
 // list and count of the points the refinement re-evaluates.
@@ -160,7 +164,7 @@ size_t far_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_eval_mixed(const Elem* el, const FarNodes* far, const float4* cjk, const double* sigma,
                               int64_t n_el, const ImageTable& img, const NearGrid& grid, const int32_t* cell_start,
                               const int32_t* cell_items, const double* pts, int64_t npts, double* phi, double* E,
-                              const MixedScratch& ms, int sms, void* part, cudaStream_t s);
+                              const MixedScratch& ms, int sms, void* part, size_t part_bytes, cudaStream_t s);
 // Tables of the two-float evaluation (the mixed fill's): element records, node records,
 // tau = t_k . frame, two-float image centroids, and the cell list with the near radius
 // kFillRatioC rho.
@@ -196,7 +200,8 @@ ErrModel default_err_model();
 // the point groups that a level splits over element chunks to keep every block busy.
 cudaError_t launch_eval_refine(const AccView& A, const ImageTable& img, const double* pts, int64_t npts,
                                double* phi, double* E, double* err, double tol, const ErrModel& em,
-                               const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part);
+                               const MixedScratch& ms, int sms, cudaStream_t s, cudaEvent_t* ev, void* part,
+                               size_t part_bytes);
 size_t elem_moments_bytes(int64_t n);
 cudaError_t launch_elem_moments(const FillEl* fe, const float4* nodes, int64_t n, float4* mom, cudaStream_t s);
 size_t refine_part_bytes(int64_t npts, int sms, int64_t n_el);

@@ -115,7 +115,7 @@ struct Server {
     DevBuf d_geoms, d_pts, d_phi, d_E, d_head, d_remaining, d_partials, d_pcount;
     DevBuf d_rpart;                           // refinement partial sums (groups split over chunks)
     // refinement: error scales, the lists of the two levels (level 1 in three: phi and E,
-    // phi only, E only; arena indices), their counts (four per slot)
+    // phi only, E only; arena indices), their counts (kRefineCounts per slot)
     DevBuf d_bound, d_list, d_list2, d_list_p, d_list_e, d_nlist;
     std::vector<int32_t> nchunks;  // element chunks per geometry
     int32_t max_chunks = 1;
@@ -189,7 +189,7 @@ struct Server {
         CK(launch_eval_refine(A, c->img, d_pts.as<double>() + 3 * r->offset, r->n,
                               r->phi ? d_phi.as<double>() + r->offset : nullptr,
                               r->E ? d_E.as<double>() + 3 * r->offset : nullptr, nullptr, c->opt.mixed_point_tol,
-                              c->err_model, ms, c->props.multiProcessorCount, refine, nullptr, part));
+                              c->err_model, ms, c->props.multiProcessorCount, refine, nullptr, part, d_rpart.bytes));
         CK(cudaEventRecord(refine_done[r->slot], refine));
         return 0;
     }
@@ -408,6 +408,15 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         s->nchunks.push_back(nc);
         s->max_chunks = std::max(s->max_chunks, nc);
     }
+    // The two areas of partial sums shrink where the device has no room for them (down to none: requests are then
+    // served by whole points, with the same results)
+    auto shrinking = [](DevBuf& b, size_t unit, size_t count, size_t* got) {
+        cudaError_t r;
+        while ((r = b.ensure(unit * count)) == cudaErrorMemoryAllocation && count > 0) count /= 2;
+        *got = count;
+        return r;
+    };
+    size_t pblocks = 0, rpart = 0;
     s->ring_cap = std::max<int64_t>(4096 + (int64_t)kPartialBlocks * s->max_chunks,
                                     2 * (cap + kItemPoints - 1) / kItemPoints);
     if ((e = s->d_geoms.ensure(sizeof(ServeGeom) * geoms.size())) != cudaSuccess ||
@@ -416,15 +425,17 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         (e = s->d_E.ensure(sizeof(double) * 3 * cap)) != cudaSuccess ||
         (e = s->d_head.ensure(3 * sizeof(unsigned long long))) != cudaSuccess ||  // claimed, finished, closing
         (e = s->d_remaining.ensure(sizeof(int) * o.max_requests)) != cudaSuccess ||
-        (e = s->d_partials.ensure((size_t)kPartialBytes * kItemPoints * (size_t)kPartialBlocks * s->max_chunks)) != cudaSuccess ||
         (e = s->d_bound.ensure(sizeof(float4) * cap)) != cudaSuccess ||
         (e = s->d_list.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_list2.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_list_p.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
         (e = s->d_list_e.ensure(sizeof(int32_t) * cap)) != cudaSuccess ||
-        (e = s->d_rpart.ensure(refine_part_bytes(cap, cs[0]->props.multiProcessorCount, max_el))) != cudaSuccess ||
         (e = s->d_nlist.ensure(kRefineCounts * sizeof(int32_t) * o.max_requests)) != cudaSuccess ||
-        (e = s->d_pcount.ensure(sizeof(int) * kPartialBlocks)) != cudaSuccess)
+        (e = s->d_pcount.ensure(sizeof(int) * kPartialBlocks)) != cudaSuccess ||
+        (e = shrinking(s->d_partials, (size_t)kPartialBytes * kItemPoints * s->max_chunks, kPartialBlocks, &pblocks)) !=
+            cudaSuccess ||
+        (e = shrinking(s->d_rpart, 1, refine_part_bytes(cap, cs[0]->props.multiProcessorCount, max_el), &rpart)) !=
+            cudaSuccess)
         return bail(cuda_fail(e, "server device buffers"));
     if ((e = cudaHostAlloc(&s->h_ring, sizeof(WorkItem) * s->ring_cap, cudaHostAllocMapped)) != cudaSuccess ||
         (e = cudaHostAlloc(&s->h_tail, 64, cudaHostAllocMapped)) != cudaSuccess ||
@@ -438,7 +449,7 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         (e = cudaMemset(s->d_head.ptr, 0, 3 * sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMemset(s->d_pcount.ptr, 0, sizeof(int) * kPartialBlocks)) != cudaSuccess)
         return bail(cuda_fail(e, "server setup copies"));
-    for (int32_t i = kPartialBlocks - 1; i >= 0; --i) s->free_pblocks.push_back(i);
+    for (int32_t i = (int32_t)pblocks - 1; i >= 0; --i) s->free_pblocks.push_back(i);
     s->arena.reset(cap);
     s->slot_gen.assign((size_t)o.max_requests, 0);
     for (int32_t i = o.max_requests - 1; i >= 0; --i) s->free_slots.push_back(i);

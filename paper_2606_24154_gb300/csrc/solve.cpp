@@ -86,6 +86,19 @@ int ensure_fill(Ctx* c, int precision, double* ms) {
     return 0;
 }
 
+int factor_f64(Ctx* c, double* A, int64_t n, int32_t* piv, DevBuf& work, int* d_info, cudaStream_t s, long long polls) {
+    const int nb = c->opt.lu_block;
+    const cudaError_t e = work.ensure(lu_work_bytes_f64(n, nb));
+    if (e == cudaErrorMemoryAllocation) {  // 4 to 5 times less, on the FP64 pipe
+        CK(work.ensure(sizeof(double) * lu_work_elems(n, nb)));
+        CK(lu_factor_f64_small(A, n, piv, nb, work.as<double>(), d_info, s));
+        return 0;
+    }
+    CK(e);
+    CK(lu_factor_f64(A, n, piv, nb, work.ptr, d_info, s, polls));
+    return 0;
+}
+
 int ensure_factors(Ctx* c, int precision, double* ms) {
     const int64_t n = c->n;
     const int nb = c->opt.lu_block;
@@ -94,13 +107,14 @@ int ensure_factors(Ctx* c, int precision, double* ms) {
         if (c->fac64_valid) return 0;
         CK(c->d_LU64.ensure(sizeof(double) * n * n));
         CK(c->d_piv64.ensure(sizeof(int32_t) * n));
-        CK(c->d_work.ensure(lu_work_bytes_f64(n, nb)));
+        c->d_work.ensure(lu_work_bytes_f64(n, nb));  // before the clock starts (factor_f64 looks at the result)
         CK(c->d_small.ensure(256));
         CK(cudaEventRecord(c->ev0, c->stream));
         CK(cudaMemcpyAsync(c->d_LU64.ptr, c->d_K.ptr, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, c->stream));
-        CK(lu_factor_f64(c->d_LU64.as<double>(), n, c->d_piv64.as<int32_t>(), nb, c->d_work.ptr,
-                         c->d_small.as<int>(), c->stream, c->opt.wait_polls));
-        int rc = elapsed_ms(c, ms);
+        int rc = factor_f64(c, c->d_LU64.as<double>(), n, c->d_piv64.as<int32_t>(), c->d_work, c->d_small.as<int>(),
+                            c->stream, c->opt.wait_polls);
+        if (rc) return rc;
+        rc = elapsed_ms(c, ms);
         if (rc) return rc;
         int h2[2] = {0, 0};
         CK(cudaMemcpy(h2, c->d_small.ptr, sizeof(h2), cudaMemcpyDeviceToHost));
@@ -326,19 +340,33 @@ int weighting_solve(Ctx* c, const int32_t* readout, int k, int precision, nebem_
     return 0;
 }
 
+// The context's scratch for `base` bytes and up to *part bytes of partial sums behind them; where the device has
+// no room for all of them, *part becomes what it has room for (the evaluation then takes longer).
+static int ensure_scratch(Ctx* c, size_t base, size_t* part) {
+    for (;;) {
+        const cudaError_t e = c->d_scratch.ensure(base + *part);
+        if (e == cudaSuccess) return 0;
+        if (e != cudaErrorMemoryAllocation || *part == 0) return cuda_fail(e, "evaluation scratch");
+        *part = *part > ((size_t)1 << 20) ? *part / 4 : 0;
+    }
+}
+
 // FP64 evaluation with stream-ordered scratch from the context's own pool: unlike the mixed
 // evaluation's scratch it is the call's own, so FP64 calls on different streams of a context
-// share nothing, and a call can be captured into a graph.
+// share nothing, and a call can be captured into a graph.  Without room for it every point's sum is
+// taken whole.
 static int eval_f64(Ctx* c, const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,
                     const double* d_pts, int64_t n, double* d_phi, double* d_E, cudaStream_t s) {
     const int sms = c->props.multiProcessorCount;
-    const size_t bytes = f64_part_bytes(n, sms, n_el);
+    size_t bytes = f64_part_bytes(n, sms, n_el);
     void* part = nullptr;
-    if (bytes > 0) {
-        CK(c->ensure_pool());
-        CK(cudaMallocFromPoolAsync(&part, bytes, c->pool, s));
+    if (bytes > 0 &&
+        (c->ensure_pool() != cudaSuccess || cudaMallocFromPoolAsync(&part, bytes, c->pool, s) != cudaSuccess)) {
+        cudaGetLastError();
+        part = nullptr;
+        bytes = 0;
     }
-    const cudaError_t e = launch_eval_f64(el, sigma, n_el, img, d_pts, n, d_phi, d_E, sms, part, s);
+    const cudaError_t e = launch_eval_f64(el, sigma, n_el, img, d_pts, n, d_phi, d_E, sms, part, bytes, s);
     const cudaError_t ef = part ? cudaFreeAsync(part, s) : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "launch_eval_f64");
     CK(ef);
@@ -350,10 +378,11 @@ int eval_set(Ctx* c, const EvalSet& es, const double* d_pts, int64_t n, double* 
     if (precision == NEBEM_MIXED) {
         const int sms = c->props.multiProcessorCount;
         const size_t ms_bytes = eval_mixed_scratch_bytes(n);
-        CK(c->d_scratch.ensure(ms_bytes + far_part_bytes(n, sms, es.n)));
+        size_t part = far_part_bytes(n, sms, es.n);
+        if (const int rc = ensure_scratch(c, ms_bytes, &part)) return rc;
         CK(launch_eval_mixed(es.el, es.far, es.cjk.as<float4>(), es.sigma, es.n, es.img, es.grid,
                              es.cell_start.as<int32_t>(), es.cell_items.as<int32_t>(), d_pts, n, d_phi, d_E,
-                             mixed_scratch(c->d_scratch.ptr, n), sms, c->d_scratch.as<char>() + ms_bytes, s));
+                             mixed_scratch(c->d_scratch.ptr, n), sms, c->d_scratch.as<char>() + ms_bytes, part, s));
     } else {
         return eval_f64(c, es.el, es.sigma, es.n, es.img, d_pts, n, d_phi, d_E, s);
     }
@@ -372,14 +401,15 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
         const size_t ms_bytes = eval_mixed_scratch_bytes(n);  // a multiple of 256
         // the FP32 pass and the refinement levels use one partial-sum area in turn
         const int sms = c->props.multiProcessorCount;
-        CK(c->d_scratch.ensure(ms_bytes + std::max(far_part_bytes(n, sms, c->n), refine_part_bytes(n, sms, c->n))));
+        size_t part_bytes = std::max(far_part_bytes(n, sms, c->n), refine_part_bytes(n, sms, c->n));
+        if (const int rc = ensure_scratch(c, ms_bytes, &part_bytes)) return rc;
         void* part = c->d_scratch.as<char>() + ms_bytes;
         const MixedScratch ms = mixed_scratch(c->d_scratch.ptr, n);
         c->eval_timed = false;
         CK(cudaEventRecord(c->ev_eval[0], s));
         CK(launch_eval_mixed(c->d_el.as<Elem>(), c->d_far.as<FarNodes>(), c->d_cjk.as<float4>(),
                              c->d_sigma.as<double>(), c->n, c->img, c->grid, c->d_cell_start.as<int32_t>(),
-                             c->d_cell_items.as<int32_t>(), d_pts, n, d_phi, d_E, ms, sms, part, s));
+                             c->d_cell_items.as<int32_t>(), d_pts, n, d_phi, d_E, ms, sms, part, part_bytes, s));
         CK(cudaEventRecord(c->ev_eval[1], s));
         if (refine || err) {
             AccView A;
@@ -399,7 +429,8 @@ int eval_elements(Ctx* c, const double* d_pts, int64_t n, double* d_phi, double*
             A.grid = c->fill_grid;
             A.cell_start = c->d_fill_cell_start.as<int32_t>();
             A.cell_items = c->d_fill_cell_items.as<int32_t>();
-            CK(launch_eval_refine(A, c->img, d_pts, n, d_phi, d_E, err, c->opt.mixed_point_tol, c->err_model, ms, sms, s, &c->ev_eval[2], part));
+            CK(launch_eval_refine(A, c->img, d_pts, n, d_phi, d_E, err, c->opt.mixed_point_tol, c->err_model, ms, sms, s,
+                                  &c->ev_eval[2], part, part_bytes));
             c->refine_list = ms.n_list;
         } else {
             CK(cudaMemsetAsync(ms.n_list, 0, 4 * sizeof(int32_t), s));
