@@ -2,6 +2,7 @@
 that only makes a call faster is done without, and the results are the same bits (FP64 LU: P A = L U within
 4 n u |L||U| per element)."""
 import contextlib
+import ctypes as C
 
 import numpy as np
 import pytest
@@ -22,18 +23,23 @@ def N():
 
 @contextlib.contextmanager
 def room(megabytes):
-    """All of the device's memory but this much taken (not touched)."""
+    """All of the device's memory but this much taken (not touched), by the runtime's own allocator: torch's
+    takes small requests in blocks of 20 MB."""
     import torch
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
-    taken = torch.empty(torch.cuda.mem_get_info()[0] - megabytes * MB, dtype=torch.uint8, device="cuda")
+    rt, taken = C.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0]), []
     try:
-        assert torch.cuda.mem_get_info()[0] <= (megabytes + 4) * MB
+        for block in (1 << 30, 32 * MB, 2 * MB):
+            while torch.cuda.mem_get_info()[0] >= megabytes * MB + block:
+                p = C.c_void_p()
+                assert rt.cudaMalloc(C.byref(p), C.c_size_t(block)) == 0
+                taken.append(p)
         yield
     finally:
         torch.cuda.synchronize()
-        del taken
-        torch.cuda.empty_cache()
+        for p in taken:
+            rt.cudaFree(p)
 
 
 def cell():
