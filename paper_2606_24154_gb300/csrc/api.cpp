@@ -60,13 +60,17 @@ cudaError_t Ctx::ensure_pool() {
     p.allocType = cudaMemAllocationTypePinned;
     p.location.type = cudaMemLocationTypeDevice;
     p.location.id = device;
+    // the call may be under capture, where both calls are refused unless the thread's capture mode is relaxed
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     cudaError_t e = cudaMemPoolCreate(&pool, &p);
-    if (e != cudaSuccess) {
-        pool = nullptr;
-        return e;
-    }
     uint64_t keep = kPoolKeep;
-    return cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e == cudaSuccess)
+        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    else
+        pool = nullptr;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
 }
 
 Ctx::~Ctx() {
