@@ -151,10 +151,15 @@ cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, c
     return cudaGetLastError();
 }
 
+cudaError_t sm_count(int* sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 cudaError_t fill_cols(int64_t n, int rows, int per_sm, int* cols) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     *cols = 64;
     while (*cols > 2 && (n + rows - 1) / rows * ((n + *cols - 1) / *cols) < 2 * (int64_t)per_sm * sms) *cols /= 2;

@@ -432,11 +432,14 @@ cudaError_t tc_apply_f64(int64_t M, int64_t N, int64_t K, int64_t c0, int64_t c1
     if (c0 % kDN || !work) return cudaErrorInvalidValue;
     const Tables64 t = tables64(M, N, work);
     // set for the current device on every call (an attribute is per device)
-    cudaError_t e = cudaFuncSetAttribute(k_tc_update_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tc_update_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
     if (e != cudaSuccess) return e;
     // column tiles per CTA: about three CTAs per SM in all, at most 8 tiles each
     const int64_t tiles_m = pad_to(M, kDM) / kDM, tile0 = c0 / kDN, tile1 = (c1 + kDN - 1) / kDN, tiles_n = tile1 - tile0;
-    const int64_t tpc = std::max<int64_t>(1, std::min<int64_t>(8, tiles_m * tiles_n / (3 * 152)));
+    const int64_t tpc = std::max<int64_t>(1, std::min<int64_t>(8, tiles_m * tiles_n / (3 * sms)));
     dim3 grid((unsigned)tiles_m, (unsigned)((tiles_n + tpc - 1) / tpc));
     k_tc_update_f64<<<grid, kDThreads, kDSmem, s>>>(M, N, (int)K, A, lda, B, ldb, t.da, t.db, t.ea, t.eb, C, ldc, tile0,
                                                     tile1, (int)tpc, err);

@@ -129,6 +129,8 @@ GeomView make_view(const Elem* el, const FarNodes* far, const float4* cjk, const
 
 // ------------------------------------------------------------------ launchers (.cu)
 // Each returns cudaSuccess or the launch error.
+// multiprocessors of the current device
+cudaError_t sm_count(int* sms);
 // The evaluations split points over pieces of the elements, whose partial sums (`part`) are at most this much
 // (10,000 elements take 450 MB, 40,000 would take 1.8 GB).  Every launcher takes less, down to none (NULL),
 // and gives the same bits: what has no room is summed whole.

@@ -394,9 +394,12 @@ cudaError_t launch_sc_eval(int precision, const double* src, const double* q, co
         // us against 43 (1,100 targets), 39 against 44 (20,000) and 205 against 178 (200,000, where the blocks'
         // targets and totals cost more than the idle SMs; 275 against 315 with 2,000 sources).  Two pairs
         // of targets per thread where that leaves a block for every SM.
+        int sms = 0;
+        const cudaError_t e = sm_count(&sms);
+        if (e != cudaSuccess) return e;
         const bool split = nsrc >= kSCSplitFrom;
         const int ns = split ? kSCSplit : 1;
-        const bool wide = ntgt * ns >= (int64_t)152 * 2 * kSCT;
+        const bool wide = ntgt * ns >= (int64_t)sms * 2 * kSCT;
         const int64_t tile = (wide ? 4 : 2) * kSCT;
         const unsigned grid = (unsigned)((ntgt + tile - 1) / tile * ns);
         auto* k = split ? (wide ? k_sc_mixed_split<2> : k_sc_mixed_split<1>) : (wide ? k_sc_mixed<2> : k_sc_mixed<1>);
