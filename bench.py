@@ -588,8 +588,9 @@ def run_native(args):
             "e2e": {"value": e2e_val, "unit": "evals/s", "h2d_bytes_per_step": int(pts_pin.numel() * 8),
                     "d2h_bytes_per_step": int((phi_pin.numel() + E_pin.numel()) * 8)},
             "cpu_baseline": cpu,
-            # per step: k_bin_keys, k_bin_scan, k_bin_scatter, k_eval_far, k_eval_near, then
-            # k_flag + k_eval_acc_far + near per refinement level
+            # per step: k_bin_keys, k_bin_sums, k_bin_scan, k_bin_scatter, k_eval_far, k_far_reduce, k_eval_near (7);
+            # k_flag by what level 1 re-evaluates (3), and for each of its three passes and level 2 (4) k_eval_acc_far,
+            # k_eval_acc_lanes, k_acc_reduce, k_eval_acc_near (16); k_flag of the three lists for level 2 (3)
             "gpu_launches": 29 * args.steps,
             "clocks": clocks,
             "wall_s_timed_region": wall,

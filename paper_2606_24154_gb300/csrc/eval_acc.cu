@@ -31,10 +31,10 @@
 // ~2e-11 of B; its estimate is 1e-9 B.  Points whose level-1 estimate still exceeds the
 // tolerance go to level 2, the arithmetic of the mixed fill (fill_mixed.cu: moments with a two-float
 // quadrupole from 40 radii on, rules truncated below ~3e-12 of each pair nearer, FP64 closed forms
-// within kFillRatioC element radii), estimate 1e-11 B.  In the frame of element j (axes ex, ey = normal, ez), a pair (point, image k) has D = P - c_j - t_k with
-// local components X = (P - c_j) . ex - tau_k.x (likewise Y, Z; tau tabulated per element
-// and image), from which the moments' series follow (twofloat.cuh); a node at offset s = centroid - node (in the element plane) sees the point at
-// D + s, so r^2 = |D|^2 + 2 (X s_x + Z s_z) + |s|^2 and
+// within kFillRatioC element radii), estimate 1e-11 B.  In the frame of element j (axes ex, ey = normal,
+// ez), a pair (point, image k) has D = P - c_j - t_k with local components X = (P - c_j) . ex - tau_k.x
+// (likewise Y, Z; tau tabulated per element and image), from which the moments' series follow
+// (twofloat.cuh); a node at offset s = centroid - node (in the element plane) sees the point at D + s, so r^2 = |D|^2 + 2 (X s_x + Z s_z) + |s|^2 and
 //   Phi' = sum w / r,   E'_local = D sum w / r^3 + (sum w s_x / r^3, 0, sum w s_z / r^3).
 // Per element the image sums are rotated to the global frame and weighted by sigma_j in
 // FP64.  Every flagged point's arithmetic depends on that point only, so its result does
@@ -233,7 +233,8 @@ __device__ __noinline__ void acc_pair_nodes(const AccView& A, const float4& hdr,
 }
 
 // Level 1, 1e6 points of the 9,996-element cell x 25 copies (320,000 of them refined): 1,490 ms with
-// every pair by Gauss nodes in two-float arithmetic, 612 ms so (540 with the units dealt as below), with an error 10 to 25 times smaller
+// every pair by Gauss nodes in two-float arithmetic, 612 ms so (540 with the units dealt as below), with an
+// error 10 to 25 times smaller
 // (E: 2.0e-10 B before, 1.7e-11 B now, the largest of 665 refined points).  The FP32 pipe is busy for
 // about two thirds of it; 5 blocks per SM (96 registers) beat 4 by 3 %, 6 are the same.
 //

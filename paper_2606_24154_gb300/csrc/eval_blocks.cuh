@@ -66,8 +66,8 @@ static_assert(kChunkEl % kLeafEl == 0 && kLeafEl % kTileMax == 0 && kLeafEl % kT
 // the first Gm groups whole, floor(G / gb) - 1 rounds of gb; the R < 2 gb left over in R * np
 // pieces (group, chunk), or (group, leaf) where the chunks would give a block fewer than
 // kSplitRounds pieces.  (With the last full round whole too, its slowest groups ran on alone:
-// 169 ms instead of 144 for the FP32 pass over 233,472 points, exactly two rounds.)  One thread walks all (element, image) pairs of its point in turn, about
-// 0.29 us a pair whatever else the SM does, so a launch cannot end before its longest piece:
+// 169 ms instead of 144 for the FP32 pass over 233,472 points, exactly two rounds.)  One thread walks all
+// (element, image) pairs of its point in turn, about 0.29 us a pair whatever else the SM does, so a launch cannot end before its longest piece:
 // 250,000 pairs (72 ms) for a whole point of a 10,000-element cell with 25 copies, 1.9 ms for a
 // chunk, 0.23 ms for a leaf.  The leaves cost eight times the chunks' partial sums (48 B per
 // point and piece), which is why they are kept for launches that are short of pieces.  Where the pieces' sums

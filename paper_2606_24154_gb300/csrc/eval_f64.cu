@@ -58,9 +58,9 @@ __global__ void __launch_bounds__(256) k_f64_reduce(const double* __restrict__ p
 // 0.619e12 a second).  Conductor rows form the potential only and interface rows the
 // field only; the row's normal is rotated into the column's frame once per (row, column), so that
 // an image of an interface row adds three products.
-__global__ void __launch_bounds__(kThreads, kFillBlocks) k_fill_f64(const Elem* __restrict__ el, const double* __restrict__ diag_in,
-                                                       int64_t n, const ImageTable img, int cols,
-                                                       double* __restrict__ K) {
+__global__ void __launch_bounds__(kThreads, kFillBlocks)
+    k_fill_f64(const Elem* __restrict__ el, const double* __restrict__ diag_in, int64_t n, const ImageTable img, int cols,
+               double* __restrict__ K) {
     __shared__ Tile64 s_t;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = i < n;

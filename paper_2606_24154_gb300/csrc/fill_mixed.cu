@@ -122,9 +122,9 @@ __host__ __device__ constexpr int fill_tile_f4(int te, int nimg) {
 // The pair (row i, element j, image k) by its tier's nodes where it is nearer than the moments reach (one
 // to three pairs in a hundred); a near pair is left to k_fill_near.
 __device__ __noinline__ void fill_pair_nodes(const float4* __restrict__ nd, const float4* __restrict__ cjk2,
-                                             const float4& hdr, const float (&ch)[3], const float (&cl)[3], const float (&Xh)[3],
-                                             const float (&Xl)[3], bool iface, const FillRow& R, float2& sh,
-                                             float2& snl) {
+                                             const float4& hdr, const float (&ch)[3], const float (&cl)[3],
+                                             const float (&Xh)[3], const float (&Xl)[3], bool iface, const FillRow& R,
+                                             float2& sh, float2& snl) {
     float dx, dy, dz;
     if (!(pair_d2(ch[0], ch[1], ch[2], cl[0], cl[1], cl[2], cjk2[0], cjk2[1], dx, dy, dz) >= hdr.z)) return;
     float d2h, d2l;
@@ -278,7 +278,8 @@ __global__ void __launch_bounds__(kFT, kFillBlocks)
                 const float l = __fadd_rn(t, __fadd_rn(Sl.x, Sl.y));
                 two_prod(h, area.x, p, e);
                 e = __fmaf_rn(h, area.y, __fmaf_rn(l, area.x, e));
-                const double acc = ((double)p + (double)e) + (((double)sh.x - (double)snl.x) + ((double)sh.y - (double)snl.y));
+                const double acc =
+                    ((double)p + (double)e) + (((double)sh.x - (double)snl.x) + ((double)sh.y - (double)snl.y));
                 K[i + j * n] = (i == j) ? fma(ke, acc, diag) : ke * acc;
             }
         }

@@ -425,13 +425,10 @@ __global__ void __launch_bounds__(kCoopThreads, 1)
 template <typename T>
 constexpr int64_t kClusterRows = sizeof(T) == 8 ? 96 : 256;
 
-// Apply the row swaps of panel rows [k0, k1) to columns outside the panel.
 // The row swaps of panel rows [k0, k1) (LAPACK order: row r with piv[r]) composed into one
-// permutation of the rows they touch (at most 2 (k1 - k0)): after it, row dst[i] holds what
-// row src[i] held before; *cnt = number of moved rows.  One warp: the touched rows are the
-// panel rows (slot r - k0) and the distinct pivot rows below the panel (found by a
-// warp-wide search of the list so far).  A pivot outside [r, n) is a row no panel wrote (its
-// panel gave up a bounded wait) and is skipped, as in the swaps themselves.
+// permutation of the rows they touch (at most 2 (k1 - k0)): perm[0] = number of moved rows, then
+// (dst, src) pairs: row dst holds afterwards what row src held before.  A pivot outside [r, n) is a row no
+// panel wrote (its panel gave up a bounded wait) and is skipped, as in the swaps themselves.
 // Each of 128 threads follows one touched row's content through the swaps: thread t < 64 the
 // panel row k0 + t, thread 64 + t the pivot row of step t below the panel, where no earlier
 // step has it.  (One warp searching its list of rows once per swap took 20 us, this 3.)
@@ -533,8 +530,6 @@ __global__ void __launch_bounds__(32 * kTriWarps) k_trtri_unit_lower(const T* __
     if (lane + 32 < nb) W[lane + 32 + (int64_t)c * nb] = x1;
 }
 
-// C = alpha * A * B + beta * C; column-major, M x N x K; 64 x 64 tiles, 256 threads, 4x4
-// register tile per thread.
 // U12 of a block row: X = L^-1 A[K0 : K0 + 64 nbk, c0 : c1] for the unit-lower L of nbk
 // diagonal 64-blocks at (K0, K0), by block forward substitution
 //   X_i = Linv_i (A_i - sum_{j < i} L_ij X_j),
@@ -615,6 +610,8 @@ __global__ void __launch_bounds__(256) k_trsm_block(T* __restrict__ A, int64_t n
     }
 }
 
+// C = alpha * A * B + beta * C; column-major, M x N x K; 64 x 64 tiles, 256 threads, 4x4
+// register tile per thread.
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm(int64_t M, int64_t N, int64_t K, T alpha, const T* __restrict__ A,
                                               int64_t lda, const T* __restrict__ B, int64_t ldb, T beta,
@@ -694,13 +691,11 @@ cudaError_t gemm(int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t l
 
 constexpr int kSuperPanels = 4;  // panels per super-panel of the two-level FP32 factorisation
 
-// work layout: [0, 4 nb*nb) unit-lower inverses; then nb*n U12 staging;
-// then kPivBlocks doubles + kPivBlocks int64 for the pivot search and one int ticket.
 // The stream on which the FP64 factorisation takes the next panel while the rest of the trailing
 // update runs.  A panel is bound by latency and leaves the SMs nearly idle: with the update of the
 // panel's columns first, the panel then beside the other columns' update (its CTAs at the higher priority,
 // beside the update's in registers and shared memory up to 8,000 rows), the LU of 6,145 rows takes 40.2 ms
-// instead of 44.4 (8,192: 65.0 and 72.6, 12,000: 151 and 164).  The two share the FP64 pipe: beside the
+// instead of 44.4 (8,192: 65.0 and 72.6, 12,000: 151 and 164; with an update by 36 digit products).  The two share the FP64 pipe: beside the
 // update a panel takes 310 us instead of 206.  Where kAheadFrom rows or more are left: below, the second
 // update launch and the events cost more (1,024 rows: 4.00 and 3.88 ms; 2,500: 11.5 and 11.4; 3,000: 14.1 and 14.3).
 constexpr int64_t kAheadFrom = 2048;
@@ -724,6 +719,8 @@ struct Ahead {
     }
 };
 
+// work layout: [0, 4 nb*nb) unit-lower inverses; then nb*n U12 staging; then kPivBlocks doubles + kPivBlocks
+// int64 for the pivot search, one int ticket and the composed row swaps.
 template <typename T>
 cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_info, void* split, void* coop,
                       cudaStream_t s, long long polls) {
@@ -744,7 +741,7 @@ cudaError_t lu_factor(T* A, int64_t n, int32_t* piv, int nb, T* work, int* d_inf
     NB_TRY(cudaFuncSetAttribute(k_laswp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, swap_smem));
     if (nb > 64) return cudaErrorInvalidValue;  // k_panel_col stages at most 64 row values
     // the whole panel in one cooperative launch when every CTA's rows fit in shared
-    // memory (R rows x 64 columns, R = max(64, rows / SMs)) and all CTAs can be resident
+    // memory (R rows x 64 columns, R = max(kCoopMinRows, rows / SMs)) and all CTAs can be resident
     int gmax = 0;
     CoopScratch<T>* cs = static_cast<CoopScratch<T>*>(coop);
     if (cs) {

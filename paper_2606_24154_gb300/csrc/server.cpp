@@ -7,8 +7,8 @@
 // items are appended to the ring in host-mapped memory before `tail` is advanced.  An
 // item is 128 points over all elements; a request of up to 16384 points instead gets one
 // item per (point block, chunk of 256 elements), so that its points still spread over
-// many CTAs (its latency would otherwise be one CTA's pass over all elements).  A persistent kernel (relaunched whenever published items wait and no
-// instance is running) claims items as they appear, so requests admitted while others
+// many CTAs (its latency would otherwise be one CTA's pass over all elements).  A persistent kernel (relaunched
+// whenever published items wait and no instance is running) claims items as they appear, so requests admitted while others
 // run join the running launch.  On completion the outputs are copied to the caller's
 // buffers and the arena range, slot and ring items are released.
 //

@@ -73,7 +73,8 @@ int ensure_fill(Ctx* c, int precision, double* ms) {
     CK(cudaEventRecord(c->ev0, c->stream));
     if (precision == NEBEM_MIXED)
         CK(launch_fill_mixed(c->d_el.as<Elem>(), c->d_fill_el.as<FillEl>(), c->d_fill_nodes.as<float4>(),
-                             c->d_fill_phimom.as<float4>(), c->d_fill_tau.as<float4>(), c->d_cjk.as<float4>(), c->d_diag.as<double>(), n, c->img,
+                             c->d_fill_phimom.as<float4>(), c->d_fill_tau.as<float4>(), c->d_cjk.as<float4>(),
+                             c->d_diag.as<double>(), n, c->img,
                              c->fill_grid, c->d_fill_cell_start.as<int32_t>(), c->d_fill_cell_items.as<int32_t>(),
                              c->d_K.as<double>(), c->stream));
     else
