@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) k_f64_reduce(const double* __restrict__ p
 }
 
 // Bound by the FP64 pipe: 4,632 elements x 25 copies take 121 ms, 4.4e9 pairs a second, where
-// the general form alone took 298 ms (about 118 FP64 instructions a pair: 0.85 of the measured
+// the general form alone took 298 ms (114 FP64 instructions a pair, counted: 0.85 of the measured
 // 0.619e12 a second).  Conductor rows form the potential only and interface rows the
 // field only; the row's normal is rotated into the column's frame once per (row, column), so that
 // an image of an interface row adds three products.

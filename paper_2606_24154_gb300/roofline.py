@@ -83,11 +83,12 @@ def mufu_peak(sm_mhz):
     return N_SM * MUFU_PER_SM * sm_mhz * 1e6
 
 
-# FP64 closed form: FP64 instructions per (point, element, image) pair of the FP64
-# evaluation kernel, from an ncu instruction count on the THGEM cell (166 DFMA, 59 DADD,
-# 53 DMUL); the FP64 pipe issues 2 such instructions per clock per SM on this GPU
+# FP64 closed forms: FP64 instructions per (point, element, image) pair of the FP64
+# evaluation kernel, from an ncu instruction count on the 9,996-element THGEM cell (78.4 DFMA, 16.8 DADD,
+# 27.6 DMUL; a triangle by series 114, a quadrilateral 155, nearer pairs more, so it depends on the
+# cell: 121.5 at 4,632 elements); the FP64 pipe issues 2 such instructions per clock per SM on this GPU
 # (1.25 TFLOP/s nominal with an FMA as 2 flops).
-FP64_INST_PER_PAIR = 118  # the series of the closed forms that most pairs take, counted from the code
+FP64_INST_PER_PAIR = 122.7
 FP64_INST_PER_SM_CLK = 2
 
 

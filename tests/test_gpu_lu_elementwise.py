@@ -105,19 +105,13 @@ def test_zero_rows_and_columns(N):
     assert (LU[:128, 200:] == 0).all() and (LU[200:, :128] == 0).all()
 
 
-@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
-@pytest.mark.parametrize("at", ["last column", "last row"])
-def test_not_finite(N, value, at):
+@pytest.mark.parametrize("value,row,col", [(np.inf, 3, 199), (-np.inf, 3, 199), (np.nan, 3, 199), (np.nan, 199, 5)])
+def test_not_finite(N, value, row, col):
     """One such value in U12's last column, or (NaN, which is never a pivot) in L21's last row: where the
     factors are not finite they are what fmas make of it, and the others keep their bound."""
     n = 200
     A = np.random.default_rng(3).normal(size=(n, n)) + 20 * np.eye(n)
-    if at == "last row":
-        if not np.isnan(value):
-            pytest.skip("an infinite entry is the column's pivot")
-        A[n - 1, 5] = value
-    else:
-        A[3, n - 1] = value
+    A[row, col] = value
     LU, perm = factor(N, A)
     ref, rperm = factor(N, A, fmas=True)
     assert np.array_equal(perm, np.arange(n)) and np.array_equal(rperm, perm)
