@@ -132,9 +132,10 @@ GeomView make_view(const Elem* el, const FarNodes* far, const float4* cjk, const
 // multiprocessors of the current device
 cudaError_t sm_count(int* sms);
 // The evaluations split points over pieces of the elements, whose partial sums (`part`) are at most this much
-// (10,000 elements take 450 MB, 40,000 would take 1.8 GB).  Every launcher takes less, down to none (NULL),
-// and gives the same bits: what has no room is summed whole.
-constexpr size_t kPartMax = (size_t)512 << 20;
+// (10,000 elements take 450 MB, 40,368 would take 1.8 GB).  Every launcher takes less, down to none (NULL),
+// and gives the same bits: what has no room is summed whole.  Level 1 of 500,000 points of a
+// 40,368-element cell: 1.61 s without a limit, 1.66 s with this one, 1.86 s with half of it.
+constexpr size_t kPartMax = (size_t)1 << 30;
 // FP64 evaluation; part: f64_part_bytes(npts, sms, n_el) bytes of device scratch
 size_t f64_part_bytes(int64_t npts, int sms, int64_t n_el);
 cudaError_t launch_eval_f64(const Elem* el, const double* sigma, int64_t n_el, const ImageTable& img,

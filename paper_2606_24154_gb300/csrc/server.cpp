@@ -49,6 +49,7 @@ constexpr int kItemPoints = 128;
 constexpr int64_t kSmallPoints = 16384;     // mixed
 constexpr int64_t kSmallPointsF64 = 16384;  // FP64
 constexpr int kPartialBlocks = 512;     // point blocks with chunk partial sums in flight
+constexpr size_t kRefinePartBytes = (size_t)512 << 20;  // refinement's partial sums: a server holds them all its life
 
 struct Interval {
     int64_t start, len;
@@ -416,7 +417,8 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         *got = count;
         return r;
     };
-    size_t pblocks = 0, rpart = 0;
+    size_t pblocks = 0, rpart = std::min<size_t>(kRefinePartBytes,
+                                                 refine_part_bytes(cap, cs[0]->props.multiProcessorCount, max_el));
     s->ring_cap = std::max<int64_t>(4096 + (int64_t)kPartialBlocks * s->max_chunks,
                                     2 * (cap + kItemPoints - 1) / kItemPoints);
     if ((e = s->d_geoms.ensure(sizeof(ServeGeom) * geoms.size())) != cudaSuccess ||
@@ -434,8 +436,7 @@ int nebem_server_create(nebem_server** out, nebem_ctx* const* ctxs, int32_t n_ct
         (e = s->d_pcount.ensure(sizeof(int) * kPartialBlocks)) != cudaSuccess ||
         (e = shrinking(s->d_partials, (size_t)kPartialBytes * kItemPoints * s->max_chunks, kPartialBlocks, &pblocks)) !=
             cudaSuccess ||
-        (e = shrinking(s->d_rpart, 1, refine_part_bytes(cap, cs[0]->props.multiProcessorCount, max_el), &rpart)) !=
-            cudaSuccess)
+        (e = shrinking(s->d_rpart, 1, rpart, &rpart)) != cudaSuccess)
         return bail(cuda_fail(e, "server device buffers"));
     if ((e = cudaHostAlloc(&s->h_ring, sizeof(WorkItem) * s->ring_cap, cudaHostAllocMapped)) != cudaSuccess ||
         (e = cudaHostAlloc(&s->h_tail, 64, cudaHostAllocMapped)) != cudaSuccess ||

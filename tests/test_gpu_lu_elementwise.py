@@ -20,10 +20,10 @@ def N():
     return nebem
 
 
-def factor(N, A, fmas=False):
+def factor(N, A, fmas=False, **opts):
     import torch
     n = A.shape[0]
-    ctx = N.Context()
+    ctx = N.Context(**opts)
     d = torch.tensor(np.asfortranarray(A).ravel(order="F"), device="cuda")
     p = torch.empty(n, dtype=torch.int32, device="cuda")
     try:
@@ -75,12 +75,13 @@ def test_weak_coupling(N, A):
     assert excess(A, *factor(N, A, fmas=True)) <= 1
 
 
+@pytest.mark.parametrize("block", [32, 64])
 @pytest.mark.parametrize("rows", [1, 8, 9, 31])
-def test_weakly_coupled_rows_of_a_warp(N, rows):
+def test_weakly_coupled_rows_of_a_warp(N, rows, block):
     """`rows` of every 32 in a group of their own: the single elements and the chains of the fma path."""
     n = 230
     A = groups(n, 1e-12, np.arange(n) % 32 < rows, rows) + 40 * np.eye(n)
-    LU, perm = factor(N, A)
+    LU, perm = factor(N, A, lu_block=block)
     assert np.array_equal(perm, np.arange(n))
     assert excess(A, LU, perm) <= 1
 
